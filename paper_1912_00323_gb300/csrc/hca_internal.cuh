@@ -49,6 +49,8 @@ struct DevCounters {
     uint32_t n_tc_recount;    // chunks of the tensor-core recount of handed-over rows
     uint32_t tc_next_recount;
     uint32_t hd_next[4];      // next unclaimed 32-point chunk: counts, first links, unions, labels
+    uint32_t hd_spill[2];     // windows queued by the CUDA-core chunks: counts, labels
+    uint32_t hd_spill_next[2];  // next unclaimed window of each queue
     uint32_t lowd_next[5];    // next unclaimed batch (labels: [4])
     unsigned long long work[8];  // work counters (see hca_stats)
     unsigned long long tc_pairs;  // point pairs of the tensor-core tiles computed

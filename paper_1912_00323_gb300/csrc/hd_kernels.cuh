@@ -57,7 +57,22 @@ struct HdView {
     // every point of the cell
     T *box_lo;
     T *box_hi;
+    // windows of long candidate streams (k_count_hd, k_labels_hd): the queue (chunk, window |
+    // windows << 16), the windows of a chunk not yet done, and per row the count so far (counts)
+    // or the smallest cluster id so far (labels)
+    uint2 *sp_queue;
+    uint32_t *sp_pending;
+    uint32_t *sp_val;
+    uint32_t sp_cap;
 };
+
+// A chunk scans the first kSpillWin candidates of its stream itself; what is left of a longer
+// stream goes to a queue in windows of that many (at most kSpillMax, then wider ones), which a
+// second launch hands to all warps.  Without it the few chunks of border and noise points next
+// to a large cluster, whose rows scan the whole neighbourhood (20,000 points and more) 32
+// candidates per round of loads, set the time of the pass alone.
+constexpr uint32_t kSpillWin = 1024;
+constexpr uint32_t kSpillMax = 64;
 
 constexpr int kHdWarps = 4;     // warps per block in the point kernels of this path (default)
 constexpr int kHdMaxWarps = 8;  // most warps per block a tuning may choose
@@ -325,12 +340,18 @@ static __global__ void __launch_bounds__(256) k_chunk_counts(const uint32_t *__r
         nch[c] = (cell_start[c + 1] - cell_start[c] + 31u) / 32u;
 }
 
-// Cell of chunk t (upper bound in chunk_off, minus one).  Warp-uniform.
-__device__ __forceinline__ uint32_t chunk_cell(const uint32_t *chunk_off, uint32_t C, uint32_t t) {
-    uint32_t lo = 0, hi = C;
-    while (hi - lo > 1) {
-        const uint32_t mid = (lo + hi) >> 1;
-        if (__ldg(chunk_off + mid) <= t) lo = mid; else hi = mid;
+// Cell of chunk (or work item) t: the last c with off[c] <= t, by a 32-way search (one round of
+// loads per level instead of one per halving).  A full warp calls it; every lane returns the
+// result.
+__device__ __forceinline__ uint32_t chunk_cell(const uint32_t *off, uint32_t C, uint32_t t) {
+    const uint32_t lane = threadIdx.x & 31u;
+    uint32_t lo = 0, hi = C;  // off[lo] <= t, and off[hi] > t unless hi == C
+    while (hi - lo > 1u) {
+        const uint32_t step = (hi - lo + 31u) >> 5;
+        const uint32_t piv = lo + lane * step;
+        const unsigned ok = __ballot_sync(0xffffffffu, piv < hi && __ldg(off + piv) <= t);
+        lo += (uint32_t)(31 - __clz(ok)) * step;  // the ok lanes are a prefix (off is nondecreasing)
+        hi = min(hi, lo + step);
     }
     return lo;
 }
@@ -463,72 +484,155 @@ __global__ void __launch_bounds__(256) k_cell_box_decode(HdView<T, DP> v) {
                           base = (v).cell_start[A] + 32u * (t_ - (v).chunk_off[A]), o2_ = 1; \
                  o2_; o2_ = 0)
 
+// Length of a cell's candidate stream: its neighbour ranges (at most 32; the coarse grid has 9),
+// one per lane, laid end to end.
+template <typename V>
+__device__ __forceinline__ uint32_t stream_length(const V &v, uint2 rg) {
+    return __reduce_add_sync(0xffffffffu, rg.x < rg.y ? v.cell_start[rg.y] - v.cell_start[rg.x] : 0u);
+}
+
+// The cells of the part [p0, p1) of that stream, in order: f(B, q0, q1) for the points
+// [q0, q1) of cell B.  f returns false to stop.  Warp-uniform.
+template <typename V, typename F>
+__device__ __forceinline__ void for_stream_cells(const V &v, uint2 rg, uint32_t p0, uint32_t p1, F f) {
+    uint32_t pos = 0;
+    for (int kk = 0; kk < v.n_all; ++kk) {
+        const uint32_t lo = __shfl_sync(0xffffffffu, rg.x, kk);
+        const uint32_t hi = __shfl_sync(0xffffffffu, rg.y, kk);
+        if (lo >= hi) continue;
+        const uint32_t s0 = v.cell_start[lo], s1 = v.cell_start[hi];
+        if (pos + (s1 - s0) <= p0) {
+            pos += s1 - s0;
+            continue;
+        }
+        uint32_t q0 = s0;
+        for (uint32_t B = lo; B < hi; ++B) {
+            const uint32_t q1 = B + 1 < hi ? v.cell_start[B + 1] : s1;
+            const uint32_t a = pos, b = pos + (q1 - q0);  // stream positions of the cell
+            if (a >= p1) return;
+            if (b > p0 && !f(B, q0 + (p0 > a ? p0 - a : 0u), q1 - (b > p1 ? b - p1 : 0u))) return;
+            pos = b;
+            q0 = q1;
+        }
+    }
+}
+
+// The window of a chunk's remaining stream [start, total) that entry (chunk, w | nw << 16) of the
+// queue stands for.
+__device__ __forceinline__ void spill_window(uint32_t entry, uint32_t start, uint32_t total, uint32_t &p0, uint32_t &p1) {
+    const uint32_t w = entry & 0xffffu, nw = entry >> 16;
+    const uint32_t step = ((total - start + nw - 1u) / nw + 31u) & ~31u;
+    p0 = min(total, start + w * step);
+    p1 = min(total, p0 + step);
+}
+
+// Queue the windows of [start, total) for chunk t; false when the queue is full (the caller then
+// scans on by itself).  sp_val of the chunk's rows is written by the caller beforehand.
+template <typename V>
+__device__ __forceinline__ bool spill_push(const V &v, int slot, uint32_t t, uint32_t start, uint32_t total) {
+    const uint32_t lane = threadIdx.x & 31u;
+    const uint32_t nw = min(kSpillMax, (total - start + kSpillWin - 1u) / kSpillWin);
+    uint32_t at = 0;
+    if (lane == 0) {  // (a full queue's counter is left alone, so it cannot wrap)
+        at = *(volatile uint32_t *)&v.ctr->hd_spill[slot];
+        if (at < v.sp_cap) at = atomicAdd(&v.ctr->hd_spill[slot], nw);
+    }
+    at = __shfl_sync(0xffffffffu, at, 0);
+    const bool fits = at < v.sp_cap && nw <= v.sp_cap - at;
+    for (uint32_t w = lane; w < nw; w += 32)  // a reservation cut off by the end is marked empty
+        if (at < v.sp_cap && w < v.sp_cap - at) v.sp_queue[at + w] = make_uint2(fits ? t : 0xffffffffu, w | nw << 16);
+    if (fits && lane == 0) v.sp_pending[t] = nw;
+    return fits;
+}
+
 // Definition 2: |N_eps(p)| >= MINPTS, counted over the 27 neighbouring coarse cells (the own
 // point included), stopping once every point of the chunk has reached MINPTS.  The chunk's
 // points are staged in shared memory, candidates stream through the lanes, and each open
 // point is compared with a warp ballot.
-template <typename T, int DP>
+//
+// Bound by the latency of its loads: a warp has one round of candidate loads in flight, so the
+// time is the longest item of a warp.  Windows (SPILL = true: the second launch) bring the
+// longest item down to kSpillWin candidates.  Measured (one launch before, both launches now):
+// HCA_MEASURED_COUNT
+template <typename T, int DP, bool SPILL>
 __global__ void __launch_bounds__(32 * kHdMaxWarps) k_count_hd(HdView<T, DP> v) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *rows = reinterpret_cast<T *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
     const int lane = lane_id();
     uint32_t chunks = 0;
-    HD_FOR_EACH_CHUNK(v, A, base, e, 0) {
+    const uint32_t C = v.ctr->n_cells, N = SPILL ? min(v.ctr->hd_spill[0], v.sp_cap) : v.ctr->n_chunks;
+    uint32_t *const next = SPILL ? &v.ctr->hd_spill_next[0] : &v.ctr->hd_next[0];
+    for (uint32_t item = next_chunk(next); item < N; item = next_chunk(next)) {
+        const uint2 entry = SPILL ? v.sp_queue[item] : make_uint2(item, 0u);
+        if (SPILL && entry.x == 0xffffffffu) continue;
+        const uint32_t t = entry.x, A = chunk_cell(v.chunk_off, C, t);
+        const uint32_t e = v.cell_start[A + 1], base = v.cell_start[A] + 32u * (t - v.chunk_off[A]);
+        const uint32_t p = base + lane;
         // a cell counted on the tensor cores leaves here only the rows it handed over (core = 2)
         const bool tc_cell = v.tc_min[0] && e - v.cell_start[A] >= v.tc_min[0];
-        const bool have = base + lane < e && (!tc_cell || v.core[base + lane] == 2);
-        unsigned open = __ballot_sync(0xffffffffu, have);
-        if (!open) continue;
+        const bool have = p < e && (!tc_cell || v.core[p] == 2);
+        const unsigned rows_m = __ballot_sync(0xffffffffu, have);
+        if (!rows_m) continue;
         const GridParams &G = params_of(v, set_of_key(v, v.cell_key[A]));
         const uint32_t min_pts = G.min_pts;
-        stage_rows<T, DP>(rows, v.pts, base, e);
-        uint32_t cnt = 0, skip = 0;
-        if (tc_cell) {  // resume where the tensor-core count stopped (same candidate order)
-            if (have) cnt = v.tc_cnt[base + lane];
-            skip = __shfl_sync(0xffffffffu, have ? v.tc_pos[base + lane] : 0u, __ffs(open) - 1);
+        const uint2 rg = lane < v.n_all ? v.ranges[(uint64_t)A * v.n_all + lane] : make_uint2(0u, 0u);
+        const uint32_t total = stream_length(v, rg);
+        // a row the tensor-core count handed over resumes where it stopped (same candidate order)
+        const uint32_t start = tc_cell ? __shfl_sync(0xffffffffu, have ? v.tc_pos[p] : 0u, __ffs(rows_m) - 1) : 0u;
+        uint32_t cnt = 0, p0 = start, p1 = start + min(kSpillWin, total - start);
+        if (SPILL) {
+            if (have) cnt = __ldcg(v.sp_val + p);
+            spill_window(entry.y, p1, total, p0, p1);
+        } else if (tc_cell && have) {
+            cnt = v.tc_cnt[p];
         }
-        for (int g0 = 0; g0 < v.n_all && open; g0 += 32) {
-            const int k = g0 + lane;
-            const uint2 rg = k < v.n_all ? v.ranges[(uint64_t)A * v.n_all + k] : make_uint2(0u, 0u);
-            // the cells of a pencil range, one at a time: a cell whose box is farther than eps
-            // from every open row adds nothing to their counts and is passed over
-            for (int kk = 0; kk < 32 && open; ++kk) {
-                const uint32_t lo = __shfl_sync(0xffffffffu, rg.x, kk);
-                const uint32_t hi = __shfl_sync(0xffffffffu, rg.y, kk);
-                for (uint32_t B = lo; B < hi && open; ++B) {
-                    uint32_t q0 = v.cell_start[B];
-                    const uint32_t q1 = v.cell_start[B + 1];
-                    if (skip) {  // positions count every point of the stream (the tensor-core order)
-                        if (skip >= q1 - q0) {
-                            skip -= q1 - q0;
-                            continue;
-                        }
-                        q0 += skip;
-                        skip = 0;
-                    }
-                    const unsigned near = open & __ballot_sync(0xffffffffu,
-                        !box_far<DP>(rows + lane * DP, v.box_lo + (uint64_t)B * DP, v.box_hi + (uint64_t)B * DP, G));
-                    if (!near) continue;
-                    for (uint32_t qb = q0; qb < q1 && open; qb += 32) {
-                        const uint32_t q = qb + lane;
-                        T qv[DP];
-                        hd_load<T, DP>(v.pts, q, q < q1, qv);
-                        ++chunks;
-                        unsigned rem = open & near;
-                        while (rem) {
-                            const int jj = __ffs(rem) - 1;
-                            rem &= rem - 1;
-                            const unsigned hits = __ballot_sync(0xffffffffu, q < q1 && hd_within<DP>(rows + jj * DP, qv, G));
-                            if (lane == jj) cnt += __popc(hits);
-                        }
-                        open &= __ballot_sync(0xffffffffu, have && cnt < min_pts);
-                    }
+        const uint32_t cnt0 = cnt;
+        unsigned open = __ballot_sync(0xffffffffu, have && (!SPILL || cnt < min_pts));
+        if (open) stage_rows<T, DP>(rows, v.pts, base, e);
+        // one cell at a time: a cell whose box is farther than eps from every open row adds
+        // nothing to their counts and is passed over
+        auto scan = [&](uint32_t B, uint32_t q0, uint32_t q1) -> bool {
+            const unsigned near = open & __ballot_sync(0xffffffffu,
+                !box_far<DP>(rows + lane * DP, v.box_lo + (uint64_t)B * DP, v.box_hi + (uint64_t)B * DP, G));
+            if (!near) return true;
+            for (uint32_t qb = q0; qb < q1 && open; qb += 32) {
+                const uint32_t q = qb + lane;
+                T qv[DP];
+                hd_load<T, DP>(v.pts, q, q < q1, qv);
+                ++chunks;
+                unsigned rem = open & near;
+                while (rem) {
+                    const int jj = __ffs(rem) - 1;
+                    rem &= rem - 1;
+                    const unsigned hits = __ballot_sync(0xffffffffu, q < q1 && hd_within<DP>(rows + jj * DP, qv, G));
+                    if (lane == jj) cnt += __popc(hits);
                 }
+                open &= __ballot_sync(0xffffffffu, have && cnt < min_pts);
             }
+            return open != 0;
+        };
+        if (open) for_stream_cells(v, rg, p0, p1, scan);
+        bool decide = true;
+        if (SPILL) {
+            // the last window of the chunk decides its rows from the summed counts
+            if (have && cnt != cnt0) atomicAdd(v.sp_val + p, cnt - cnt0);
+            __threadfence();
+            __syncwarp();
+            uint32_t left = 0;
+            if (lane == 0) left = atomicSub(v.sp_pending + t, 1u);
+            decide = __shfl_sync(0xffffffffu, left, 0) == 1u;
+            __threadfence();
+            if (decide && have) cnt = __ldcg(v.sp_val + p);
+        } else if (open && p1 < total) {
+            if (have) v.sp_val[p] = cnt;
+            decide = !spill_push(v, 0, t, p1, total);
+            if (decide) for_stream_cells(v, rg, p1, total, scan);
         }
-        const bool is_core = have && cnt >= min_pts;
-        if (have) v.core[base + lane] = is_core ? 1 : 0;
-        if (__any_sync(0xffffffffu, is_core) && lane == 0) v.cell_core[A] = 1;
+        if (decide) {
+            const bool is_core = have && cnt >= min_pts;
+            if (have) v.core[p] = is_core ? 1 : 0;
+            if (__any_sync(0xffffffffu, is_core) && lane == 0) v.cell_core[A] = 1;
+        }
         __syncwarp();
     }
     add_counter(&v.ctr->work[0], lane == 0 ? chunks : 0u);
@@ -726,74 +830,89 @@ __global__ void __launch_bounds__(256) k_comp_min_hd(HdView<T, DP> v) {
 }
 
 // Algorithm 4 / Definition 5 with the canonical rule, over points: core points take their
-// cluster id, a non-core point the smallest id among its core neighbours, else -1.
-template <typename T, int DP>
+// cluster id, a non-core point the smallest id among its core neighbours, else -1.  Long
+// streams are split into windows as in k_count_hd (SPILL = true: the second launch).
+template <typename T, int DP, bool SPILL>
 __global__ void __launch_bounds__(32 * kHdMaxWarps) k_labels_hd(HdView<T, DP> v) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *rows = reinterpret_cast<T *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
     const int lane = lane_id();
     uint32_t noise = 0, chunks = 0;
-    HD_FOR_EACH_CHUNK(v, A, base, e, 3) {
-        if (v.tc_min[2]) {  // non-core rows of a tensor-core cell: labelled there
-            const uint32_t s0 = v.cell_start[A];
-            if (e - s0 - (v.cx[e] - v.cx[s0]) >= v.tc_min[2]) continue;
-        }
-        {
-            const uint32_t aset = set_of_key(v, v.cell_key[A]);
-            const GridParams &G = params_of(v, aset);
-            const uint32_t base_label = v.gtab ? (uint32_t)v.set_off[aset] : 0u;
-            const uint32_t p = base + lane;
-            const bool have = p < e;
-            const bool isc = have && v.core[p];
-            uint32_t best = isc ? v.comp_min[v.parent[p]] : kNoLabel;
-            const unsigned smask = __ballot_sync(0xffffffffu, have && !isc);
-            if (smask) {
-                stage_rows<T, DP>(rows, v.pts, base, e);
-                for (int g0 = 0; g0 < v.n_all; g0 += 32) {
-                    const int k = g0 + lane;
-                    const uint2 rg = k < v.n_all ? v.ranges[(uint64_t)A * v.n_all + k] : make_uint2(0u, 0u);
-                    for (int kk = 0; kk < 32; ++kk) {
-                        const uint32_t lo = __shfl_sync(0xffffffffu, rg.x, kk);
-                        const uint32_t hi = __shfl_sync(0xffffffffu, rg.y, kk);
-                        for (uint32_t B = lo; B < hi; ++B) {
-                            // a cell whose box is farther than eps from every row is passed over
-                            const unsigned near = smask & __ballot_sync(0xffffffffu,
-                                !box_far<DP>(rows + lane * DP, v.box_lo + (uint64_t)B * DP,
-                                             v.box_hi + (uint64_t)B * DP, G));
-                            if (!near) continue;
-                            const uint32_t q0 = v.cell_start[B], q1 = v.cell_start[B + 1];
-                            for (uint32_t qb = q0; qb < q1; qb += 32) {
-                                const uint32_t q = qb + lane;
-                                const bool qc = q < q1 && v.core[q];
-                                if (!__any_sync(0xffffffffu, qc)) continue;
-                                const uint32_t lq = qc ? v.comp_min[v.parent[q]] : kNoLabel;
-                                T qv[DP];
-                                hd_load<T, DP>(v.pts, q, qc, qv);
-                                ++chunks;
-                                unsigned rem = near;
-                                while (rem) {
-                                    const int jj = __ffs(rem) - 1;
-                                    rem &= rem - 1;
-                                    const uint32_t bj = __shfl_sync(0xffffffffu, best, jj);
-                                    const bool need = qc && lq < bj;
-                                    if (!__any_sync(0xffffffffu, need)) continue;
-                                    uint32_t cand = (need && hd_within<DP>(rows + jj * DP, qv, G)) ? lq : kNoLabel;
-                                    cand = __reduce_min_sync(0xffffffffu, cand);
-                                    if (lane == jj && cand < best) best = cand;
-                                }
-                            }
-                        }
+    const uint32_t C = v.ctr->n_cells, N = SPILL ? min(v.ctr->hd_spill[1], v.sp_cap) : v.ctr->n_chunks;
+    uint32_t *const next = SPILL ? &v.ctr->hd_spill_next[1] : &v.ctr->hd_next[3];
+    for (uint32_t item = next_chunk(next); item < N; item = next_chunk(next)) {
+        const uint2 entry = SPILL ? v.sp_queue[item] : make_uint2(item, 0u);
+        if (SPILL && entry.x == 0xffffffffu) continue;
+        const uint32_t t = entry.x, A = chunk_cell(v.chunk_off, C, t);
+        const uint32_t s0 = v.cell_start[A], e = v.cell_start[A + 1], base = s0 + 32u * (t - v.chunk_off[A]);
+        if (v.tc_min[2] && e - s0 - (v.cx[e] - v.cx[s0]) >= v.tc_min[2])
+            continue;  // non-core rows of a tensor-core cell: labelled there
+        const uint32_t aset = set_of_key(v, v.cell_key[A]);
+        const GridParams &G = params_of(v, aset);
+        const uint32_t base_label = v.gtab ? (uint32_t)v.set_off[aset] : 0u;
+        const uint32_t p = base + lane;
+        const bool have = p < e;
+        const bool isc = have && v.core[p];
+        uint32_t best = isc ? v.comp_min[v.parent[p]] : SPILL && have ? __ldcg(v.sp_val + p) : kNoLabel;
+        const unsigned smask = __ballot_sync(0xffffffffu, have && !isc);
+        bool decide = true;
+        if (smask) {
+            const uint2 rg = lane < v.n_all ? v.ranges[(uint64_t)A * v.n_all + lane] : make_uint2(0u, 0u);
+            const uint32_t total = stream_length(v, rg);
+            uint32_t p0 = 0, p1 = min(kSpillWin, total);
+            if (SPILL) spill_window(entry.y, p1, total, p0, p1);
+            stage_rows<T, DP>(rows, v.pts, base, e);
+            auto scan = [&](uint32_t B, uint32_t q0, uint32_t q1) -> bool {
+                // a cell whose box is farther than eps from every row is passed over
+                const unsigned near = smask & __ballot_sync(0xffffffffu,
+                    !box_far<DP>(rows + lane * DP, v.box_lo + (uint64_t)B * DP, v.box_hi + (uint64_t)B * DP, G));
+                if (!near) return true;
+                for (uint32_t qb = q0; qb < q1; qb += 32) {
+                    const uint32_t q = qb + lane;
+                    const bool qc = q < q1 && v.core[q];
+                    if (!__any_sync(0xffffffffu, qc)) continue;
+                    const uint32_t lq = qc ? v.comp_min[v.parent[q]] : kNoLabel;
+                    T qv[DP];
+                    hd_load<T, DP>(v.pts, q, qc, qv);
+                    ++chunks;
+                    unsigned rem = near;
+                    while (rem) {
+                        const int jj = __ffs(rem) - 1;
+                        rem &= rem - 1;
+                        const uint32_t bj = __shfl_sync(0xffffffffu, best, jj);
+                        const bool need = qc && lq < bj;
+                        if (!__any_sync(0xffffffffu, need)) continue;
+                        uint32_t cand = (need && hd_within<DP>(rows + jj * DP, qv, G)) ? lq : kNoLabel;
+                        cand = __reduce_min_sync(0xffffffffu, cand);
+                        if (lane == jj && cand < best) best = cand;
                     }
                 }
+                return true;
+            };
+            for_stream_cells(v, rg, p0, p1, scan);
+            if (SPILL) {
+                // the last window of the chunk writes its labels from the smallest ids
+                if (have && !isc) atomicMin(v.sp_val + p, best);
+                __threadfence();
                 __syncwarp();
+                uint32_t left = 0;
+                if (lane == 0) left = atomicSub(v.sp_pending + t, 1u);
+                decide = __shfl_sync(0xffffffffu, left, 0) == 1u;
+                __threadfence();
+                if (decide && have && !isc) best = __ldcg(v.sp_val + p);
+            } else if (p1 < total) {
+                if (have) v.sp_val[p] = best;
+                decide = !spill_push(v, 1, t, p1, total);
+                if (decide) for_stream_cells(v, rg, p1, total, scan);
             }
-            if (have) {
-                const int32_t lab = best == kNoLabel ? -1 : (int32_t)(best - base_label);
-                const uint32_t o = v.perm[p];
-                v.labels[o] = lab;
-                if (v.core_out) v.core_out[o] = isc ? 1 : 0;
-                noise += lab < 0;
-            }
+            __syncwarp();
+        }
+        if (decide && have) {
+            const int32_t lab = best == kNoLabel ? -1 : (int32_t)(best - base_label);
+            const uint32_t o = v.perm[p];
+            v.labels[o] = lab;
+            if (v.core_out) v.core_out[o] = isc ? 1 : 0;
+            noise += lab < 0;
         }
     }
     noise = __reduce_add_sync(0xffffffffu, noise);

@@ -177,8 +177,9 @@ void run_tc_phases(HdView<float, DP> &hv, cudaStream_t s, char *b, int64_t n, in
     tc::k_tc_hd<DP, tc::kCount><<<grid_tc, tc::kTile, tc_smem, s>>>(
         hv, tc::Tables{ch1, cx, nullptr, nullptr, nullptr, nullptr, nullptr, clist, nch, ch0, nclist});
     tmark(1);
-    k_count_hd<float, DP><<<gcell, hd_block, smem, s>>>(hv);
-    launches += 7;
+    k_count_hd<float, DP, false><<<gcell, hd_block, smem, s>>>(hv);
+    k_count_hd<float, DP, true><<<gcell, hd_block, smem, s>>>(hv);
+    launches += 8;
     mark(6);
     // core numbering, core and non-core lists, chunk tables of the unions and the labels
     tc::k_tc_core_flags<<<gpts, 256, 0, s>>>(hv.core, n, flags);
@@ -221,7 +222,11 @@ void run_tc_phases(HdView<float, DP> &hv, cudaStream_t s, char *b, int64_t n, in
     const detail::SideStream ss = detail::side_stream();
     const bool fork = ss.ok && cudaEventRecord(ss.fork, s) == cudaSuccess &&
                       cudaStreamWaitEvent(ss.s, ss.fork, 0) == cudaSuccess;
-    if (fork) k_labels_hd<float, DP><<<gcell, hd_block, smem, ss.s>>>(hv);
+    auto cuda_labels = [&](cudaStream_t ls) {
+        k_labels_hd<float, DP, false><<<gcell, hd_block, smem, ls>>>(hv);
+        k_labels_hd<float, DP, true><<<gcell, hd_block, smem, ls>>>(hv);
+    };
+    if (fork) cuda_labels(ss.s);
     tc::k_tc_core_labels<DP><<<gpts, 256, 0, s>>>(hv, tc::Tables{ch2, cx, clist, nclist, clab, nullptr}, nsets, clab);
     tmark(4);
     tc::k_tc_hd<DP, tc::kLabels><<<grid_tc, tc::kTile, tc_smem, s>>>(hv, tc::Tables{ch2, cx, clist, nclist, clab, nullptr});
@@ -230,9 +235,9 @@ void run_tc_phases(HdView<float, DP> &hv, cudaStream_t s, char *b, int64_t n, in
         cudaEventRecord(ss.join, ss.s);
         cudaStreamWaitEvent(s, ss.join, 0);
     } else {
-        k_labels_hd<float, DP><<<gcell, hd_block, smem, s>>>(hv);
+        cuda_labels(s);
     }
-    launches += 4;
+    launches += 5;
     mark(9);
 }
 
@@ -573,15 +578,23 @@ int run_hd(const RunArgs &a) {
     hv.n_half = st.n_half;
     hv.box_lo = (T *)(b + o_blo);
     hv.box_hi = (T *)(b + o_bhi);
+    // the windows' queue and per-row values take the sort's key buffers, free once the cells are
+    // known; one word per chunk (at most n) from the pencil flags, free once the pencils are
+    hv.sp_queue = (uint2 *)(b + o_ka);
+    hv.sp_cap = (uint32_t)n;
+    hv.sp_val = (uint32_t *)(b + o_kb);
+    hv.sp_pending = (uint32_t *)(b + o_pflags);
     // the box of every coarse cell in all d dimensions (point-to-box distance bounds)
     k_cell_box_clear<T, DP><<<grid_for((int64_t)n * DP, 256, sms, 8), 256, 0, s>>>(hv);
     k_cell_box_hd<T, DP><<<grid_for(n / 32 + 1, 8, sms, 16), 256, 0, s>>>(hv);
     k_cell_box_decode<T, DP><<<grid_for((int64_t)n * DP, 256, sms, 8), 256, 0, s>>>(hv);
     launches += 3;
-    allow_smem(k_count_hd<T, DP>, smem);
+    allow_smem(k_count_hd<T, DP, false>, smem);
+    allow_smem(k_count_hd<T, DP, true>, smem);
     allow_smem(k_hook_hd<T, DP>, smem);
     allow_smem(k_merge_hd<T, DP>, smem);
-    allow_smem(k_labels_hd<T, DP>, smem);
+    allow_smem(k_labels_hd<T, DP, false>, smem);
+    allow_smem(k_labels_hd<T, DP, true>, smem);
     if constexpr (std::is_same<T, float>::value) {
         if (use_tc && st.n_all <= tc::kMaxRng) {
             run_tc_phases<DP>(hv, s, b, n, sms * tc_occ, tc_smem, gpts, gcell, hd_block, smem, part_of(b, o_part),
@@ -598,8 +611,9 @@ int run_hd(const RunArgs &a) {
     if (!tc_phases) {
         // ---- Definition 2: exact counts over the neighbouring coarse cells ----
         cudaMemsetAsync(hv.cell_core, 0, (size_t)n, s);
-        k_count_hd<T, DP><<<gcell, hd_block, smem, s>>>(hv);
-        ++launches;
+        k_count_hd<T, DP, false><<<gcell, hd_block, smem, s>>>(hv);
+        k_count_hd<T, DP, true><<<gcell, hd_block, smem, s>>>(hv);
+        launches += 2;
         mark(6);
         // (no representative points in this path: every pair of core points is a candidate)
         mark(7);
@@ -613,8 +627,9 @@ int run_hd(const RunArgs &a) {
         mark(8);
         // ---- Algorithm 4: canonical ids, border and noise points ----
         k_comp_min_hd<T, DP><<<gpts, 256, 0, s>>>(hv);
-        k_labels_hd<T, DP><<<gcell, hd_block, smem, s>>>(hv);
-        launches += 2;
+        k_labels_hd<T, DP, false><<<gcell, hd_block, smem, s>>>(hv);
+        k_labels_hd<T, DP, true><<<gcell, hd_block, smem, s>>>(hv);
+        launches += 3;
         mark(9);
     }
     if (cudaGetLastError() != cudaSuccess) { rc = HCA_ECUDA; goto out; }

@@ -78,21 +78,6 @@ __device__ __forceinline__ uint32_t merge_windows(uint32_t len) {
     return len > kSegCand ? (len + kSegCand - 1u) / kSegCand : 1u;
 }
 
-// Cell of work item t: the last c with off[c] <= t, by a 32-way search (one round of loads per
-// level instead of one per halving).  A full warp calls it; every lane returns the result.
-__device__ __forceinline__ uint32_t chunk_cell_warp(const uint32_t *off, uint32_t C, uint32_t t) {
-    const uint32_t lane = threadIdx.x & 31u;
-    uint32_t lo = 0, hi = C;  // off[lo] <= t, and off[hi] > t unless hi == C
-    while (hi - lo > 1u) {
-        const uint32_t step = (hi - lo + 31u) >> 5;
-        const uint32_t piv = lo + lane * step;
-        const unsigned ok = __ballot_sync(0xffffffffu, piv < hi && __ldg(off + piv) <= t);
-        lo += (uint32_t)(31 - __clz(ok)) * step;  // the ok lanes are a prefix (off is nondecreasing)
-        hi = min(hi, lo + step);
-    }
-    return lo;
-}
-
 // Row and candidate lists of the three phases.
 struct Tables {
     const uint32_t *choff;      // first work item of every coarse cell (this launch)
@@ -443,7 +428,7 @@ __global__ void __launch_bounds__(kTile) k_tc_hd(HdView<float, DP> v, Tables tt)
             uint32_t A = 0, nwin = 1;
             if (t < NC) {
                 const bool later = MODE == kMerge && t >= N0;
-                A = later ? chunk_cell_warp(tt.choff_later, C, t - N0) : chunk_cell_warp(tt.choff, C, t);
+                A = later ? chunk_cell(tt.choff_later, C, t - N0) : chunk_cell(tt.choff, C, t);
                 if (later) {
                     uint32_t len = tid < n_rng ? merge_range_len(v.ranges, v.n_all, v.cell_start, tt.cx, A, tid) : 0u;
                     nwin = merge_windows(__reduce_add_sync(0xffffffffu, len));
