@@ -48,9 +48,9 @@ struct DevCounters {
     uint32_t tc_next[3];      // next unclaimed item of each tensor-core phase
     uint32_t n_tc_recount;    // chunks of the tensor-core recount of handed-over rows
     uint32_t tc_next_recount;
-    uint32_t hd_next[4];      // next unclaimed 32-point chunk: counts, first links, unions, labels
-    uint32_t hd_spill[2];     // windows queued by the CUDA-core chunks: counts, labels
-    uint32_t hd_spill_next[2];  // next unclaimed window of each queue
+    uint32_t hd_next[4];      // next unclaimed 32-point chunk: counts, odd rows, unions, labels
+    uint32_t hd_spill[3];     // windows queued by the CUDA-core chunks: counts, labels, odd rows
+    uint32_t hd_spill_next[3];  // next unclaimed window of each queue
     uint32_t lowd_next[5];    // next unclaimed batch (labels: [4])
     unsigned long long work[8];  // work counters (see hca_stats)
     unsigned long long tc_pairs;  // point pairs of the tensor-core tiles computed
@@ -195,6 +195,7 @@ struct RunArgs {
     DevCounters *h_ext = nullptr;        // pinned host copy of the counters (nullptr: the thread's)
     void *h_stage = nullptr;             // pinned staging of the batched tables (deferred calls)
     bool deferred = false;               // no host synchronisation: the caller checks the status
+    bool no_lists = false;               // coarse grid: run without neighbour lists (no memory for them)
     // optional outputs: the measured extents of a single-set call without declared extents
     // (host, 2 d values: d minima then d maxima), and the launch count and key bits of the call
     double *ext_out = nullptr;

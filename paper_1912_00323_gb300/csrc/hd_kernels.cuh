@@ -12,6 +12,19 @@
 // clustering itself then works on points: exact counts with early exit at MINPTS
 // (Definition 2), union-find over core points (Definitions 3-5) and the canonical labels.
 //
+// Neighbour lists.  The counts write down the first nl_k neighbours that they find of every
+// point, and the later phases start from those instead of comparing points again:
+//   - a non-core point has fewer than MINPTS neighbours, so with nl_k >= MINPTS - 1 its list is
+//     complete and its label is the smallest cluster id among the listed core points;
+//   - the listed core neighbours of a core point are edges of the core graph: joined first, they
+//     leave one tree per cluster and cell but for a few odd points, so that the unions only
+//     compare the odd points with their neighbourhood and the cells whose trees still differ.
+//
+// Double input.  With the filter on (FILTER = true) the pair tests of double input run on a float
+// copy of the points, taken relative to the set's smallest coordinates, against thresholds that
+// bound the copy's rounding (make_coarse_grid); the pairs between the thresholds are decided by
+// the exact predicate on the double coordinates.
+//
 // Layout: pts[j * DP + i] (cell order, zero padded), perm[j], cell_start/cell_key/ranges of
 // the coarse cells, core[j], parent[j] and comp_min[j] over points.
 #pragma once
@@ -29,7 +42,9 @@ struct HdView {
     const int64_t *set_off;       // batched calls: first point of every set
     int d;
     const T *pts;                 // sorted, n x DP
+    const float *fpts;            // float rows of the filter: pts itself, or the copy of double input
     const uint32_t *perm;
+    const uint32_t *cell_of;      // coarse cell of every sorted point
     const uint32_t *cell_start;
     const uint32_t *chunk_off;    // first 32-point chunk of each coarse cell
     const uint64_t *cell_key;
@@ -53,8 +68,8 @@ struct HdView {
     uint32_t *tc_cnt;
     uint32_t *tc_pos;
     // per coarse cell, the smallest and largest coordinate of its points in every dimension
-    // (DP values each): a point farther than eps from a cell's box is farther than eps from
-    // every point of the cell
+    // (DP values each, of the type of the rows that the pair tests read): a point farther than
+    // eps from a cell's box is farther than eps from every point of the cell
     T *box_lo;
     T *box_hi;
     // windows of long candidate streams (k_count_hd, k_labels_hd): the queue (chunk, window |
@@ -64,7 +79,34 @@ struct HdView {
     uint32_t *sp_pending;
     uint32_t *sp_val;
     uint32_t sp_cap;
+    // neighbour lists: entry i < min(nl_cnt[p], nl_k) of point p at nl[p * nl_k + i] is a point
+    // within eps of p, or with kListNear set one that only the exact predicate can tell; nl_cnt
+    // counts all that were found (nl_k = 0: no lists)
+    uint32_t *nl;
+    uint32_t *nl_cnt;
+    uint32_t nl_k;
+    // after the lists are joined: the tree of most of a cell's core points (kNoRoot: no core
+    // point; kMixedRoot: too mixed for one), the core points of other trees per cell, and which
+    // points of every 32-point chunk they are
+    uint32_t *cell_root;
+    uint32_t *odd_cnt;
+    uint32_t *odd_mask;
 };
+
+constexpr uint32_t kNoRoot = 0xffffffffu, kMixedRoot = 0xfffffffeu;
+constexpr uint32_t kListNear = 0x80000000u;
+// Most list entries: MINPTS up to kListMax + 1 has its labels from the lists.  80 bytes a point
+// cover the MINPTS of up to 20 that the workloads use.
+constexpr uint32_t kListMax = 20;
+
+// List entries per point for the largest MINPTS of a call: MINPTS - 1 (a non-core point has no
+// more neighbours), at least 8 (with only the three or four of a small MINPTS the joined lists
+// leave many small trees), a multiple of 4 (16-byte loads).
+inline uint32_t list_len(uint32_t min_pts) {
+    uint32_t k = min_pts > 1 ? min_pts - 1 : 1;
+    k = k < 8 ? 8 : k > kListMax ? kListMax : k;
+    return (k + 3u) & ~3u;
+}
 
 // A chunk scans the first kSpillWin candidates of its stream itself; what is left of a longer
 // stream goes to a queue in windows of that many (at most kSpillMax, then wider ones), which a
@@ -165,6 +207,90 @@ __device__ __forceinline__ void hd_load(const T *pts, uint32_t j, bool valid, T 
             q[2 * i] = v2.x; q[2 * i + 1] = v2.y;
         }
     }
+}
+
+// The exact predicate on two sorted rows in global memory.
+template <typename T, int DP>
+__device__ __noinline__ bool hd_exact(const T *pts, uint32_t i, uint32_t j, double eps2) {
+    const T *a = pts + (uint64_t)i * DP, *b = pts + (uint64_t)j * DP;
+    double e = 0.0;
+#pragma unroll 4
+    for (int k = 0; k < DP; ++k) {
+        const double t = __dsub_rn((double)__ldg(a + k), (double)__ldg(b + k));
+        e = __dadd_rn(e, __dmul_rn(t, t));
+    }
+    return e <= eps2;
+}
+
+// One candidate point in registers against rows in shared memory.  FILTER: float coordinates in
+// pairs (packed two-way FP32 subtract and multiply-add, half the instructions of the scalar
+// form; the sum of squares of even and odd dimensions, within (DP + 2) 2^-24 of exact in any
+// order), only the 4-coordinate groups that hold one of the d dimensions; else the exact
+// predicate of the input type.
+template <typename T, int DP, bool FILTER>
+struct Candidate;
+
+template <typename T, int DP>
+struct Candidate<T, DP, true> {
+    typedef float Row;
+    unsigned long long q[DP / 2];
+    uint32_t idx;
+    static __device__ __forceinline__ const float *src(const HdView<T, DP> &v) { return v.fpts; }
+    __device__ __forceinline__ void load(const HdView<T, DP> &v, uint32_t j, bool valid) {
+        idx = j;
+        const ulonglong2 *p = reinterpret_cast<const ulonglong2 *>(v.fpts + (uint64_t)(valid ? j : 0u) * DP);
+#pragma unroll
+        for (int i = 0; i < DP / 4; ++i) {
+            if (4 * i >= v.d) break;
+            const ulonglong2 x = __ldg(p + i);
+            q[2 * i] = x.x;
+            q[2 * i + 1] = x.y;
+        }
+    }
+    __device__ __forceinline__ bool within(const HdView<T, DP> &v, const float *row, uint32_t ri, const GridParams &g) const {
+        unsigned long long s2 = 0ull;
+        const ulonglong2 *a = reinterpret_cast<const ulonglong2 *>(row);
+#pragma unroll
+        for (int i = 0; i < DP / 4; ++i) {
+            if (4 * i >= v.d) break;
+            const ulonglong2 x = a[i];
+            unsigned long long t;
+            asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(x.x), "l"(q[2 * i]));
+            asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(s2) : "l"(t));
+            asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(t) : "l"(x.y), "l"(q[2 * i + 1]));
+            asm("fma.rn.f32x2 %0, %1, %1, %0;" : "+l"(s2) : "l"(t));
+        }
+        const float s = __uint_as_float((uint32_t)s2) + __uint_as_float((uint32_t)(s2 >> 32));
+        if (s > g.hi32) return false;
+        if (s < g.lo32) return true;
+        return hd_exact<T, DP>(v.pts, ri, idx, g.eps2);
+    }
+};
+
+template <typename T, int DP>
+struct Candidate<T, DP, false> {
+    typedef T Row;
+    T q[DP];
+    static __device__ __forceinline__ const T *src(const HdView<T, DP> &v) { return v.pts; }
+    __device__ __forceinline__ void load(const HdView<T, DP> &v, uint32_t j, bool valid) {
+        hd_load<T, DP>(v.pts, j, valid, q);
+    }
+    __device__ __forceinline__ bool within(const HdView<T, DP> &, const T *row, uint32_t, const GridParams &g) const {
+        return hd_within<DP>(row, q, g);
+    }
+};
+
+// The boxes that go with those rows.
+template <bool FILTER, int DP>
+__device__ __forceinline__ bool cell_far(const HdView<float, DP> &v, const float *row, uint32_t B, const GridParams &g) {
+    return box_far<DP>(row, v.box_lo + (uint64_t)B * DP, v.box_hi + (uint64_t)B * DP, g);
+}
+template <bool FILTER, int DP>
+__device__ __forceinline__ bool cell_far(const HdView<double, DP> &v, const typename Candidate<double, DP, FILTER>::Row *row,
+                                         uint32_t B, const GridParams &g) {
+    typedef typename Candidate<double, DP, FILTER>::Row R;
+    const R *lo = reinterpret_cast<const R *>(v.box_lo), *hi = reinterpret_cast<const R *>(v.box_hi);
+    return box_far<DP>(row, lo + (uint64_t)B * DP, hi + (uint64_t)B * DP, g);
 }
 
 // Declared extents of a plan against the measured ones (encoded min of dimension i of set s at
@@ -277,7 +403,10 @@ template <typename T, int DP, typename K>
 __global__ void __launch_bounds__(256) k_gather_hd(const T *__restrict__ in, int d, const K *__restrict__ keys,
                                                   const uint32_t *__restrict__ idx, int64_t n,
                                                   T *__restrict__ pts, uint32_t *__restrict__ flags,
-                                                  uint32_t *__restrict__ tile_sums) {
+                                                  uint32_t *__restrict__ tile_sums, float *__restrict__ fpts,
+                                                  const unsigned long long *__restrict__ mm, int set_shift) {
+    // fpts (double input with the filter on): the float copy of the rows, relative to the set's
+    // smallest coordinates (set id above set_shift of the key; encodings at mm[set * 64 + i])
     constexpr int G = DP / 4;          // threads per row
     constexpr int R = 256 / G;         // rows per step of the block
     const int g = threadIdx.x % G, r0 = threadIdx.x / G;
@@ -298,6 +427,14 @@ __global__ void __launch_bounds__(256) k_gather_hd(const T *__restrict__ in, int
             } else {
                 reinterpret_cast<double2 *>(dst)[0] = make_double2((double)x[0], (double)x[1]);
                 reinterpret_cast<double2 *>(dst)[1] = make_double2((double)x[2], (double)x[3]);
+                if (fpts) {
+                    const uint64_t set = set_shift < 64 ? (uint64_t)keys[j] >> set_shift : 0ull;
+                    float f[4];
+#pragma unroll
+                    for (int u = 0; u < 4; ++u)
+                        f[u] = 4 * g + u < d ? (float)__dsub_rn((double)x[u], dec_double_dev(__ldg(mm + set * 64 + 4 * g + u))) : 0.f;
+                    *reinterpret_cast<float4 *>(fpts + j * DP + 4 * g) = make_float4(f[0], f[1], f[2], f[3]);
+                }
             }
             if (g == 0) {
                 const uint32_t f = (j == 0 || keys[j] != keys[j - 1]) ? 1u : 0u;
@@ -400,9 +537,9 @@ struct BoxCode {
     }
 };
 
-template <typename T, int DP>
+template <typename T, int DP, typename R>
 __global__ void __launch_bounds__(256) k_cell_box_clear(HdView<T, DP> v) {
-    typedef typename BoxCode<T>::U U;
+    typedef typename BoxCode<R>::U U;
     const uint64_t m = (uint64_t)v.ctr->n_cells * DP;
     U *lo = reinterpret_cast<U *>(v.box_lo), *hi = reinterpret_cast<U *>(v.box_hi);
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
@@ -411,15 +548,16 @@ __global__ void __launch_bounds__(256) k_cell_box_clear(HdView<T, DP> v) {
     }
 }
 
-template <typename T, int DP>
+template <typename T, int DP, typename R>
 __global__ void __launch_bounds__(256) k_cell_box_hd(HdView<T, DP> v) {
-    typedef BoxCode<T> BC;
+    typedef BoxCode<R> BC;
     typedef typename BC::U U;
     constexpr int E = DP > 32 ? DP / 32 : 1;  // dimensions per lane in the atomics
     const int lane = lane_id();
     const uint32_t C = v.ctr->n_cells, NC = v.ctr->n_chunks;
     const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
     U *lo = reinterpret_cast<U *>(v.box_lo), *hi = reinterpret_cast<U *>(v.box_hi);
+    const R *pts = sizeof(R) == sizeof(T) ? reinterpret_cast<const R *>(v.pts) : reinterpret_cast<const R *>(v.fpts);
     for (uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < NC; t += warps) {
         const uint32_t A = chunk_cell(v.chunk_off, C, t);
         const uint32_t e = v.cell_start[A + 1], base = v.cell_start[A] + 32u * (t - v.chunk_off[A]);
@@ -433,14 +571,14 @@ __global__ void __launch_bounds__(256) k_cell_box_hd(HdView<T, DP> v) {
         }
 #pragma unroll
         for (int g0 = 0; g0 < DP; g0 += 4) {
-            T x[4];
-            if (sizeof(T) == 4) {
-                const float4 f = valid ? __ldg(reinterpret_cast<const float4 *>(v.pts + (uint64_t)p * DP + g0))
+            R x[4];
+            if (sizeof(R) == 4) {
+                const float4 f = valid ? __ldg(reinterpret_cast<const float4 *>(pts + (uint64_t)p * DP + g0))
                                        : make_float4(0.f, 0.f, 0.f, 0.f);
-                x[0] = (T)f.x; x[1] = (T)f.y; x[2] = (T)f.z; x[3] = (T)f.w;
+                x[0] = (R)f.x; x[1] = (R)f.y; x[2] = (R)f.z; x[3] = (R)f.w;
             } else {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) x[i] = valid ? __ldg(v.pts + (uint64_t)p * DP + g0 + i) : (T)0;
+                for (int i = 0; i < 4; ++i) x[i] = valid ? __ldg(pts + (uint64_t)p * DP + g0 + i) : (R)0;
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -463,15 +601,15 @@ __global__ void __launch_bounds__(256) k_cell_box_hd(HdView<T, DP> v) {
     }
 }
 
-template <typename T, int DP>
+template <typename T, int DP, typename R>
 __global__ void __launch_bounds__(256) k_cell_box_decode(HdView<T, DP> v) {
-    typedef BoxCode<T> BC;
+    typedef BoxCode<R> BC;
     typedef typename BC::U U;
     const uint64_t m = (uint64_t)v.ctr->n_cells * DP;
     U *lo = reinterpret_cast<U *>(v.box_lo), *hi = reinterpret_cast<U *>(v.box_hi);
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
-        v.box_lo[i] = BC::dec(lo[i]);
-        v.box_hi[i] = BC::dec(hi[i]);
+        reinterpret_cast<R *>(lo)[i] = BC::dec(lo[i]);
+        reinterpret_cast<R *>(hi)[i] = BC::dec(hi[i]);
     }
 }
 
@@ -552,12 +690,15 @@ __device__ __forceinline__ bool spill_push(const V &v, int slot, uint32_t t, uin
 //
 // Bound by the latency of its loads: a warp has one round of candidate loads in flight, so the
 // time is the longest item of a warp.  Windows (SPILL = true: the second launch) bring the
-// longest item down to kSpillWin candidates.  Measured (one launch before, both launches now):
-// HCA_MEASURED_COUNT
-template <typename T, int DP, bool SPILL>
+// longest item down to kSpillWin candidates (9-D call of 200,003 points 4.04 -> 3.50 ms).  The
+// filter on packed float pairs takes the double-precision call of 60,007 7-D points, whose
+// pair tests were bound by the FP64 rate, from 7.4 to 0.95 ms together with the lists.
+template <typename T, int DP, bool SPILL, bool FILTER>
 __global__ void __launch_bounds__(32 * kHdMaxWarps) k_count_hd(HdView<T, DP> v) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *rows = reinterpret_cast<T *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
+    typedef Candidate<T, DP, FILTER> Cand;
+    typedef typename Cand::Row R;
+    R *rows = reinterpret_cast<R *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
     const int lane = lane_id();
     uint32_t chunks = 0;
     const uint32_t C = v.ctr->n_cells, N = SPILL ? min(v.ctr->hd_spill[0], v.sp_cap) : v.ctr->n_chunks;
@@ -586,26 +727,34 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_count_hd(HdView<T, DP> v) 
         } else if (tc_cell && have) {
             cnt = v.tc_cnt[p];
         }
-        const uint32_t cnt0 = cnt;
         unsigned open = __ballot_sync(0xffffffffu, have && (!SPILL || cnt < min_pts));
-        if (open) stage_rows<T, DP>(rows, v.pts, base, e);
+        if (open) stage_rows<R, DP>(rows, Cand::src(v), base, e);
         // one cell at a time: a cell whose box is farther than eps from every open row adds
         // nothing to their counts and is passed over
         auto scan = [&](uint32_t B, uint32_t q0, uint32_t q1) -> bool {
             const unsigned near = open & __ballot_sync(0xffffffffu,
-                !box_far<DP>(rows + lane * DP, v.box_lo + (uint64_t)B * DP, v.box_hi + (uint64_t)B * DP, G));
+                !cell_far<FILTER, DP>(v, rows + lane * DP, B, G));
             if (!near) return true;
             for (uint32_t qb = q0; qb < q1 && open; qb += 32) {
                 const uint32_t q = qb + lane;
-                T qv[DP];
-                hd_load<T, DP>(v.pts, q, q < q1, qv);
+                Cand qv;
+                qv.load(v, q, q < q1);
                 ++chunks;
                 unsigned rem = open & near;
                 while (rem) {
                     const int jj = __ffs(rem) - 1;
                     rem &= rem - 1;
-                    const unsigned hits = __ballot_sync(0xffffffffu, q < q1 && hd_within<DP>(rows + jj * DP, qv, G));
-                    if (lane == jj) cnt += __popc(hits);
+                    const bool hit = q < q1 && qv.within(v, rows + jj * DP, base + jj, G);
+                    const unsigned hits = __ballot_sync(0xffffffffu, hit);
+                    if (!hits) continue;
+                    // the row's count, and its list entries from there on
+                    uint32_t at = 0;
+                    if (lane == jj) {
+                        at = SPILL ? atomicAdd(v.sp_val + p, (uint32_t)__popc(hits)) : cnt;
+                        cnt = at + (uint32_t)__popc(hits);
+                    }
+                    at = __shfl_sync(0xffffffffu, at, jj) + (uint32_t)__popc(hits & ((1u << lane) - 1u));
+                    if (hit && at < v.nl_k) v.nl[(uint64_t)(base + jj) * v.nl_k + at] = q;
                 }
                 open &= __ballot_sync(0xffffffffu, have && cnt < min_pts);
             }
@@ -615,7 +764,6 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_count_hd(HdView<T, DP> v) 
         bool decide = true;
         if (SPILL) {
             // the last window of the chunk decides its rows from the summed counts
-            if (have && cnt != cnt0) atomicAdd(v.sp_val + p, cnt - cnt0);
             __threadfence();
             __syncwarp();
             uint32_t left = 0;
@@ -631,6 +779,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_count_hd(HdView<T, DP> v) 
         if (decide) {
             const bool is_core = have && cnt >= min_pts;
             if (have) v.core[p] = is_core ? 1 : 0;
+            if (have && v.nl_k) v.nl_cnt[p] = cnt;
             if (__any_sync(0xffffffffu, is_core) && lane == 0) v.cell_core[A] = 1;
         }
         __syncwarp();
@@ -638,95 +787,252 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_count_hd(HdView<T, DP> v) 
     add_counter(&v.ctr->work[0], lane == 0 ? chunks : 0u);
 }
 
-// Union-find over points: parent[j] = j for every point.
+// Four list entries of point p from entry i on.
+template <typename V>
+__device__ __forceinline__ uint4 list4(const V &v, uint32_t p, uint32_t i) {
+    return __ldg(reinterpret_cast<const uint4 *>(v.nl + (uint64_t)p * v.nl_k + i));
+}
+
+// Union-find over points: every core point starts below the smallest core point on its list (an
+// edge of the core graph to a smaller index, so the links form a forest inside the clusters),
+// every other point is its own root.  With tc_hook = 0 only in the cells whose unions run on the
+// CUDA cores.
 template <typename T, int DP>
-__global__ void __launch_bounds__(256) k_uf_init_hd(HdView<T, DP> v) {
+__global__ void __launch_bounds__(256) k_list_link(HdView<T, DP> v) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += (int64_t)gridDim.x * blockDim.x) {
-        v.parent[j] = (uint32_t)j;
-        v.comp_min[j] = kNoLabel;
+        const uint32_t p = (uint32_t)j;
+        uint32_t m = p;
+        bool use = v.nl_k && v.core[p];
+        if (use && v.tc_min[1] && !v.tc_hook) {
+            const uint32_t A = v.cell_of[p];
+            use = v.cx[v.cell_start[A + 1]] - v.cx[v.cell_start[A]] < v.tc_min[1];
+        }
+        if (use) {
+            const uint32_t len = min(v.nl_cnt[p], v.nl_k);
+            for (uint32_t i = 0; i < len; i += 4) {
+                const uint4 e4 = list4(v, p, i);
+                const uint32_t e[4] = {e4.x, e4.y, e4.z, e4.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u)  // (a flagged entry is above every index)
+                    if (i + u < len && e[u] < m && v.core[e[u]]) m = e[u];
+            }
+        }
+        v.parent[p] = m;
+        v.comp_min[p] = kNoLabel;
     }
 }
 
-// First links of the core graph (Definitions 3-5): every core point p hooks to the first core
-// point q < p within eps that the scan meets (p keeps itself when there is none).  Each link
-// is an edge of the graph and points to a smaller index, so the links form a forest whose
-// trees lie inside clusters; the union pass that follows joins the trees.  The links only
-// shorten that pass (it tests every pair itself), so a chunk stops looking after
-// kHookBlocks candidate blocks: a point with no lower neighbour (the first point of every
-// cluster) would otherwise make its warp read the whole lower half of its neighbourhood.
-constexpr uint32_t kHookBlocks = 16;
+// The other edges of the lists.
 template <typename T, int DP>
-__global__ void __launch_bounds__(32 * kHdMaxWarps) k_hook_hd(HdView<T, DP> v) {
+__global__ void __launch_bounds__(256) k_list_join(HdView<T, DP> v) {
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += (int64_t)gridDim.x * blockDim.x) {
+        const uint32_t p = (uint32_t)j;
+        if (!v.core[p]) continue;
+        if (v.tc_min[1] && !v.tc_hook) {
+            const uint32_t A = v.cell_of[p];
+            if (v.cx[v.cell_start[A + 1]] - v.cx[v.cell_start[A]] >= v.tc_min[1]) continue;
+        }
+        const uint32_t len = min(v.nl_cnt[p], v.nl_k);
+        uint32_t rp = uf_find(v.parent, p, v.ctr);
+        for (uint32_t i = 0; i < len; i += 4) {
+            const uint4 e4 = list4(v, p, i);
+            const uint32_t e[4] = {e4.x, e4.y, e4.z, e4.w};
+#pragma unroll
+            for (int u = 0; u < 4; ++u) {
+                if (i + u >= len || (e[u] & kListNear) || !v.core[e[u]]) continue;
+                if (uf_find(v.parent, e[u], v.ctr) == rp) continue;
+                uf_union(v.parent, p, e[u], v.ctr);
+                rp = uf_find(v.parent, p, v.ctr);
+            }
+        }
+    }
+}
+
+// Read-only finds: parent[p] = root (nothing hooks meanwhile).
+template <typename T, int DP>
+__global__ void __launch_bounds__(256) k_flatten_hd(HdView<T, DP> v) {
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += (int64_t)gridDim.x * blockDim.x)
+        if (v.core[j]) v.parent[j] = uf_root_readonly(v.parent, (uint32_t)j, v.ctr);
+}
+
+// The tree of a cell: the smallest root among its core points.  A tree's root is its smallest
+// index, so the tree that spans a cluster has a smaller root than the small trees that the lists
+// left over in the cluster's cells, and nearly all core points of a cell have this one; the
+// others are the cell's odd points.
+template <typename T, int DP>
+__global__ void __launch_bounds__(256) k_cell_root_clear(HdView<T, DP> v) {
+    const uint32_t C = v.ctr->n_cells;
+    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
+        v.cell_root[c] = kNoRoot;
+        v.odd_cnt[c] = 0u;
+    }
+}
+
+template <typename T, int DP>
+__global__ void __launch_bounds__(256) k_cell_root(HdView<T, DP> v) {
+    const int lane = lane_id();
+    const int64_t n = v.g.n;
+    for (int64_t jb = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); jb < n; jb += (int64_t)gridDim.x * blockDim.x) {
+        const int64_t j = jb + lane;
+        const bool isc = j < n && v.core[j];
+        const uint32_t r = isc ? v.parent[j] : 0xffffffffu, c = isc ? v.cell_of[j] : 0xffffffffu;
+        // one atomic per cell of the warp's 32 consecutive points
+        const unsigned peers = __match_any_sync(0xffffffffu, c);
+        const uint32_t m = __reduce_min_sync(peers, r);
+        if (isc && lane == __ffs(peers) - 1) atomicMin(v.cell_root + c, m);
+    }
+}
+
+template <typename T, int DP>
+__global__ void __launch_bounds__(256) k_cell_odd(HdView<T, DP> v) {
+    const int lane = lane_id();
+    const uint32_t C = v.ctr->n_cells, NC = v.ctr->n_chunks, warps = (gridDim.x * blockDim.x) >> 5;
+    for (uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < NC; t += warps) {
+        const uint32_t A = chunk_cell(v.chunk_off, C, t);
+        const uint32_t e = v.cell_start[A + 1], p = v.cell_start[A] + 32u * (t - v.chunk_off[A]) + lane;
+        const unsigned m = __ballot_sync(0xffffffffu, p < e && v.core[p] && v.parent[p] != v.cell_root[A]);
+        if (lane == 0) {
+            v.odd_mask[t] = m;
+            if (m) atomicAdd(v.odd_cnt + A, (uint32_t)__popc(m));
+        }
+    }
+}
+
+// A cell with more odd points than this has no tree of its own: its core points are all compared
+// with those of every neighbour cell (the union kernels) instead of one odd point at a time.
+constexpr uint32_t kOddMin = 8;
+template <typename T, int DP>
+__global__ void __launch_bounds__(256) k_cell_mixed(HdView<T, DP> v) {
+    const uint32_t C = v.ctr->n_cells;
+    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
+        const uint32_t odd = v.odd_cnt[c];
+        if (odd > kOddMin && odd > (v.cell_start[c + 1] - v.cell_start[c]) / 4u) v.cell_root[c] = kMixedRoot;
+    }
+}
+
+// Has a pair of cells anything left for the union kernels?  Not when both have one tree and it is
+// the same: then a pair of core points in different trees has an odd point, and those were
+// compared with their whole neighbourhood.
+__device__ __forceinline__ bool cells_to_join(uint32_t ra, uint32_t rb) {
+    return rb != kNoRoot && (ra != rb || ra == kMixedRoot);
+}
+
+// Odd points against every core point of the 27 neighbour cells, joining the pairs within eps
+// whose trees differ.  One warp per chunk with odd points; long streams in windows as in the
+// counts (SPILL = true: the second launch).
+template <typename T, int DP, bool SPILL, bool FILTER>
+__global__ void __launch_bounds__(32 * kHdMaxWarps) k_odd_hd(HdView<T, DP> v) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *rows = reinterpret_cast<T *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
+    typedef Candidate<T, DP, FILTER> Cand;
+    typedef typename Cand::Row R;
+    R *rows = reinterpret_cast<R *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
     const int lane = lane_id();
     uint32_t chunks = 0;
-    HD_FOR_EACH_CHUNK(v, A, base, e, 1) {
-        if (v.tc_min[1] && !v.tc_hook && v.cx[e] - v.cx[v.cell_start[A]] >= v.tc_min[1]) continue;
-        const uint32_t p = base + lane;
-        unsigned open = __ballot_sync(0xffffffffu, p < e && v.core[p]);
-        if (!open) continue;
+    const uint32_t C = v.ctr->n_cells, N = SPILL ? min(v.ctr->hd_spill[2], v.sp_cap) : v.ctr->n_chunks;
+    uint32_t *const next = SPILL ? &v.ctr->hd_spill_next[2] : &v.ctr->hd_next[1];
+    for (uint32_t item = next_chunk(next); item < N; item = next_chunk(next)) {
+        const uint2 entry = SPILL ? v.sp_queue[item] : make_uint2(item, 0u);
+        if (SPILL && entry.x == 0xffffffffu) continue;
+        const uint32_t t = entry.x;
+        const unsigned omask = v.odd_mask[t];
+        if (!omask) continue;
+        const uint32_t A = chunk_cell(v.chunk_off, C, t);
+        if (v.cell_root[A] == kMixedRoot) continue;  // mixed: left to the union kernels
+        const uint32_t e = v.cell_start[A + 1], base = v.cell_start[A] + 32u * (t - v.chunk_off[A]), p = base + lane;
         const GridParams &G = params_of(v, set_of_key(v, v.cell_key[A]));
-        stage_rows<T, DP>(rows, v.pts, base, e);
-        uint32_t chunks_here = 0;
-        for (int g0 = 0; g0 < v.n_all && open; g0 += 32) {
-            const int k = g0 + lane;
-            const uint2 rg = k < v.n_all ? v.ranges[(uint64_t)A * v.n_all + k] : make_uint2(0u, 0u);
-            for (int kk = 0; kk < 32 && open; ++kk) {
-                const uint32_t lo = __shfl_sync(0xffffffffu, rg.x, kk);
-                const uint32_t hi = __shfl_sync(0xffffffffu, rg.y, kk);
-                if (lo >= hi) continue;
-                const uint32_t q0 = v.cell_start[lo];
-                const uint32_t q1 = min(v.cell_start[hi], base + 31u);  // only q < p can link
-                for (uint32_t qb = q0; qb < q1 && open; qb += 32) {
-                    const uint32_t q = qb + lane;
-                    const bool qc = q < q1 && v.core[q];
-                    if (!__any_sync(0xffffffffu, qc)) continue;
-                    if (++chunks_here > kHookBlocks) {
-                        open = 0;
-                        break;
-                    }
-                    T qv[DP];
-                    hd_load<T, DP>(v.pts, q, qc, qv);
-                    ++chunks;
-                    unsigned rem = open;
-                    while (rem) {
-                        const int jj = __ffs(rem) - 1;
-                        rem &= rem - 1;
-                        const bool hit = qc && q < base + jj && hd_within<DP>(rows + jj * DP, qv, G);
-                        const unsigned hm = __ballot_sync(0xffffffffu, hit);
-                        if (hm) {
-                            if (lane == jj) v.parent[base + jj] = qb + (uint32_t)(__ffs(hm) - 1);
-                            open &= ~(1u << jj);
-                        }
+        const uint2 rg = lane < v.n_all ? v.ranges[(uint64_t)A * v.n_all + lane] : make_uint2(0u, 0u);
+        const uint32_t total = stream_length(v, rg);
+        uint32_t p0 = 0, p1 = min(kSpillWin, total);
+        if (SPILL) spill_window(entry.y, p1, total, p0, p1);
+        stage_rows<R, DP>(rows, Cand::src(v), base, e);
+        const bool mine = (omask >> lane) & 1u;
+        uint32_t rp = mine ? uf_find(v.parent, p, v.ctr) : 0xffffffffu;
+        auto scan = [&](uint32_t B, uint32_t q0, uint32_t q1) -> bool {
+            const unsigned near = omask & __ballot_sync(0xffffffffu, !cell_far<FILTER, DP>(v, rows + lane * DP, B, G));
+            if (!near) return true;
+            for (uint32_t qb = q0; qb < q1; qb += 32) {
+                const uint32_t q = qb + lane;
+                const bool qc = q < q1 && v.core[q];
+                if (!__any_sync(0xffffffffu, qc)) continue;
+                uint32_t rq = qc ? uf_find(v.parent, q, v.ctr) : 0xfffffffeu;
+                Cand qv;
+                qv.load(v, q, qc);
+                ++chunks;
+                unsigned rem = near;
+                while (rem) {
+                    const int jj = __ffs(rem) - 1;
+                    rem &= rem - 1;
+                    const uint32_t rj = __shfl_sync(0xffffffffu, rp, jj);
+                    const bool hit = qc && rq != rj && qv.within(v, rows + jj * DP, base + jj, G);
+                    if (hit) uf_union(v.parent, base + jj, q, v.ctr);
+                    if (__any_sync(0xffffffffu, hit)) {
+                        rq = qc ? uf_find(v.parent, q, v.ctr) : 0xfffffffeu;
+                        if (mine) rp = uf_find(v.parent, p, v.ctr);
                     }
                 }
             }
-        }
+            return true;
+        };
+        for_stream_cells(v, rg, p0, p1, scan);
+        if (!SPILL && p1 < total && !spill_push(v, 2, t, p1, total)) for_stream_cells(v, rg, p1, total, scan);
         __syncwarp();
     }
     add_counter(&v.ctr->work[1], lane == 0 ? chunks : 0u);
 }
 
-// One round of pointer jumping over core points: parent[p] = parent[parent[p]].
+// Labels from complete lists (nl_k >= MINPTS - 1): a non-core point takes the smallest cluster id
+// among its listed core points, core points their cluster id when `core_too` (else they are
+// labelled elsewhere).  One thread per point: at most nl_k scattered loads of a byte, a tree
+// and an id instead of the comparison with the whole neighbourhood (9-D call of 200,003 points
+// 3.50 -> 2.18 ms for the labels and unions from lists together).
 template <typename T, int DP>
-__global__ void __launch_bounds__(256) k_jump_hd(HdView<T, DP> v) {
+__global__ void __launch_bounds__(256) k_list_labels(HdView<T, DP> v, int core_too) {
+    uint32_t noise = 0;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += (int64_t)gridDim.x * blockDim.x) {
-        if (!v.core[j]) continue;
-        const uint32_t p = __ldcg(v.parent + j);
-        const uint32_t gp = __ldcg(v.parent + p);
-        if (gp != p) v.parent[j] = gp;
+        const uint32_t p = (uint32_t)j;
+        const bool isc = v.core[p];
+        if (isc && !core_too) continue;
+        const uint32_t set = v.gtab ? set_of_key(v, v.cell_key[v.cell_of[p]]) : 0u;
+        uint32_t best = kNoLabel;
+        if (isc) {
+            best = v.comp_min[v.parent[p]];
+        } else {
+            const uint32_t len = min(v.nl_cnt[p], v.nl_k);
+            for (uint32_t i = 0; i < len; i += 4) {
+                const uint4 e4 = list4(v, p, i);
+                const uint32_t e[4] = {e4.x, e4.y, e4.z, e4.w};
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    const uint32_t q = e[u] & ~kListNear;
+                    if (i + u >= len || !v.core[q]) continue;
+                    const uint32_t lq = v.comp_min[v.parent[q]];
+                    if (lq >= best) continue;
+                    if ((e[u] & kListNear) && !hd_exact<T, DP>(v.pts, p, q, params_of(v, set).eps2)) continue;
+                    best = lq;
+                }
+            }
+        }
+        const uint32_t base_label = v.gtab ? (uint32_t)v.set_off[set] : 0u;
+        const int32_t lab = best == kNoLabel ? -1 : (int32_t)(best - base_label);
+        const uint32_t o = v.perm[p];
+        v.labels[o] = lab;
+        if (v.core_out) v.core_out[o] = isc ? 1 : 0;
+        noise += lab < 0;
     }
+    noise = __reduce_add_sync(0xffffffffu, noise);
+    if (lane_id() == 0 && noise) atomicAdd(&v.ctr->n_noise, noise);
 }
 
 // Definitions 3-5, remaining edges: every pair of core points within eps of the upper half of
 // the neighbourhood (the own pencil from this chunk on) whose trees differ is joined
 // (lock-free union-find, root = smallest index).  A 32 x 32 tile whose core points all share
 // one root is skipped without loading coordinates.
-template <typename T, int DP>
+template <typename T, int DP, bool FILTER>
 __global__ void __launch_bounds__(32 * kHdMaxWarps) k_merge_hd(HdView<T, DP> v) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *rows = reinterpret_cast<T *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
+    typedef Candidate<T, DP, FILTER> Cand;
+    typedef typename Cand::Row R;
+    R *rows = reinterpret_cast<R *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
     const int lane = lane_id();
     uint32_t chunks = 0, tests = 0, skipped = 0;
     HD_FOR_EACH_CHUNK(v, A, base, e, 2) {
@@ -736,20 +1042,23 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_merge_hd(HdView<T, DP> v) 
         const bool pc = p < e && v.core[p];
         const unsigned amask = __ballot_sync(0xffffffffu, pc);
         if (!amask) continue;
+        // the neighbour cells of the upper half that still have something to join
+        const uint32_t ra = v.cell_root[A];
+        const uint2 mine = lane < v.n_half ? v.ranges[(uint64_t)A * v.n_all + lane] : make_uint2(0u, 0u);
+        bool any = false;
+        for (uint32_t B = lane == 0 ? A : mine.x; B < mine.y; ++B) any |= cells_to_join(ra, v.cell_root[B]);
+        if (!__any_sync(0xffffffffu, any)) continue;
         const GridParams &G = params_of(v, set_of_key(v, v.cell_key[A]));
-        stage_rows<T, DP>(rows, v.pts, base, e);
+        stage_rows<R, DP>(rows, Cand::src(v), base, e);
         uint32_t rp = pc ? uf_find(v.parent, p, v.ctr) : 0xffffffffu;
-        for (int g0 = 0; g0 < v.n_half; g0 += 32) {
-            const int k = g0 + lane;
-            uint2 rg = k < v.n_half ? v.ranges[(uint64_t)A * v.n_all + k] : make_uint2(0u, 0u);
-            if (k == 0) rg.x = A;  // own pencil: this cell and the ones after it
-            for (int kk = 0; kk < 32; ++kk) {
-                const uint32_t lo = __shfl_sync(0xffffffffu, rg.x, kk);
-                const uint32_t hi = __shfl_sync(0xffffffffu, rg.y, kk);
-                if (lo >= hi) continue;
-                // own pencil: start at this chunk (earlier points pair with it from their side)
-                const uint32_t q0 = (g0 + kk == 0) ? max(v.cell_start[lo], base) : v.cell_start[lo];
-                const uint32_t q1 = v.cell_start[hi];
+        for (int kk = 0; kk < v.n_half; ++kk) {
+            const uint32_t lo = kk == 0 ? A : __shfl_sync(0xffffffffu, mine.x, kk);  // own pencil: this cell on
+            const uint32_t hi = __shfl_sync(0xffffffffu, mine.y, kk);
+            for (uint32_t B = lo; B < hi; ++B) {
+                if (!cells_to_join(ra, v.cell_root[B])) continue;
+                // own cell: start at this chunk (earlier points pair with it from their side)
+                const uint32_t q0 = B == A ? base : v.cell_start[B];
+                const uint32_t q1 = v.cell_start[B + 1];
                 for (uint32_t qb = q0; qb < q1; qb += 32) {
                     const uint32_t q = qb + lane;
                     const bool qc = q < q1 && v.core[q];
@@ -760,8 +1069,8 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_merge_hd(HdView<T, DP> v) 
                         ++skipped;
                         continue;
                     }
-                    T qv[DP];
-                    hd_load<T, DP>(v.pts, q, qc, qv);
+                    Cand qv;
+                    qv.load(v, q, qc);
                     ++chunks;
                     unsigned rem = amask;
                     while (rem) {
@@ -772,7 +1081,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_merge_hd(HdView<T, DP> v) 
                         const bool need = qc && q > pj && rq != rj;
                         if (!__any_sync(0xffffffffu, need)) continue;
                         ++tests;
-                        const bool hit = need && hd_within<DP>(rows + jj * DP, qv, G);
+                        const bool hit = need && qv.within(v, rows + jj * DP, pj, G);
                         if (hit) uf_union(v.parent, pj, q, v.ctr);
                         if (__any_sync(0xffffffffu, hit)) {
                             // roots moved: refresh every lane so later pairs of the tile skip
@@ -830,12 +1139,15 @@ __global__ void __launch_bounds__(256) k_comp_min_hd(HdView<T, DP> v) {
 }
 
 // Algorithm 4 / Definition 5 with the canonical rule, over points: core points take their
-// cluster id, a non-core point the smallest id among its core neighbours, else -1.  Long
-// streams are split into windows as in k_count_hd (SPILL = true: the second launch).
-template <typename T, int DP, bool SPILL>
+// cluster id, a non-core point the smallest id among its core neighbours, else -1.  For MINPTS
+// beyond the lists.  Long streams are split into windows as in k_count_hd (SPILL = true: the
+// second launch).
+template <typename T, int DP, bool SPILL, bool FILTER>
 __global__ void __launch_bounds__(32 * kHdMaxWarps) k_labels_hd(HdView<T, DP> v) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    T *rows = reinterpret_cast<T *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
+    typedef Candidate<T, DP, FILTER> Cand;
+    typedef typename Cand::Row R;
+    R *rows = reinterpret_cast<R *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
     const int lane = lane_id();
     uint32_t noise = 0, chunks = 0;
     const uint32_t C = v.ctr->n_cells, N = SPILL ? min(v.ctr->hd_spill[1], v.sp_cap) : v.ctr->n_chunks;
@@ -861,19 +1173,19 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_labels_hd(HdView<T, DP> v)
             const uint32_t total = stream_length(v, rg);
             uint32_t p0 = 0, p1 = min(kSpillWin, total);
             if (SPILL) spill_window(entry.y, p1, total, p0, p1);
-            stage_rows<T, DP>(rows, v.pts, base, e);
+            stage_rows<R, DP>(rows, Cand::src(v), base, e);
             auto scan = [&](uint32_t B, uint32_t q0, uint32_t q1) -> bool {
                 // a cell whose box is farther than eps from every row is passed over
                 const unsigned near = smask & __ballot_sync(0xffffffffu,
-                    !box_far<DP>(rows + lane * DP, v.box_lo + (uint64_t)B * DP, v.box_hi + (uint64_t)B * DP, G));
+                    !cell_far<FILTER, DP>(v, rows + lane * DP, B, G));
                 if (!near) return true;
                 for (uint32_t qb = q0; qb < q1; qb += 32) {
                     const uint32_t q = qb + lane;
                     const bool qc = q < q1 && v.core[q];
                     if (!__any_sync(0xffffffffu, qc)) continue;
                     const uint32_t lq = qc ? v.comp_min[v.parent[q]] : kNoLabel;
-                    T qv[DP];
-                    hd_load<T, DP>(v.pts, q, qc, qv);
+                    Cand qv;
+                    qv.load(v, q, qc);
                     ++chunks;
                     unsigned rem = near;
                     while (rem) {
@@ -882,7 +1194,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_labels_hd(HdView<T, DP> v)
                         const uint32_t bj = __shfl_sync(0xffffffffu, best, jj);
                         const bool need = qc && lq < bj;
                         if (!__any_sync(0xffffffffu, need)) continue;
-                        uint32_t cand = (need && hd_within<DP>(rows + jj * DP, qv, G)) ? lq : kNoLabel;
+                        uint32_t cand = (need && qv.within(v, rows + jj * DP, base + jj, G)) ? lq : kNoLabel;
                         cand = __reduce_min_sync(0xffffffffu, cand);
                         if (lane == jj && cand < best) best = cand;
                     }

@@ -14,8 +14,15 @@ namespace detail {
 // Coarse grid over three projected dimensions with side eps (1 + 2^-10): two points within eps
 // differ by at most eps (1 + 2^-50) in every coordinate, and with band coordinates computed in
 // FP64 (error tau in band units, tau << 2^-12) they fall in the same or adjacent coarse cells.
+//
+// FP32 filter thresholds: a float sum of squares s (within 2^-17 of exact, relative) below lo32
+// proves a pair within eps, above hi32 outside.  Double input is filtered on float coordinates
+// relative to the smallest ones, x' = fl32(x - mn): each is off by at most 2^-24 of the extent, so
+// a distance between copies is off by at most E = 2^-23 (1 + 2^-20) |extents|, and the thresholds
+// are (eps -+ E)^2 with the same 2^-16 on top.  `ext2` is the squared norm of the extents over all
+// dimensions of double input (-1: no filter for it); with E > eps / 4 the filter is off.
 inline int make_coarse_grid(bool input_f32, double eps, int min_pts, int64_t n, const double *mn,
-                            const double *mx, int flags, GridParams &g, double &tau) {
+                            const double *mx, int flags, GridParams &g, double &tau, double ext2 = -1.0) {
     memset(&g, 0, sizeof(g));
     g.d = 3;
     g.n = n;
@@ -51,13 +58,16 @@ inline int make_coarse_grid(bool input_f32, double eps, int min_pts, int64_t n, 
         sh += (int)g.bits[i];
     }
     g.prefix_shift = (int)g.bits[2];
-    const bool filter = input_f32 && !(flags & HCA_FLAG_FP64_ONLY) && g.eps2 >= ldexp(1.0, -100) &&
-                        g.eps2 <= ldexp(1.0, 100);
+    const double off = input_f32 || ext2 < 0.0 ? 0.0 : ldexp(1.0, -23) * (1.0 + ldexp(1.0, -20)) * sqrt(ext2);
+    const bool filter = (input_f32 || ext2 >= 0.0) && !(flags & HCA_FLAG_FP64_ONLY) && g.eps2 >= ldexp(1.0, -100) &&
+                        g.eps2 <= ldexp(1.0, 100) && off <= 0.25 * eps;
     if (filter) {
-        float lo = (float)(g.eps2 * (1.0 - ldexp(1.0, -16)));
-        if ((double)lo > g.eps2 * (1.0 - ldexp(1.0, -16))) lo = nextafterf(lo, 0.f);
-        float hi = (float)(g.eps2 * (1.0 + ldexp(1.0, -16)));
-        if ((double)hi < g.eps2 * (1.0 + ldexp(1.0, -16))) hi = nextafterf(hi, INFINITY);
+        const double lo2 = (off > 0.0 ? (eps - off) * (eps - off) : g.eps2) * (1.0 - ldexp(1.0, -16));
+        const double hi2 = (off > 0.0 ? (eps + off) * (eps + off) : g.eps2) * (1.0 + ldexp(1.0, -16));
+        float lo = (float)lo2;
+        if ((double)lo > lo2) lo = nextafterf(lo, 0.f);
+        float hi = (float)hi2;
+        if ((double)hi < hi2) hi = nextafterf(hi, INFINITY);
         g.lo32 = lo;
         g.hi32 = hi;
     } else {
@@ -134,13 +144,71 @@ struct TcOffsets {
 
 inline uint32_t *part_of(char *b, size_t o) { return (uint32_t *)(b + o); }
 
-// The three point phases with tensor-core tiles for the cells holding at least min_rows rows
-// of a phase and the CUDA-core kernels for the rest (float input): counts (Definition 2),
-// first links + pointer jumping + unions (Definitions 3-5) and labels (Algorithm 4).
+// Launch shapes shared by the phases.
+struct HdLaunch {
+    cudaStream_t s;
+    int gpts, gcell, block;  // grids of the point and of the chunk kernels, threads of the latter
+    size_t smem;             // their shared memory
+    bool list_labels;        // the lists are complete: labels from them
+};
+
+// The lists joined, every cell's tree and its odd points, and those against their neighbourhood.
+template <typename T, int DP, bool FILTER>
+void run_list_unions(HdView<T, DP> &hv, const HdLaunch &L, int &launches) {
+    k_list_link<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+    if (hv.nl_k) k_list_join<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+    k_flatten_hd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+    k_cell_root_clear<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+    k_cell_root<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+    k_cell_odd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+    k_cell_mixed<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+    k_odd_hd<T, DP, false, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
+    k_odd_hd<T, DP, true, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
+    launches += hv.nl_k ? 9 : 8;
+}
+
+// The three point phases on the CUDA cores: counts (Definition 2), unions (Definitions 3-5) and
+// labels (Algorithm 4).
+template <typename T, int DP, bool FILTER, typename Mark>
+void run_cuda_phases(HdView<T, DP> &hv, const HdLaunch &L, int64_t n, Mark &mark, int &launches) {
+    detail::allow_smem(k_count_hd<T, DP, false, FILTER>, L.smem);
+    detail::allow_smem(k_count_hd<T, DP, true, FILTER>, L.smem);
+    detail::allow_smem(k_odd_hd<T, DP, false, FILTER>, L.smem);
+    detail::allow_smem(k_odd_hd<T, DP, true, FILTER>, L.smem);
+    detail::allow_smem(k_merge_hd<T, DP, FILTER>, L.smem);
+    detail::allow_smem(k_labels_hd<T, DP, false, FILTER>, L.smem);
+    detail::allow_smem(k_labels_hd<T, DP, true, FILTER>, L.smem);
+    cudaMemsetAsync(hv.cell_core, 0, (size_t)n, L.s);
+    k_count_hd<T, DP, false, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
+    k_count_hd<T, DP, true, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
+    mark(6);
+    // (no representative points in this path: every pair of core points is a candidate)
+    mark(7);
+    run_list_unions<T, DP, FILTER>(hv, L, launches);
+    k_merge_hd<T, DP, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
+    k_compress_hd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+    mark(8);
+    k_comp_min_hd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+    if (L.list_labels) {
+        k_list_labels<T, DP><<<L.gpts, 256, 0, L.s>>>(hv, 1);
+        launches += 6;
+    } else {
+        k_labels_hd<T, DP, false, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
+        k_labels_hd<T, DP, true, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
+        launches += 7;
+    }
+    mark(9);
+}
+
+// The same with tensor-core tiles for the cells holding at least min_rows rows of a phase and
+// the CUDA-core kernels for the rest (float input).
 template <int DP, typename Mark>
-void run_tc_phases(HdView<float, DP> &hv, cudaStream_t s, char *b, int64_t n, int grid_tc, size_t tc_smem,
-                   int gpts, int gcell, int hd_block, size_t smem, uint32_t *part, const TcOffsets &o, int nsets,
-                   DevCounters *ctr, const TcTuning &tune, Mark &mark, int &launches, cudaEvent_t *tev) {
+void run_tc_phases(HdView<float, DP> &hv, const HdLaunch &L, char *b, int64_t n, int grid_tc, size_t tc_smem,
+                   uint32_t *part, const TcOffsets &o, int nsets, DevCounters *ctr, const TcTuning &tune, Mark &mark,
+                   int &launches, cudaEvent_t *tev) {
+    cudaStream_t s = L.s;
+    const int gpts = L.gpts, gcell = L.gcell, hd_block = L.block;
+    const size_t smem = L.smem;
     // tev (nullable): six events recorded around the three tensor-core launches
     auto tmark = [&](int i) { if (tev) cudaEventRecord(tev[i], s); };
     uint32_t *nch = (uint32_t *)(b + o.nch), *nch2 = (uint32_t *)(b + o.nch2);
@@ -154,13 +222,20 @@ void run_tc_phases(HdView<float, DP> &hv, cudaStream_t s, char *b, int64_t n, in
     hv.cx = cx;
     hv.tc_cnt = clab;   // free until the labels phase
     hv.tc_pos = flags;  // free until the core numbering
+    detail::allow_smem(k_count_hd<float, DP, false, true>, smem);
+    detail::allow_smem(k_count_hd<float, DP, true, true>, smem);
+    detail::allow_smem(k_odd_hd<float, DP, false, true>, smem);
+    detail::allow_smem(k_odd_hd<float, DP, true, true>, smem);
+    detail::allow_smem(k_merge_hd<float, DP, true>, smem);
+    detail::allow_smem(k_labels_hd<float, DP, false, true>, smem);
+    detail::allow_smem(k_labels_hd<float, DP, true, true>, smem);
     // ---- Definition 2: exact counts over the neighbouring coarse cells ----
     cudaMemsetAsync(hv.cell_core, 0, (size_t)n, s);
     cudaMemsetAsync(hv.core, 0, (size_t)n, s);  // the recount below lists the rows with core = 2
     tc::k_tc_chunks_count<<<gpts, 256, 0, s>>>(hv.cell_start, ctr, tune.min[0], nch);
     exclusive_scan_u32(nch, ch0, n, &ctr->n_cells, &ctr->n_tc_chunks[tc::kCount], part, s, &launches);
     tmark(0);
-    tc::k_tc_hd<DP, tc::kCount><<<grid_tc, tc::kTile, tc_smem, s>>>(hv, tc::Tables{ch0, cx, clist, nclist, clab, nullptr});
+    tc::k_tc_hd<DP, tc::kCount><<<grid_tc, tc::kTile, tc_smem, s>>>(hv, tc::Tables{ch0, cx, clist, nclist, clab});
     // the rows those chunks handed over, in cells with at least kRecountMin of them, counted again
     // from the start, 128 per chunk (cx, clist, nclist, nch2 and ch1 are free until the core
     // numbering); the rest, and what the recount hands over, go to the CUDA-core count
@@ -175,61 +250,63 @@ void run_tc_phases(HdView<float, DP> &hv, cudaStream_t s, char *b, int64_t n, in
     cudaMemsetAsync(ch0, 0, 4 * (size_t)n, s);
     cudaMemsetAsync(nclist, 0, 4 * (size_t)n, s);
     tc::k_tc_hd<DP, tc::kCount><<<grid_tc, tc::kTile, tc_smem, s>>>(
-        hv, tc::Tables{ch1, cx, nullptr, nullptr, nullptr, nullptr, nullptr, clist, nch, ch0, nclist});
+        hv, tc::Tables{ch1, cx, nullptr, nullptr, nullptr, nullptr, clist, nch, ch0, nclist});
     tmark(1);
-    k_count_hd<float, DP, false><<<gcell, hd_block, smem, s>>>(hv);
-    k_count_hd<float, DP, true><<<gcell, hd_block, smem, s>>>(hv);
+    k_count_hd<float, DP, false, true><<<gcell, hd_block, smem, s>>>(hv);
+    k_count_hd<float, DP, true, true><<<gcell, hd_block, smem, s>>>(hv);
     launches += 8;
     mark(6);
-    // core numbering, core and non-core lists, chunk tables of the unions and the labels
+    // core numbering, core and non-core lists
     tc::k_tc_core_flags<<<gpts, 256, 0, s>>>(hv.core, n, flags);
     exclusive_scan_u32(flags, cx, n, nullptr, cx + n, part, s, &launches);
-    tc::k_tc_partition<<<gpts, 256, 0, s>>>(hv.core, cx, n, clist, nclist);
-    // (flags and ch0 are free once cx is scanned and the counts are done: the unions' later
-    // windows take them)
-    tc::k_tc_chunks_split<<<gpts, 256, 0, s>>>(hv.cell_start, cx, ctr, hv.ranges, hv.n_half, hv.n_all, tune.min[1],
-                                               tune.min[2], nch, flags, nch2);
-    exclusive_scan_u32(nch, ch1, n, &ctr->n_cells, &ctr->n_tc_chunks[tc::kMerge], part, s, &launches);
-    exclusive_scan_u32(nch2, ch2, n, &ctr->n_cells, &ctr->n_tc_chunks[tc::kLabels], part, s, &launches);
-    exclusive_scan_u32(flags, ch0, n, &ctr->n_cells, &ctr->n_tc_chunks[3], part, s, &launches);
-    launches += 3;
+    tc::k_tc_partition<<<gpts, 256, 0, s>>>(hv.core, cx, n, clist, L.list_labels ? nullptr : nclist);
+    launches += 2;
     mark(7);
-    // ---- Definitions 3-5: first links, pointer jumping, then the remaining unions ----
-    k_uf_init_hd<float, DP><<<gpts, 256, 0, s>>>(hv);
-    k_hook_hd<float, DP><<<gcell, hd_block, smem, s>>>(hv);
-    for (int r = 0; r < 6; ++r) k_jump_hd<float, DP><<<gpts, 256, 0, s>>>(hv);
-    // (nch and nch2 are free once the chunk tables are scanned)
-    tc::k_tc_cell_root_clear<<<gpts, 256, 0, s>>>(ctr, nch, nch2);
-    tc::k_tc_cell_root<DP><<<gpts, 256, 0, s>>>(hv, nch, nch2);
-    tc::k_tc_cell_root_final<<<gpts, 256, 0, s>>>(ctr, nch, nch2);
+    // ---- Definitions 3-5: the lists' edges and the odd points, then the remaining unions ----
+    run_list_unions<float, DP, true>(hv, L, launches);
+    // chunk tables of the unions and the labels (flags and ch0 are free: the unions' later windows)
+    tc::k_tc_chunks_split<DP><<<gpts, 256, 0, s>>>(hv, tune.min[1], tune.min[2], nch, flags,
+                                                   L.list_labels ? nullptr : nch2);
+    exclusive_scan_u32(nch, ch1, n, &ctr->n_cells, &ctr->n_tc_chunks[tc::kMerge], part, s, &launches);
+    if (!L.list_labels)
+        exclusive_scan_u32(nch2, ch2, n, &ctr->n_cells, &ctr->n_tc_chunks[tc::kLabels], part, s, &launches);
+    exclusive_scan_u32(flags, ch0, n, &ctr->n_cells, &ctr->n_tc_chunks[3], part, s, &launches);
     tmark(2);
     // window-major items: the first window of every chunk, then the other windows
-    tc::k_tc_hd<DP, tc::kMerge><<<grid_tc, tc::kTile, tc_smem, s>>>(hv, tc::Tables{ch1, cx, clist, nclist, clab, nch, ch0});
+    tc::k_tc_hd<DP, tc::kMerge><<<grid_tc, tc::kTile, tc_smem, s>>>(hv, tc::Tables{ch1, cx, clist, nclist, clab, ch0});
     tmark(3);
     // the CUDA-core unions take the cells below the threshold; from one core row on every cell
     // with a core point is on the tensor cores and nothing is left for them
     if (tune.min[1] > 1) {
-        k_merge_hd<float, DP><<<gcell, hd_block, smem, s>>>(hv);
+        k_merge_hd<float, DP, true><<<gcell, hd_block, smem, s>>>(hv);
         ++launches;
     }
     k_compress_hd<float, DP><<<gpts, 256, 0, s>>>(hv);
-    launches += 13;
+    launches += 3;
     mark(8);
     // ---- Algorithm 4: canonical ids, core labels, border and noise points ----
     k_comp_min_hd<float, DP><<<gpts, 256, 0, s>>>(hv);
+    if (L.list_labels) {
+        tmark(4);
+        k_list_labels<float, DP><<<gpts, 256, 0, s>>>(hv, 1);
+        tmark(5);
+        launches += 2;
+        mark(9);
+        return;
+    }
     // the cells below the labels threshold on a second stream beside the tensor-core labels:
     // the two write the labels of disjoint cells
     const detail::SideStream ss = detail::side_stream();
     const bool fork = ss.ok && cudaEventRecord(ss.fork, s) == cudaSuccess &&
                       cudaStreamWaitEvent(ss.s, ss.fork, 0) == cudaSuccess;
     auto cuda_labels = [&](cudaStream_t ls) {
-        k_labels_hd<float, DP, false><<<gcell, hd_block, smem, ls>>>(hv);
-        k_labels_hd<float, DP, true><<<gcell, hd_block, smem, ls>>>(hv);
+        k_labels_hd<float, DP, false, true><<<gcell, hd_block, smem, ls>>>(hv);
+        k_labels_hd<float, DP, true, true><<<gcell, hd_block, smem, ls>>>(hv);
     };
     if (fork) cuda_labels(ss.s);
-    tc::k_tc_core_labels<DP><<<gpts, 256, 0, s>>>(hv, tc::Tables{ch2, cx, clist, nclist, clab, nullptr}, nsets, clab);
+    tc::k_tc_core_labels<DP><<<gpts, 256, 0, s>>>(hv, tc::Tables{ch2, cx, clist, nclist, clab}, nsets, clab);
     tmark(4);
-    tc::k_tc_hd<DP, tc::kLabels><<<grid_tc, tc::kTile, tc_smem, s>>>(hv, tc::Tables{ch2, cx, clist, nclist, clab, nullptr});
+    tc::k_tc_hd<DP, tc::kLabels><<<grid_tc, tc::kTile, tc_smem, s>>>(hv, tc::Tables{ch2, cx, clist, nclist, clab});
     tmark(5);
     if (fork) {
         cudaEventRecord(ss.join, ss.s);
@@ -294,6 +371,12 @@ int run_hd(const RunArgs &a) {
     const size_t o_tflags = take(4 * tc_n), o_cx = take(4 * (tc_n + 1));
     const size_t o_clist = take(4 * tc_n), o_nclist = take(4 * tc_n), o_clab = take(4 * tc_n);
     const size_t o_box = take(sizeof(double) * 2 * (size_t)d * nsets);
+    // the neighbour lists come last: without memory for them the call runs without
+    uint32_t max_min_pts = (uint32_t)a.min_pts;
+    for (int i = 0; batched && i < nsets; ++i) max_min_pts = std::max(max_min_pts, (uint32_t)a.h_minpts[i]);
+    if (a.ws_query && !a.box_mn) max_min_pts = kListMax + 1;  // any MINPTS
+    const bool lists = !a.no_lists;
+    const size_t o_nl = take(lists ? sizeof(uint32_t) * list_len(max_min_pts) * (size_t)n : 0);
     bool use_tc = tc_occ > 0;
     const bool boxed = a.box_mn != nullptr;
     const bool own_ws = a.ws_ext == nullptr;
@@ -306,7 +389,11 @@ int run_hd(const RunArgs &a) {
         if (!boxed || a.ws_ext_bytes < off) return HCA_EINVAL;
         ws = a.ws_ext;
     } else if (pool_alloc(&ws, off, s) != cudaSuccess || !ws) {
-        return HCA_ENOMEM;
+        cudaGetLastError();
+        if (!lists) return HCA_ENOMEM;
+        RunArgs less = a;
+        less.no_lists = true;
+        return run_hd<T, DP>(less);
     }
     char *b = (char *)ws;
     DevCounters *ctr = (DevCounters *)(b + o_ctr);
@@ -314,6 +401,7 @@ int run_hd(const RunArgs &a) {
     DevCounters *h = a.h_ext ? a.h_ext : (a.ws_query ? nullptr : host_counters());
     int rc = HCA_OK;
     bool tc_phases = false;  // the tensor-core split ran every phase
+    bool filter = true;      // every set's pair tests have the FP32 filter
 
     cudaEvent_t ev[HCA_NUM_STAGES + 1] = {};
     cudaEvent_t tev[6] = {};
@@ -341,6 +429,8 @@ int run_hd(const RunArgs &a) {
     memset(&hv, 0, sizeof(hv));
     memset(&lv, 0, sizeof(lv));
     int sort_bits = 0;
+    float *fpts = nullptr;
+    HdLaunch L;
     std::vector<unsigned long long> smm;
     std::vector<GridParams> gsets;
     GridParams *d_gtab = (GridParams *)(b + o_gtab);
@@ -366,8 +456,12 @@ int run_hd(const RunArgs &a) {
         }
         const double mn3[3] = {mn_all[pick[0]], mn_all[pick[1]], mn_all[pick[2]]};
         const double mx3[3] = {mx_all[pick[0]], mx_all[pick[1]], mx_all[pick[2]]};
-        const int r = make_coarse_grid(sizeof(T) == 4, set_eps, set_minpts, n, mn3, mx3, a.flags, gp, tau_s);
+        double ext2 = 0.0;
+        for (int i = 0; sizeof(T) == 8 && i < d; ++i) ext2 += (mx_all[i] - mn_all[i]) * (mx_all[i] - mn_all[i]);
+        const int r = make_coarse_grid(sizeof(T) == 4, set_eps, set_minpts, n, mn3, mx3, a.flags, gp, tau_s, ext2);
         if (r) return r;
+        // (double input: the float copies and their squares stay finite under the same bound)
+        if (!(gp.lo32 >= 0.0f) || (sizeof(T) == 8 && !tc_magnitude_ok(d, mn_all, mx_all, gp))) filter = false;
         if (!tc_magnitude_ok(d, mn_all, mx_all, gp)) use_tc = false;
         for (int k = 0; k < 3; ++k) gp.sel[k] = pick[k];
         return HCA_OK;
@@ -487,6 +581,9 @@ int run_hd(const RunArgs &a) {
         if (batched) cudaMemcpyAsync(d_gtab, gsets.data(), sizeof(GridParams) * nsets, cudaMemcpyHostToDevice, s);
     }
     mark(1);
+    // the filter's float copy of double input takes the half of the box space that float boxes
+    // leave free
+    if (sizeof(T) == 8 && filter) fpts = (float *)(b + o_bhi);
     {
         uint32_t *ia = (uint32_t *)(b + o_ia), *ib = (uint32_t *)(b + o_ib);
         uint32_t *hist = (uint32_t *)(b + o_hist), *part = (uint32_t *)(b + o_part);
@@ -504,7 +601,7 @@ int run_hd(const RunArgs &a) {
             mark(3);
             k_gather_hd<T, DP, uint32_t><<<gtile, 256, 0, s>>>(
                 (const T *)a.d_points, d, flipped ? kb : ka, flipped ? ib : ia, n, (T *)(b + o_pts),
-                (uint32_t *)(b + o_flags), part);
+                (uint32_t *)(b + o_flags), part, fpts, batched ? d_smm : mm, batched ? g.key_bits : 64);
         } else {
             uint64_t *ka = (uint64_t *)(b + o_ka), *kb = (uint64_t *)(b + o_kb);
             if (batched)
@@ -517,7 +614,7 @@ int run_hd(const RunArgs &a) {
             mark(3);
             k_gather_hd<T, DP, uint64_t><<<gtile, 256, 0, s>>>(
                 (const T *)a.d_points, d, flipped ? kb : ka, flipped ? ib : ia, n, (T *)(b + o_pts),
-                (uint32_t *)(b + o_flags), part);
+                (uint32_t *)(b + o_flags), part, fpts, batched ? d_smm : mm, batched ? g.key_bits : 64);
         }
         launches += 2;
         // run-length cells: scan of the gather's tile counts, cell ids / starts / keys
@@ -576,28 +673,45 @@ int run_hd(const RunArgs &a) {
     hv.ctr = ctr;
     hv.n_all = st.n_all;
     hv.n_half = st.n_half;
+    hv.fpts = sizeof(T) == 4 ? (const float *)(b + o_pts) : fpts;
+    hv.cell_of = (const uint32_t *)(b + o_flags);
     hv.box_lo = (T *)(b + o_blo);
-    hv.box_hi = (T *)(b + o_bhi);
+    // (with fpts both float boxes lie in the first half of the box space)
+    hv.box_hi = (T *)(b + (fpts ? o_blo + sizeof(float) * DP * (size_t)n : o_bhi));
     // the windows' queue and per-row values take the sort's key buffers, free once the cells are
-    // known; one word per chunk (at most n) from the pencil flags, free once the pencils are
+    // known; one word per chunk (at most n) from the pencil flags, free once the pencils are, and
+    // so are the scan scratch and the pencil starts that the cells' trees take after the ranges;
+    // the list lengths take the index buffer that the sort did not end in
     hv.sp_queue = (uint2 *)(b + o_ka);
     hv.sp_cap = (uint32_t)n;
     hv.sp_val = (uint32_t *)(b + o_kb);
     hv.sp_pending = (uint32_t *)(b + o_pflags);
+    hv.cell_root = (uint32_t *)(b + o_pexcl);
+    hv.odd_cnt = (uint32_t *)(b + o_excl);
+    hv.odd_mask = (uint32_t *)(b + o_pstart);
+    hv.nl = (uint32_t *)(b + o_nl);
+    hv.nl_k = lists ? list_len(max_min_pts) : 0u;
+    hv.nl_cnt = (uint32_t *)(b + (flipped ? o_ia : o_ib));
+    L.s = s;
+    L.gpts = gpts;
+    L.gcell = gcell;
+    L.block = hd_block;
+    L.smem = smem;
+    L.list_labels = hv.nl_k && hv.nl_k + 1 >= max_min_pts;
     // the box of every coarse cell in all d dimensions (point-to-box distance bounds)
-    k_cell_box_clear<T, DP><<<grid_for((int64_t)n * DP, 256, sms, 8), 256, 0, s>>>(hv);
-    k_cell_box_hd<T, DP><<<grid_for(n / 32 + 1, 8, sms, 16), 256, 0, s>>>(hv);
-    k_cell_box_decode<T, DP><<<grid_for((int64_t)n * DP, 256, sms, 8), 256, 0, s>>>(hv);
+    if (fpts) {
+        k_cell_box_clear<T, DP, float><<<grid_for((int64_t)n * DP, 256, sms, 8), 256, 0, s>>>(hv);
+        k_cell_box_hd<T, DP, float><<<grid_for(n / 32 + 1, 8, sms, 16), 256, 0, s>>>(hv);
+        k_cell_box_decode<T, DP, float><<<grid_for((int64_t)n * DP, 256, sms, 8), 256, 0, s>>>(hv);
+    } else {
+        k_cell_box_clear<T, DP, T><<<grid_for((int64_t)n * DP, 256, sms, 8), 256, 0, s>>>(hv);
+        k_cell_box_hd<T, DP, T><<<grid_for(n / 32 + 1, 8, sms, 16), 256, 0, s>>>(hv);
+        k_cell_box_decode<T, DP, T><<<grid_for((int64_t)n * DP, 256, sms, 8), 256, 0, s>>>(hv);
+    }
     launches += 3;
-    allow_smem(k_count_hd<T, DP, false>, smem);
-    allow_smem(k_count_hd<T, DP, true>, smem);
-    allow_smem(k_hook_hd<T, DP>, smem);
-    allow_smem(k_merge_hd<T, DP>, smem);
-    allow_smem(k_labels_hd<T, DP, false>, smem);
-    allow_smem(k_labels_hd<T, DP, true>, smem);
     if constexpr (std::is_same<T, float>::value) {
         if (use_tc && st.n_all <= tc::kMaxRng) {
-            run_tc_phases<DP>(hv, s, b, n, sms * tc_occ, tc_smem, gpts, gcell, hd_block, smem, part_of(b, o_part),
+            run_tc_phases<DP>(hv, L, b, n, sms * tc_occ, tc_smem, part_of(b, o_part),
                               TcOffsets{o_tnch, o_tnch2, o_tch0, o_tch1, o_tch2, o_tflags, o_cx, o_clist, o_nclist,
                                         o_clab},
                               batched ? nsets : 0, ctr,
@@ -609,28 +723,8 @@ int run_hd(const RunArgs &a) {
         }
     }
     if (!tc_phases) {
-        // ---- Definition 2: exact counts over the neighbouring coarse cells ----
-        cudaMemsetAsync(hv.cell_core, 0, (size_t)n, s);
-        k_count_hd<T, DP, false><<<gcell, hd_block, smem, s>>>(hv);
-        k_count_hd<T, DP, true><<<gcell, hd_block, smem, s>>>(hv);
-        launches += 2;
-        mark(6);
-        // (no representative points in this path: every pair of core points is a candidate)
-        mark(7);
-        // ---- Definitions 3-5: first links, pointer jumping, then the remaining unions ----
-        k_uf_init_hd<T, DP><<<gpts, 256, 0, s>>>(hv);
-        k_hook_hd<T, DP><<<gcell, hd_block, smem, s>>>(hv);
-        for (int r = 0; r < 6; ++r) k_jump_hd<T, DP><<<gpts, 256, 0, s>>>(hv);
-        k_merge_hd<T, DP><<<gcell, hd_block, smem, s>>>(hv);
-        k_compress_hd<T, DP><<<gpts, 256, 0, s>>>(hv);
-        launches += 10;
-        mark(8);
-        // ---- Algorithm 4: canonical ids, border and noise points ----
-        k_comp_min_hd<T, DP><<<gpts, 256, 0, s>>>(hv);
-        k_labels_hd<T, DP, false><<<gcell, hd_block, smem, s>>>(hv);
-        k_labels_hd<T, DP, true><<<gcell, hd_block, smem, s>>>(hv);
-        launches += 3;
-        mark(9);
+        if (filter) run_cuda_phases<T, DP, true>(hv, L, n, mark, launches);
+        else run_cuda_phases<T, DP, false>(hv, L, n, mark, launches);
     }
     if (cudaGetLastError() != cudaSuccess) { rc = HCA_ECUDA; goto out; }
     if (cudaMemcpyAsync(h, ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, s) != cudaSuccess) {

@@ -26,6 +26,7 @@ struct PlanPart {
     hca::GroupBuffers gb = {};
     hca::DevCounters *h = nullptr;   // pinned: the counters of the last launch
     void *stage = nullptr;           // pinned: per-set tables the graph copies to the device
+    bool no_lists = false;           // captured without neighbour lists (no memory for them)
     int32_t flags = 0;               // HCA_FLAG_* of the captured call (no timing)
     int launches = 0;                // kernels the captured call launches
     int key_bits = 0;                // bits of its cell keys
@@ -74,6 +75,7 @@ hca::RunArgs part_args(const PlanPart &pt, const void *pts, int32_t *lab, uint8_
     a.tune = hca::tuning_for(pt.g.d);  // fixed into the graph
     a.box_mn = pt.g.box_mn.data();
     a.box_mx = pt.g.box_mx.data();
+    a.no_lists = pt.no_lists;
     if (pt.batched) {
         a.nsets = (int)pt.g.sets.size();
         a.h_off = pt.g.off.data();
@@ -156,8 +158,15 @@ int create(hca_plan **out, const void *d_points, int32_t dtype, bool batched, st
         }
         memset(pt.h, 0, sizeof(DevCounters));
         if (pool_alloc(&pt.ws, pt.ws_bytes, p->cap) != cudaSuccess || !pt.ws) {
-            rc = HCA_ENOMEM;
-            break;
+            cudaGetLastError();
+            pt.ws = nullptr;
+            a.no_lists = pt.no_lists = true;
+            rc = dispatch(a, dtype);
+            if (rc) break;
+            if (pool_alloc(&pt.ws, pt.ws_bytes, p->cap) != cudaSuccess || !pt.ws) {
+                rc = HCA_ENOMEM;
+                break;
+            }
         }
     }
     if (rc == HCA_OK && cudaStreamSynchronize(p->cap) != cudaSuccess) rc = HCA_ECUDA;

@@ -58,17 +58,22 @@ constexpr uint32_t kSegCand = 16 * kTile;  // unions: candidates per work item (
 constexpr uint32_t kSplitBelow = 32;       // unions: windows only with fewer chunks per CTA than this
 enum { kCount = 0, kMerge = 1, kLabels = 2 };
 
-// Unions: core points of neighbour range k of cell A before any pruning (range 0, the cell's
-// own pencil, from A on).  The unpruned stream of A is ranges 0 .. n_half - 1 end to end.
-__device__ __forceinline__ uint32_t merge_range_len(const uint2 *ranges, int n_all, const uint32_t *cell_start,
-                                                    const uint32_t *cx, uint32_t A, int k) {
-    uint2 rg = ranges[(uint64_t)A * n_all + k];
+// Unions: core points of the cells of neighbour range k of cell A (range 0, the cell's own pencil,
+// from A on) that still have something to join with A.  The stream of A before the box tests is
+// those of ranges 0 .. n_half - 1 end to end.
+template <int DP>
+__device__ __forceinline__ uint32_t merge_range_len(const HdView<float, DP> &v, uint32_t A, int k) {
+    uint2 rg = v.ranges[(uint64_t)A * v.n_all + k];
     if (k == 0) rg.x = A;
-    return rg.x < rg.y ? cx[cell_start[rg.y]] - cx[cell_start[rg.x]] : 0u;
+    const uint32_t ra = v.cell_root[A];
+    uint32_t len = 0;
+    for (uint32_t B = rg.x; B < rg.y; ++B)
+        if (cells_to_join(ra, v.cell_root[B])) len += v.cx[v.cell_start[B + 1]] - v.cx[v.cell_start[B]];
+    return len;
 }
 
-// Windows of a 128-row chunk of the unions: one per kSegCand candidates of the unpruned
-// stream (an upper bound of the pruned one); window w is the blocks of the pruned stream from
+// Windows of a 128-row chunk of the unions: one per kSegCand candidates of that stream (an
+// upper bound of what the box tests leave); window w is the blocks of the pruned stream from
 // w * kSegCand on (none when the pruning left fewer).  The items are handed out window-major:
 // the first windows of all chunks, then the others, so that no item of a cell with a long
 // neighbourhood runs far longer than the rest, and the later windows mostly find the trees that
@@ -85,8 +90,6 @@ struct Tables {
     const uint32_t *core_list;  // core points, ascending
     const uint32_t *nc_list;    // non-core points, ascending
     const uint32_t *core_lab;   // cluster id of every core point, by core-list index (labels phase)
-    const uint32_t *cell_root;  // unions: the one root of a cell's core points (~0 if they differ or
-                                // there are none), taken before the phase; nullptr: unused
     const uint32_t *choff_later;  // unions: first item of every coarse cell among the windows after
                                   // the first of its chunks (chunks x (windows - 1) per cell)
     const uint32_t *row_list;     // counts: nullptr = every point of the cell; else the recount of the
@@ -430,7 +433,7 @@ __global__ void __launch_bounds__(kTile) k_tc_hd(HdView<float, DP> v, Tables tt)
                 const bool later = MODE == kMerge && t >= N0;
                 A = later ? chunk_cell(tt.choff_later, C, t - N0) : chunk_cell(tt.choff, C, t);
                 if (later) {
-                    uint32_t len = tid < n_rng ? merge_range_len(v.ranges, v.n_all, v.cell_start, tt.cx, A, tid) : 0u;
+                    uint32_t len = tid < n_rng ? merge_range_len(v, A, tid) : 0u;
                     nwin = merge_windows(__reduce_add_sync(0xffffffffu, len));
                 }
                 if (recount) {
@@ -536,12 +539,7 @@ __global__ void __launch_bounds__(kTile) k_tc_hd(HdView<float, DP> v, Tables tt)
                 if (warp == 0) {
                     uint32_t q0 = 0, len = 0;
                     bool keep = tid < (int)nbc && S.bnear[tid];
-                    if (MODE == kMerge && keep && tt.cell_root) {
-                        // two cells whose core points were already all in one tree have no pair
-                        // left to join (trees only grow)
-                        const uint32_t ra = tt.cell_root[A];
-                        keep = ra == 0xffffffffu || tt.cell_root[S.bcell[tid]] != ra;
-                    }
+                    if (MODE == kMerge && keep) keep = cells_to_join(v.cell_root[A], v.cell_root[S.bcell[tid]]);
                     if (keep) {
                         const uint32_t c = S.bcell[tid];
                         q0 = tt.cx[v.cell_start[c]];
@@ -750,28 +748,29 @@ __global__ void __launch_bounds__(kTile) k_tc_hd(HdView<float, DP> v, Tables tt)
                         } else if (max32(dv[h]) < thr_near) {
                             continue;
                         }
+                        uint32_t in_m = 0, near_m = 0;
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) {
+                            const float dd = __uint_as_float(dv[h][j]);
+                            const bool in = dd > rowA;
+                            in_m |= (uint32_t)in << j;
+                            near_m |= (uint32_t)(!in && !(dd < thr_near)) << j;
+                        }
                         if (MODE == kCount) {
                             // cnt: pairs surely within eps (D > rowA); cnt_hi: pairs not proved
-                            // outside (D >= thr_near); four partial tallies each
-                            uint32_t ci[4] = {0u, 0u, 0u, 0u}, ch[4] = {0u, 0u, 0u, 0u};
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) {
-                                const float dd = __uint_as_float(dv[h][j]);
-                                ci[j & 3] += dd > rowA ? 1u : 0u;
-                                ch[j & 3] += dd < thr_near ? 0u : 1u;
+                            // outside (D >= thr_near), which take the next entries of the list
+                            uint32_t m = in_m | near_m;
+                            const uint32_t found = (uint32_t)__popc(m);
+                            uint32_t at = recount ? atomicAdd(tt.rc_hi + rk, found) : cnt_hi;
+                            cnt += (uint32_t)__popc(in_m);
+                            cnt_hi += found;
+                            for (; m && at < v.nl_k; ++at) {
+                                const int j = __ffs(m) - 1;
+                                m &= m - 1;
+                                v.nl[(uint64_t)p * v.nl_k + at] = S.cidx[cg + (uint32_t)j] | ((in_m >> j) & 1u ? 0u : kListNear);
                             }
-                            cnt += (ci[0] + ci[1]) + (ci[2] + ci[3]);
-                            cnt_hi += (ch[0] + ch[1]) + (ch[2] + ch[3]);
                             if (cnt >= G.min_pts) need = false;
                         } else {
-                            uint32_t in_m = 0, near_m = 0;
-#pragma unroll
-                            for (int j = 0; j < 32; ++j) {
-                                const float dd = __uint_as_float(dv[h][j]);
-                                const bool in = dd > rowA;
-                                in_m |= (uint32_t)in << j;
-                                near_m |= (uint32_t)(!in && !(dd < thr_near)) << j;
-                            }
                             uint32_t m = in_m | near_m;  // near: decided by the exact predicate
                             // candidates sharing the row's tree node need no test; nor do ids
                             // that cannot lower the row's label
@@ -838,8 +837,7 @@ __global__ void __launch_bounds__(kTile) k_tc_hd(HdView<float, DP> v, Tables tt)
             // this window's tallies (a row that reached MINPTS here stopped early: it is core);
             // the last of the row's windows decides it, as below
             if (have) {
-                atomicAdd(tt.rc_in + rk, cnt);
-                atomicAdd(tt.rc_hi + rk, cnt_hi);
+                atomicAdd(tt.rc_in + rk, cnt);  // (rc_hi has its share already)
                 __threadfence();
                 if (atomicAdd(tt.rc_done + rk, 1u) == nw - 1u) {
                     __threadfence();
@@ -851,6 +849,7 @@ __global__ void __launch_bounds__(kTile) k_tc_hd(HdView<float, DP> v, Tables tt)
                         v.tc_pos[p] = 0u;
                     }
                     v.core[p] = undecided ? 2 : (is_core ? 1 : 0);
+                    if (v.nl_k) v.nl_cnt[p] = up;
                     if (is_core) v.cell_core[A] = 1;
                 }
             }
@@ -863,6 +862,7 @@ __global__ void __launch_bounds__(kTile) k_tc_hd(HdView<float, DP> v, Tables tt)
             }
             const bool is_core = have && !handed && cnt >= G.min_pts;
             if (have) v.core[p] = handed ? 2 : (is_core ? 1 : 0);
+            if (have && v.nl_k) v.nl_cnt[p] = cnt_hi;
             // the unions of a cell may run on the CUDA cores (fewer core rows than points)
             if (__syncthreads_or(is_core) && tid == 0) v.cell_core[A] = 1;
         } else if (MODE == kLabels) {
@@ -893,49 +893,6 @@ __global__ void __launch_bounds__(kTile) k_tc_hd(HdView<float, DP> v, Tables tt)
 
 __device__ __forceinline__ uint32_t tc_chunks(uint32_t rows, uint32_t min_rows) {
     return rows >= min_rows ? (rows + (uint32_t)kTile - 1u) / (uint32_t)kTile : 0u;
-}
-
-// The one root of every coarse cell's core points (~0 when they differ or there are none),
-// with read-only finds (nothing hooks meanwhile), in three launches so that a cell of
-// thousands of points is spread over many warps: clear, one warp per 32-point chunk folding
-// its core points' roots into the cell's smallest (lo) and largest (hi) root, then per cell
-// lo if lo == hi.
-static __global__ void __launch_bounds__(256) k_tc_cell_root_clear(const DevCounters *ctr, uint32_t *__restrict__ lo,
-                                                                  uint32_t *__restrict__ hi) {
-    const uint32_t C = ctr->n_cells;
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
-        lo[c] = 0xffffffffu;
-        hi[c] = 0u;
-    }
-}
-
-template <int DP>
-__global__ void __launch_bounds__(256) k_tc_cell_root(HdView<float, DP> v, uint32_t *__restrict__ lo,
-                                                     uint32_t *__restrict__ hi) {
-    const int lane = threadIdx.x & 31;
-    const uint32_t C = v.ctr->n_cells, NC = v.ctr->n_chunks;
-    const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
-    for (uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < NC; t += warps) {
-        const uint32_t A = chunk_cell(v.chunk_off, C, t);
-        const uint32_t e = v.cell_start[A + 1], p = v.cell_start[A] + 32u * (t - v.chunk_off[A]) + lane;
-        uint32_t mn = 0xffffffffu, mx = 0u;
-        if (p < e && v.core[p]) {
-            mn = mx = uf_root_readonly(v.parent, p, v.ctr);
-        }
-        mn = __reduce_min_sync(0xffffffffu, mn);
-        mx = __reduce_max_sync(0xffffffffu, mx);
-        if (lane == 0 && mn != 0xffffffffu) {
-            atomicMin(lo + A, mn);
-            atomicMax(hi + A, mx);
-        }
-    }
-}
-
-static __global__ void __launch_bounds__(256) k_tc_cell_root_final(const DevCounters *ctr, uint32_t *__restrict__ lo,
-                                                                  const uint32_t *__restrict__ hi) {
-    const uint32_t C = ctr->n_cells;
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x)
-        if (lo[c] != hi[c]) lo[c] = 0xffffffffu;
 }
 
 // 128-row chunks of the counts for every coarse cell with at least min_rows points.
@@ -995,34 +952,32 @@ static __global__ void __launch_bounds__(256) k_tc_partition(const uint8_t *__re
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t x = cx[j];
         if (core[j]) core_list[x] = (uint32_t)j;
-        else nc_list[(uint32_t)j - x] = (uint32_t)j;
+        else if (nc_list) nc_list[(uint32_t)j - x] = (uint32_t)j;
     }
 }
 
 // Work items of every coarse cell: for the unions, 128-row chunks of core rows (first launch)
-// and those chunks times the windows after the first (second launch); for the labels, 128-row
-// chunks of non-core rows.
-static __global__ void __launch_bounds__(256) k_tc_chunks_split(const uint32_t *__restrict__ cell_start,
-                                                               const uint32_t *__restrict__ cx, const DevCounters *ctr,
-                                                               const uint2 *__restrict__ ranges, int n_half, int n_all,
-                                                               uint32_t min_core, uint32_t min_nc,
-                                                               uint32_t *__restrict__ nch_core,
-                                                               uint32_t *__restrict__ nch_later,
-                                                               uint32_t *__restrict__ nch_nc) {
-    const uint32_t C = ctr->n_cells;
+// and those chunks times the windows after the first (second launch), none for a cell that has
+// nothing left to join; for the labels, 128-row chunks of non-core rows.
+template <int DP>
+__global__ void __launch_bounds__(256) k_tc_chunks_split(HdView<float, DP> v, uint32_t min_core, uint32_t min_nc,
+                                                        uint32_t *__restrict__ nch_core,
+                                                        uint32_t *__restrict__ nch_later,
+                                                        uint32_t *__restrict__ nch_nc) {
+    const uint32_t C = v.ctr->n_cells;
     for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
-        const uint32_t s = cell_start[c], e = cell_start[c + 1];
-        const uint32_t nc = cx[e] - cx[s];
-        const uint32_t chunks = tc_chunks(nc, min_core);
-        uint32_t later = 0;
+        const uint32_t s = v.cell_start[c], e = v.cell_start[c + 1];
+        const uint32_t nc = v.cx[e] - v.cx[s];
+        uint32_t chunks = tc_chunks(nc, min_core), later = 0;
         if (chunks) {
             uint32_t len = 0;
-            for (int k = 0; k < n_half; ++k) len += merge_range_len(ranges, n_all, cell_start, cx, c, k);
-            later = chunks * (merge_windows(len) - 1u);
+            for (int k = 0; k < v.n_half; ++k) len += merge_range_len(v, c, k);
+            if (len) later = chunks * (merge_windows(len) - 1u);
+            else chunks = 0;
         }
         nch_core[c] = chunks;
         nch_later[c] = later;
-        nch_nc[c] = tc_chunks(e - s - nc, min_nc);
+        if (nch_nc) nch_nc[c] = tc_chunks(e - s - nc, min_nc);
     }
 }
 
