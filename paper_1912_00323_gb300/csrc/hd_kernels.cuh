@@ -822,37 +822,138 @@ __global__ void __launch_bounds__(256) k_list_link(HdView<T, DP> v) {
     }
 }
 
-// The other edges of the lists.
-template <typename T, int DP>
-__global__ void __launch_bounds__(256) k_list_join(HdView<T, DP> v) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t p = (uint32_t)j;
-        if (!v.core[p]) continue;
-        if (v.tc_min[1] && !v.tc_hook) {
-            const uint32_t A = v.cell_of[p];
-            if (v.cx[v.cell_start[A + 1]] - v.cx[v.cell_start[A]] >= v.tc_min[1]) continue;
-        }
-        const uint32_t len = min(v.nl_cnt[p], v.nl_k);
-        uint32_t rp = uf_find(v.parent, p, v.ctr);
-        for (uint32_t i = 0; i < len; i += 4) {
-            const uint4 e4 = list4(v, p, i);
-            const uint32_t e[4] = {e4.x, e4.y, e4.z, e4.w};
-#pragma unroll
-            for (int u = 0; u < 4; ++u) {
-                if (i + u >= len || (e[u] & kListNear) || !v.core[e[u]]) continue;
-                if (uf_find(v.parent, e[u], v.ctr) == rp) continue;
-                uf_union(v.parent, p, e[u], v.ctr);
-                rp = uf_find(v.parent, p, v.ctr);
-            }
-        }
-    }
-}
-
 // Read-only finds: parent[p] = root (nothing hooks meanwhile).
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_flatten_hd(HdView<T, DP> v) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += (int64_t)gridDim.x * blockDim.x)
         if (v.core[j]) v.parent[j] = uf_root_readonly(v.parent, (uint32_t)j, v.ctr);
+}
+
+// Four list entries of one point and its tree against theirs (k_list_hook, k_list_join): the tree
+// nodes of the point (rp) and of the entries (r[u], rp itself where there is no edge).
+template <typename V>
+__device__ __forceinline__ void load_edges(const V &v, int64_t j, int64_t m, uint32_t &rp, uint32_t (&r)[4]) {
+    const uint32_t quads = v.nl_k / 4;
+    const uint32_t p = (uint32_t)(min(j, m - 1) / quads), i = 4u * (uint32_t)(j % quads);
+    uint32_t len = j < m && v.core[p] ? min(v.nl_cnt[p], v.nl_k) : 0u;
+    if (len > i && v.tc_min[1] && !v.tc_hook) {
+        const uint32_t A = v.cell_of[p];
+        if (v.cx[v.cell_start[A + 1]] - v.cx[v.cell_start[A]] >= v.tc_min[1]) len = 0u;
+    }
+    const uint4 e4 = len > i ? list4(v, p, i) : make_uint4(p, p, p, p);
+    const uint32_t e[4] = {e4.x, e4.y, e4.z, e4.w};
+    rp = __ldcg(v.parent + p);
+    bool c[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
+        const bool ok = i + u < len && !(e[u] & kListNear);
+        const uint32_t q = ok ? e[u] : p;
+        c[u] = ok && v.core[q];
+        r[u] = __ldcg(v.parent + q);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u)
+        if (!c[u]) r[u] = rp;
+}
+
+// The other edges of the lists, one thread per four entries, in two passes.  The first puts every
+// tree below the smallest tree that one of its edges leads to: one minimum per edge between two
+// trees, nothing waited for, and of two minima on one root the larger is lost.  The second
+// joins what that left.  Joining at once is bound by the roots that everybody wants: when it
+// starts, the large trees have thousands of edges between them, and every one of them tries to
+// hook the same root.
+template <typename T, int DP>
+__global__ void __launch_bounds__(256) k_list_hook(HdView<T, DP> v) {
+    const int64_t m = v.g.n * (v.nl_k / 4);
+    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
+        uint32_t rp, r[4];
+        load_edges(v, j, m, rp, r);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            const uint32_t lo = min(rp, r[u]), hi = max(rp, r[u]);
+            if (lo != hi && __ldcg(v.parent + hi) > lo) atomicMin(v.parent + hi, lo);
+        }
+    }
+}
+
+template <typename T, int DP>
+__global__ void __launch_bounds__(256) k_list_join(HdView<T, DP> v) {
+    const uint32_t lane = lane_id();
+    const int64_t m = v.g.n * (v.nl_k / 4);
+    for (int64_t jb = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); jb < m; jb += (int64_t)gridDim.x * blockDim.x) {
+        uint32_t rp, r[4];
+        load_edges(v, jb + lane, m, rp, r);
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+            bool need = r[u] != rp;
+            if (!__any_sync(0xffffffffu, need)) continue;
+            if (need) {
+                rp = uf_root_readonly(v.parent, rp, v.ctr);
+                r[u] = uf_root_readonly(v.parent, r[u], v.ctr);
+                need = r[u] != rp;
+            }
+            // the lanes with the same two roots leave the join to one of them
+            const unsigned active = __ballot_sync(0xffffffffu, need);
+            if (!need) continue;
+            const uint32_t lo = min(rp, r[u]), hi = max(rp, r[u]);
+            const unsigned same = __match_any_sync(active, (unsigned long long)hi << 32 | lo);
+            if ((int)lane == __ffs(same) - 1) uf_join_readonly(v.parent, lo, hi, v.ctr);
+        }
+    }
+}
+
+// One edge for every pair of neighbouring cells (upper half) whose first core points are in
+// different trees: the first 32 points of one against the first 32 of the other.  The lists
+// of a dense cluster hold the first points of the stream, so they join its points along each
+// pencil but hardly across pencils; between dense cells nearly every such sample has an edge.
+template <typename T, int DP, bool FILTER>
+__global__ void __launch_bounds__(32 * kHdMaxWarps) k_cell_link(HdView<T, DP> v) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    typedef Candidate<T, DP, FILTER> Cand;
+    typedef typename Cand::Row R;
+    R *rows = reinterpret_cast<R *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
+    const int lane = lane_id();
+    const uint64_t N = (uint64_t)v.ctr->n_cells * v.n_half;  // one warp per cell and neighbour pencil
+    for (uint64_t w = global_warp(); w < N; w += total_warps()) {
+        const uint32_t A = (uint32_t)(w / v.n_half);
+        const int kk = (int)(w % v.n_half);
+        if (!v.cell_core[A]) continue;
+        const uint2 rg = v.ranges[(uint64_t)A * v.n_all + kk];
+        const uint32_t lo = kk == 0 ? A + 1 : rg.x;
+        if (lo >= rg.y) continue;
+        const uint32_t s = v.cell_start[A], e = min(v.cell_start[A + 1], s + 32u), p = s + lane;
+        const bool pc = p < e && v.core[p];
+        const unsigned amask = __ballot_sync(0xffffffffu, pc);
+        if (!amask) continue;
+        const uint32_t a0 = s + (uint32_t)__ffs(amask) - 1u;
+        const GridParams &G = params_of(v, set_of_key(v, v.cell_key[A]));
+        bool staged = false;
+        for (uint32_t B = lo; B < rg.y; ++B) {
+            if (!v.cell_core[B]) continue;
+            const uint32_t q = v.cell_start[B] + lane;
+            const bool qc = q < v.cell_start[B + 1] && v.core[q];
+            const unsigned bmask = __ballot_sync(0xffffffffu, qc);
+            if (!bmask) continue;
+            uint32_t r = 0;  // the roots of the two first core points
+            if (lane == 0) r = uf_find(v.parent, a0, v.ctr);
+            if (lane == 1) r = uf_find(v.parent, v.cell_start[B] + (uint32_t)__ffs(bmask) - 1u, v.ctr);
+            if (__shfl_sync(0xffffffffu, r, 0) == __shfl_sync(0xffffffffu, r, 1)) continue;
+            if (!staged) stage_rows<R, DP>(rows, Cand::src(v), s, e);
+            staged = true;
+            Cand qv;
+            qv.load(v, q, qc);
+            unsigned rem = amask;
+            while (rem) {
+                const int jj = __ffs(rem) - 1;
+                rem &= rem - 1;
+                const unsigned hm = __ballot_sync(0xffffffffu, qc && qv.within(v, rows + jj * DP, s + jj, G));
+                if (!hm) continue;
+                if (lane == __ffs(hm) - 1) uf_union(v.parent, s + jj, q, v.ctr);
+                break;
+            }
+        }
+        __syncwarp();
+    }
 }
 
 // The tree of a cell: the smallest root among its core points.  A tree's root is its smallest

@@ -156,7 +156,13 @@ struct HdLaunch {
 template <typename T, int DP, bool FILTER>
 void run_list_unions(HdView<T, DP> &hv, const HdLaunch &L, int &launches) {
     k_list_link<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
-    if (hv.nl_k) k_list_join<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+    if (hv.nl_k) {
+        k_flatten_hd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+        k_list_hook<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+        k_flatten_hd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+        k_list_join<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+        k_cell_link<T, DP, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
+    }
     k_flatten_hd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
     k_cell_root_clear<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
     k_cell_root<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
@@ -164,7 +170,7 @@ void run_list_unions(HdView<T, DP> &hv, const HdLaunch &L, int &launches) {
     k_cell_mixed<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
     k_odd_hd<T, DP, false, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
     k_odd_hd<T, DP, true, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
-    launches += hv.nl_k ? 9 : 8;
+    launches += hv.nl_k ? 13 : 8;
 }
 
 // The three point phases on the CUDA cores: counts (Definition 2), unions (Definitions 3-5) and
@@ -173,6 +179,7 @@ template <typename T, int DP, bool FILTER, typename Mark>
 void run_cuda_phases(HdView<T, DP> &hv, const HdLaunch &L, int64_t n, Mark &mark, int &launches) {
     detail::allow_smem(k_count_hd<T, DP, false, FILTER>, L.smem);
     detail::allow_smem(k_count_hd<T, DP, true, FILTER>, L.smem);
+    detail::allow_smem(k_cell_link<T, DP, FILTER>, L.smem);
     detail::allow_smem(k_odd_hd<T, DP, false, FILTER>, L.smem);
     detail::allow_smem(k_odd_hd<T, DP, true, FILTER>, L.smem);
     detail::allow_smem(k_merge_hd<T, DP, FILTER>, L.smem);
@@ -224,6 +231,7 @@ void run_tc_phases(HdView<float, DP> &hv, const HdLaunch &L, char *b, int64_t n,
     hv.tc_pos = flags;  // free until the core numbering
     detail::allow_smem(k_count_hd<float, DP, false, true>, smem);
     detail::allow_smem(k_count_hd<float, DP, true, true>, smem);
+    detail::allow_smem(k_cell_link<float, DP, true>, smem);
     detail::allow_smem(k_odd_hd<float, DP, false, true>, smem);
     detail::allow_smem(k_odd_hd<float, DP, true, true>, smem);
     detail::allow_smem(k_merge_hd<float, DP, true>, smem);

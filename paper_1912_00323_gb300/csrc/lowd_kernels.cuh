@@ -297,6 +297,18 @@ __device__ __forceinline__ void uf_union(uint32_t *parent, uint32_t a, uint32_t 
     set_error(ctr, kErrLoop);
 }
 
+// uf_union with finds that do not write.
+__device__ __forceinline__ void uf_join_readonly(uint32_t *parent, uint32_t a, uint32_t b, DevCounters *ctr) {
+    for (uint32_t it = 0; it < kLoopLimit; ++it) {
+        a = uf_root_readonly(parent, a, ctr);
+        b = uf_root_readonly(parent, b, ctr);
+        if (a == b) return;
+        if (a > b) { uint32_t t = a; a = b; b = t; }
+        if (atomicCAS(parent + b, b, a) == b) return;
+    }
+    set_error(ctr, kErrLoop);
+}
+
 // ------------------------------------------------------------------------------------------
 // Cell boxes and flattened neighbour lists
 // ------------------------------------------------------------------------------------------

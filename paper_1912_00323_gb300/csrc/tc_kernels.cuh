@@ -207,17 +207,11 @@ __device__ __forceinline__ float fmax3(float a, float b, float c) {
     return r;
 }
 
-// Largest of 32 FP32 values, as a tree of three-input maxima (17 instructions, four dependent
-// steps, instead of a chain of 31).
-__device__ __forceinline__ float max32(const uint32_t (&v)[32]) {
-    float a[11];
-#pragma unroll
-    for (int j = 0; j < 10; ++j)
-        a[j] = fmax3(__uint_as_float(v[3 * j]), __uint_as_float(v[3 * j + 1]), __uint_as_float(v[3 * j + 2]));
-    a[10] = fmaxf(__uint_as_float(v[30]), __uint_as_float(v[31]));
-    const float b0 = fmax3(a[0], a[1], a[2]), b1 = fmax3(a[3], a[4], a[5]), b2 = fmax3(a[6], a[7], a[8]);
-    const float b3 = fmaxf(a[9], a[10]);
-    return fmaxf(fmax3(b0, b1, b2), b3);
+// Largest of 8 FP32 values, as three-input maxima.
+__device__ __forceinline__ float max8(const uint32_t *v) {
+    const float a = fmax3(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]));
+    const float b = fmax3(__uint_as_float(v[3]), __uint_as_float(v[4]), __uint_as_float(v[5]));
+    return fmax3(a, b, fmaxf(__uint_as_float(v[6]), __uint_as_float(v[7])));
 }
 
 template <int DP>
@@ -230,8 +224,9 @@ struct Smem {
     float cen[DP];             // the centre c (row 0 of the chunk, original coordinates)
     uint32_t cpay[kTile];      // per candidate: tree node (unions) or cluster id (labels)
     uint32_t cidx[kTile];      // per candidate: list index
-    uint32_t gsum[4];          // per 32 candidates: unions: bit mask of the candidates whose tree node
-                               // differs from ref; labels: the smallest cluster id
+    uint32_t gsum[4];          // labels, per 32 candidates: the smallest cluster id
+    uint2 groot[4][4];         // unions, per 32 candidates: up to four of their tree nodes, each with
+                               // the mask of the candidates below it
     uint32_t rq0[kMaxRng];     // first list index of each span (a neighbour range, or a kept cell)
     uint32_t rpre[kMaxRng + 1];  // stream offset of each span; [kMaxRng] = stream length
     uint32_t bcell[kMaxRng];   // unions, labels: the neighbour cells, range by range
@@ -389,7 +384,7 @@ __device__ __forceinline__ uint32_t stream_index(const uint32_t *rpre, const uin
 //   kLabels: rows = non-core points, candidates = core points of the 27 cells; the row takes
 //            the smallest cluster id among the candidates within eps, else -1.
 template <int DP, int MODE>
-__global__ void __launch_bounds__(kTile) k_tc_hd(HdView<float, DP> v, Tables tt) {
+__global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float, DP> v, Tables tt) {
     constexpr int KP = Smem<DP>::KP;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     Smem<DP> &S = *reinterpret_cast<Smem<DP> *>(smem_raw);
@@ -674,8 +669,12 @@ __global__ void __launch_bounds__(kTile) k_tc_hd(HdView<float, DP> v, Tables tt)
                     continue;
                 }
                 S.cpay[tid] = rq;
-                const unsigned dm = __ballot_sync(0xffffffffu, cin && rq != ref);
-                if ((tid & 31) == 0) S.gsum[warp] = dm;  // read after the barrier of the MMA wait
+                // (read after the barrier of the MMA wait)
+                const unsigned peers = __match_any_sync(0xffffffffu, rq);
+                const unsigned first = __ballot_sync(0xffffffffu, (tid & 31) == __ffs(peers) - 1);
+                const uint32_t slot = (uint32_t)__popc(first & ((1u << (tid & 31)) - 1u));
+                if ((tid & 31) == __ffs(peers) - 1 && slot < 4u) S.groot[warp][slot] = make_uint2(rq, peers);
+                if ((tid & 31) < 4 && (tid & 31) >= __popc(first)) S.groot[warp][tid & 31] = make_uint2(0u, 0u);
             }
             // stage the prefetched block
             {
@@ -737,25 +736,23 @@ __global__ void __launch_bounds__(kTile) k_tc_hd(HdView<float, DP> v, Tables tt)
                     for (int h = 0; h < NH; ++h) {
                         const uint32_t cg = c0 + 32u * (uint32_t)h;
                         if (cg >= nq || !need) continue;
-                        // 32 candidates all proved outside (the common case for the rows that
-                        // scan their whole neighbourhood: noise and border points) cost one
-                        // maximum each instead of the classification
-                        if (MODE == kMerge) {  // the tree's registers push the union loop into spills
-                            float mx = __uint_as_float(dv[h][0]);
-#pragma unroll
-                            for (int j = 1; j < 32; ++j) mx = fmaxf(mx, __uint_as_float(dv[h][j]));
-                            if (mx < thr_near) continue;
-                        } else if (max32(dv[h]) < thr_near) {
-                            continue;
-                        }
+                        // eight candidates all proved outside (the common case: a row of a large
+                        // cluster has a few neighbours among thousands of candidates, and noise
+                        // and border rows hardly any) cost one maximum each instead of the two
+                        // comparisons and mask bits, all on the ALU pipe that bounds the epilogue
                         uint32_t in_m = 0, near_m = 0;
 #pragma unroll
-                        for (int j = 0; j < 32; ++j) {
-                            const float dd = __uint_as_float(dv[h][j]);
-                            const bool in = dd > rowA;
-                            in_m |= (uint32_t)in << j;
-                            near_m |= (uint32_t)(!in && !(dd < thr_near)) << j;
+                        for (int j8 = 0; j8 < 32; j8 += 8) {
+                            if (max8(&dv[h][j8]) < thr_near) continue;
+#pragma unroll
+                            for (int j = j8; j < j8 + 8; ++j) {
+                                const float dd = __uint_as_float(dv[h][j]);
+                                if (!(dd < thr_near)) near_m |= 1u << j;
+                                if (dd > rowA) in_m |= 1u << j;
+                            }
                         }
+                        near_m &= ~in_m;
+                        if (!(in_m | near_m)) continue;
                         if (MODE == kCount) {
                             // cnt: pairs surely within eps (D > rowA); cnt_hi: pairs not proved
                             // outside (D >= thr_near), which take the next entries of the list
@@ -774,7 +771,16 @@ __global__ void __launch_bounds__(kTile) k_tc_hd(HdView<float, DP> v, Tables tt)
                             uint32_t m = in_m | near_m;  // near: decided by the exact predicate
                             // candidates sharing the row's tree node need no test; nor do ids
                             // that cannot lower the row's label
-                            if (MODE == kMerge && rp == ref) m &= S.gsum[cg >> 5];
+                            if (MODE == kMerge) {
+                                // (a tile of two clusters' points has hundreds of pairs inside
+                                // either tree: one comparison per node drops them, where the loop
+                                // below took 10 us a tile)
+#pragma unroll
+                                for (int k2 = 0; k2 < 4; ++k2) {
+                                    const uint2 gr = S.groot[cg >> 5][k2];
+                                    if (gr.x == rp) m &= ~gr.y;
+                                }
+                            }
                             if (MODE == kLabels && S.gsum[cg >> 5] >= best) m = 0;
                             while (m) {
                                 const int j = __ffs(m) - 1;
