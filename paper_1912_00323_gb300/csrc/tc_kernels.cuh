@@ -147,6 +147,26 @@ __device__ __forceinline__ void mma_tf32(uint32_t d_tmem, uint64_t a, uint64_t b
         "l"(a), "l"(b), "r"(idesc), "r"(acc));
 }
 
+// The MMAs of a 128 x 128 tile: hi.hi + hi.lo + lo.hi per coordinate step, and hi.hi of the threshold
+// step.  The operands' descriptors differ by a constant per step (2 kLBO bytes), so the issuing
+// thread only adds: building each descriptor from its address took it 650 cycles a tile, with
+// the CTA waiting behind it.
+struct TileDesc {
+    uint64_t ah, al, bh, bl;  // step 0 of the four operands
+};
+template <int DP>
+__device__ __forceinline__ void mma_tile(uint32_t d, const TileDesc &t, uint32_t idesc) {
+#pragma unroll
+    for (int ks = 0; ks < DP / 8 + 1; ++ks) {
+        const uint64_t o = (uint64_t)(ks * 2 * kLBO >> 4);
+        mma_tf32(d, t.ah + o, t.bh + o, idesc, ks > 0 ? 1u : 0u);
+        if (ks < DP / 8) {  // the threshold columns have no lo parts
+            mma_tf32(d, t.ah + o, t.bl + o, idesc, 1u);
+            mma_tf32(d, t.al + o, t.bh + o, idesc, 1u);
+        }
+    }
+}
+
 __device__ __forceinline__ void mma_commit(uint32_t mbar) {
     asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(mbar)
                  : "memory");
@@ -200,18 +220,59 @@ __device__ __forceinline__ void reg_tie(uint32_t (&v)[32]) {
                  : "memory");
 }
 
-// Three-input maximum (PTX max.f32 with three sources).
-__device__ __forceinline__ float fmax3(float a, float b, float c) {
+// Three-input minimum of magnitudes (PTX min.f32 with three sources).
+__device__ __forceinline__ float fmin3_abs(float a, float b, float c) {
     float r;
-    asm("max.f32 %0, %1, %2, %3;" : "=f"(r) : "f"(a), "f"(b), "f"(c));
+    asm("{\n .reg .f32 x, y;\n abs.f32 x, %2;\n abs.f32 y, %3;\n min.f32 %0, %1, x, y;\n}" : "=f"(r) : "f"(a), "f"(b), "f"(c));
     return r;
 }
 
-// Largest of 8 FP32 values, as three-input maxima.
-__device__ __forceinline__ float max8(const uint32_t *v) {
-    const float a = fmax3(__uint_as_float(v[0]), __uint_as_float(v[1]), __uint_as_float(v[2]));
-    const float b = fmax3(__uint_as_float(v[3]), __uint_as_float(v[4]), __uint_as_float(v[5]));
-    return fmax3(a, b, fmaxf(__uint_as_float(v[6]), __uint_as_float(v[7])));
+// The two thresholds of a row as classify32 takes them: the middle between them and half their
+// distance, rounded up by more than the rounding of the middle and of a difference from it.
+struct RowTest {
+    float row_a, thr_near, mid, half;
+    __device__ __forceinline__ RowTest(float a, float t) : row_a(a), thr_near(t) {
+        mid = 0.5f * (a + t);
+        half = 0.5f * (a - t) * (1.0f + 0x1p-18f) + fabsf(mid) * 0x1p-21f;
+    }
+};
+
+// The 32 values of one load against a row's thresholds: bit j of `in` = pair surely within eps
+// (value > row_a), of `near` = neither that nor proved outside (value >= thr_near).  No branch but
+// for a value between the thresholds: the signs of the differences from the middle are collected
+// into the mask (a packed subtraction per two values, one funnel shift each, four chains of eight),
+// and the smallest difference tells whether a value lies between (one three-input minimum
+// per two).  Of 32 values of 32 rows one is usually inside, so skipping the ones below by
+// branches or votes leaves the warp waiting instead (a tile of the counts took 2.9 us a CTA
+// with eight values per branch, 2.4 us with two tallies and no masks).
+__device__ __forceinline__ void classify32(const uint32_t (&v)[32], const RowTest &t, uint32_t &in, uint32_t &near) {
+    const unsigned long long mid2 = (unsigned long long)__float_as_uint(t.mid) << 32 | __float_as_uint(t.mid);
+    uint32_t m[4] = {0u, 0u, 0u, 0u};
+    float least[4] = {3.0e38f, 3.0e38f, 3.0e38f, 3.0e38f};
+#pragma unroll
+    for (int j = 6; j >= 0; j -= 2) {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+            const unsigned long long x = (unsigned long long)v[8 * c + j + 1] << 32 | v[8 * c + j];
+            unsigned long long y;
+            asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(y) : "l"(x), "l"(mid2));
+            const uint32_t y0 = (uint32_t)y, y1 = (uint32_t)(y >> 32);
+            m[c] = __funnelshift_l(y1, m[c], 1);
+            m[c] = __funnelshift_l(y0, m[c], 1);
+            least[c] = fmin3_abs(least[c], __uint_as_float(y0), __uint_as_float(y1));
+        }
+    }
+    in = ~(m[0] | m[1] << 8 | m[2] << 16 | m[3] << 24);
+    near = 0u;
+    if (fminf(fminf(least[0], least[1]), fminf(least[2], least[3])) <= t.half) {
+        in = 0u;
+#pragma unroll
+        for (int j = 0; j < 32; ++j) {
+            const float d = __uint_as_float(v[j]);
+            in |= (uint32_t)(d > t.row_a) << j;
+            near |= (uint32_t)(!(d > t.row_a) && !(d < t.thr_near)) << j;
+        }
+    }
 }
 
 template <int DP>
@@ -235,7 +296,7 @@ struct Smem {
     uint32_t cell, nwin;       // the item's coarse cell; unions: windows per chunk of it
     uint32_t la[3], pad3;      // unions: blocks of a look-ahead round not skippable (rotating)
     uint64_t mbar;
-    uint32_t taddr, ref, next, pad;
+    uint32_t taddr, ref, next, fail;
 };
 
 template <int DP>
@@ -246,16 +307,16 @@ inline size_t smem_bytes() {
 // FP32 value truncated to TF32 (10 stored mantissa bits); x - tf32_trunc(x) is exact in FP32.
 __device__ __forceinline__ float tf32_trunc(float x) { return __uint_as_float(__float_as_uint(x) & 0xFFFFE000u); }
 
-// Centre a row (4 coordinates per float4) on c, split it into TF32 hi and lo parts, store both
-// in the operand layout (columns [0, DP) of KP) and return the squared norm (FP32) of the
-// centred row; an invalid row becomes the zero row.
-template <int DP, int KP>
-__device__ __forceinline__ float stage_split(float *hi_op, float *lo_op, int row, const float4 (&q)[DP / 4],
-                                             const float *c, bool valid) {
+// Centre the coordinates [k0, k0 + 4 N) of a row (4 per float4) on c, split them into TF32 hi and lo
+// parts, store both in the operand layout of KP columns and return the squared norm (FP32) of
+// what is left; an invalid row becomes zero.
+template <int KP, int N>
+__device__ __forceinline__ float stage_coords(float *hi_op, float *lo_op, int row, int k0, const float4 (&q)[N],
+                                              const float4 (&c)[N], bool valid) {
     float nrm = 0.f;
 #pragma unroll
-    for (int k = 0; k < DP / 4; ++k) {
-        const float4 cc = *reinterpret_cast<const float4 *>(c + 4 * k);
+    for (int k = 0; k < N; ++k) {
+        const float4 cc = c[k];
         float4 w = make_float4(0.f, 0.f, 0.f, 0.f);
         if (valid) {
             w.x = __fsub_rn(q[k].x, cc.x);
@@ -269,23 +330,43 @@ __device__ __forceinline__ float stage_split(float *hi_op, float *lo_op, int row
         nrm = __fmaf_rn(w.w, w.w, nrm);
         const float4 h = make_float4(tf32_trunc(w.x), tf32_trunc(w.y), tf32_trunc(w.z), tf32_trunc(w.w));
         const float4 l = make_float4(__fsub_rn(w.x, h.x), __fsub_rn(w.y, h.y), __fsub_rn(w.z, h.z), __fsub_rn(w.w, h.w));
-        const uint32_t off = op_offset<KP>(row, 4 * k);
+        const uint32_t off = op_offset<KP>(row, k0 + 4 * k);
         *reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(hi_op) + off) = h;
         *reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(lo_op) + off) = l;
     }
     return nrm;
 }
 
+// A whole row of DP coordinates, the centre in registers or in shared memory; part of a row.
+template <int DP, int KP>
+__device__ __forceinline__ float stage_split_c(float *hi_op, float *lo_op, int row, const float4 (&q)[DP / 4],
+                                               const float4 (&c)[DP / 4], bool valid) {
+    return stage_coords<KP, DP / 4>(hi_op, lo_op, row, 0, q, c, valid);
+}
+template <int KP, int N>
+__device__ __forceinline__ float stage_part(float *hi_op, float *lo_op, int row, int k0, const float4 (&q)[N],
+                                            const float *c, bool valid) {
+    float4 cc[N];
+#pragma unroll
+    for (int k = 0; k < N; ++k) cc[k] = *reinterpret_cast<const float4 *>(c + 4 * k);
+    return stage_coords<KP, N>(hi_op, lo_op, row, k0, q, cc, valid);
+}
+template <int DP, int KP>
+__device__ __forceinline__ float stage_split(float *hi_op, float *lo_op, int row, const float4 (&q)[DP / 4],
+                                             const float *c, bool valid) {
+    return stage_part<KP, DP / 4>(hi_op, lo_op, row, 0, q, c, valid);
+}
+
 // Columns [DP, DP + 8) of the hi operand, set once per CTA: the rows' (1, 1, 0, ...) and the
 // candidates' trailing zeros (columns DP + 4 .. DP + 7).  The lo operands' threshold columns
 // are never read (the threshold K step multiplies the hi parts only).
 template <int DP, int KP>
-__device__ __forceinline__ void stage_extra_const(float *a_hi, float *b_hi, int row) {
+__device__ __forceinline__ void stage_extra_const(float *a_hi, float *b_hi, int row, int b_row) {
     const float4 z = make_float4(0.f, 0.f, 0.f, 0.f);
     const uint32_t o0 = op_offset<KP>(row, DP), o1 = op_offset<KP>(row, DP + 4);
     *reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(a_hi) + o0) = make_float4(1.f, 1.f, 0.f, 0.f);
     *reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(a_hi) + o1) = z;
-    *reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(b_hi) + o1) = z;
+    *reinterpret_cast<float4 *>(reinterpret_cast<unsigned char *>(b_hi) + op_offset<KP>(b_row, DP + 4)) = z;
 }
 
 // The candidate's threshold columns: (-colA_hi, -colA_lo, 0, 0) at columns DP .. DP + 3.
@@ -393,19 +474,22 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
     if (tid == 0) {
         asm volatile("mbarrier.init.shared::cta.b64 [%0], 1;" ::"r"(mbar));
         asm volatile("fence.mbarrier_init.release.cluster;");
+        S.fail = 0u;
     }
     if (warp == 0) {
         asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&S.taddr)),
                      "r"(kTile));
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;");
     }
-    stage_extra_const<DP, KP>(S.a_hi, S.b_hi, tid);  // made visible to the MMA by each block's proxy fence
+    stage_extra_const<DP, KP>(S.a_hi, S.b_hi, tid, tid);  // made visible to the MMA by each block's proxy fence
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
     const uint32_t taddr = S.taddr;
     const uint32_t t_lane = taddr + ((uint32_t)(warp * 32) << 16);
     const uint32_t idesc = idesc_tf32();
+    const TileDesc td = {smem_desc<KP>(smem_u32(S.a_hi)), smem_desc<KP>(smem_u32(S.a_lo)),
+                         smem_desc<KP>(smem_u32(S.b_hi)), smem_desc<KP>(smem_u32(S.b_lo))};
     const bool recount = MODE == kCount && tt.row_list != nullptr;
     const uint32_t C = v.ctr->n_cells, N0 = recount ? v.ctr->n_tc_recount : v.ctr->n_tc_chunks[MODE];
     uint32_t *const next = recount ? &v.ctr->tc_next_recount : &v.ctr->tc_next[MODE];
@@ -597,6 +681,7 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
         const float hi = (float)(G.eps2 * (1.0 + 0x1p-20));
         const float rowA = 0.5f * __fsub_rn(__fmul_rn(na, 1.000244140625f), lo);  // (1 + 2^-12) |x|^2
         const float thr_near = __fsub_rn(0.5f * __fsub_rn(na, hi), 0x1p-11f * __fadd_rn(na, hi));
+        const RowTest rt(rowA, thr_near);
         uint32_t cnt = 0, cnt_hi = 0, rp = 0, best = kNoLabel;
         if (MODE == kMerge && have) rp = uf_find(v.parent, p, v.ctr);
         bool done = !have;    // counts: the row surely has MINPTS neighbours
@@ -604,10 +689,19 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
         // registers of the next candidate block (loaded one block ahead)
         uint32_t pre_k = 0, pre_pay = 0;
         bool pre_in = false;
+        // the span of this thread's candidate (positions only grow, so it moves forward from there;
+        // a search in shared memory per block took 600 cycles)
+        int span = -1;
+        uint32_t span_end = 0, span_off = 0;
         auto prefetch = [&](uint32_t ub) {
             const uint32_t u = ub + (uint32_t)tid;
             pre_in = u < L;
-            pre_k = pre_in ? stream_index(S.rpre, S.rq0, nspan, u) : 0u;
+            while (pre_in && u >= span_end) {  // L is the end of the last span or below it
+                ++span;
+                span_end = span + 1 < nspan ? S.rpre[span + 1] : S.rpre[kMaxRng];
+                span_off = S.rq0[span] - S.rpre[span];
+            }
+            pre_k = pre_in ? span_off + u : 0u;
             // past the stream: list index 0 (a valid point), zeroed when staged; the loads are
             // not waited for here (no select on their values) but at the staging of the block
             const uint32_t qp = MODE == kCount ? pre_k : __ldg(tt.core_list + pre_k);
@@ -696,37 +790,65 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
             __syncthreads();
             asm volatile("tcgen05.fence::after_thread_sync;");
             if (tid == 0) {
-                const uint32_t ah = smem_u32(S.a_hi), al = smem_u32(S.a_lo);
-                const uint32_t bh = smem_u32(S.b_hi), bl = smem_u32(S.b_lo);
-#pragma unroll
-                for (int ks = 0; ks < KP / 8; ++ks) {
-                    const uint32_t o = ks * 2 * kLBO;
-                    mma_tf32(taddr, smem_desc<KP>(ah + o), smem_desc<KP>(bh + o), idesc, ks > 0 ? 1u : 0u);
-                    if (ks < DP / 8) {  // the threshold columns have no lo parts
-                        mma_tf32(taddr, smem_desc<KP>(ah + o), smem_desc<KP>(bl + o), idesc, 1u);
-                        mma_tf32(taddr, smem_desc<KP>(al + o), smem_desc<KP>(bh + o), idesc, 1u);
-                    }
-                }
+                mma_tile<DP>(taddr, td, idesc);
                 mma_commit(mbar);
             }
             if (ub + kTile < L) prefetch(ub + kTile);  // overlaps the MMA and the classification
-            const bool ok = mbar_wait(mbar, phase);
-            if (__syncthreads_or(!ok)) {
-                failed = true;
-                if (tid == 0) set_error(v.ctr, kErrLoop);
-                break;
-            }
+            if (!mbar_wait(mbar, phase)) *(volatile uint32_t *)&S.fail = 1u;  // read after the block's last barrier
             phase ^= 1u;
             asm volatile("tcgen05.fence::after_thread_sync;");
             ++n_tiles;
             if (tid == 0) n_pairs += (unsigned long long)min((uint32_t)kTile, rend - k0) * nq;
             bool need = have && (MODE != kCount || !done);
-            if (__any_sync(0xffffffffu, need)) {
-                // counts and labels: 64 columns per wait, the second 32 read even past nq
-                // (allocated columns; their values are not used); unions: 32 (the registers
-                // of a second set slowed the union-find loop)
+            if (MODE == kCount && __any_sync(0xffffffffu, need)) {
+                // 64 columns per wait, the second 32 read even past nq (allocated columns; an empty
+                // candidate's value is below every threshold)
+                uint32_t in_m[4] = {0u, 0u, 0u, 0u}, near_m[4] = {0u, 0u, 0u, 0u};
+#pragma unroll
+                for (int c = 0; c < 4; c += 2) {
+                    if (32u * c >= nq) break;
+                    __syncwarp();
+                    uint32_t dv[2][32];
+                    tmem_ld32_issue(t_lane + 32 * c, dv[0]);
+                    tmem_ld32_issue(t_lane + 32 * c + 32, dv[1]);
+                    tmem_ld_wait(dv[0]);
+                    reg_tie(dv[1]);
+                    classify32(dv[0], rt, in_m[c], near_m[c]);
+                    classify32(dv[1], rt, in_m[c + 1], near_m[c + 1]);
+                }
+                uint32_t m_in = 0, found = 0;
+#pragma unroll
+                for (int c = 0; c < 4; ++c) {
+                    m_in += (uint32_t)__popc(in_m[c]);
+                    found += (uint32_t)__popc(in_m[c] | near_m[c]);
+                }
+                if (need && found) {
+                    // cnt: pairs surely within eps; cnt_hi: pairs not proved outside, which take the
+                    // next entries of the list
+                    uint32_t at = recount ? atomicAdd(tt.rc_hi + rk, found) : cnt_hi;
+                    cnt += m_in;
+                    cnt_hi += found;
+                    // (one loop over the 128 columns: its trip count is the most hits of a lane)
+                    unsigned long long m0 = (unsigned long long)(in_m[1] | near_m[1]) << 32 | in_m[0] | near_m[0];
+                    unsigned long long m1 = (unsigned long long)(in_m[3] | near_m[3]) << 32 | in_m[2] | near_m[2];
+                    const unsigned long long n0 = (unsigned long long)near_m[1] << 32 | near_m[0];
+                    const unsigned long long n1 = (unsigned long long)near_m[3] << 32 | near_m[2];
+                    for (; at < v.nl_k && (m0 | m1); ++at) {
+                        const bool low = m0 != 0ull;
+                        const unsigned long long m = low ? m0 : m1, n = low ? n0 : n1;
+                        const int j = __ffsll((long long)m) - 1;
+                        if (low) m0 &= m0 - 1ull;
+                        else m1 &= m1 - 1ull;
+                        v.nl[(uint64_t)p * v.nl_k + at] = S.cidx[j + (low ? 0 : 64)] | ((n >> j) & 1ull ? kListNear : 0u);
+                    }
+                }
+            }
+            if (MODE != kCount && __any_sync(0xffffffffu, need)) {
+                // labels: 64 columns per wait; unions: 32 (the registers of a second set slowed the
+                // union-find loop)
                 constexpr int NH = MODE == kMerge ? 1 : 2;
                 for (uint32_t c0 = 0; c0 < nq; c0 += 32u * NH) {
+                    __syncwarp();
                     uint32_t dv[NH][32];
                     tmem_ld32_issue(t_lane + c0, dv[0]);
                     if (NH == 2) tmem_ld32_issue(t_lane + c0 + 32, dv[NH - 1]);
@@ -735,91 +857,68 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
 #pragma unroll
                     for (int h = 0; h < NH; ++h) {
                         const uint32_t cg = c0 + 32u * (uint32_t)h;
-                        if (cg >= nq || !need) continue;
-                        // eight candidates all proved outside (the common case: a row of a large
-                        // cluster has a few neighbours among thousands of candidates, and noise
-                        // and border rows hardly any) cost one maximum each instead of the two
-                        // comparisons and mask bits, all on the ALU pipe that bounds the epilogue
-                        uint32_t in_m = 0, near_m = 0;
+                        if (cg >= nq) break;
+                        uint32_t in_m, near_m;
+                        classify32(dv[h], rt, in_m, near_m);
+                        uint32_t m = need ? in_m | near_m : 0u;  // near: decided by the exact predicate
+                        // candidates sharing the row's tree node need no test; nor do ids
+                        // that cannot lower the row's label
+                        if (MODE == kMerge) {
+                            // (a tile of two clusters' points has hundreds of pairs inside
+                            // either tree: one comparison per node drops them, where the loop
+                            // below took 10 us a tile)
 #pragma unroll
-                        for (int j8 = 0; j8 < 32; j8 += 8) {
-                            if (max8(&dv[h][j8]) < thr_near) continue;
-#pragma unroll
-                            for (int j = j8; j < j8 + 8; ++j) {
-                                const float dd = __uint_as_float(dv[h][j]);
-                                if (!(dd < thr_near)) near_m |= 1u << j;
-                                if (dd > rowA) in_m |= 1u << j;
+                            for (int k2 = 0; k2 < 4; ++k2) {
+                                const uint2 gr = S.groot[cg >> 5][k2];
+                                if (gr.x == rp) m &= ~gr.y;
                             }
                         }
-                        near_m &= ~in_m;
-                        if (!(in_m | near_m)) continue;
-                        if (MODE == kCount) {
-                            // cnt: pairs surely within eps (D > rowA); cnt_hi: pairs not proved
-                            // outside (D >= thr_near), which take the next entries of the list
-                            uint32_t m = in_m | near_m;
-                            const uint32_t found = (uint32_t)__popc(m);
-                            uint32_t at = recount ? atomicAdd(tt.rc_hi + rk, found) : cnt_hi;
-                            cnt += (uint32_t)__popc(in_m);
-                            cnt_hi += found;
-                            for (; m && at < v.nl_k; ++at) {
-                                const int j = __ffs(m) - 1;
-                                m &= m - 1;
-                                v.nl[(uint64_t)p * v.nl_k + at] = S.cidx[cg + (uint32_t)j] | ((in_m >> j) & 1u ? 0u : kListNear);
-                            }
-                            if (cnt >= G.min_pts) need = false;
-                        } else {
-                            uint32_t m = in_m | near_m;  // near: decided by the exact predicate
-                            // candidates sharing the row's tree node need no test; nor do ids
-                            // that cannot lower the row's label
+                        if (MODE == kLabels && S.gsum[cg >> 5] >= best) m = 0;
+                        while (m) {
+                            const int j = __ffs(m) - 1;
+                            m &= m - 1;
+                            const uint32_t col = cg + (uint32_t)j;
+                            const bool inside = (in_m >> j) & 1u;
+                            const uint32_t ck2 = S.cidx[col];
                             if (MODE == kMerge) {
-                                // (a tile of two clusters' points has hundreds of pairs inside
-                                // either tree: one comparison per node drops them, where the loop
-                                // below took 10 us a tile)
-#pragma unroll
-                                for (int k2 = 0; k2 < 4; ++k2) {
-                                    const uint2 gr = S.groot[cg >> 5][k2];
-                                    if (gr.x == rp) m &= ~gr.y;
+                                if (ck2 <= rk || S.cpay[col] == rp) continue;
+                                const uint32_t qp = __ldg(tt.core_list + ck2);
+                                bool hit = inside;
+                                if (!hit) {
+                                    ++n_re;
+                                    hit = within_pts<DP>(v.pts, p, qp, G);
                                 }
-                            }
-                            if (MODE == kLabels && S.gsum[cg >> 5] >= best) m = 0;
-                            while (m) {
-                                const int j = __ffs(m) - 1;
-                                m &= m - 1;
-                                const uint32_t col = cg + (uint32_t)j;
-                                const bool inside = (in_m >> j) & 1u;
-                                const uint32_t ck2 = S.cidx[col];
-                                if (MODE == kMerge) {
-                                    if (ck2 <= rk || S.cpay[col] == rp) continue;
-                                    const uint32_t qp = __ldg(tt.core_list + ck2);
-                                    bool hit = inside;
-                                    if (!hit) {
-                                        ++n_re;
-                                        hit = within_pts<DP>(v.pts, p, qp, G);
-                                    }
-                                    if (hit) {
-                                        uf_union(v.parent, p, qp, v.ctr);
-                                        rp = uf_find(v.parent, p, v.ctr);
-                                        S.cpay[col] = rp;  // now an ancestor of qp too: later rows skip it
-                                    }
-                                } else {
-                                    const uint32_t lq = S.cpay[col];
-                                    if (lq >= best) continue;
-                                    bool hit = inside;
-                                    if (!hit) {
-                                        ++n_re;
-                                        hit = within_pts<DP>(v.pts, p, __ldg(tt.core_list + ck2), G);
-                                    }
-                                    if (hit) best = lq;
+                                if (hit) {
+                                    uf_union(v.parent, p, qp, v.ctr);
+                                    rp = uf_find(v.parent, p, v.ctr);
+                                    S.cpay[col] = rp;  // now an ancestor of qp too: later rows skip it
                                 }
+                            } else {
+                                const uint32_t lq = S.cpay[col];
+                                if (lq >= best) continue;
+                                bool hit = inside;
+                                if (!hit) {
+                                    ++n_re;
+                                    hit = within_pts<DP>(v.pts, p, __ldg(tt.core_list + ck2), G);
+                                }
+                                if (hit) best = lq;
                             }
                         }
                     }
                 }
+                __syncwarp();
             }
             if (MODE == kCount) done = done || cnt >= G.min_pts;
             asm volatile("tcgen05.fence::before_thread_sync;");
+            int open = 0;
+            if (MODE == kCount) open = __syncthreads_count(!done);
+            else __syncthreads();
+            if (*(volatile uint32_t *)&S.fail) {  // uniform: the next wait comes after another barrier
+                failed = true;
+                if (tid == 0) set_error(v.ctr, kErrLoop);
+                break;
+            }
             if (MODE == kCount) {
-                const int open = __syncthreads_count(!done);
                 if (open == 0) break;
                 if (!recount && open <= (int)v.tc_handoff && ub + 2 * kTile < L) {
                     // few rows left and more than one block to go: the recount or the CUDA-core
@@ -834,8 +933,6 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
                     }
                     break;
                 }
-            } else {
-                __syncthreads();
             }
         }
         if (failed) continue;  // the loop head ends this CTA
@@ -882,7 +979,7 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
             }
         }
     }
-    if (failed) mbar_wait(mbar, phase);  // the MMA that did not complete in time, bounded again
+    if (failed) mbar_wait(mbar, phase ^ 1u);  // the MMA that did not complete in time, bounded again
     asm volatile("tcgen05.fence::before_thread_sync;");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;");
