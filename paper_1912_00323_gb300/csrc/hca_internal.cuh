@@ -40,7 +40,8 @@ struct DevCounters {
     uint32_t n_noise;
     uint32_t n_core_cells;  // cells holding a core point (hypercube path)
     uint32_t n_list[3];     // hypercube path: cells to count, cells with core points, cells to label
-    uint64_t minmax_enc[2 * kMaxD];  // order-preserving encodings of min (first kMaxD) / max per dim
+    uint64_t minmax_enc[2 * kMaxD];  // order-preserving encodings per dim: complement of the min's (first
+                                     // kMaxD; so that both halves start at 0 and grow) and the max's
     uint32_t nan_seen;
     uint32_t n_chunks;     // 32-point chunks of the coarse cells (high-dimensional path)
     uint32_t n_tc_chunks[4];  // work items of the tensor-core phases: counts, unions (the first window of
@@ -111,12 +112,8 @@ struct Workspace {
 // Primitives implemented in sort.cu / scan.cu
 // ---------------------------------------------------------------------------------------
 
-// Exclusive scan of uint32 in[0, m) into out[0, m); total into *total (device, may be null).
-// If m_dev is non-null the length is min(*m_dev, m_max); elements past it are left untouched.
-// partials: device scratch of scan_partials_size(m_max) uint32.
+// Scratch words of cells_from_flags for m_max elements.
 size_t scan_partials_size(int64_t m_max);
-void exclusive_scan_u32(const uint32_t *in, uint32_t *out, int64_t m_max, const uint32_t *m_dev,
-                        uint32_t *total, uint32_t *partials, cudaStream_t s, int *launches);
 
 // Elements per tile of the scan (the tile sums in `partials` are per this many elements).
 constexpr int kScanTileElems = 2048;
@@ -154,12 +151,12 @@ constexpr size_t sort_hist_elems(int64_t n) {
 inline size_t sort_hist_size(int64_t n) { return sort_hist_elems(n); }
 uint32_t *sort_status_word(uint32_t *hist, int64_t n);
 // digit_counts (optional, device): counts of every 8-bit digit of every pass, [pass][256],
-// already computed by the caller.
+// already computed by the caller.  hist_cleared: the caller has cleared hist.
 template <typename K>
 bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, int64_t n,
                       int begin_bit, int end_bit, uint32_t *hist, uint32_t *partials,
                       cudaStream_t s, int *launches, uint32_t *err_out = nullptr,
-                      const uint32_t *digit_counts = nullptr);
+                      const uint32_t *digit_counts = nullptr, bool hist_cleared = false);
 
 // Pool allocation (stream ordered) used by api.cu and the pipelines.
 cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t s);

@@ -293,8 +293,8 @@ __device__ __forceinline__ bool cell_far(const HdView<double, DP> &v, const type
     return box_far<DP>(row, lo + (uint64_t)B * DP, hi + (uint64_t)B * DP, g);
 }
 
-// Declared extents of a plan against the measured ones (encoded min of dimension i of set s at
-// mm[s * 64 + i], max at mm[(nsets + s) * 64 + i]; boxes: mins [s * d + i], maxes
+// Declared extents of a plan against the measured ones (complement of the encoded min of dimension
+// i of set s at mm[s * 64 + i], encoded max at mm[(nsets + s) * 64 + i]; boxes: mins [s * d + i], maxes
 // [(nsets + s) * d + i]): a point outside its box, or a NaN, sets status bit kErrBox.
 static __global__ void __launch_bounds__(256) k_box_check_hd(const double *__restrict__ boxes, int nsets, int d,
                                                             const int64_t *__restrict__ set_off,
@@ -305,7 +305,7 @@ static __global__ void __launch_bounds__(256) k_box_check_hd(const double *__res
          k += (int64_t)gridDim.x * blockDim.x) {
         const int set = (int)(k / d), i = (int)(k % d);
         if (set_off && set_off[set + 1] == set_off[set]) continue;
-        const double lo = dec_double_dev(mm[(size_t)set * 64 + i]);
+        const double lo = dec_double_dev(~mm[(size_t)set * 64 + i]);
         const double hi = dec_double_dev(mm[((size_t)nsets + set) * 64 + i]);
         if (lo < boxes[(size_t)set * d + i] || hi > boxes[((size_t)nsets + set) * d + i])
             atomicOr(&ctr->status, kErrBox);
@@ -323,7 +323,7 @@ __global__ void __launch_bounds__(256) k_minmax_rt(const T *__restrict__ in, int
     __shared__ unsigned long long smn[64], smx[64];
     __shared__ int snan;
     for (int i = threadIdx.x; i < 64; i += blockDim.x) {
-        smn[i] = ~0ull;
+        smn[i] = 0ull;  // complements of minima, so that both grow from 0
         smx[i] = 0ull;
     }
     if (threadIdx.x == 0) snan = 0;
@@ -364,22 +364,44 @@ __global__ void __launch_bounds__(256) k_minmax_rt(const T *__restrict__ in, int
             mx[0] = mx[u] > mx[0] ? mx[u] : mx[0];
         }
         const int dim = (int)(tid % d);
-        atomicMin(&smn[dim], (unsigned long long)enc_double((double)mn[0]));
+        atomicMax(&smn[dim], ~(unsigned long long)enc_double((double)mn[0]));
         atomicMax(&smx[dim], (unsigned long long)enc_double((double)mx[0]));
         if (nan) snan = 1;
     }
     __syncthreads();
     for (int i = threadIdx.x; i < d; i += blockDim.x) {
-        if (smn[i] != ~0ull) atomicMin(&mm[i], smn[i]);
+        if (smn[i] != 0ull) atomicMax(&mm[i], smn[i]);
         if (smx[i] != 0ull) atomicMax(&mm[64 + i], smx[i]);
     }
     if (threadIdx.x == 0 && snan) atomicOr(&ctr->nan_seen, 1u);
 }
 
-// Coarse cell keys from the three projected dimensions (Algorithm 1 on a grid of side >= eps).
+// Digit counts of every radix pass, gathered per block in shared memory (h, cleared by the block).
+__device__ __forceinline__ void count_digits_begin(uint32_t (&h)[8][256]) {
+    for (int i = threadIdx.x; i < 8 * 256; i += blockDim.x) (&h[0][0])[i] = 0;
+    __syncthreads();
+}
+__device__ __forceinline__ void count_digits(uint32_t (&h)[8][256], uint64_t key, int passes) {
+    for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(uint32_t)(key >> (8 * p)) & 0xffu], 1u);
+}
+__device__ __forceinline__ void count_digits_end(uint32_t (&h)[8][256], int passes, uint32_t *digit_counts) {
+    __syncthreads();
+    for (int i = threadIdx.x; i < passes * 256; i += blockDim.x) {
+        const uint32_t c = (&h[0][0])[i];
+        if (c) atomicAdd(&digit_counts[i], c);
+    }
+}
+
+// Coarse cell keys from the three projected dimensions (Algorithm 1 on a grid of side >= eps),
+// with the radix digit counts of the sort that follows.
 template <typename T, typename K>
 __global__ void __launch_bounds__(256) k_bin_proj(const T *__restrict__ in, int d, int3 sel, GridParams g,
-                                                 K *__restrict__ keys, uint32_t *__restrict__ idx) {
+                                                 K *__restrict__ keys, uint32_t *__restrict__ idx,
+                                                 uint32_t *__restrict__ digit_counts, FillList fill) {
+    __shared__ uint32_t h[8][256];
+    fill_regions(fill);
+    count_digits_begin(h);
+    const int passes = (g.key_bits + 7) / 8;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < g.n;
          j += (int64_t)gridDim.x * blockDim.x) {
         const int dims[3] = {sel.x, sel.y, sel.z};
@@ -393,59 +415,53 @@ __global__ void __launch_bounds__(256) k_bin_proj(const T *__restrict__ in, int 
         }
         keys[j] = (K)key;
         idx[j] = (uint32_t)j;
+        count_digits(h, key, passes);
     }
+    count_digits_end(h, passes, digit_counts);
 }
 
-// Gather the points into cell order, padded to DP coordinates, and flag the first point of
-// every coarse cell; one block per tile of kScanTileElems rows, DP / 4 threads per row (four
-// coordinates each, one vector store), the tile's flag count to tile_sums[block].
+// Gather the points into cell order, padded to DP coordinates, and the coarse cells and pencils; one
+// block per tile of kScanTileElems rows, DP / 4 threads per row (four coordinates each, one vector
+// store).  Also clears the core flags of the points and cells, and with fpts (double input with the
+// filter on) writes the float copy of the rows, relative to the set's smallest coordinates (set
+// id above set_shift of the key; complements of their encodings at mm[set * 64 + i]).
 template <typename T, int DP, typename K>
-__global__ void __launch_bounds__(256) k_gather_hd(const T *__restrict__ in, int d, const K *__restrict__ keys,
-                                                  const uint32_t *__restrict__ idx, int64_t n,
-                                                  T *__restrict__ pts, uint32_t *__restrict__ flags,
-                                                  uint32_t *__restrict__ tile_sums, float *__restrict__ fpts,
-                                                  const unsigned long long *__restrict__ mm, int set_shift) {
-    // fpts (double input with the filter on): the float copy of the rows, relative to the set's
-    // smallest coordinates (set id above set_shift of the key; encodings at mm[set * 64 + i])
+__global__ void __launch_bounds__(kTileThreads) k_cells_hd(const T *__restrict__ in, int d, CellsArgs<K> a,
+                                                          T *__restrict__ pts, uint8_t *__restrict__ core,
+                                                          uint8_t *__restrict__ cell_core, float *__restrict__ fpts,
+                                                          const unsigned long long *__restrict__ mm, int set_shift) {
     constexpr int G = DP / 4;          // threads per row
     constexpr int R = 256 / G;         // rows per step of the block
     const int g = threadIdx.x % G, r0 = threadIdx.x / G;
-    const int64_t base = (int64_t)blockIdx.x * kScanTileElems;
-    uint32_t cnt = 0;
+    const uint32_t tile = take_tile(a.l, 0u);
+    const int64_t base = (int64_t)tile * kScanTileElems;
 #pragma unroll 4
     for (int k = 0; k < kScanTileElems / R; ++k) {
         const int64_t j = base + (int64_t)k * R + r0;
-        if (j < n) {
-            const uint32_t o = idx[j];
-            const T *src = in + (int64_t)o * d;
-            T x[4];
+        if (j >= a.n) break;
+        const uint32_t o = a.idx[j];
+        const T *src = in + (int64_t)o * d;
+        T x[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = 4 * g + u < d ? src[4 * g + u] : T(0);
-            T *dst = pts + j * DP + 4 * g;
-            if (sizeof(T) == 4) {
-                *reinterpret_cast<float4 *>(dst) = make_float4((float)x[0], (float)x[1], (float)x[2], (float)x[3]);
-            } else {
-                reinterpret_cast<double2 *>(dst)[0] = make_double2((double)x[0], (double)x[1]);
-                reinterpret_cast<double2 *>(dst)[1] = make_double2((double)x[2], (double)x[3]);
-                if (fpts) {
-                    const uint64_t set = set_shift < 64 ? (uint64_t)keys[j] >> set_shift : 0ull;
-                    float f[4];
+        for (int u = 0; u < 4; ++u) x[u] = 4 * g + u < d ? src[4 * g + u] : T(0);
+        T *dst = pts + j * DP + 4 * g;
+        if (sizeof(T) == 4) {
+            *reinterpret_cast<float4 *>(dst) = make_float4((float)x[0], (float)x[1], (float)x[2], (float)x[3]);
+        } else {
+            reinterpret_cast<double2 *>(dst)[0] = make_double2((double)x[0], (double)x[1]);
+            reinterpret_cast<double2 *>(dst)[1] = make_double2((double)x[2], (double)x[3]);
+            if (fpts) {
+                const uint64_t set = set_shift < 64 ? (uint64_t)a.keys[j] >> set_shift : 0ull;
+                float f[4];
 #pragma unroll
-                    for (int u = 0; u < 4; ++u)
-                        f[u] = 4 * g + u < d ? (float)__dsub_rn((double)x[u], dec_double_dev(__ldg(mm + set * 64 + 4 * g + u))) : 0.f;
-                    *reinterpret_cast<float4 *>(fpts + j * DP + 4 * g) = make_float4(f[0], f[1], f[2], f[3]);
-                }
-            }
-            if (g == 0) {
-                const uint32_t f = (j == 0 || keys[j] != keys[j - 1]) ? 1u : 0u;
-                flags[j] = f;
-                cnt += f;
+                for (int u = 0; u < 4; ++u)
+                    f[u] = 4 * g + u < d ? (float)__dsub_rn((double)x[u], dec_double_dev(~__ldg(mm + set * 64 + 4 * g + u))) : 0.f;
+                *reinterpret_cast<float4 *>(fpts + j * DP + 4 * g) = make_float4(f[0], f[1], f[2], f[3]);
             }
         }
+        if (g == 0) core[j] = 0;
     }
-    uint32_t total;
-    block_exclusive_scan<256>(cnt, &total);
-    if (threadIdx.x == 0) tile_sums[blockIdx.x] = total;
+    cells_tile(a, tile, [cell_core](uint32_t c) { cell_core[c] = 0; });
 }
 
 template <typename T, int DP>
@@ -470,12 +486,12 @@ __device__ __forceinline__ void stage_rows(T *rows, const T *pts, uint32_t base,
 // Work is scheduled in chunks of 32 consecutive points of one coarse cell (a coarse cell can
 // hold a whole cluster, so one warp per cell would leave the largest cell to a single warp).
 // chunk_off[c] = first chunk of cell c (exclusive scan of ceil(size / 32)).
-static __global__ void __launch_bounds__(256) k_chunk_counts(const uint32_t *__restrict__ cell_start,
-                                                     const DevCounters *ctr, uint32_t *__restrict__ nch) {
-    const uint32_t C = ctr->n_cells;
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x)
-        nch[c] = (cell_start[c + 1] - cell_start[c] + 31u) / 32u;
-}
+// The scan also clears the cell's box (codes; see BoxCode).
+template <typename V>
+struct ChunkCount {
+    V v;
+    __device__ uint32_t operator()(int64_t c) const { return (v.cell_start[c + 1] - v.cell_start[c] + 31u) / 32u; }
+};
 
 // Cell of chunk (or work item) t: the last c with off[c] <= t, by a 32-way search (one round of
 // loads per level instead of one per halving).  A full warp calls it; every lane returns the
@@ -493,8 +509,8 @@ __device__ __forceinline__ uint32_t chunk_cell(const uint32_t *off, uint32_t C, 
     return lo;
 }
 
-// Box of every coarse cell in three launches: clear, accumulate over 32-point chunks (one
-// warp per chunk, so a large cell is spread over many warps), decode.  Coordinates are
+// Box of every coarse cell: cleared by the scan of the chunk counts, accumulated over 32-point
+// chunks (one warp per chunk, so a large cell is spread over many warps), decoded.  Coordinates are
 // accumulated as order-preserving unsigned integers (sign bit flipped for x >= 0, every bit
 // for x < 0), so min / max of the codes is min / max of the values and the warps of one cell
 // combine with atomicMin / atomicMax.
@@ -538,15 +554,18 @@ struct BoxCode {
 };
 
 template <typename T, int DP, typename R>
-__global__ void __launch_bounds__(256) k_cell_box_clear(HdView<T, DP> v) {
-    typedef typename BoxCode<R>::U U;
-    const uint64_t m = (uint64_t)v.ctr->n_cells * DP;
-    U *lo = reinterpret_cast<U *>(v.box_lo), *hi = reinterpret_cast<U *>(v.box_hi);
-    for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
-        lo[i] = ~(U)0;
-        hi[i] = (U)0;
+struct BoxClear {
+    HdView<T, DP> v;
+    __device__ void operator()(int64_t c, uint32_t, uint32_t) const {
+        uint4 *lo = reinterpret_cast<uint4 *>(reinterpret_cast<R *>(v.box_lo) + c * DP);
+        uint4 *hi = reinterpret_cast<uint4 *>(reinterpret_cast<R *>(v.box_hi) + c * DP);
+#pragma unroll
+        for (int i = 0; i < DP * (int)sizeof(R) / 16; ++i) {
+            lo[i] = make_uint4(~0u, ~0u, ~0u, ~0u);
+            hi[i] = make_uint4(0u, 0u, 0u, 0u);
+        }
     }
-}
+};
 
 template <typename T, int DP, typename R>
 __global__ void __launch_bounds__(256) k_cell_box_hd(HdView<T, DP> v) {
@@ -799,6 +818,12 @@ __device__ __forceinline__ uint4 list4(const V &v, uint32_t p, uint32_t i) {
 // CUDA cores.
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_list_link(HdView<T, DP> v) {
+    // (the cells' trees and odd counts are cleared here too)
+    const uint32_t C = v.ctr->n_cells;
+    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
+        v.cell_root[c] = kNoRoot;
+        v.odd_cnt[c] = 0u;
+    }
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t p = (uint32_t)j;
         uint32_t m = p;
@@ -960,15 +985,6 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_cell_link(HdView<T, DP> v)
 // index, so the tree that spans a cluster has a smaller root than the small trees that the lists
 // left over in the cluster's cells, and nearly all core points of a cell have this one; the
 // others are the cell's odd points.
-template <typename T, int DP>
-__global__ void __launch_bounds__(256) k_cell_root_clear(HdView<T, DP> v) {
-    const uint32_t C = v.ctr->n_cells;
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
-        v.cell_root[c] = kNoRoot;
-        v.odd_cnt[c] = 0u;
-    }
-}
-
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_cell_root(HdView<T, DP> v) {
     const int lane = lane_id();
@@ -1200,30 +1216,20 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_merge_hd(HdView<T, DP> v) 
     add_counter(&v.ctr->work[2], lane == 0 ? skipped : 0u);
 }
 
-// Flatten the point union-find (read-only finds), count roots, canonical ids.
-template <typename T, int DP>
-__global__ void __launch_bounds__(256) k_compress_hd(HdView<T, DP> v) {
-    uint32_t roots = 0;
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += (int64_t)gridDim.x * blockDim.x) {
-        if (!v.core[j]) continue;
-        const uint32_t r = uf_root_readonly(v.parent, (uint32_t)j, v.ctr);
-        v.parent[j] = r;
-        roots += (r == (uint32_t)j);
-    }
-    roots = __reduce_add_sync(0xffffffffu, roots);
-    if (lane_id() == 0 && roots) atomicAdd(&v.ctr->n_clusters, roots);
-}
-
+// Flatten the point union-find (read-only finds; the only writes are parent[j] = root), count the
+// roots and the core points, canonical ids.
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_comp_min_hd(HdView<T, DP> v) {
     const int64_t n = v.g.n;
     const int lane = lane_id();
-    uint32_t ncore = 0;
+    uint32_t ncore = 0, roots = 0;
     for (int64_t base = (int64_t)blockIdx.x * blockDim.x + (threadIdx.x & ~31); base < n;
          base += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j = base + lane;
         const bool valid = j < n && v.core[j];
-        const uint32_t r = valid ? v.parent[j] : 0xffffffffu;
+        const uint32_t r = valid ? uf_root_readonly(v.parent, (uint32_t)j, v.ctr) : 0xffffffffu;
+        if (valid) v.parent[j] = r;
+        roots += (valid && r == (uint32_t)j) ? 1u : 0u;
         uint32_t val = valid ? v.perm[j] : kNoLabel;
         const unsigned vm = __ballot_sync(0xffffffffu, valid);
         if (!vm) continue;
@@ -1237,6 +1243,8 @@ __global__ void __launch_bounds__(256) k_comp_min_hd(HdView<T, DP> v) {
         }
     }
     if (lane == 0 && ncore) atomicAdd(&v.ctr->n_core, ncore);
+    roots = __reduce_add_sync(0xffffffffu, roots);
+    if (lane == 0 && roots) atomicAdd(&v.ctr->n_clusters, roots);
 }
 
 // Algorithm 4 / Definition 5 with the canonical rule, over points: core points take their
@@ -1334,8 +1342,8 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_labels_hd(HdView<T, DP> v)
 }
 
 
-// Batched calls: per-set min / max of every dimension (mm[set * 64 + i] min encodings,
-// mm[(nsets + set) * 64 + i] max encodings), by seg_minmax.
+// Batched calls: per-set min / max of every dimension (mm[set * 64 + i] complements of the min
+// encodings, mm[(nsets + set) * 64 + i] max encodings), by seg_minmax.
 template <typename T>
 __global__ void __launch_bounds__(256) k_minmax_rt_seg(const T *__restrict__ in, int64_t n, int d,
                                                       const int64_t *set_off, int nsets,
@@ -1348,7 +1356,12 @@ __global__ void __launch_bounds__(256) k_minmax_rt_seg(const T *__restrict__ in,
 template <typename T, typename K>
 __global__ void __launch_bounds__(256) k_bin_proj_seg(const T *__restrict__ in, int64_t n, int d,
                                                      const int64_t *set_off, int nsets, const GridParams *gtab,
-                                                     int key_bits, K *__restrict__ keys, uint32_t *__restrict__ idx) {
+                                                     int key_bits, K *__restrict__ keys, uint32_t *__restrict__ idx,
+                                                     uint32_t *__restrict__ digit_counts, int total_bits, FillList fill) {
+    __shared__ uint32_t h[8][256];
+    fill_regions(fill);
+    count_digits_begin(h);
+    const int passes = (total_bits + 7) / 8;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n;
          j += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t set = set_of_point(set_off, nsets, j);
@@ -1363,7 +1376,9 @@ __global__ void __launch_bounds__(256) k_bin_proj_seg(const T *__restrict__ in, 
         }
         keys[j] = (K)key;
         idx[j] = (uint32_t)j;
+        count_digits(h, key, passes);
     }
+    count_digits_end(h, passes, digit_counts);
 }
 
 }  // namespace hca

@@ -142,8 +142,6 @@ struct TcOffsets {
     size_t nch, nch2, ch0, ch1, ch2, flags, cx, clist, nclist, clab;
 };
 
-inline uint32_t *part_of(char *b, size_t o) { return (uint32_t *)(b + o); }
-
 // Launch shapes shared by the phases.
 struct HdLaunch {
     cudaStream_t s;
@@ -164,19 +162,18 @@ void run_list_unions(HdView<T, DP> &hv, const HdLaunch &L, int &launches) {
         k_cell_link<T, DP, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
     }
     k_flatten_hd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
-    k_cell_root_clear<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
     k_cell_root<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
     k_cell_odd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
     k_cell_mixed<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
     k_odd_hd<T, DP, false, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
     k_odd_hd<T, DP, true, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
-    launches += hv.nl_k ? 13 : 8;
+    launches += hv.nl_k ? 12 : 7;
 }
 
 // The three point phases on the CUDA cores: counts (Definition 2), unions (Definitions 3-5) and
 // labels (Algorithm 4).
 template <typename T, int DP, bool FILTER, typename Mark>
-void run_cuda_phases(HdView<T, DP> &hv, const HdLaunch &L, int64_t n, Mark &mark, int &launches) {
+void run_cuda_phases(HdView<T, DP> &hv, const HdLaunch &L, Mark &mark, int &launches) {
     detail::allow_smem(k_count_hd<T, DP, false, FILTER>, L.smem);
     detail::allow_smem(k_count_hd<T, DP, true, FILTER>, L.smem);
     detail::allow_smem(k_cell_link<T, DP, FILTER>, L.smem);
@@ -185,7 +182,8 @@ void run_cuda_phases(HdView<T, DP> &hv, const HdLaunch &L, int64_t n, Mark &mark
     detail::allow_smem(k_merge_hd<T, DP, FILTER>, L.smem);
     detail::allow_smem(k_labels_hd<T, DP, false, FILTER>, L.smem);
     detail::allow_smem(k_labels_hd<T, DP, true, FILTER>, L.smem);
-    cudaMemsetAsync(hv.cell_core, 0, (size_t)n, L.s);
+    typedef typename Candidate<T, DP, FILTER>::Row R;
+    k_cell_box_decode<T, DP, R><<<L.gpts, 256, 0, L.s>>>(hv);
     k_count_hd<T, DP, false, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
     k_count_hd<T, DP, true, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
     mark(6);
@@ -193,7 +191,6 @@ void run_cuda_phases(HdView<T, DP> &hv, const HdLaunch &L, int64_t n, Mark &mark
     mark(7);
     run_list_unions<T, DP, FILTER>(hv, L, launches);
     k_merge_hd<T, DP, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
-    k_compress_hd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
     mark(8);
     k_comp_min_hd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
     if (L.list_labels) {
@@ -211,7 +208,7 @@ void run_cuda_phases(HdView<T, DP> &hv, const HdLaunch &L, int64_t n, Mark &mark
 // the CUDA-core kernels for the rest (float input).
 template <int DP, typename Mark>
 void run_tc_phases(HdView<float, DP> &hv, const HdLaunch &L, char *b, int64_t n, int grid_tc, size_t tc_smem,
-                   uint32_t *part, const TcOffsets &o, int nsets, DevCounters *ctr, const TcTuning &tune, Mark &mark,
+                   Scans &scans, const TcOffsets &o, int nsets, DevCounters *ctr, const TcTuning &tune, Mark &mark,
                    int &launches, cudaEvent_t *tev) {
     cudaStream_t s = L.s;
     const int gpts = L.gpts, gcell = L.gcell, hd_block = L.block;
@@ -238,47 +235,35 @@ void run_tc_phases(HdView<float, DP> &hv, const HdLaunch &L, char *b, int64_t n,
     detail::allow_smem(k_labels_hd<float, DP, false, true>, smem);
     detail::allow_smem(k_labels_hd<float, DP, true, true>, smem);
     // ---- Definition 2: exact counts over the neighbouring coarse cells ----
-    cudaMemsetAsync(hv.cell_core, 0, (size_t)n, s);
-    cudaMemsetAsync(hv.core, 0, (size_t)n, s);  // the recount below lists the rows with core = 2
-    tc::k_tc_chunks_count<<<gpts, 256, 0, s>>>(hv.cell_start, ctr, tune.min[0], nch);
-    exclusive_scan_u32(nch, ch0, n, &ctr->n_cells, &ctr->n_tc_chunks[tc::kCount], part, s, &launches);
+    scans.run(tc::CountChunks<DP>{hv, tune.min[0]}, tc::BoxDecode<DP>{hv}, ch0, n, &ctr->n_cells,
+              &ctr->n_tc_chunks[tc::kCount]);
     tmark(0);
     tc::k_tc_hd<DP, tc::kCount><<<grid_tc, tc::kTile, tc_smem, s>>>(hv, tc::Tables{ch0, cx, clist, nclist, clab});
     // the rows those chunks handed over, in cells with at least kRecountMin of them, counted again
-    // from the start, 128 per chunk (cx, clist, nclist, nch2 and ch1 are free until the core
-    // numbering); the rest, and what the recount hands over, go to the CUDA-core count
-    tc::k_tc_handed_flags<<<gpts, 256, 0, s>>>(hv.core, n, nclist);
-    exclusive_scan_u32(nclist, cx, n, nullptr, cx + n, part, s, &launches);
-    tc::k_tc_handed_list<<<gpts, 256, 0, s>>>(hv.core, cx, n, clist);
-    tc::k_tc_chunks_recount<<<gpts, 256, 0, s>>>(hv.cell_start, cx, ctr, hv.ranges, hv.n_all, tc::kRecountMin, nch2);
-    exclusive_scan_u32(nch2, ch1, n, &ctr->n_cells, &ctr->n_tc_recount, part, s, &launches);
-    // per listed row: the tallies summed over its windows and the windows done (nch, ch0 and
-    // nclist are free once scanned / once the first count is done)
-    cudaMemsetAsync(nch, 0, 4 * (size_t)n, s);
-    cudaMemsetAsync(ch0, 0, 4 * (size_t)n, s);
-    cudaMemsetAsync(nclist, 0, 4 * (size_t)n, s);
+    // from the start, 128 per chunk (cx, clist, nclist and ch1 are free until the core numbering); the
+    // rest, and what the recount hands over, go to the CUDA-core count.  Per listed row the
+    // tallies summed over its windows and the windows done are in nch, ch0 and nclist.
+    scans.run(tc::HandedFlag{hv.core}, tc::HandedList{clist, nch, ch0, nclist}, cx, n, nullptr, cx + n);
+    scans.run(tc::RecountItems{hv.cell_start, cx, hv.ranges, hv.n_all, tc::kRecountMin}, tc::NoEmit{}, ch1, n,
+              &ctr->n_cells, &ctr->n_tc_recount);
     tc::k_tc_hd<DP, tc::kCount><<<grid_tc, tc::kTile, tc_smem, s>>>(
         hv, tc::Tables{ch1, cx, nullptr, nullptr, nullptr, nullptr, clist, nch, ch0, nclist});
     tmark(1);
     k_count_hd<float, DP, false, true><<<gcell, hd_block, smem, s>>>(hv);
     k_count_hd<float, DP, true, true><<<gcell, hd_block, smem, s>>>(hv);
-    launches += 8;
+    launches += 4;
     mark(6);
     // core numbering, core and non-core lists
-    tc::k_tc_core_flags<<<gpts, 256, 0, s>>>(hv.core, n, flags);
-    exclusive_scan_u32(flags, cx, n, nullptr, cx + n, part, s, &launches);
-    tc::k_tc_partition<<<gpts, 256, 0, s>>>(hv.core, cx, n, clist, L.list_labels ? nullptr : nclist);
-    launches += 2;
+    scans.run(tc::CoreFlag{hv.core}, tc::CoreLists{clist, L.list_labels ? nullptr : nclist}, cx, n, nullptr, cx + n);
     mark(7);
     // ---- Definitions 3-5: the lists' edges and the odd points, then the remaining unions ----
     run_list_unions<float, DP, true>(hv, L, launches);
     // chunk tables of the unions and the labels (flags and ch0 are free: the unions' later windows)
-    tc::k_tc_chunks_split<DP><<<gpts, 256, 0, s>>>(hv, tune.min[1], tune.min[2], nch, flags,
-                                                   L.list_labels ? nullptr : nch2);
-    exclusive_scan_u32(nch, ch1, n, &ctr->n_cells, &ctr->n_tc_chunks[tc::kMerge], part, s, &launches);
+    scans.run(tc::MergeChunks<DP>{hv, tune.min[1], tune.min[2], flags, L.list_labels ? nullptr : nch2}, tc::NoEmit{},
+              ch1, n, &ctr->n_cells, &ctr->n_tc_chunks[tc::kMerge]);
     if (!L.list_labels)
-        exclusive_scan_u32(nch2, ch2, n, &ctr->n_cells, &ctr->n_tc_chunks[tc::kLabels], part, s, &launches);
-    exclusive_scan_u32(flags, ch0, n, &ctr->n_cells, &ctr->n_tc_chunks[3], part, s, &launches);
+        scans.run(tc::Stored{nch2}, tc::NoEmit{}, ch2, n, &ctr->n_cells, &ctr->n_tc_chunks[tc::kLabels]);
+    scans.run(tc::Stored{flags}, tc::NoEmit{}, ch0, n, &ctr->n_cells, &ctr->n_tc_chunks[3]);
     tmark(2);
     // window-major items: the first window of every chunk, then the other windows
     tc::k_tc_hd<DP, tc::kMerge><<<grid_tc, tc::kTile, tc_smem, s>>>(hv, tc::Tables{ch1, cx, clist, nclist, clab, ch0});
@@ -289,8 +274,7 @@ void run_tc_phases(HdView<float, DP> &hv, const HdLaunch &L, char *b, int64_t n,
         k_merge_hd<float, DP, true><<<gcell, hd_block, smem, s>>>(hv);
         ++launches;
     }
-    k_compress_hd<float, DP><<<gpts, 256, 0, s>>>(hv);
-    launches += 3;
+    launches += 1;
     mark(8);
     // ---- Algorithm 4: canonical ids, core labels, border and noise points ----
     k_comp_min_hd<float, DP><<<gpts, 256, 0, s>>>(hv);
@@ -344,21 +328,20 @@ int run_hd(const RunArgs &a) {
     int64_t cap_max = 64;
     while (cap_max < 2 * n) cap_max <<= 1;
     const size_t hist_elems = sort_hist_size(n);
-    const int64_t scan_max = n > (int64_t)hist_elems ? n : (int64_t)hist_elems;
     const size_t o_ctr = take(sizeof(DevCounters));
     const size_t o_mm = take(sizeof(unsigned long long) * 128);
     const size_t o_ka = take(8 * n), o_kb = take(8 * n), o_ia = take(4 * n), o_ib = take(4 * n);
     const size_t o_hist = take(4 * hist_elems);
-    const size_t o_part = take(4 * scan_partials_size(scan_max));
+    const size_t o_look = take(look_bytes(n)), o_scan = take(look_bytes(n));
     const size_t o_pts = take(sizeof(T) * DP * (size_t)n);
-    const size_t o_flags = take(4 * n), o_excl = take(4 * n);
+    const size_t o_flags = take(4 * n), o_odd = take(4 * n);
     const size_t o_cstart = take(4 * (n + 1)), o_ckey = take(8 * n);
-    const size_t o_pflags = take(4 * n), o_pexcl = take(4 * n), o_pstart = take(4 * (n + 1));
+    const size_t o_pend = take(4 * n), o_croot = take(4 * n), o_pstart = take(4 * (n + 1));
     const size_t o_hk = take(8 * cap_max), o_hv = take(4 * cap_max);
     const size_t o_core = take(n), o_ccore = take(n);
     const size_t o_parent = take(4 * n), o_cmin = take(4 * n);
     const size_t o_ranges = take(sizeof(uint2) * 9 * (size_t)n);
-    const size_t o_nch = take(4 * n), o_choff = take(4 * n);
+    const size_t o_choff = take(4 * n);
     const size_t o_blo = take(sizeof(T) * DP * (size_t)n), o_bhi = take(sizeof(T) * DP * (size_t)n);
     const bool batched = a.nsets > 0;
     const int nsets = batched ? a.nsets : 1;
@@ -438,7 +421,9 @@ int run_hd(const RunArgs &a) {
     memset(&lv, 0, sizeof(lv));
     int sort_bits = 0;
     float *fpts = nullptr;
+    uint32_t *ptab = nullptr;
     HdLaunch L;
+    Scans scans;
     std::vector<unsigned long long> smm;
     std::vector<GridParams> gsets;
     GridParams *d_gtab = (GridParams *)(b + o_gtab);
@@ -541,15 +526,12 @@ int run_hd(const RunArgs &a) {
         if (rc) goto out;
     }
     mark(0);
-    cudaMemsetAsync(ctr, 0, sizeof(DevCounters), s);
+    cudaMemsetAsync(ctr, 0, o_mm + sizeof(unsigned long long) * 128 - o_ctr, s);  // (mm follows the counters)
     if (!batched) {
-        cudaMemsetAsync(mm, 0xff, sizeof(unsigned long long) * 64, s);
-        cudaMemsetAsync(mm + 64, 0, sizeof(unsigned long long) * 64, s);
         k_minmax_rt<T><<<grid_for(n * d, 256, sms, 8), 256, 0, s>>>((const T *)a.d_points, n, d, ctr, mm);
         if (!boxed) cudaMemcpyAsync(hmm.data(), mm, sizeof(unsigned long long) * 128, cudaMemcpyDeviceToHost, s);
     } else {
-        cudaMemsetAsync(d_smm, 0xff, sizeof(unsigned long long) * 64 * nsets, s);
-        cudaMemsetAsync(d_smm + (size_t)64 * nsets, 0, sizeof(unsigned long long) * 64 * nsets, s);
+        cudaMemsetAsync(d_smm, 0, sizeof(unsigned long long) * 2 * 64 * nsets, s);
         upload(d_setoff, a.h_off, sizeof(int64_t) * (nsets + 1), stage_setoff);
         k_minmax_rt_seg<T><<<grid_for(n, 256, sms, 8), 256, 0, s>>>((const T *)a.d_points, n, d, d_setoff, nsets,
                                                                    d_smm, ctr);
@@ -571,19 +553,19 @@ int run_hd(const RunArgs &a) {
             d_box, nsets, d, batched ? d_setoff : nullptr, batched ? d_smm : mm, ctr);
         ++launches;
     } else {
-        if (cudaMemcpyAsync(h, ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        if (cudaMemcpyAsync(h, ctr, kCountersRead, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess) { rc = HCA_ECUDA; goto out; }
         if (h->nan_seen) { rc = HCA_EINVAL; goto out; }
         if (a.ext_out && !batched)
             for (int i = 0; i < d; ++i) {
-                a.ext_out[i] = dec_double(hmm[i]);
+                a.ext_out[i] = dec_double(~hmm[i]);
                 a.ext_out[d + i] = dec_double(hmm[64 + i]);
             }
         if (batched)
-            rc = build_grids([&](int set, int i) { return dec_double(smm[(size_t)set * 64 + i]); },
+            rc = build_grids([&](int set, int i) { return dec_double(~smm[(size_t)set * 64 + i]); },
                              [&](int set, int i) { return dec_double(smm[((size_t)nsets + set) * 64 + i]); });
         else
-            rc = build_grids([&](int, int i) { return dec_double(hmm[i]); },
+            rc = build_grids([&](int, int i) { return dec_double(~hmm[i]); },
                              [&](int, int i) { return dec_double(hmm[64 + i]); });
         if (rc) goto out;
         if (batched) cudaMemcpyAsync(d_gtab, gsets.data(), sizeof(GridParams) * nsets, cudaMemcpyHostToDevice, s);
@@ -593,75 +575,68 @@ int run_hd(const RunArgs &a) {
     // leave free
     if (sizeof(T) == 8 && filter) fpts = (float *)(b + o_bhi);
     {
-        uint32_t *ia = (uint32_t *)(b + o_ia), *ib = (uint32_t *)(b + o_ib);
-        uint32_t *hist = (uint32_t *)(b + o_hist), *part = (uint32_t *)(b + o_part);
-        const bool use32 = sort_bits <= 32;
-        const int gtile = (int)((n + kScanTileElems - 1) / kScanTileElems);  // gather: one block per scan tile
-        if (use32) {
-            uint32_t *ka = (uint32_t *)(b + o_ka), *kb = (uint32_t *)(b + o_kb);
+        uint32_t *ia = (uint32_t *)(b + o_ia), *ib = (uint32_t *)(b + o_ib), *hist = (uint32_t *)(b + o_hist);
+        ptab = pencil_table(sort_bits - g.prefix_shift, cap_max, b + o_hk);
+        FillList fill = {};
+        fill.add(hist, sizeof(uint32_t) * hist_elems, 0u);
+        fill.add(b + o_look, o_scan + look_bytes(n) - o_look, 0u);
+        if (ptab) fill.add(ptab, sizeof(uint32_t) << (sort_bits - g.prefix_shift), 0xffffffffu);
+        auto front = [&](auto *ka, auto *kb) {
+            typedef typename std::remove_reference<decltype(*ka)>::type K;
             if (batched)
-                k_bin_proj_seg<T, uint32_t><<<gpts, 256, 0, s>>>((const T *)a.d_points, n, d, d_setoff, nsets, d_gtab,
-                                                                 g.key_bits, ka, ia);
+                k_bin_proj_seg<T, K><<<gpts, 256, 0, s>>>((const T *)a.d_points, n, d, d_setoff, nsets, d_gtab,
+                                                         g.key_bits, ka, ia, ctr->digit_counts, sort_bits, fill);
             else
-                k_bin_proj<T, uint32_t><<<gpts, 256, 0, s>>>((const T *)a.d_points, d, sel, g, ka, ia);
+                k_bin_proj<T, K><<<gpts, 256, 0, s>>>((const T *)a.d_points, d, sel, g, ka, ia, ctr->digit_counts, fill);
             mark(2);
-            flipped = radix_sort_pairs<uint32_t>(ka, ia, kb, ib, n, 0, sort_bits, hist, part, s, &launches, &ctr->status);
+            flipped = radix_sort_pairs<K>(ka, ia, kb, ib, n, 0, sort_bits, hist, nullptr, s, &launches, &ctr->status,
+                                          ctr->digit_counts, true);
             mark(3);
-            k_gather_hd<T, DP, uint32_t><<<gtile, 256, 0, s>>>(
-                (const T *)a.d_points, d, flipped ? kb : ka, flipped ? ib : ia, n, (T *)(b + o_pts),
-                (uint32_t *)(b + o_flags), part, fpts, batched ? d_smm : mm, batched ? g.key_bits : 64);
-        } else {
-            uint64_t *ka = (uint64_t *)(b + o_ka), *kb = (uint64_t *)(b + o_kb);
-            if (batched)
-                k_bin_proj_seg<T, uint64_t><<<gpts, 256, 0, s>>>((const T *)a.d_points, n, d, d_setoff, nsets, d_gtab,
-                                                                 g.key_bits, ka, ia);
-            else
-                k_bin_proj<T, uint64_t><<<gpts, 256, 0, s>>>((const T *)a.d_points, d, sel, g, ka, ia);
-            mark(2);
-            flipped = radix_sort_pairs<uint64_t>(ka, ia, kb, ib, n, 0, sort_bits, hist, part, s, &launches, &ctr->status);
-            mark(3);
-            k_gather_hd<T, DP, uint64_t><<<gtile, 256, 0, s>>>(
-                (const T *)a.d_points, d, flipped ? kb : ka, flipped ? ib : ia, n, (T *)(b + o_pts),
-                (uint32_t *)(b + o_flags), part, fpts, batched ? d_smm : mm, batched ? g.key_bits : 64);
-        }
-        launches += 2;
-        // run-length cells: scan of the gather's tile counts, cell ids / starts / keys
-        if (use32)
-            cells_from_flags<uint32_t>((const uint32_t *)(b + (flipped ? o_kb : o_ka)), (uint32_t *)(b + o_flags), n,
-                                       part, &ctr->n_cells, (uint32_t *)(b + o_cstart), (uint64_t *)(b + o_ckey), s,
-                                       &launches);
-        else
-            cells_from_flags<uint64_t>((const uint64_t *)(b + (flipped ? o_kb : o_ka)), (uint32_t *)(b + o_flags), n,
-                                       part, &ctr->n_cells, (uint32_t *)(b + o_cstart), (uint64_t *)(b + o_ckey), s,
-                                       &launches);
+            CellsArgs<K> ca;
+            ca.keys = flipped ? kb : ka;
+            ca.idx = flipped ? ib : ia;
+            ca.n = n;
+            ca.prefix_shift = g.prefix_shift;
+            ca.cell_of = (uint32_t *)(b + o_flags);
+            ca.cell_start = (uint32_t *)(b + o_cstart);
+            ca.cell_key = (uint64_t *)(b + o_ckey);
+            ca.pencil_start = (uint32_t *)(b + o_pstart);
+            ca.ptab = ptab;
+            ca.l = LookBack::at(b + o_look);
+            ca.ctr = ctr;
+            k_cells_hd<T, DP, K><<<(unsigned)((n + kScanTileElems - 1) / kScanTileElems), kTileThreads, 0, s>>>(
+                (const T *)a.d_points, d, ca, (T *)(b + o_pts), (uint8_t *)(b + o_core), (uint8_t *)(b + o_ccore), fpts,
+                batched ? d_smm : mm, batched ? g.key_bits : 64);
+            launches += 2;
+        };
+        if (sort_bits <= 32) front((uint32_t *)(b + o_ka), (uint32_t *)(b + o_kb));
+        else front((uint64_t *)(b + o_ka), (uint64_t *)(b + o_kb));
         hv.perm = flipped ? ib : ia;
     }
     mark(4);
-    {
-        uint32_t *part = (uint32_t *)(b + o_part);
-        k_pencil_flags<<<gpts, 256, 0, s>>>((const uint64_t *)(b + o_ckey), g.prefix_shift, ctr,
-                                            (uint32_t *)(b + o_pflags));
-        exclusive_scan_u32((uint32_t *)(b + o_pflags), (uint32_t *)(b + o_pexcl), n, &ctr->n_cells,
-                           &ctr->n_pencils, part, s, &launches);
+    if (!ptab) {
         k_hash_init<<<grid_for(cap_max, 256, sms, 8), 256, 0, s>>>((uint64_t *)(b + o_hk), ctr);
         k_pencils<<<gpts, 256, 0, s>>>((const uint64_t *)(b + o_ckey), g.prefix_shift,
-                                       (const uint32_t *)(b + o_pflags), (const uint32_t *)(b + o_pexcl),
-                                       (uint32_t *)(b + o_pstart), (uint64_t *)(b + o_hk),
+                                       (const uint32_t *)(b + o_pstart), (uint64_t *)(b + o_hk),
                                        (uint32_t *)(b + o_hv), ctr);
-        lv.g = g;
-        lv.gtab = batched ? d_gtab : nullptr;
-        lv.cell_key = (const uint64_t *)(b + o_ckey);
-        lv.pencil_start = (const uint32_t *)(b + o_pstart);
-        lv.hkeys = (uint64_t *)(b + o_hk);
-        lv.hvals = (uint32_t *)(b + o_hv);
-        lv.ranges = (uint2 *)(b + o_ranges);
-        lv.ctr = ctr;
-        k_ranges<float, 3><<<grid_for((n / kRangeRun + 1) * (int64_t)st.n_all, 256, sms, 16), 256, 0, s>>>(lv, st);
-        k_chunk_counts<<<gpts, 256, 0, s>>>((const uint32_t *)(b + o_cstart), ctr, (uint32_t *)(b + o_nch));
-        exclusive_scan_u32((uint32_t *)(b + o_nch), (uint32_t *)(b + o_choff), n, &ctr->n_cells,
-                           &ctr->n_chunks, part, s, &launches);
-        launches += 5;
+        launches += 2;
     }
+    lv.g = g;
+    lv.gtab = batched ? d_gtab : nullptr;
+    lv.cell_key = (const uint64_t *)(b + o_ckey);
+    lv.pencil_start = (const uint32_t *)(b + o_pstart);
+    lv.hkeys = (uint64_t *)(b + o_hk);
+    lv.hvals = (uint32_t *)(b + o_hv);
+    lv.ptab = ptab;
+    lv.ranges = (uint2 *)(b + o_ranges);
+    lv.ctr = ctr;
+    k_ranges<float, 3><<<grid_for((n / kRangeRun + 1) * (int64_t)st.n_all, 256, sms, 16), 256, 0, s>>>(lv, st);
+    ++launches;
+    scans.l = LookBack::at(b + o_scan);
+    scans.err = &ctr->status;
+    scans.epoch = 1;
+    scans.s = s;
+    scans.launches = &launches;
     mark(5);
     hv.g = g;
     hv.gtab = batched ? d_gtab : nullptr;
@@ -687,15 +662,14 @@ int run_hd(const RunArgs &a) {
     // (with fpts both float boxes lie in the first half of the box space)
     hv.box_hi = (T *)(b + (fpts ? o_blo + sizeof(float) * DP * (size_t)n : o_bhi));
     // the windows' queue and per-row values take the sort's key buffers, free once the cells are
-    // known; one word per chunk (at most n) from the pencil flags, free once the pencils are, and
-    // so are the scan scratch and the pencil starts that the cells' trees take after the ranges;
-    // the list lengths take the index buffer that the sort did not end in
+    // known; the odd masks (one word per chunk, at most n) the pencil starts, free after the ranges;
+    // the list lengths the index buffer that the sort did not end in
     hv.sp_queue = (uint2 *)(b + o_ka);
     hv.sp_cap = (uint32_t)n;
     hv.sp_val = (uint32_t *)(b + o_kb);
-    hv.sp_pending = (uint32_t *)(b + o_pflags);
-    hv.cell_root = (uint32_t *)(b + o_pexcl);
-    hv.odd_cnt = (uint32_t *)(b + o_excl);
+    hv.sp_pending = (uint32_t *)(b + o_pend);
+    hv.cell_root = (uint32_t *)(b + o_croot);
+    hv.odd_cnt = (uint32_t *)(b + o_odd);
     hv.odd_mask = (uint32_t *)(b + o_pstart);
     hv.nl = (uint32_t *)(b + o_nl);
     hv.nl_k = lists ? list_len(max_min_pts) : 0u;
@@ -706,20 +680,22 @@ int run_hd(const RunArgs &a) {
     L.block = hd_block;
     L.smem = smem;
     L.list_labels = hv.nl_k && hv.nl_k + 1 >= max_min_pts;
-    // the box of every coarse cell in all d dimensions (point-to-box distance bounds)
-    if (fpts) {
-        k_cell_box_clear<T, DP, float><<<grid_for((int64_t)n * DP, 256, sms, 8), 256, 0, s>>>(hv);
-        k_cell_box_hd<T, DP, float><<<grid_for(n / 32 + 1, 8, sms, 16), 256, 0, s>>>(hv);
-        k_cell_box_decode<T, DP, float><<<grid_for((int64_t)n * DP, 256, sms, 8), 256, 0, s>>>(hv);
-    } else {
-        k_cell_box_clear<T, DP, T><<<grid_for((int64_t)n * DP, 256, sms, 8), 256, 0, s>>>(hv);
-        k_cell_box_hd<T, DP, T><<<grid_for(n / 32 + 1, 8, sms, 16), 256, 0, s>>>(hv);
-        k_cell_box_decode<T, DP, T><<<grid_for((int64_t)n * DP, 256, sms, 8), 256, 0, s>>>(hv);
+    // the chunks and the box of every coarse cell in all d dimensions (point-to-box distance bounds)
+    {
+        uint32_t *choff = (uint32_t *)(b + o_choff);
+        const ChunkCount<HdView<T, DP>> chunks{hv};
+        if (fpts) {
+            scans.run(chunks, BoxClear<T, DP, float>{hv}, choff, n, &ctr->n_cells, &ctr->n_chunks);
+            k_cell_box_hd<T, DP, float><<<grid_for(n / 32 + 1, 8, sms, 16), 256, 0, s>>>(hv);
+        } else {
+            scans.run(chunks, BoxClear<T, DP, T>{hv}, choff, n, &ctr->n_cells, &ctr->n_chunks);
+            k_cell_box_hd<T, DP, T><<<grid_for(n / 32 + 1, 8, sms, 16), 256, 0, s>>>(hv);
+        }
+        ++launches;
     }
-    launches += 3;
     if constexpr (std::is_same<T, float>::value) {
         if (use_tc && st.n_all <= tc::kMaxRng) {
-            run_tc_phases<DP>(hv, L, b, n, sms * tc_occ, tc_smem, part_of(b, o_part),
+            run_tc_phases<DP>(hv, L, b, n, sms * tc_occ, tc_smem, scans,
                               TcOffsets{o_tnch, o_tnch2, o_tch0, o_tch1, o_tch2, o_tflags, o_cx, o_clist, o_nclist,
                                         o_clab},
                               batched ? nsets : 0, ctr,
@@ -731,11 +707,11 @@ int run_hd(const RunArgs &a) {
         }
     }
     if (!tc_phases) {
-        if (filter) run_cuda_phases<T, DP, true>(hv, L, n, mark, launches);
-        else run_cuda_phases<T, DP, false>(hv, L, n, mark, launches);
+        if (filter) run_cuda_phases<T, DP, true>(hv, L, mark, launches);
+        else run_cuda_phases<T, DP, false>(hv, L, mark, launches);
     }
     if (cudaGetLastError() != cudaSuccess) { rc = HCA_ECUDA; goto out; }
-    if (cudaMemcpyAsync(h, ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, s) != cudaSuccess) {
+    if (cudaMemcpyAsync(h, ctr, kCountersRead, cudaMemcpyDeviceToHost, s) != cudaSuccess) {
         rc = HCA_ECUDA;
         goto out;
     }

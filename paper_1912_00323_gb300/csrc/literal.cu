@@ -271,7 +271,6 @@ int run_literal(const T *d_points, int64_t n, double eps, int32_t *d_labels, cud
     const int gpts = grid_for(n, 256, sms, 8);
     bool flipped = false;
     cudaMemsetAsync(ctr, 0, sizeof(DevCounters), s);
-    cudaMemsetAsync(ctr->minmax_enc, 0xff, sizeof(uint64_t) * kMaxD, s);
     k_minmax<T, D><<<grid_for(n, 256, sms, 2), 256, 0, s>>>(d_points, n, ctr);
     ++launches;
     if (cudaMemcpyAsync(h, ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
@@ -283,7 +282,7 @@ int run_literal(const T *d_points, int64_t n, double eps, int32_t *d_labels, cud
     {
         int sh = 0;
         for (int i = D - 1; i >= 0; --i) {
-            p.origin[i] = dec_double(h->minmax_enc[i]);
+            p.origin[i] = dec_double(~h->minmax_enc[i]);
             const double mx = dec_double(h->minmax_enc[kMaxD + i]);
             if (!isfinite(p.origin[i]) || !isfinite(mx)) { rc = HCA_EINVAL; goto out; }
             const double t = floor((mx - p.origin[i]) / p.side);

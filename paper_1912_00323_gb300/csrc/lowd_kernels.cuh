@@ -16,8 +16,7 @@
 
 #include <float.h>
 
-#include "block_scan.cuh"
-#include "hca_internal.cuh"
+#include "cells.cuh"
 
 namespace hca {
 
@@ -35,6 +34,7 @@ struct LowdView {
     const uint32_t *pencil_start;
     uint64_t *hkeys;
     uint32_t *hvals;
+    const uint32_t *ptab;         // direct table pencil key -> pencil id (~0: none); NULL: the hash table
     uint8_t *core;
     uint8_t *cell_core;
     uint32_t *parent;
@@ -230,6 +230,12 @@ __device__ __forceinline__ uint32_t hash_lookup(const uint64_t *hkeys, const uin
         h = (h + 1) & mask;
     }
     return 0xffffffffu;
+}
+
+// The pencil of a key, ~0 when there is none.
+template <typename V>
+__device__ __forceinline__ uint32_t pencil_of(const V &v, uint64_t key) {
+    return v.ptab ? __ldg(v.ptab + key) : hash_lookup(v.hkeys, v.hvals, v.ctr->hash_mask, key);
 }
 
 // First position in [a, e) of a pencil's cells (keys ascending) whose key is not below kt
@@ -489,7 +495,7 @@ __global__ void __launch_bounds__(256) k_minmax(const T *__restrict__ in, int64_
             b = smx[w][i] > b ? smx[w][i] : b;
         }
         uint64_t *mm = ctr->minmax_enc;
-        atomicMin((unsigned long long *)&mm[i], (unsigned long long)enc_double((double)a));
+        atomicMax((unsigned long long *)&mm[i], ~(unsigned long long)enc_double((double)a));
         atomicMax((unsigned long long *)&mm[kMaxD + i], (unsigned long long)enc_double((double)b));
     }
     if (threadIdx.x == 0 && snan) atomicOr(&ctr->nan_seen, 1u);
@@ -502,8 +508,9 @@ __global__ void __launch_bounds__(256) k_minmax(const T *__restrict__ in, int64_
 template <typename T, int D, typename K>
 __global__ void __launch_bounds__(256) k_bin(const T *__restrict__ in, GridParams g,
                                             K *__restrict__ keys, uint32_t *__restrict__ idx,
-                                            uint32_t *__restrict__ digit_counts) {
+                                            uint32_t *__restrict__ digit_counts, FillList fill) {
     constexpr int P = VecPts<T, D>::pts;
+    fill_regions(fill);
     // digit counts of every radix pass, for the sort that follows
     __shared__ uint32_t h[8][256];
     const int passes = (g.key_bits + 7) / 8;
@@ -566,45 +573,29 @@ __global__ void __launch_bounds__(256) k_bin(const T *__restrict__ in, GridParam
     }
 }
 
-// Gather the points into cell order and flag the first point of every cell; one block per
-// tile of kScanTileElems points, whose flag count goes to tile_sums[block] for the run-length
-// cells that follow (cells_from_flags).
+// Gather the points into cell order, and the cells and pencils, one block per tile of
+// kScanTileElems points.
 template <typename T, int D, typename K>
-__global__ void __launch_bounds__(256) k_gather(const T *__restrict__ in, const K *__restrict__ keys,
-                                               const uint32_t *__restrict__ idx, int64_t n,
-                                               Pt<T, D> *__restrict__ pts, uint32_t *__restrict__ flags,
-                                               uint32_t *__restrict__ tile_sums) {
-    const int64_t base = (int64_t)blockIdx.x * kScanTileElems;
-    uint32_t cnt = 0;
+__global__ void __launch_bounds__(kTileThreads) k_cells(const T *__restrict__ in, CellsArgs<K> a,
+                                                       Pt<T, D> *__restrict__ pts) {
+    const uint32_t tile = take_tile(a.l, 0u);
+    const int64_t base = (int64_t)tile * kScanTileElems;
 #pragma unroll
-    for (int k = 0; k < kScanTileElems / 256; ++k) {
-        const int64_t j = base + k * 256 + threadIdx.x;
-        if (j < n) {
-            const uint32_t o = idx[j];
+    for (int k = 0; k < kTileItems; ++k) {
+        const int64_t j = base + k * kTileThreads + threadIdx.x;
+        if (j < a.n) {
+            const uint32_t o = a.idx[j];
             Pt<T, D> p = zero_pt<T, D>();
 #pragma unroll
             for (int i = 0; i < D; ++i) p.x[i] = in[(int64_t)o * D + i];
             pts[j] = p;
-            const uint32_t f = (j == 0 || keys[j] != keys[j - 1]) ? 1u : 0u;
-            flags[j] = f;
-            cnt += f;
         }
     }
-    uint32_t total;
-    block_exclusive_scan<256>(cnt, &total);
-    if (threadIdx.x == 0) tile_sums[blockIdx.x] = total;
+    cells_tile(a, tile, [](uint32_t) {});
 }
 
-// First cell of every pencil (cells sharing all coordinates but the last).
-static __global__ void __launch_bounds__(256) k_pencil_flags(const uint64_t *__restrict__ cell_key,
-                                                            int prefix_shift, const DevCounters *ctr,
-                                                            uint32_t *__restrict__ pflags) {
-    const uint32_t C = ctr->n_cells;
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x)
-        pflags[c] = (c == 0 || (cell_key[c] >> prefix_shift) != (cell_key[c - 1] >> prefix_shift)) ? 1u : 0u;
-}
-
-// Clear the used part of the hash table (capacity = power of two >= 2 P).
+// The hash table of the pencils, when their keys span too much for a direct table: clear the used
+// part (capacity = power of two >= 2 P), then insert.
 static __global__ void __launch_bounds__(256) k_hash_init(uint64_t *__restrict__ hkeys, DevCounters *ctr) {
     const uint32_t P = ctr->n_pencils;
     uint32_t cap = 64;
@@ -614,19 +605,13 @@ static __global__ void __launch_bounds__(256) k_hash_init(uint64_t *__restrict__
     if (blockIdx.x == 0 && threadIdx.x == 0) ctr->hash_mask = cap - 1;
 }
 
-static __global__ void __launch_bounds__(256) k_pencils(const uint64_t *__restrict__ cell_key,
-                                                       int prefix_shift, const uint32_t *__restrict__ pflags,
-                                                       const uint32_t *__restrict__ pexcl,
-                                                       uint32_t *__restrict__ pencil_start,
-                                                       uint64_t *hkeys, uint32_t *hvals, DevCounters *ctr) {
-    const uint32_t C = ctr->n_cells;
+static __global__ void __launch_bounds__(256) k_pencils(const uint64_t *__restrict__ cell_key, int prefix_shift,
+                                                       const uint32_t *__restrict__ pencil_start, uint64_t *hkeys,
+                                                       uint32_t *hvals, DevCounters *ctr) {
+    const uint32_t P = ctr->n_pencils;
     const uint32_t mask = ctr->hash_mask;
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
-        if (c == C - 1) pencil_start[pexcl[c] + pflags[c]] = C;
-        if (!pflags[c]) continue;
-        const uint32_t p = pexcl[c];
-        pencil_start[p] = c;
-        const uint64_t key = cell_key[c] >> prefix_shift;
+    for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
+        const uint64_t key = cell_key[pencil_start[p]] >> prefix_shift;
         uint32_t h = (uint32_t)mix64(key) & mask;
         bool placed = false;
         for (uint32_t it = 0; it <= mask; ++it) {
@@ -687,7 +672,7 @@ __global__ void __launch_bounds__(256) k_ranges(LowdView<T, D> v, Stencil st_in)
                     if (cc < 0 || cc >= (int)g.ncell[i]) ok = false;
                     pkey |= (uint64_t)(cc & ((1 << g.bits[i]) - 1)) << (g.shift[i] - g.prefix_shift);
                 }
-                const uint32_t q = ok ? hash_lookup(v.hkeys, v.hvals, v.ctr->hash_mask, pkey) : 0xffffffffu;
+                const uint32_t q = ok ? pencil_of(v, pkey) : 0xffffffffu;
                 ok = q != 0xffffffffu;
                 lo = hi = ok ? v.pencil_start[q] : 0u;
                 qe = ok ? v.pencil_start[q + 1] : 0u;
@@ -1192,15 +1177,14 @@ __global__ void __launch_bounds__(256) k_hook(LowdView<T, D> v, int n_all, int n
     }
 }
 
-// One round of pointer jumping over cells with core points: parent[c] = parent[parent[c]].
+// The first links flattened: parent[c] = root of every cell with core points, by finds that do not
+// write on the way (nothing hooks meanwhile; the links run a few cells far).
 template <typename T, int D>
-__global__ void __launch_bounds__(256) k_jump(LowdView<T, D> v) {
-    const uint32_t C = v.ctr->n_cells;
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
-        if (!v.cell_core[c]) continue;
-        const uint32_t p = __ldcg(v.parent + c);
-        const uint32_t gp = __ldcg(v.parent + p);
-        if (gp != p) v.parent[c] = gp;
+__global__ void __launch_bounds__(256) k_flatten(LowdView<T, D> v) {
+    const uint32_t NL = v.ctr->n_list[1];
+    for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < NL; w += gridDim.x * blockDim.x) {
+        const uint32_t c = v.list_core[w];
+        v.parent[c] = uf_root_readonly(v.parent, c, v.ctr);
     }
 }
 
@@ -1279,37 +1263,28 @@ __global__ void __launch_bounds__(256) k_merge(LowdView<T, D> v, int n_all, int 
     add_counter(&v.ctr->work[4], lane == 0 ? chunks : 0u);
 }
 
-// Flatten the union-find: parent[c] = root for every cell with core points; count roots.
-// The only writes are parent[c] = root, so every pointer ends at its root.
-template <typename T, int D>
-__global__ void __launch_bounds__(256) k_compress(LowdView<T, D> v, int count_roots) {
-    const uint32_t C = v.ctr->n_cells;
-    uint32_t roots = 0;
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
-        if (!v.cell_core[c]) continue;
-        const uint32_t r = uf_root_readonly(v.parent, c, v.ctr);
-        v.parent[c] = r;
-        roots += (r == c);
-    }
-    roots = __reduce_add_sync(0xffffffffu, roots);
-    if (count_roots && lane_id() == 0 && roots) atomicAdd(&v.ctr->n_clusters, roots);
-}
-
-// Canonical cluster id (Algorithm 4 numbers clusters in traversal order; the fixed rule
-// here is the smallest input index among the cluster's core points).  The radix sort is
-// stable and starts from input order, so inside a cell the points keep their input order and
-// the first core point of a cell holds the cell's smallest core index: one atomicMin per cell
-// with core points.
+// Flatten the union-find (the only writes are parent[c] = root, so every pointer ends at its root),
+// count the roots, and the canonical cluster id (Algorithm 4 numbers clusters in traversal order;
+// the fixed rule here is the smallest input index among the cluster's core points).  The radix
+// sort is stable and starts from input order, so inside a cell the points keep their input
+// order and the first core point of a cell holds the cell's smallest core index: one atomicMin
+// per cell with core points.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_comp_min(LowdView<T, D> v) {
     const uint32_t NL = v.ctr->n_list[1];
+    uint32_t roots = 0;
     for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < NL; w += gridDim.x * blockDim.x) {
         const uint32_t A = v.list_core[w];
+        const uint32_t r = uf_root_readonly(v.parent, A, v.ctr);
+        v.parent[A] = r;
+        roots += (r == A);
         const uint32_t e = v.cell_start[A + 1];
         uint32_t i = v.cell_start[A];
         while (i < e && !v.core[i]) ++i;
-        if (i < e) atomicMin(&v.comp_min[v.parent[A]], v.perm[i]);
+        if (i < e) atomicMin(&v.comp_min[r], v.perm[i]);
     }
+    roots = __reduce_add_sync(0xffffffffu, roots);
+    if (lane_id() == 0 && roots) atomicAdd(&v.ctr->n_clusters, roots);
 }
 
 // Cluster ids of core points, point-parallel (a cell can hold tens of thousands of points);
@@ -1479,7 +1454,7 @@ __global__ void __launch_bounds__(256) k_box_check(BoxArgs single, const double 
         if (blockIdx.x != 0 || threadIdx.x >= D) return;
         const int i = threadIdx.x;
         const uint64_t *enc = ctr->minmax_enc;
-        if (dec_double_dev(enc[i]) < single.mn[i] || dec_double_dev(enc[kMaxD + i]) > single.mx[i])
+        if (dec_double_dev(~enc[i]) < single.mn[i] || dec_double_dev(enc[kMaxD + i]) > single.mx[i])
             atomicOr(&ctr->status, kErrBox);
         return;
     }
@@ -1487,7 +1462,7 @@ __global__ void __launch_bounds__(256) k_box_check(BoxArgs single, const double 
          k += (int64_t)gridDim.x * blockDim.x) {
         const int set = (int)(k / D), i = (int)(k % D);
         if (set_off[set + 1] == set_off[set]) continue;
-        const double lo = dec_double_dev(mm[(size_t)set * kMaxD + i]);
+        const double lo = dec_double_dev(~mm[(size_t)set * kMaxD + i]);
         const double hi = dec_double_dev(mm[(size_t)kMaxD * nsets + (size_t)set * kMaxD + i]);
         if (lo < boxes[(size_t)set * D + i] || hi > boxes[(size_t)(nsets + set) * D + i])
             atomicOr(&ctr->status, kErrBox);
@@ -1496,7 +1471,7 @@ __global__ void __launch_bounds__(256) k_box_check(BoxArgs single, const double 
 
 // Per-set min / max of every dimension for a batched call (set s = points [set_off[s],
 // set_off[s + 1]), d values each; mm[s * stride + i] and mm[(nsets + s) * stride + i] receive
-// the order-preserving codes of the minimum and maximum of dimension i).  Each warp takes a
+// the complement of the minimum's order-preserving code and the maximum's code of dimension i).  Each warp takes a
 // contiguous run of points, so it crosses few set boundaries: lanes hold running minima and
 // maxima of fixed dimensions (lane % d, for d <= 32 and 32 / d points per step; dimensions
 // lane and lane + 32 for larger d), and the warp folds them into the set's words with one
@@ -1533,16 +1508,16 @@ __device__ __forceinline__ void seg_minmax(const T *__restrict__ in, int64_t n, 
                     }
                 }
                 if (lane < d) {
-                    atomicMin(&mm[(uint64_t)set * stride + lane], (unsigned long long)enc_double((double)mn0));
+                    atomicMax(&mm[(uint64_t)set * stride + lane], ~(unsigned long long)enc_double((double)mn0));
                     atomicMax(&mm[((uint64_t)nsets + set) * stride + lane], (unsigned long long)enc_double((double)mx0));
                 }
             } else {
                 if (lane < d) {
-                    atomicMin(&mm[(uint64_t)set * stride + lane], (unsigned long long)enc_double((double)mn0));
+                    atomicMax(&mm[(uint64_t)set * stride + lane], ~(unsigned long long)enc_double((double)mn0));
                     atomicMax(&mm[((uint64_t)nsets + set) * stride + lane], (unsigned long long)enc_double((double)mx0));
                 }
                 if (lane + 32 < d) {
-                    atomicMin(&mm[(uint64_t)set * stride + lane + 32], (unsigned long long)enc_double((double)mn1));
+                    atomicMax(&mm[(uint64_t)set * stride + lane + 32], ~(unsigned long long)enc_double((double)mn1));
                     atomicMax(&mm[((uint64_t)nsets + set) * stride + lane + 32],
                               (unsigned long long)enc_double((double)mx1));
                 }
@@ -1625,7 +1600,8 @@ template <typename T, int D, typename K>
 __global__ void __launch_bounds__(256) k_bin_seg(const T *__restrict__ in, int64_t n, const int64_t *set_off,
                                                 int nsets, const GridParams *gtab, int key_bits,
                                                 K *__restrict__ keys, uint32_t *__restrict__ idx,
-                                                uint32_t *__restrict__ digit_counts, int total_bits) {
+                                                uint32_t *__restrict__ digit_counts, int total_bits, FillList fill) {
+    fill_regions(fill);
     __shared__ uint32_t h[8][256];
     const int passes = (total_bits + 7) / 8;
     for (int i = threadIdx.x; i < 8 * 256; i += blockDim.x) (&h[0][0])[i] = 0;

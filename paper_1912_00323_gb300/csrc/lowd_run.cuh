@@ -3,9 +3,11 @@
 #pragma once
 
 #include <math.h>
+#include <stddef.h>
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "lowd_kernels.cuh"
@@ -278,6 +280,17 @@ inline int grid_for(int64_t work, int per_block, int sms, int max_per_sm) {
     return (int)b;
 }
 
+// The part of the counters that the host reads (the digit counts after it stay on the device).
+constexpr size_t kCountersRead = offsetof(DevCounters, digit_counts);
+
+// The direct table of pencil keys of `bits` bits, in the space of the hash keys (8 cap_max bytes) when
+// it fits there: one load per lookup and one store per pencil, made in the pass that finds the
+// pencils, instead of two launches and a probe.  NULL: the keys span too much (many sets, four
+// spread-out dimensions), the hash table is used.
+inline uint32_t *pencil_table(int bits, int64_t cap_max, void *space) {
+    return bits < 40 && ((uint64_t)4 << bits) <= (uint64_t)8 * (uint64_t)cap_max ? (uint32_t *)space : nullptr;
+}
+
 }  // namespace detail
 
 template <typename T, int D>
@@ -299,15 +312,13 @@ int run_lowd(const RunArgs &a) {
     int64_t cap_max = 64;
     while (cap_max < 2 * n) cap_max <<= 1;
     const size_t hist_elems = sort_hist_size(n);
-    const int64_t scan_max = n > (int64_t)hist_elems ? n : (int64_t)hist_elems;
     const size_t o_ctr = take(sizeof(DevCounters));
     const size_t o_ka = take(8 * n), o_kb = take(8 * n), o_ia = take(4 * n), o_ib = take(4 * n);
     const size_t o_hist = take(4 * hist_elems);
-    const size_t o_part = take(4 * scan_partials_size(scan_max));
+    const size_t o_look = take(look_bytes(n));
     const size_t o_pts = take(sizeof(Pt<T, D>) * n);
-    const size_t o_flags = take(4 * n), o_excl = take(4 * n);
-    const size_t o_cstart = take(4 * (n + 1)), o_ckey = take(8 * n);
-    const size_t o_pflags = take(4 * n), o_pexcl = take(4 * n), o_pstart = take(4 * (n + 1));
+    const size_t o_flags = take(4 * n), o_lcount = take(4 * n), o_lcore = take(4 * n), o_llabel = take(4 * n);
+    const size_t o_cstart = take(4 * (n + 1)), o_ckey = take(8 * n), o_pstart = take(4 * (n + 1));
     const size_t o_hk = take(8 * cap_max), o_hv = take(4 * cap_max);
     const size_t o_core = take(n), o_ccore = take(n);
     const size_t o_parent = take(4 * n), o_cmin = take(4 * n);
@@ -341,6 +352,7 @@ int run_lowd(const RunArgs &a) {
     memset(&v, 0, sizeof(v));
     bool flipped = false;
     int sort_bits = 0;
+    uint32_t *ptab = nullptr;
     std::vector<GridParams> gsets;
     std::vector<uint64_t> hmm;
     GridParams *d_gtab = nullptr;
@@ -454,12 +466,10 @@ int run_lowd(const RunArgs &a) {
 
     mark(0);
     cudaMemsetAsync(ctr, 0, sizeof(DevCounters), s);
-    cudaMemsetAsync(ctr->minmax_enc, 0xff, sizeof(uint64_t) * kMaxD, s);
     if (!batched) {
         k_minmax<T, D><<<grid_for(n, 256, sms, 2), 256, 0, s>>>((const T *)a.d_points, n, ctr);
     } else {
-        cudaMemsetAsync(d_mm, 0xff, sizeof(uint64_t) * kMaxD * nsets, s);
-        cudaMemsetAsync(d_mm + (size_t)kMaxD * nsets, 0, sizeof(uint64_t) * kMaxD * nsets, s);
+        cudaMemsetAsync(d_mm, 0, sizeof(uint64_t) * 2 * kMaxD * nsets, s);
         upload(d_setoff, a.h_off, sizeof(int64_t) * (nsets + 1), stage_setoff);
         k_minmax_seg<T, D><<<grid_for(n, 256, sms, 8), 256, 0, s>>>((const T *)a.d_points, n, d_setoff, nsets,
                                                                   (unsigned long long *)d_mm, ctr);
@@ -491,19 +501,19 @@ int run_lowd(const RunArgs &a) {
             one, d_box, nsets, d_setoff, (const unsigned long long *)d_mm, ctr);
         ++launches;
     } else {
-        if (cudaMemcpyAsync(h, ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+        if (cudaMemcpyAsync(h, ctr, kCountersRead, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
             cudaStreamSynchronize(s) != cudaSuccess) { rc = HCA_ECUDA; goto out; }
         if (h->nan_seen) { rc = HCA_EINVAL; goto out; }
         if (a.ext_out && !batched)
             for (int i = 0; i < D; ++i) {
-                a.ext_out[i] = dec_double(h->minmax_enc[i]);
+                a.ext_out[i] = dec_double(~h->minmax_enc[i]);
                 a.ext_out[D + i] = dec_double(h->minmax_enc[kMaxD + i]);
             }
         if (batched)
-            rc = build_grids([&](int set, int i) { return dec_double(hmm[(size_t)set * kMaxD + i]); },
+            rc = build_grids([&](int set, int i) { return dec_double(~hmm[(size_t)set * kMaxD + i]); },
                              [&](int set, int i) { return dec_double(hmm[(size_t)kMaxD * nsets + (size_t)set * kMaxD + i]); });
         else
-            rc = build_grids([&](int, int i) { return dec_double(h->minmax_enc[i]); },
+            rc = build_grids([&](int, int i) { return dec_double(~h->minmax_enc[i]); },
                              [&](int, int i) { return dec_double(h->minmax_enc[kMaxD + i]); });
         if (rc) goto out;
         if (batched) cudaMemcpyAsync(d_gtab, gsets.data(), sizeof(GridParams) * nsets, cudaMemcpyHostToDevice, s);
@@ -516,67 +526,53 @@ int run_lowd(const RunArgs &a) {
         }
     }
     mark(1);
-    // ---- Algorithm 1: cell keys; pre-sort (Sec. 2) by a radix sort of (key, index) ----
+    // ---- Algorithm 1: cell keys; pre-sort (Sec. 2) by a radix sort of (key, index); the points
+    // in cell order, cells and pencils ----
     {
-        uint32_t *ia = (uint32_t *)(b + o_ia), *ib = (uint32_t *)(b + o_ib);
-        uint32_t *hist = (uint32_t *)(b + o_hist), *part = (uint32_t *)(b + o_part);
-        const bool use32 = sort_bits <= 32;
-        const int gtile = (int)((n + kScanTileElems - 1) / kScanTileElems);  // gather: one block per scan tile
-        if (use32) {
-            uint32_t *ka = (uint32_t *)(b + o_ka), *kb = (uint32_t *)(b + o_kb);
+        uint32_t *ia = (uint32_t *)(b + o_ia), *ib = (uint32_t *)(b + o_ib), *hist = (uint32_t *)(b + o_hist);
+        ptab = pencil_table(sort_bits - g.prefix_shift, cap_max, b + o_hk);
+        FillList fill = {};
+        fill.add(hist, sizeof(uint32_t) * hist_elems, 0u);
+        fill.add(b + o_look, look_bytes(n), 0u);
+        if (ptab) fill.add(ptab, sizeof(uint32_t) << (sort_bits - g.prefix_shift), 0xffffffffu);
+        auto front = [&](auto *ka, auto *kb) {
+            typedef typename std::remove_reference<decltype(*ka)>::type K;
             if (batched)
-                k_bin_seg<T, D, uint32_t><<<gpts, 256, 0, s>>>((const T *)a.d_points, n, d_setoff, nsets, d_gtab,
-                                                               g.key_bits, ka, ia, ctr->digit_counts, sort_bits);
+                k_bin_seg<T, D, K><<<gpts, 256, 0, s>>>((const T *)a.d_points, n, d_setoff, nsets, d_gtab, g.key_bits,
+                                                       ka, ia, ctr->digit_counts, sort_bits, fill);
             else
-                k_bin<T, D, uint32_t><<<gpts, 256, 0, s>>>((const T *)a.d_points, g, ka, ia, ctr->digit_counts);
-            ++launches;
+                k_bin<T, D, K><<<gpts, 256, 0, s>>>((const T *)a.d_points, g, ka, ia, ctr->digit_counts, fill);
             mark(2);
-            flipped = radix_sort_pairs<uint32_t>(ka, ia, kb, ib, n, 0, sort_bits, hist, part, s, &launches, &ctr->status, ctr->digit_counts);
+            flipped = radix_sort_pairs<K>(ka, ia, kb, ib, n, 0, sort_bits, hist, nullptr, s, &launches, &ctr->status,
+                                          ctr->digit_counts, true);
             mark(3);
-            k_gather<T, D, uint32_t><<<gtile, 256, 0, s>>>((const T *)a.d_points, flipped ? kb : ka,
-                                                           flipped ? ib : ia, n, (Pt<T, D> *)(b + o_pts),
-                                                           (uint32_t *)(b + o_flags), part);
-        } else {
-            uint64_t *ka = (uint64_t *)(b + o_ka), *kb = (uint64_t *)(b + o_kb);
-            if (batched)
-                k_bin_seg<T, D, uint64_t><<<gpts, 256, 0, s>>>((const T *)a.d_points, n, d_setoff, nsets, d_gtab,
-                                                               g.key_bits, ka, ia, ctr->digit_counts, sort_bits);
-            else
-                k_bin<T, D, uint64_t><<<gpts, 256, 0, s>>>((const T *)a.d_points, g, ka, ia, ctr->digit_counts);
-            ++launches;
-            mark(2);
-            flipped = radix_sort_pairs<uint64_t>(ka, ia, kb, ib, n, 0, sort_bits, hist, part, s, &launches, &ctr->status, ctr->digit_counts);
-            mark(3);
-            k_gather<T, D, uint64_t><<<gtile, 256, 0, s>>>((const T *)a.d_points, flipped ? kb : ka,
-                                                           flipped ? ib : ia, n, (Pt<T, D> *)(b + o_pts),
-                                                           (uint32_t *)(b + o_flags), part);
-        }
-        ++launches;
-        // run-length cells: scan of the gather's tile counts, cell ids / starts / keys
-        if (use32)
-            cells_from_flags<uint32_t>((const uint32_t *)(b + (flipped ? o_kb : o_ka)), (uint32_t *)(b + o_flags), n,
-                                       part, &ctr->n_cells, (uint32_t *)(b + o_cstart), (uint64_t *)(b + o_ckey), s,
-                                       &launches);
-        else
-            cells_from_flags<uint64_t>((const uint64_t *)(b + (flipped ? o_kb : o_ka)), (uint32_t *)(b + o_flags), n,
-                                       part, &ctr->n_cells, (uint32_t *)(b + o_cstart), (uint64_t *)(b + o_ckey), s,
-                                       &launches);
+            CellsArgs<K> ca;
+            ca.keys = flipped ? kb : ka;
+            ca.idx = flipped ? ib : ia;
+            ca.n = n;
+            ca.prefix_shift = g.prefix_shift;
+            ca.cell_of = (uint32_t *)(b + o_flags);
+            ca.cell_start = (uint32_t *)(b + o_cstart);
+            ca.cell_key = (uint64_t *)(b + o_ckey);
+            ca.pencil_start = (uint32_t *)(b + o_pstart);
+            ca.ptab = ptab;
+            ca.l = LookBack::at(b + o_look);
+            ca.ctr = ctr;
+            k_cells<T, D, K><<<(unsigned)((n + kScanTileElems - 1) / kScanTileElems), kTileThreads, 0, s>>>(
+                (const T *)a.d_points, ca, (Pt<T, D> *)(b + o_pts));
+            launches += 2;
+        };
+        if (sort_bits <= 32) front((uint32_t *)(b + o_ka), (uint32_t *)(b + o_kb));
+        else front((uint64_t *)(b + o_ka), (uint64_t *)(b + o_kb));
         v.perm = flipped ? ib : ia;
     }
     mark(4);
-    // ---- pencils and their hash table ----
-    {
-        uint32_t *part = (uint32_t *)(b + o_part);
-        k_pencil_flags<<<gpts, 256, 0, s>>>((const uint64_t *)(b + o_ckey), g.prefix_shift, ctr,
-                                            (uint32_t *)(b + o_pflags));
-        exclusive_scan_u32((uint32_t *)(b + o_pflags), (uint32_t *)(b + o_pexcl), n, &ctr->n_cells,
-                           &ctr->n_pencils, part, s, &launches);
+    if (!ptab) {
         k_hash_init<<<grid_for(cap_max, 256, sms, 8), 256, 0, s>>>((uint64_t *)(b + o_hk), ctr);
         k_pencils<<<gpts, 256, 0, s>>>((const uint64_t *)(b + o_ckey), g.prefix_shift,
-                                       (const uint32_t *)(b + o_pflags), (const uint32_t *)(b + o_pexcl),
-                                       (uint32_t *)(b + o_pstart), (uint64_t *)(b + o_hk),
+                                       (const uint32_t *)(b + o_pstart), (uint64_t *)(b + o_hk),
                                        (uint32_t *)(b + o_hv), ctr);
-        launches += 3;
+        launches += 2;
     }
     v.g = g;
     v.gtab = batched ? d_gtab : nullptr;
@@ -589,15 +585,16 @@ int run_lowd(const RunArgs &a) {
     v.pencil_start = (const uint32_t *)(b + o_pstart);
     v.hkeys = (uint64_t *)(b + o_hk);
     v.hvals = (uint32_t *)(b + o_hv);
+    v.ptab = ptab;
     v.core = (uint8_t *)(b + o_core);
     v.cell_core = (uint8_t *)(b + o_ccore);
     v.parent = (uint32_t *)(b + o_parent);
     v.reps = (uint64_t *)(b + o_reps);
     v.comp_min = (uint32_t *)(b + o_cmin);
     v.ranges = (uint2 *)ws_ranges;
-    v.list_count = (uint32_t *)(b + o_excl);   // the scan scratch of the cell and pencil passes is free now
-    v.list_core = (uint32_t *)(b + o_pflags);
-    v.list_label = (uint32_t *)(b + o_pexcl);
+    v.list_count = (uint32_t *)(b + o_lcount);
+    v.list_core = (uint32_t *)(b + o_lcore);
+    v.list_label = (uint32_t *)(b + o_llabel);
     v.rep_pts = (Pt<T, D> *)((char *)ws_ranges + align_up(sizeof(uint2) * (size_t)n * st.n_all));
     v.labels = a.d_labels;
     v.core_out = a.d_core;
@@ -620,11 +617,9 @@ int run_lowd(const RunArgs &a) {
     launches += 2;
     // ---- Algorithm 3: first links, pointer jumping, then one merge pass over every pair ----
     k_hook<T, D><<<gwarp, 256, 0, s>>>(v, st.n_all, st.n_half);
-    for (int r = 0; r < 3; ++r) k_jump<T, D><<<gpts, 256, 0, s>>>(v);
-    launches += 4;
+    k_flatten<T, D><<<gpts, 256, 0, s>>>(v);
     k_merge<T, D><<<gwarp, 256, 0, s>>>(v, st.n_all, st.n_half, 2);
-    k_compress<T, D><<<gpts, 256, 0, s>>>(v, 1);
-    launches += 2;
+    launches += 3;
     mark(8);
     // ---- Algorithm 4: cluster ids, border and noise ----
     k_comp_min<T, D><<<gpts, 256, 0, s>>>(v);
@@ -645,7 +640,7 @@ int run_lowd(const RunArgs &a) {
     launches += 3;
     mark(9);
     if (cudaGetLastError() != cudaSuccess) { rc = HCA_ECUDA; goto out; }
-    if (cudaMemcpyAsync(h, ctr, sizeof(DevCounters), cudaMemcpyDeviceToHost, s) != cudaSuccess) {
+    if (cudaMemcpyAsync(h, ctr, kCountersRead, cudaMemcpyDeviceToHost, s) != cudaSuccess) {
         rc = HCA_ECUDA;
         goto out;
     }

@@ -330,7 +330,8 @@ uint32_t *sort_status_word(uint32_t *hist, int64_t n) {
 template <typename K>
 bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, int64_t n,
                       int begin_bit, int end_bit, uint32_t *hist, uint32_t *partials,
-                      cudaStream_t s, int *launches, uint32_t *err_out, const uint32_t *digit_counts) {
+                      cudaStream_t s, int *launches, uint32_t *err_out, const uint32_t *digit_counts,
+                      bool hist_cleared) {
     (void)partials;
     if (n <= 1 || end_bit <= begin_bit) return false;
     const int nb = (int)sort_tiles(n);
@@ -339,7 +340,7 @@ bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, 
     uint32_t *ghist = hist + 2 * (size_t)nb * kRadix;
     uint32_t *tickets = ghist + kMaxPasses * kRadix;
     uint32_t *err = err_out ? err_out : sort_status_word(hist, n);
-    cudaMemsetAsync(hist, 0, sizeof(uint32_t) * sort_hist_size(n), s);
+    if (!hist_cleared) cudaMemsetAsync(hist, 0, sizeof(uint32_t) * sort_hist_size(n), s);
     if (digit_counts) {
         ghist = const_cast<uint32_t *>(digit_counts);
     } else {
@@ -368,9 +369,9 @@ bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, 
 
 template bool radix_sort_pairs<uint32_t>(uint32_t *, uint32_t *, uint32_t *, uint32_t *, int64_t,
                                          int, int, uint32_t *, uint32_t *, cudaStream_t, int *, uint32_t *,
-                                         const uint32_t *);
+                                         const uint32_t *, bool);
 template bool radix_sort_pairs<uint64_t>(uint64_t *, uint32_t *, uint64_t *, uint32_t *, int64_t,
                                          int, int, uint32_t *, uint32_t *, cudaStream_t, int *, uint32_t *,
-                                         const uint32_t *);
+                                         const uint32_t *, bool);
 
 }  // namespace hca

@@ -998,91 +998,110 @@ __device__ __forceinline__ uint32_t tc_chunks(uint32_t rows, uint32_t min_rows) 
     return rows >= min_rows ? (rows + (uint32_t)kTile - 1u) / (uint32_t)kTile : 0u;
 }
 
-// 128-row chunks of the counts for every coarse cell with at least min_rows points.
-static __global__ void __launch_bounds__(256) k_tc_chunks_count(const uint32_t *__restrict__ cell_start,
-                                                               const DevCounters *ctr, uint32_t min_rows,
-                                                               uint32_t *__restrict__ nch) {
-    const uint32_t C = ctr->n_cells;
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x)
-        nch[c] = tc_chunks(cell_start[c + 1] - cell_start[c], min_rows);
-}
+// Values and callbacks of the scans between the phases (k_scan_fn).
+struct NoEmit {
+    __device__ void operator()(int64_t, uint32_t, uint32_t) const {}
+};
 
-// The recount of handed-over rows: their flags (core = 2, set only by the tensor-core count; the
-// other cells' flags are still 0), their list (ascending) from the scan hx of the flags, and the
-// 128-row chunks of every cell with at least min_rows of them.
-static __global__ void __launch_bounds__(256) k_tc_handed_flags(const uint8_t *__restrict__ core, int64_t n,
-                                                               uint32_t *__restrict__ f) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
-        f[j] = core[j] == 2 ? 1u : 0u;
-}
+// 128-row chunks of the counts for every coarse cell with at least min_rows points; the callback
+// decodes the cell's box.
+template <int DP>
+struct CountChunks {
+    HdView<float, DP> v;
+    uint32_t min_rows;
+    __device__ uint32_t operator()(int64_t c) const { return tc_chunks(v.cell_start[c + 1] - v.cell_start[c], min_rows); }
+};
+template <int DP>
+struct BoxDecode {
+    HdView<float, DP> v;
+    __device__ void operator()(int64_t c, uint32_t, uint32_t) const {
+        uint4 *lo = reinterpret_cast<uint4 *>(v.box_lo + c * DP), *hi = reinterpret_cast<uint4 *>(v.box_hi + c * DP);
+        auto dec = [](uint4 x) {
+            return make_uint4(__float_as_uint(BoxCode<float>::dec(x.x)), __float_as_uint(BoxCode<float>::dec(x.y)),
+                              __float_as_uint(BoxCode<float>::dec(x.z)), __float_as_uint(BoxCode<float>::dec(x.w)));
+        };
+#pragma unroll
+        for (int i = 0; i < DP / 4; ++i) {
+            lo[i] = dec(lo[i]);
+            hi[i] = dec(hi[i]);
+        }
+    }
+};
 
-static __global__ void __launch_bounds__(256) k_tc_handed_list(const uint8_t *__restrict__ core,
-                                                              const uint32_t *__restrict__ hx, int64_t n,
-                                                              uint32_t *__restrict__ list) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
-        if (core[j] == 2) list[hx[j]] = (uint32_t)j;
-}
-
-static __global__ void __launch_bounds__(256) k_tc_chunks_recount(const uint32_t *__restrict__ cell_start,
-                                                                 const uint32_t *__restrict__ hx,
-                                                                 const DevCounters *ctr,
-                                                                 const uint2 *__restrict__ ranges, int n_all,
-                                                                 uint32_t min_rows, uint32_t *__restrict__ nch) {
-    const uint32_t C = ctr->n_cells;
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
+// The recount of handed-over rows: their list (ascending; core = 2, set only by the tensor-core
+// count, the other cells' flags are still 0) with its tallies cleared, and the work items of every
+// cell with at least min_rows of them.
+struct HandedFlag {
+    const uint8_t *core;
+    __device__ uint32_t operator()(int64_t j) const { return core[j] == 2 ? 1u : 0u; }
+};
+struct HandedList {
+    uint32_t *list, *in, *hi, *done;
+    __device__ void operator()(int64_t j, uint32_t f, uint32_t x) const {
+        if (!f) return;
+        list[x] = (uint32_t)j;
+        in[x] = 0u;
+        hi[x] = 0u;
+        done[x] = 0u;
+    }
+};
+struct RecountItems {
+    const uint32_t *cell_start, *hx;
+    const uint2 *ranges;
+    int n_all;
+    uint32_t min_rows;
+    __device__ uint32_t operator()(int64_t c) const {
         uint32_t items = tc_chunks(hx[cell_start[c + 1]] - hx[cell_start[c]], min_rows);
         if (items) {
             uint32_t len = 0;
-            for (int k = 0; k < n_all; ++k) len += count_range_len(ranges, n_all, cell_start, c, k);
+            for (int k = 0; k < n_all; ++k) len += count_range_len(ranges, n_all, cell_start, (uint32_t)c, k);
             items *= merge_windows(len);
         }
-        nch[c] = items;
+        return items;
     }
-}
+};
 
-// Core flags as uint32 for the scan that numbers the core points.
-static __global__ void __launch_bounds__(256) k_tc_core_flags(const uint8_t *__restrict__ core, int64_t n,
-                                                             uint32_t *__restrict__ f) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
-        f[j] = core[j];
-}
-
-// Core and non-core point lists (ascending) from the scan cx of the core flags.
-static __global__ void __launch_bounds__(256) k_tc_partition(const uint8_t *__restrict__ core,
-                                                            const uint32_t *__restrict__ cx, int64_t n,
-                                                            uint32_t *__restrict__ core_list,
-                                                            uint32_t *__restrict__ nc_list) {
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t x = cx[j];
-        if (core[j]) core_list[x] = (uint32_t)j;
+// Core numbering: core and (nullable) non-core point lists, ascending.
+struct CoreFlag {
+    const uint8_t *core;
+    __device__ uint32_t operator()(int64_t j) const { return core[j]; }
+};
+struct CoreLists {
+    uint32_t *core_list, *nc_list;
+    __device__ void operator()(int64_t j, uint32_t f, uint32_t x) const {
+        if (f) core_list[x] = (uint32_t)j;
         else if (nc_list) nc_list[(uint32_t)j - x] = (uint32_t)j;
     }
-}
+};
 
-// Work items of every coarse cell: for the unions, 128-row chunks of core rows (first launch)
-// and those chunks times the windows after the first (second launch), none for a cell that has
-// nothing left to join; for the labels, 128-row chunks of non-core rows.
+// Work items of every coarse cell: for the unions, 128-row chunks of core rows (first scan; none for
+// a cell that has nothing left to join) and those chunks times the windows after the first (left
+// in `later` for the second scan); for the labels, 128-row chunks of non-core rows (left in `nc`,
+// nullable, for the third).
 template <int DP>
-__global__ void __launch_bounds__(256) k_tc_chunks_split(HdView<float, DP> v, uint32_t min_core, uint32_t min_nc,
-                                                        uint32_t *__restrict__ nch_core,
-                                                        uint32_t *__restrict__ nch_later,
-                                                        uint32_t *__restrict__ nch_nc) {
-    const uint32_t C = v.ctr->n_cells;
-    for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
+struct MergeChunks {
+    HdView<float, DP> v;
+    uint32_t min_core, min_nc;
+    uint32_t *later, *nc;
+    __device__ uint32_t operator()(int64_t c) const {
         const uint32_t s = v.cell_start[c], e = v.cell_start[c + 1];
-        const uint32_t nc = v.cx[e] - v.cx[s];
-        uint32_t chunks = tc_chunks(nc, min_core), later = 0;
+        const uint32_t rows = v.cx[e] - v.cx[s];
+        uint32_t chunks = tc_chunks(rows, min_core), more = 0;
         if (chunks) {
             uint32_t len = 0;
-            for (int k = 0; k < v.n_half; ++k) len += merge_range_len(v, c, k);
-            if (len) later = chunks * (merge_windows(len) - 1u);
+            for (int k = 0; k < v.n_half; ++k) len += merge_range_len(v, (uint32_t)c, k);
+            if (len) more = chunks * (merge_windows(len) - 1u);
             else chunks = 0;
         }
-        nch_core[c] = chunks;
-        nch_later[c] = later;
-        if (nch_nc) nch_nc[c] = tc_chunks(e - s - nc, min_nc);
+        later[c] = more;
+        if (nc) nc[c] = tc_chunks(e - s - rows, min_nc);
+        return chunks;
     }
-}
+};
+struct Stored {
+    const uint32_t *x;
+    __device__ uint32_t operator()(int64_t i) const { return x[i]; }
+};
 
 // Cluster id of every core point (by core-list index, for the labels phase), its label and
 // the core flag output.
