@@ -63,8 +63,16 @@ __device__ __forceinline__ void fill_regions(const FillList &f) {
     }
 }
 
-// Sum of the earlier tiles' values; publishes this tile's (PAIR: the cells' words, two counts of 31
-// bits; else 32 bits and the epoch).  One full warp calls it; every lane returns the result.
+// A tile's own value (PAIR: the cells' words, two counts of 31 bits; else 32 bits and the epoch).
+template <bool PAIR>
+__device__ __forceinline__ void look_publish(const LookBack &l, uint32_t epoch, uint32_t tile, unsigned long long own) {
+    constexpr int kShift = PAIR ? 62 : 56;
+    const unsigned long long tag = PAIR ? 0ull : (unsigned long long)epoch << 58;
+    ((volatile unsigned long long *)l.words)[tile] = tag | (tile == 0 ? 2ull : 1ull) << kShift | own;
+}
+
+// Sum of the earlier tiles' values, and the sum with this tile's published.  One full warp calls it
+// after look_publish; every lane returns the result.
 template <bool PAIR>
 __device__ __forceinline__ unsigned long long look_back(const LookBack &l, uint32_t epoch, uint32_t tile,
                                                         unsigned long long own, uint32_t *err) {
@@ -74,7 +82,6 @@ __device__ __forceinline__ unsigned long long look_back(const LookBack &l, uint3
     constexpr unsigned long long kAgg = 1ull << kShift, kPrefix = 2ull << kShift;
     constexpr unsigned long long kValue = PAIR ? kAgg - 1ull : 0xffffffffull;
     const unsigned long long tag = PAIR ? 0ull : (unsigned long long)epoch << 58;
-    if (lane == 0) st[tile] = tag | (tile == 0 ? kPrefix : kAgg) | own;
     unsigned long long sum = 0;
     int64_t base = (int64_t)tile - 1;
     uint32_t spins = 0;
@@ -138,6 +145,7 @@ __global__ void __launch_bounds__(kTileThreads) k_scan_fn(F f, E emit, uint32_t 
     uint32_t all;
     uint32_t run = block_exclusive_scan<kTileThreads>(sum, &all);
     if (threadIdx.x < 32) {
+        if (threadIdx.x == 0) look_publish<false>(l, epoch, tile, all);
         const uint32_t b = (uint32_t)look_back<false>(l, epoch, tile, all, err);
         if (threadIdx.x == 0) {
             s_base = b;
@@ -194,9 +202,11 @@ struct CellsArgs {
     DevCounters *ctr;
 };
 
-// One tile (all 256 threads of the block).  on_cell(c) for every first point of a cell.
-template <typename K, typename F>
-__device__ __forceinline__ void cells_tile(const CellsArgs<K> &a, uint32_t tile, F on_cell) {
+// One tile (all 256 threads of the block): `between` runs after the tile's counts are published and
+// before the earlier tiles' are read, so that its loads cover the wait; on_cell(c) for every
+// first point of a cell.
+template <typename K, typename B, typename F>
+__device__ __forceinline__ void cells_tile(const CellsArgs<K> &a, uint32_t tile, B between, F on_cell) {
     constexpr int kWarps = kTileThreads / 32, kGroups = kTileItems * kWarps;  // 32-point groups
     static_assert(kGroups == 64, "two groups per lane of the scanning warp");
     __shared__ uint32_t s_cnt[kGroups];  // pencils << 16 | cells, then their exclusive sums
@@ -204,24 +214,27 @@ __device__ __forceinline__ void cells_tile(const CellsArgs<K> &a, uint32_t tile,
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t base = (int64_t)tile * kScanTileElems;
     unsigned cb[kTileItems], pb[kTileItems];
-    K key[kTileItems];
+    {
+        K key[kTileItems];
 #pragma unroll
-    for (int k = 0; k < kTileItems; ++k) {
-        const int64_t j = base + k * kTileThreads + threadIdx.x;
-        key[k] = j < a.n ? a.keys[j] : K(0);
-    }
+        for (int k = 0; k < kTileItems; ++k) {
+            const int64_t j = base + k * kTileThreads + threadIdx.x;
+            key[k] = j < a.n ? a.keys[j] : K(0);
+        }
 #pragma unroll
-    for (int k = 0; k < kTileItems; ++k) {
-        const int64_t j = base + k * kTileThreads + threadIdx.x;
-        K prev = __shfl_up_sync(0xffffffffu, key[k], 1);
-        if (lane == 0 && j > 0 && j < a.n) prev = a.keys[j - 1];
-        const bool c = j < a.n && (j == 0 || key[k] != prev);
-        const bool p = c && (j == 0 || ((uint64_t)key[k] >> a.prefix_shift) != ((uint64_t)prev >> a.prefix_shift));
-        cb[k] = __ballot_sync(0xffffffffu, c);
-        pb[k] = __ballot_sync(0xffffffffu, p);
-        if (lane == 0) s_cnt[k * kWarps + warp] = (uint32_t)__popc(pb[k]) << 16 | (uint32_t)__popc(cb[k]);
+        for (int k = 0; k < kTileItems; ++k) {
+            const int64_t j = base + k * kTileThreads + threadIdx.x;
+            K prev = __shfl_up_sync(0xffffffffu, key[k], 1);
+            if (lane == 0 && j > 0 && j < a.n) prev = a.keys[j - 1];
+            const bool c = j < a.n && (j == 0 || key[k] != prev);
+            const bool p = c && (j == 0 || ((uint64_t)key[k] >> a.prefix_shift) != ((uint64_t)prev >> a.prefix_shift));
+            cb[k] = __ballot_sync(0xffffffffu, c);
+            pb[k] = __ballot_sync(0xffffffffu, p);
+            if (lane == 0) s_cnt[k * kWarps + warp] = (uint32_t)__popc(pb[k]) << 16 | (uint32_t)__popc(cb[k]);
+        }
     }
     __syncthreads();
+    unsigned long long own = 0;
     if (warp == 0) {
         const uint32_t x0 = s_cnt[2 * lane], x1 = s_cnt[2 * lane + 1];  // (a tile has at most 2048 of each)
         const uint32_t incl = warp_inclusive_scan(x0 + x1);
@@ -229,7 +242,11 @@ __device__ __forceinline__ void cells_tile(const CellsArgs<K> &a, uint32_t tile,
         s_cnt[2 * lane] = incl - x0 - x1;
         s_cnt[2 * lane + 1] = incl - x1;
         // (fewer than 2^31 points: either count fits its 31 bits)
-        const unsigned long long own = (unsigned long long)(all >> 16) << 31 | (all & 0xffffu);
+        own = (unsigned long long)(all >> 16) << 31 | (all & 0xffffu);
+        if (lane == 0) look_publish<true>(a.l, 0u, tile, own);
+    }
+    between();
+    if (warp == 0) {
         const unsigned long long b = look_back<true>(a.l, 0u, tile, own, &a.ctr->status);
         if (lane == 0) {
             s_cells = (uint32_t)(b & 0x7fffffffull);
@@ -246,15 +263,16 @@ __device__ __forceinline__ void cells_tile(const CellsArgs<K> &a, uint32_t tile,
         const unsigned upto = lane == 31 ? 0xffffffffu : (2u << lane) - 1u;
         const uint32_t c = c0 + (off & 0xffffu) + (uint32_t)__popc(cb[k] & upto) - 1u;
         a.cell_of[j] = c;
-        if ((cb[k] >> lane) & 1u) {
-            a.cell_start[c] = (uint32_t)j;
-            a.cell_key[c] = (uint64_t)key[k];
-            on_cell(c);
-        }
         const uint32_t p = p0 + (off >> 16) + (uint32_t)__popc(pb[k] & upto) - 1u;
-        if ((pb[k] >> lane) & 1u) {
-            a.pencil_start[p] = c;
-            if (a.ptab) a.ptab[(uint64_t)key[k] >> a.prefix_shift] = p;
+        if ((cb[k] >> lane) & 1u) {
+            const uint64_t key = (uint64_t)a.keys[j];
+            a.cell_start[c] = (uint32_t)j;
+            a.cell_key[c] = key;
+            on_cell(c);
+            if ((pb[k] >> lane) & 1u) {
+                a.pencil_start[p] = c;
+                if (a.ptab) a.ptab[key >> a.prefix_shift] = p;
+            }
         }
         if (j == a.n - 1) {
             a.cell_start[c + 1] = (uint32_t)a.n;

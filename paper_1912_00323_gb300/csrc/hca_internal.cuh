@@ -132,14 +132,24 @@ void cells_from_flags(const K *keys, uint32_t *flags_cell_of, int64_t n, uint32_
 // most passes a call can make.  The scratch of a sort of n pairs is sort_hist_elems(n)
 // uint32: two words per tile and digit for the look-back, the digit counts of every pass,
 // one ticket per pass and a status word.
-constexpr int kSortTileKeys = 13312;
+constexpr int kSortThreads = 1024;
 constexpr int kSortRadix = 256;
 constexpr int kSortMaxPasses = 8;
+// Keys per thread of a tile: 13 for large sorts, and below about two million keys the fewest of 2,
+// 4 and 8 that still leave one tile per SM (152) or less, so that the passes of a small sort are
+// spread over the chip and each tile ranks fewer keys in turn.
+constexpr int sort_items_for(int64_t n) {
+    return n <= 150 * kSortThreads * 2 ? 2 : n <= 150 * kSortThreads * 4 ? 4 : n <= 150 * kSortThreads * 8 ? 8 : 13;
+}
 constexpr int64_t sort_tiles_for(int64_t n) {
-    return n <= kSortTileKeys ? 1 : (n + kSortTileKeys - 1) / kSortTileKeys;
+    const int64_t tile = (int64_t)sort_items_for(n) * kSortThreads;
+    return n <= tile ? 1 : (n + tile - 1) / tile;
 }
 constexpr size_t sort_hist_elems(int64_t n) {
-    return (size_t)(2 * sort_tiles_for(n) * kSortRadix + kSortMaxPasses * kSortRadix + kSortMaxPasses + 2);
+    // (where the tiles grow their number drops; the scratch keeps growing with n)
+    int64_t tiles = sort_tiles_for(n);
+    if (n > 150 * kSortThreads * 2 && tiles < 150) tiles = 150;
+    return (size_t)(2 * tiles * kSortRadix + kSortMaxPasses * kSortRadix + kSortMaxPasses + 2);
 }
 
 // LSD radix sort of (key, value) pairs by bits [begin_bit, end_bit), 8 bits per pass.
@@ -151,12 +161,13 @@ constexpr size_t sort_hist_elems(int64_t n) {
 inline size_t sort_hist_size(int64_t n) { return sort_hist_elems(n); }
 uint32_t *sort_status_word(uint32_t *hist, int64_t n);
 // digit_counts (optional, device): counts of every 8-bit digit of every pass, [pass][256],
-// already computed by the caller.  hist_cleared: the caller has cleared hist.
+// already computed by the caller.  hist_cleared: the caller has cleared hist.  identity: the values
+// are 0 .. n - 1 and vals need not hold them.
 template <typename K>
 bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, int64_t n,
                       int begin_bit, int end_bit, uint32_t *hist, uint32_t *partials,
                       cudaStream_t s, int *launches, uint32_t *err_out = nullptr,
-                      const uint32_t *digit_counts = nullptr, bool hist_cleared = false);
+                      const uint32_t *digit_counts = nullptr, bool hist_cleared = false, bool identity = false);
 
 // Pool allocation (stream ordered) used by api.cu and the pipelines.
 cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t s);

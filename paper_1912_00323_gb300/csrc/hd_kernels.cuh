@@ -396,8 +396,8 @@ __device__ __forceinline__ void count_digits_end(uint32_t (&h)[8][256], int pass
 // with the radix digit counts of the sort that follows.
 template <typename T, typename K>
 __global__ void __launch_bounds__(256) k_bin_proj(const T *__restrict__ in, int d, int3 sel, GridParams g,
-                                                 K *__restrict__ keys, uint32_t *__restrict__ idx,
-                                                 uint32_t *__restrict__ digit_counts, FillList fill) {
+                                                 K *__restrict__ keys, uint32_t *__restrict__ digit_counts,
+                                                 FillList fill) {
     __shared__ uint32_t h[8][256];
     fill_regions(fill);
     count_digits_begin(h);
@@ -414,7 +414,6 @@ __global__ void __launch_bounds__(256) k_bin_proj(const T *__restrict__ in, int 
             key |= (uint64_t)c << g.shift[i];
         }
         keys[j] = (K)key;
-        idx[j] = (uint32_t)j;
         count_digits(h, key, passes);
     }
     count_digits_end(h, passes, digit_counts);
@@ -435,33 +434,34 @@ __global__ void __launch_bounds__(kTileThreads) k_cells_hd(const T *__restrict__
     const int g = threadIdx.x % G, r0 = threadIdx.x / G;
     const uint32_t tile = take_tile(a.l, 0u);
     const int64_t base = (int64_t)tile * kScanTileElems;
+    cells_tile(a, tile, [&]() {
 #pragma unroll 4
-    for (int k = 0; k < kScanTileElems / R; ++k) {
-        const int64_t j = base + (int64_t)k * R + r0;
-        if (j >= a.n) break;
-        const uint32_t o = a.idx[j];
-        const T *src = in + (int64_t)o * d;
-        T x[4];
+        for (int k = 0; k < kScanTileElems / R; ++k) {
+            const int64_t j = base + (int64_t)k * R + r0;
+            if (j >= a.n) break;
+            const uint32_t o = a.idx[j];
+            const T *src = in + (int64_t)o * d;
+            T x[4];
 #pragma unroll
-        for (int u = 0; u < 4; ++u) x[u] = 4 * g + u < d ? src[4 * g + u] : T(0);
-        T *dst = pts + j * DP + 4 * g;
-        if (sizeof(T) == 4) {
-            *reinterpret_cast<float4 *>(dst) = make_float4((float)x[0], (float)x[1], (float)x[2], (float)x[3]);
-        } else {
-            reinterpret_cast<double2 *>(dst)[0] = make_double2((double)x[0], (double)x[1]);
-            reinterpret_cast<double2 *>(dst)[1] = make_double2((double)x[2], (double)x[3]);
-            if (fpts) {
-                const uint64_t set = set_shift < 64 ? (uint64_t)a.keys[j] >> set_shift : 0ull;
-                float f[4];
+            for (int u = 0; u < 4; ++u) x[u] = 4 * g + u < d ? src[4 * g + u] : T(0);
+            T *dst = pts + j * DP + 4 * g;
+            if (sizeof(T) == 4) {
+                *reinterpret_cast<float4 *>(dst) = make_float4((float)x[0], (float)x[1], (float)x[2], (float)x[3]);
+            } else {
+                reinterpret_cast<double2 *>(dst)[0] = make_double2((double)x[0], (double)x[1]);
+                reinterpret_cast<double2 *>(dst)[1] = make_double2((double)x[2], (double)x[3]);
+                if (fpts) {
+                    const uint64_t set = set_shift < 64 ? (uint64_t)a.keys[j] >> set_shift : 0ull;
+                    float f[4];
 #pragma unroll
-                for (int u = 0; u < 4; ++u)
-                    f[u] = 4 * g + u < d ? (float)__dsub_rn((double)x[u], dec_double_dev(~__ldg(mm + set * 64 + 4 * g + u))) : 0.f;
-                *reinterpret_cast<float4 *>(fpts + j * DP + 4 * g) = make_float4(f[0], f[1], f[2], f[3]);
+                    for (int u = 0; u < 4; ++u)
+                        f[u] = 4 * g + u < d ? (float)__dsub_rn((double)x[u], dec_double_dev(~__ldg(mm + set * 64 + 4 * g + u))) : 0.f;
+                    *reinterpret_cast<float4 *>(fpts + j * DP + 4 * g) = make_float4(f[0], f[1], f[2], f[3]);
+                }
             }
+            if (g == 0) core[j] = 0;
         }
-        if (g == 0) core[j] = 0;
-    }
-    cells_tile(a, tile, [cell_core](uint32_t c) { cell_core[c] = 0; });
+    }, [cell_core](uint32_t c) { cell_core[c] = 0; });
 }
 
 template <typename T, int DP>
@@ -1356,7 +1356,7 @@ __global__ void __launch_bounds__(256) k_minmax_rt_seg(const T *__restrict__ in,
 template <typename T, typename K>
 __global__ void __launch_bounds__(256) k_bin_proj_seg(const T *__restrict__ in, int64_t n, int d,
                                                      const int64_t *set_off, int nsets, const GridParams *gtab,
-                                                     int key_bits, K *__restrict__ keys, uint32_t *__restrict__ idx,
+                                                     int key_bits, K *__restrict__ keys,
                                                      uint32_t *__restrict__ digit_counts, int total_bits, FillList fill) {
     __shared__ uint32_t h[8][256];
     fill_regions(fill);
@@ -1375,7 +1375,6 @@ __global__ void __launch_bounds__(256) k_bin_proj_seg(const T *__restrict__ in, 
             key |= (uint64_t)c << g.shift[i];
         }
         keys[j] = (K)key;
-        idx[j] = (uint32_t)j;
         count_digits(h, key, passes);
     }
     count_digits_end(h, passes, digit_counts);

@@ -585,12 +585,12 @@ int run_hd(const RunArgs &a) {
             typedef typename std::remove_reference<decltype(*ka)>::type K;
             if (batched)
                 k_bin_proj_seg<T, K><<<gpts, 256, 0, s>>>((const T *)a.d_points, n, d, d_setoff, nsets, d_gtab,
-                                                         g.key_bits, ka, ia, ctr->digit_counts, sort_bits, fill);
+                                                         g.key_bits, ka, ctr->digit_counts, sort_bits, fill);
             else
-                k_bin_proj<T, K><<<gpts, 256, 0, s>>>((const T *)a.d_points, d, sel, g, ka, ia, ctr->digit_counts, fill);
+                k_bin_proj<T, K><<<gpts, 256, 0, s>>>((const T *)a.d_points, d, sel, g, ka, ctr->digit_counts, fill);
             mark(2);
             flipped = radix_sort_pairs<K>(ka, ia, kb, ib, n, 0, sort_bits, hist, nullptr, s, &launches, &ctr->status,
-                                          ctr->digit_counts, true);
+                                          ctr->digit_counts, true, true);
             mark(3);
             CellsArgs<K> ca;
             ca.keys = flipped ? kb : ka;

@@ -503,12 +503,11 @@ __global__ void __launch_bounds__(256) k_minmax(const T *__restrict__ in, int64_
 
 // Algorithm 1: band index of every coordinate, c_i = floor((x_i - o_i) / side), packed into a
 // key whose order is lexicographic in (c_0, ..., c_{d-1}).  Each thread step bins
-// VecPts::pts consecutive points read with 16-byte loads and stores their keys and indices
-// together.
+// VecPts::pts consecutive points read with 16-byte loads and stores their keys together.
 template <typename T, int D, typename K>
 __global__ void __launch_bounds__(256) k_bin(const T *__restrict__ in, GridParams g,
-                                            K *__restrict__ keys, uint32_t *__restrict__ idx,
-                                            uint32_t *__restrict__ digit_counts, FillList fill) {
+                                            K *__restrict__ keys, uint32_t *__restrict__ digit_counts,
+                                            FillList fill) {
     constexpr int P = VecPts<T, D>::pts;
     fill_regions(fill);
     // digit counts of every radix pass, for the sort that follows
@@ -544,25 +543,19 @@ __global__ void __launch_bounds__(256) k_bin(const T *__restrict__ in, GridParam
                 for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(uint32_t)(key >> (8 * p)) & 0xffu], 1u);
         }
         if (j0 + P <= g.n && sizeof(K) * P == 16) {
-            // P keys (16 bytes) and P indices at once
+            // P keys (16 bytes) at once
             if (sizeof(K) == 4) {
                 *reinterpret_cast<uint4 *>(keys + j0) =
                     make_uint4((uint32_t)kk[0], (uint32_t)kk[P > 1 ? 1 : 0], (uint32_t)kk[P > 2 ? 2 : 0],
                                (uint32_t)kk[P > 3 ? 3 : 0]);
-                *reinterpret_cast<uint4 *>(idx + j0) =
-                    make_uint4((uint32_t)j0, (uint32_t)j0 + 1u, (uint32_t)j0 + 2u, (uint32_t)j0 + 3u);
             } else {
                 *reinterpret_cast<ulonglong2 *>(keys + j0) =
                     make_ulonglong2((unsigned long long)kk[0], (unsigned long long)kk[P > 1 ? 1 : 0]);
-                *reinterpret_cast<uint2 *>(idx + j0) = make_uint2((uint32_t)j0, (uint32_t)j0 + 1u);
             }
         } else {
 #pragma unroll
             for (int t = 0; t < P; ++t) {
-                if (j0 + t < g.n) {
-                    keys[j0 + t] = kk[t];
-                    idx[j0 + t] = (uint32_t)(j0 + t);
-                }
+                if (j0 + t < g.n) keys[j0 + t] = kk[t];
             }
         }
     }
@@ -580,18 +573,23 @@ __global__ void __launch_bounds__(kTileThreads) k_cells(const T *__restrict__ in
                                                        Pt<T, D> *__restrict__ pts) {
     const uint32_t tile = take_tile(a.l, 0u);
     const int64_t base = (int64_t)tile * kScanTileElems;
+    cells_tile(a, tile, [&]() {
+        uint32_t o[kTileItems];
 #pragma unroll
-    for (int k = 0; k < kTileItems; ++k) {
-        const int64_t j = base + k * kTileThreads + threadIdx.x;
-        if (j < a.n) {
-            const uint32_t o = a.idx[j];
+        for (int k = 0; k < kTileItems; ++k) {
+            const int64_t j = base + k * kTileThreads + threadIdx.x;
+            o[k] = j < a.n ? a.idx[j] : 0u;
+        }
+#pragma unroll
+        for (int k = 0; k < kTileItems; ++k) {
+            const int64_t j = base + k * kTileThreads + threadIdx.x;
+            if (j >= a.n) continue;
             Pt<T, D> p = zero_pt<T, D>();
 #pragma unroll
-            for (int i = 0; i < D; ++i) p.x[i] = in[(int64_t)o * D + i];
+            for (int i = 0; i < D; ++i) p.x[i] = in[(int64_t)o[k] * D + i];
             pts[j] = p;
         }
-    }
-    cells_tile(a, tile, [](uint32_t) {});
+    }, [](uint32_t) {});
 }
 
 // The hash table of the pencils, when their keys span too much for a direct table: clear the used
@@ -902,7 +900,7 @@ __global__ void __launch_bounds__(256) k_core(LowdView<T, D> v, Stencil st_in) {
 
 // Algorithm 2: for every cell with core points and every direction delta, the core point
 // nearest to the ideal position of delta, and that point's coordinates (rep_pts).
-// The points are in cell order, so the pass walks them in windows of kRepWin consecutive
+// The points are in cell order, so the pass walks them in windows of WIN consecutive
 // points, one warp per window: every load of a window is issued at once (point, core flag,
 // cell id, then the cell key), which keeps the pass a stream over the sorted points.  Lane r
 // of a group of `width` lanes takes direction r and scans the group's core points in order,
@@ -912,7 +910,11 @@ __global__ void __launch_bounds__(256) k_core(LowdView<T, D> v, Stencil st_in) {
 // (distance bits, sorted index) (non-negative float bits order like the floats) and gets its
 // coordinates from k_rep_fix.  The representative only decides which pair a merge tests
 // first, never a label.
-constexpr uint32_t kRepWin = 128;     // points per warp window
+// Points per warp window: 64 (at 128 the window's shared memory leaves too few warps on an SM: 83
+// against 57 us at two million points); below kRepSmall points 32, since there are not enough
+// windows of 64 to fill the chip (18 -> 8 us at 10,000 points of d = 2).
+constexpr uint32_t kRepWin = 64, kRepWinSmall = 32;
+constexpr int64_t kRepSmall = 500000;
 constexpr int kRepWarps = 4;          // warps per block
 
 template <int NDIR>
@@ -920,34 +922,35 @@ struct RepWidth {  // lanes per direction group: the power of two >= NDIR
     static constexpr int value = NDIR <= 2 ? 2 : NDIR <= 4 ? 4 : NDIR <= 8 ? 8 : NDIR <= 16 ? 16 : 32;
 };
 
-template <int D>
+template <int D, uint32_t WIN>
 struct RepGeom {
     static constexpr int ndir = RepDirs<D>::value;
     static constexpr int width = RepWidth<ndir>::value;
     static constexpr int groups = 32 / width;
-    static constexpr uint32_t sub = kRepWin / groups;  // points scanned by one group
+    static constexpr uint32_t sub = WIN / groups;  // points scanned by one group
 };
 
 // Bits of the 32-point slice `it` of a window that fall in group g's range [g sub, (g+1) sub).
-template <int D>
+template <int D, uint32_t WIN>
 __device__ __forceinline__ unsigned rep_group_bits(int it, int g) {
-    constexpr int sub = (int)RepGeom<D>::sub;
+    constexpr int sub = (int)RepGeom<D, WIN>::sub;
     const int lo = max(g * sub - 32 * it, 0), hi = min((g + 1) * sub - 32 * it, 32);
     if (hi <= lo) return 0u;
     const unsigned upto = hi == 32 ? 0xffffffffu : ((1u << hi) - 1u);
     return upto & ~((1u << lo) - 1u);
 }
 
-template <typename T, int D>
+template <typename T, int D, uint32_t WIN>
 __global__ void __launch_bounds__(32 * kRepWarps) k_reps(LowdView<T, D> v, int64_t n) {
-    using Geo = RepGeom<D>;
+    using Geo = RepGeom<D, WIN>;
     constexpr int ndir = Geo::ndir;
-    constexpr int kPer = (int)(kRepWin / 32);
-    __shared__ float2 s_lh[kRepWarps][kRepWin][D];    // (lo2, hi2) of every dimension
-    __shared__ Pt<T, D> s_pt[kRepWarps][kRepWin];
-    __shared__ uint32_t s_cell[kRepWarps][kRepWin + 2];  // cell ids of points w0 - 1 .. w0 + kRepWin
+    constexpr int kPer = (int)(WIN / 32);
+    // per point and dimension 0, lo^2, hi^2: the term of a direction with delta_i = 0, -1, +1
+    __shared__ float s_t[kRepWarps][WIN][3 * D];
+    __shared__ Pt<T, D> s_pt[kRepWarps][WIN];
+    __shared__ uint32_t s_cell[kRepWarps][WIN + 2];  // cell ids of points w0 - 1 .. w0 + WIN
     const int lane = lane_id(), wib = threadIdx.x >> 5;
-    const int64_t w0 = ((int64_t)blockIdx.x * kRepWarps + wib) * kRepWin;
+    const int64_t w0 = ((int64_t)blockIdx.x * kRepWarps + wib) * WIN;
     if (w0 >= n) return;
     // ---- loads: cell ids, core flags and points of the window, then the cells' keys ----
     uint32_t cid[kPer];
@@ -962,16 +965,18 @@ __global__ void __launch_bounds__(32 * kRepWarps) k_reps(LowdView<T, D> v, int64
         pp[it] = in ? v.pts[j] : zero_pt<T, D>();
     }
     if (lane == 0) s_cell[wib][0] = w0 > 0 ? v.cell_of[w0 - 1] : 0xffffffffu;
-    if (lane == 1) s_cell[wib][kRepWin + 1] = w0 + kRepWin < n ? v.cell_of[w0 + kRepWin] : 0xffffffffu;
+    if (lane == 1) s_cell[wib][WIN + 1] = w0 + WIN < n ? v.cell_of[w0 + WIN] : 0xffffffffu;
     uint64_t key[kPer];
 #pragma unroll
     for (int it = 0; it < kPer; ++it) key[it] = cf[it] ? v.cell_key[cid[it]] : 0ull;
-    unsigned cmask[kPer];
+    unsigned cmask[kPer], smask[kPer];  // core points; points that start a cell (or the slice)
 #pragma unroll
     for (int it = 0; it < kPer; ++it) {
         const int p = lane + 32 * it;
         s_cell[wib][p + 1] = cid[it];
         cmask[it] = __ballot_sync(0xffffffffu, cf[it] != 0);
+        const uint32_t before = __shfl_up_sync(0xffffffffu, cid[it], 1);
+        smask[it] = __ballot_sync(0xffffffffu, lane == 0 || cid[it] != before);
         if (cf[it]) {
             const GridParams &G = params_of(v, set_of_key(v, key[it]));
             int ac[D];
@@ -981,7 +986,9 @@ __global__ void __launch_bounds__(32 * kRepWarps) k_reps(LowdView<T, D> v, int64
 #pragma unroll
             for (int k = 0; k < D; ++k) {
                 const float x = u[k] - (float)ac[k];
-                s_lh[wib][p][k] = make_float2(x * x, (1.f - x) * (1.f - x));
+                s_t[wib][p][3 * k] = 0.f;
+                s_t[wib][p][3 * k + 1] = x * x;
+                s_t[wib][p][3 * k + 2] = (1.f - x) * (1.f - x);
             }
             s_pt[wib][p] = pp[it];
         }
@@ -990,15 +997,17 @@ __global__ void __launch_bounds__(32 * kRepWarps) k_reps(LowdView<T, D> v, int64
     // ---- scan: lane r of group g takes direction r over the group's points.  The squared
     // distance of a point at cell-local position x to the ideal position of direction delta
     // (the face / edge / corner of the cube, Sec. 2) sums (1 - x_i)^2 over the dimensions with
-    // delta_i = +1 and x_i^2 over those with delta_i = -1: weights whi / wlo of the lane ----
+    // delta_i = +1 and x_i^2 over those with delta_i = -1.
+    // Bound by instruction issue: each term is one shared-memory load at the lane's offset (three
+    // words per point and dimension, so the lanes never conflict), and a run of core points of
+    // one cell is a loop of loads, two additions and a minimum without looking at masks or cell
+    // ids.  As six multiply-adds with lane weights per point and a mask step each, a point took 32
+    // instructions and the pass 79 us at two million points (490 us at 16 million); now 57 (349) ----
     const int g = lane / Geo::width, r = lane % Geo::width;
     const bool active = r < ndir;
-    float wlo[D], whi[D];
+    int off[D];
 #pragma unroll
-    for (int k = 0; k < D; ++k) {
-        wlo[k] = 0.f;
-        whi[k] = 0.f;
-    }
+    for (int k = 0; k < D; ++k) off[k] = 3 * k;
     if (active) {
         if (D <= 3) {
             int code = r < (ndir / 2) ? r : r + 1;
@@ -1006,16 +1015,10 @@ __global__ void __launch_bounds__(32 * kRepWarps) k_reps(LowdView<T, D> v, int64
             for (int k = 0; k < D; ++k) {
                 const int sgn = code % 3 - 1;
                 code /= 3;
-                if (sgn > 0) whi[k] = 1.f;
-                if (sgn < 0) wlo[k] = 1.f;
+                off[k] += sgn < 0 ? 1 : sgn > 0 ? 2 : 0;
             }
         } else {
-#pragma unroll
-            for (int k = 0; k < D; ++k)
-                if (k == (r >> 1)) {
-                    if (r & 1) whi[k] = 1.f;
-                    else wlo[k] = 1.f;
-                }
+            off[0] = 3 * (r >> 1) + ((r & 1) ? 2 : 1);  // axis directions: one term
         }
     }
     // cells of the points just before and just after the group's range: a run of either
@@ -1035,28 +1038,44 @@ __global__ void __launch_bounds__(32 * kRepWarps) k_reps(LowdView<T, D> v, int64
             v.rep_pts[slot] = s_pt[wib][bp];
         }
     };
+    auto take = [&](int p) {
+        const float *t = s_t[wib][p];
+        float dd = t[off[0]];
+        if (D <= 3) {
+#pragma unroll
+            for (int k = 1; k < D; ++k) dd += t[off[k]];
+        }
+        if (dd < best) {
+            best = dd;
+            bp = p;
+        }
+    };
 #pragma unroll
     for (int it = 0; it < kPer; ++it) {
-        unsigned mm = cmask[it] & rep_group_bits<D>(it, g);
+        unsigned mm = cmask[it] & rep_group_bits<D, WIN>(it, g);
         while (mm) {
-            const int p = 32 * it + __ffs(mm) - 1;
-            mm &= mm - 1;
-            const uint32_t c = s_cell[wib][p + 1];
+            const int b = __ffs(mm) - 1;
+            const uint32_t c = s_cell[wib][32 * it + b + 1];
             if (c != cur) {
                 if (cur != 0xffffffffu) flush();
                 cur = c;
                 best = FLT_MAX;
             }
-            float dd = 0.f;
+            // the core points of this cell in the slice: up to the next cell's first point
+            const unsigned later = smask[it] & ~((2u << b) - 1u);
+            const unsigned seg = b == 31 || !later ? mm : mm & ((later & (0u - later)) - 1u);
+            mm &= ~seg;
+            const int m = __popc(seg);
+            if (32 - __clz(seg) - b == m) {  // without a gap
+                int p = 32 * it + b;
+                const int e = p + m;
+                for (; p + 4 <= e; p += 4) {
 #pragma unroll
-            for (int i = 0; i < D; ++i) {
-                const float2 lh = s_lh[wib][p][i];
-                dd = __fmaf_rn(wlo[i], lh.x, dd);
-                dd = __fmaf_rn(whi[i], lh.y, dd);
-            }
-            if (dd < best) {
-                best = dd;
-                bp = p;
+                    for (int u = 0; u < 4; ++u) take(p + u);
+                }
+                for (; p < e; ++p) take(p);
+            } else {
+                for (unsigned x = seg; x; x &= x - 1) take(32 * it + __ffs(x) - 1);
             }
         }
     }
@@ -1066,9 +1085,9 @@ __global__ void __launch_bounds__(32 * kRepWarps) k_reps(LowdView<T, D> v, int64
 // Coordinates of the representatives of the cells that cross a scan-range boundary of
 // k_reps (their pieces were combined by atomicMin): one thread per (boundary, direction).
 // A cell that crosses several boundaries is written several times with the same values.
-template <typename T, int D>
+template <typename T, int D, uint32_t WIN>
 __global__ void __launch_bounds__(256) k_rep_fix(LowdView<T, D> v, int64_t n) {
-    using Geo = RepGeom<D>;
+    using Geo = RepGeom<D, WIN>;
     constexpr int ndir = Geo::ndir;
     const int64_t nb = (n + Geo::sub - 1) / Geo::sub;
     for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < nb * ndir;
@@ -1206,6 +1225,7 @@ __global__ void __launch_bounds__(256) k_merge(LowdView<T, D> v, int n_all, int 
         const uint64_t akey = v.cell_key[A];
         unpack_key<D>(akey, v.g, ac);
         const GridParams &G = params_of(v, set_of_key(v, akey));
+        const uint32_t pa = __ldcg(v.parent + A);
         for (int g0 = 0; g0 < n_half; g0 += 32) {
             const int k = g0 + lane;
             uint2 rg = k < n_half ? v.ranges[(uint64_t)A * n_all + k] : make_uint2(0u, 0u);
@@ -1214,8 +1234,12 @@ __global__ void __launch_bounds__(256) k_merge(LowdView<T, D> v, int n_all, int 
             for (uint32_t f0 = 0; f0 < lr.total; f0 += 32) {
                 const uint32_t f = f0 + lane;
                 const uint32_t B = flat_cell(lr, f < lr.total ? f : 0u);
-                const uint64_t bkey = f < lr.total ? v.cell_key[B] : 0ull;  // loaded with the core flag
-                bool pending = f < lr.total && v.cell_core[B];
+                // key, tree node and core flag in one round of loads; after the flattening two cells
+                // of one tree have the same node, and most pairs end here (walking both cells to
+                // their roots first took two more rounds)
+                const uint64_t bkey = f < lr.total ? v.cell_key[B] : 0ull;
+                const uint32_t pb = f < lr.total ? __ldcg(v.parent + B) : pa;
+                bool pending = f < lr.total && v.cell_core[B] && pb != pa;
                 int bc[D], delta[D];
                 if (pending) {
                     unpack_key<D>(bkey, v.g, bc);
@@ -1599,8 +1623,8 @@ __global__ void __launch_bounds__(256) k_minmax_seg(const T *__restrict__ in, in
 template <typename T, int D, typename K>
 __global__ void __launch_bounds__(256) k_bin_seg(const T *__restrict__ in, int64_t n, const int64_t *set_off,
                                                 int nsets, const GridParams *gtab, int key_bits,
-                                                K *__restrict__ keys, uint32_t *__restrict__ idx,
-                                                uint32_t *__restrict__ digit_counts, int total_bits, FillList fill) {
+                                                K *__restrict__ keys, uint32_t *__restrict__ digit_counts,
+                                                int total_bits, FillList fill) {
     fill_regions(fill);
     __shared__ uint32_t h[8][256];
     const int passes = (total_bits + 7) / 8;
@@ -1626,7 +1650,6 @@ __global__ void __launch_bounds__(256) k_bin_seg(const T *__restrict__ in, int64
             key |= (uint64_t)c << g.shift[i];
         }
         keys[j] = (K)key;
-        idx[j] = (uint32_t)j;
         for (int p = 0; p < passes; ++p) atomicAdd(&h[p][(uint32_t)(key >> (8 * p)) & 0xffu], 1u);
     }
     __syncthreads();

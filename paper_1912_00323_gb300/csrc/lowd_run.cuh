@@ -539,12 +539,12 @@ int run_lowd(const RunArgs &a) {
             typedef typename std::remove_reference<decltype(*ka)>::type K;
             if (batched)
                 k_bin_seg<T, D, K><<<gpts, 256, 0, s>>>((const T *)a.d_points, n, d_setoff, nsets, d_gtab, g.key_bits,
-                                                       ka, ia, ctr->digit_counts, sort_bits, fill);
+                                                       ka, ctr->digit_counts, sort_bits, fill);
             else
-                k_bin<T, D, K><<<gpts, 256, 0, s>>>((const T *)a.d_points, g, ka, ia, ctr->digit_counts, fill);
+                k_bin<T, D, K><<<gpts, 256, 0, s>>>((const T *)a.d_points, g, ka, ctr->digit_counts, fill);
             mark(2);
             flipped = radix_sort_pairs<K>(ka, ia, kb, ib, n, 0, sort_bits, hist, nullptr, s, &launches, &ctr->status,
-                                          ctr->digit_counts, true);
+                                          ctr->digit_counts, true, true);
             mark(3);
             CellsArgs<K> ca;
             ca.keys = flipped ? kb : ka;
@@ -610,12 +610,19 @@ int run_lowd(const RunArgs &a) {
     // ---- Algorithm 2: representative points and their coordinates (the stage times k_reps
     // alone; the coordinates of boundary-crossing cells are counted with the merge stage) ----
     mark(6);
-    k_reps<T, D><<<(unsigned)((n + (int64_t)kRepWin * kRepWarps - 1) / ((int64_t)kRepWin * kRepWarps)),
-                   32 * kRepWarps, 0, s>>>(v, n);
-    mark(7);
-    k_rep_fix<T, D><<<grid_for((n / RepGeom<D>::sub + 1) * ndir, 256, sms, 8), 256, 0, s>>>(v, n);
+    {
+        auto reps = [&](auto win) {
+            constexpr uint32_t W = decltype(win)::value;
+            k_reps<T, D, W><<<(unsigned)((n + (int64_t)W * kRepWarps - 1) / ((int64_t)W * kRepWarps)), 32 * kRepWarps,
+                              0, s>>>(v, n);
+            mark(7);
+            k_rep_fix<T, D, W><<<grid_for((n / RepGeom<D, W>::sub + 1) * ndir, 256, sms, 8), 256, 0, s>>>(v, n);
+        };
+        if (n < kRepSmall) reps(std::integral_constant<uint32_t, kRepWinSmall>());
+        else reps(std::integral_constant<uint32_t, kRepWin>());
+    }
     launches += 2;
-    // ---- Algorithm 3: first links, pointer jumping, then one merge pass over every pair ----
+    // ---- Algorithm 3: first links, flattened, then one merge pass over every pair ----
     k_hook<T, D><<<gwarp, 256, 0, s>>>(v, st.n_all, st.n_half);
     k_flatten<T, D><<<gpts, 256, 0, s>>>(v);
     k_merge<T, D><<<gwarp, 256, 0, s>>>(v, st.n_all, st.n_half, 2);

@@ -2,8 +2,8 @@
 //
 // A first kernel counts the digits of every pass over all keys (the counts do not depend on
 // the order, so one read of the keys serves all passes); a caller that produced the keys may
-// pass these counts in instead.  Each pass kernel then takes a tile of 13,312 keys (1024
-// threads x 13), ranks every key stably among the keys of its tile with the same digit (the
+// pass these counts in instead.  Each pass kernel then takes a tile of 1024 threads x 2, 4, 8
+// or 13 keys (sort_items_for), ranks every key stably among the keys of its tile with the same digit (the
 // lanes of a warp with one digit found by a match instruction or by shared-memory OR masks,
 // per-warp digit counters, an exclusive scan across warps), publishes the tile's digit
 // counts, scatters the tile through shared memory in digit order, learns how many keys of each
@@ -11,7 +11,10 @@
 // coalesced stores.
 //
 // Tile size.  A tile is one CTA per SM (its shared memory holds the whole tile), so at two
-// million keys the ~150 tiles all run at once.  With every tile running together a published
+// million keys the ~150 tiles of 13,312 all run at once.  A smaller sort takes smaller tiles, so
+// that it spreads over as many SMs and each ranks fewer keys in turn: four passes over 300,001
+// keys 70 -> 46 us, two over 10,000 28 -> 19 us (one tile of 13,312 before).  Two CTAs of 512
+// threads per SM instead were slower (two million keys 76 -> 109 us).  With every tile running together a published
 // prefix reaches the later tiles only through their own reads, so the look-back reads 64
 // predecessors per round trip (four thread quarters of 16 words per digit): the last tile of
 // two million keys needs three round trips instead of the dozens that a 4096-key tile with a
@@ -31,6 +34,8 @@
 // epoch (pass number + 1) makes words left by an earlier pass invisible.  Words are tile-major
 // (the 256 digits of one tile are consecutive), so a warp reads 32 digits of a tile in one
 // coalesced 256-byte access.
+#include <type_traits>
+
 #include "block_scan.cuh"
 #include "hca_internal.cuh"
 
@@ -38,16 +43,12 @@ namespace hca {
 
 namespace {
 
-constexpr int kSortThreads = 1024;
-constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kSortItems = 13;  // per lane: a warp covers 416 consecutive keys
-constexpr int kSortTile = kSortThreads * kSortItems;
 constexpr int kRadix = kSortRadix;
 constexpr int kMaxPasses = kSortMaxPasses;
-constexpr int kQuarters = kSortThreads / kRadix;  // threads per digit in the look-back
 constexpr int kLbWords = 16;                      // predecessors per thread per round trip
 constexpr int kHistThreads = 256;
-static_assert(kSortTile == kSortTileKeys, "tile size shared with the scratch sizing");
+constexpr int kSortWarps = kSortThreads / 32;
+constexpr int kQuarters = kSortThreads / kRadix;  // threads per digit in the look-back
 static_assert(kQuarters * kRadix == kSortThreads, "whole quarters of digits");
 constexpr uint32_t kSpinLimit = 1u << 24;
 // Up to this many tiles a tile sums the counts of all earlier tiles instead of the decoupled
@@ -88,35 +89,37 @@ __global__ void __launch_bounds__(kHistThreads) k_os_hist(const K *__restrict__ 
 }
 
 // Shared memory of a pass (dynamic, 16-byte aligned).
-template <typename K>
+template <typename K, int ITEMS>
 struct PassSmem {
-    uint32_t whist[kSortWarps][kRadix];   // per-warp digit counts, then per-warp digit offsets
-    uint32_t part[kQuarters][kRadix];     // counts of warps [8q, 8q + 8), per digit
-    uint32_t lstart[kRadix];              // first position of each digit in the tile
-    uint32_t goff[kRadix];                // global position of the tile's first key of each digit
+    static constexpr int tile = ITEMS * kSortThreads;
+    uint32_t whist[kSortWarps][kRadix];       // per-warp digit counts, then per-warp digit offsets
+    uint32_t part[kQuarters][kRadix];     // counts of a quarter's warps, per digit
+    uint32_t lstart[kRadix];                // first position of each digit in the tile
+    uint32_t goff[kRadix];                  // global position of the tile's first key of each digit
     uint32_t lb_sum[kQuarters][kRadix];   // look-back: AGG sum of a quarter's window
     uint32_t lb_used[kQuarters][kRadix];  // predecessors the quarter consumed
     uint32_t lb_kind[kQuarters][kRadix];  // 0 window read through, 1 met a PREFIX, 2 met an unpublished word
-    int32_t lb_next[kRadix];              // nearest predecessor not yet added, per digit (-1: done)
+    int32_t lb_next[kRadix];                // nearest predecessor not yet added, per digit (-1: done)
     uint32_t tile_id, pad[3];
     union {
-        uint32_t wmask[kSortWarps][kRadix];  // ranking: per-warp lane masks of each digit
-        K keys[kSortTile];                   // then: the tile in digit order
+        uint32_t wmask[kSortWarps][kRadix];   // ranking: per-warp lane masks of each digit
+        K keys[tile];                       // then: the tile in digit order
     };
-    uint32_t vals[kSortTile];
+    uint32_t vals[tile];
 };
-static_assert(sizeof(uint32_t) * kSortWarps * kRadix <= sizeof(uint32_t) * kSortTile, "masks fit the key array");
 
 // One pass: rank within the tile, publish the tile's digit counts, scatter the tile into
 // shared memory in digit order, look back for the counts of the earlier tiles, write out.
-template <typename K>
+// IDENT: the values are the positions (first pass of a sort of indices; vals_in is not read).
+template <typename K, int ITEMS, bool IDENT>
 __global__ void __launch_bounds__(kSortThreads, 1) k_os_pass(
     const K *__restrict__ keys_in, const uint32_t *__restrict__ vals_in, K *__restrict__ keys_out,
     uint32_t *__restrict__ vals_out, int64_t n, int shift, int mask_bits,
     const uint32_t *__restrict__ ghist_pass, unsigned long long *status, uint32_t *ticket, uint32_t epoch,
     uint32_t *err, bool full_sum) {
+    constexpr int kSortItems = ITEMS, kSortTile = ITEMS * kSortThreads;
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    PassSmem<K> &S = *reinterpret_cast<PassSmem<K> *>(sm_raw);
+    PassSmem<K, ITEMS> &S = *reinterpret_cast<PassSmem<K, ITEMS> *>(sm_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int dg = threadIdx.x & (kRadix - 1), q = threadIdx.x / kRadix;
     const uint32_t mask = (1u << mask_bits) - 1u;
@@ -144,7 +147,7 @@ __global__ void __launch_bounds__(kSortThreads, 1) k_os_pass(
     for (int r = 0; r < kSortItems; ++r) {
         const int64_t i = wbase + r * 32 + lane;
         const bool valid = i < n;
-        v[r] = valid ? vals_in[i] : 0u;
+        v[r] = IDENT ? (uint32_t)i : valid ? vals_in[i] : 0u;
         const uint32_t d = valid ? ((uint32_t)(k[r] >> shift) & mask) : (uint32_t)kRadix;
         // the lanes holding the same digit: a match instruction when lane 0's digit recurs
         // often (few distinct digits), else one shared-memory OR per lane into the warp's
@@ -319,23 +322,49 @@ __global__ void __launch_bounds__(kSortThreads, 1) k_os_pass(
     }
 }
 
-int64_t sort_tiles(int64_t n) { return sort_tiles_for(n); }
+// The passes of one sort.
+template <typename K, int ITEMS>
+bool run_passes(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, int64_t n, int begin_bit, int end_bit,
+                const uint32_t *ghist, unsigned long long *status, uint32_t *tickets, uint32_t *err, bool identity,
+                cudaStream_t s) {
+    const int nb = (int)((n + (int64_t)ITEMS * kSortThreads - 1) / ((int64_t)ITEMS * kSortThreads));
+    const int passes = (end_bit - begin_bit + 7) / 8;
+    const size_t smem = sizeof(PassSmem<K, ITEMS>);
+    cudaFuncSetAttribute(k_os_pass<K, ITEMS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_os_pass<K, ITEMS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    bool flipped = false;
+    K *kin = keys, *kout = keys_alt;
+    uint32_t *vin = vals, *vout = vals_alt;
+    for (int p = 0; p < passes; ++p) {
+        const int shift = begin_bit + 8 * p;
+        const int bits = (end_bit - shift) < 8 ? (end_bit - shift) : 8;
+        auto kern = p == 0 && identity ? k_os_pass<K, ITEMS, true> : k_os_pass<K, ITEMS, false>;
+        kern<<<nb, kSortThreads, smem, s>>>(kin, vin, kout, vout, n, shift, bits, ghist + p * kRadix, status, tickets + p,
+                                            (uint32_t)(p + 1), err, nb <= kFullSumTiles);
+        K *tk = kin; kin = kout; kout = tk;
+        uint32_t *tv = vin; vin = vout; vout = tv;
+        flipped = !flipped;
+    }
+    return flipped;
+}
 
 }  // namespace
 
 uint32_t *sort_status_word(uint32_t *hist, int64_t n) {
-    return hist + 2 * sort_tiles(n) * kRadix + kMaxPasses * kRadix + kMaxPasses;
+    return hist + 2 * sort_tiles_for(n) * kRadix + kMaxPasses * kRadix + kMaxPasses;
 }
 
 template <typename K>
 bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, int64_t n,
                       int begin_bit, int end_bit, uint32_t *hist, uint32_t *partials,
                       cudaStream_t s, int *launches, uint32_t *err_out, const uint32_t *digit_counts,
-                      bool hist_cleared) {
+                      bool hist_cleared, bool identity) {
     (void)partials;
-    if (n <= 1 || end_bit <= begin_bit) return false;
-    const int nb = (int)sort_tiles(n);
-    const int passes = (end_bit - begin_bit + 7) / 8;
+    if (n <= 1 || end_bit <= begin_bit) {
+        if (identity && n == 1) cudaMemsetAsync(vals, 0, sizeof(uint32_t), s);
+        return false;
+    }
+    const int64_t nb = sort_tiles_for(n);
     unsigned long long *status = reinterpret_cast<unsigned long long *>(hist);  // 8-byte aligned
     uint32_t *ghist = hist + 2 * (size_t)nb * kRadix;
     uint32_t *tickets = ghist + kMaxPasses * kRadix;
@@ -348,30 +377,24 @@ bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, 
         k_os_hist<K><<<hb < 1216 ? (int)hb : 1216, kHistThreads, 0, s>>>(keys, n, begin_bit, end_bit, ghist);
         if (launches) *launches += 1;
     }
-    const size_t smem = sizeof(PassSmem<K>);
-    cudaFuncSetAttribute(k_os_pass<K>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    bool flipped = false;
-    K *kin = keys, *kout = keys_alt;
-    uint32_t *vin = vals, *vout = vals_alt;
-    for (int p = 0; p < passes; ++p) {
-        const int shift = begin_bit + 8 * p;
-        const int bits = (end_bit - shift) < 8 ? (end_bit - shift) : 8;
-        k_os_pass<K><<<nb, kSortThreads, smem, s>>>(kin, vin, kout, vout, n, shift, bits, ghist + p * kRadix,
-                                                    status, tickets + p, (uint32_t)(p + 1), err,
-                                                    nb <= kFullSumTiles);
-        K *tk = kin; kin = kout; kout = tk;
-        uint32_t *tv = vin; vin = vout; vout = tv;
-        flipped = !flipped;
+    if (launches) *launches += (end_bit - begin_bit + 7) / 8;
+    auto run = [&](auto items) {
+        return run_passes<K, decltype(items)::value>(keys, vals, keys_alt, vals_alt, n, begin_bit, end_bit, ghist, status,
+                                                     tickets, err, identity, s);
+    };
+    switch (sort_items_for(n)) {
+        case 2: return run(std::integral_constant<int, 2>());
+        case 4: return run(std::integral_constant<int, 4>());
+        case 8: return run(std::integral_constant<int, 8>());
     }
-    if (launches) *launches += passes;
-    return flipped;
+    return run(std::integral_constant<int, 13>());
 }
 
 template bool radix_sort_pairs<uint32_t>(uint32_t *, uint32_t *, uint32_t *, uint32_t *, int64_t,
                                          int, int, uint32_t *, uint32_t *, cudaStream_t, int *, uint32_t *,
-                                         const uint32_t *, bool);
+                                         const uint32_t *, bool, bool);
 template bool radix_sort_pairs<uint64_t>(uint64_t *, uint32_t *, uint64_t *, uint32_t *, int64_t,
                                          int, int, uint32_t *, uint32_t *, cudaStream_t, int *, uint32_t *,
-                                         const uint32_t *, bool);
+                                         const uint32_t *, bool, bool);
 
 }  // namespace hca
