@@ -117,6 +117,7 @@ template <typename F, typename E>
 __global__ void __launch_bounds__(kTileThreads) k_scan_fn(F f, E emit, uint32_t *out, int64_t m_max,
                                                          const uint32_t *m_dev, uint32_t *total, LookBack l,
                                                          uint32_t epoch, uint32_t *err) {
+    pdl_enter();
     __shared__ uint32_t s_val[kScanTileElems];
     __shared__ uint32_t s_tile, s_base;
     const int64_t m = m_dev ? min((int64_t)*m_dev, m_max) : m_max;
@@ -180,7 +181,7 @@ struct Scans {
     template <typename F, typename E>
     void run(F f, E emit, uint32_t *out, int64_t m_max, const uint32_t *m_dev, uint32_t *total) {
         const unsigned tiles = (unsigned)((m_max + kScanTileElems - 1) / kScanTileElems);
-        k_scan_fn<F, E><<<tiles ? tiles : 1u, kTileThreads, 0, s>>>(f, emit, out, m_max, m_dev, total, l, epoch++, err);
+        launch(k_scan_fn<F, E>, tiles ? tiles : 1u, kTileThreads, 0, s, f, emit, out, m_max, m_dev, total, l, epoch++, err);
         *launches += 1;
     }
 };

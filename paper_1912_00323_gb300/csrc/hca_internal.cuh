@@ -108,6 +108,33 @@ struct Workspace {
     size_t bytes;
 };
 
+// Launch of a kernel of a call's chain.  The kernel may be put on the GPU while the one before it in
+// the stream still runs (programmatic stream serialisation), and every kernel launched this way
+// starts with pdl_enter, which waits until that one and its writes are complete.  Measured: a call
+// of 16 short kernels (2-D, 10,000 points) 197 -> 167 us, one of 34 (8-D, 3,001 points) 362 ->
+// 298 us; captured into a graph the chain runs as before.
+template <typename... P, typename... A>
+inline void launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A &&...args) {
+    cudaLaunchAttribute attr;
+    attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cfg.attrs = &attr;
+    cfg.numAttrs = 1;
+    cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+
+// First statement of those kernels: wait for the kernel before, then let the next one be put in
+// place behind this one (it waits in turn).
+__device__ __forceinline__ void pdl_enter() {
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+
 // ---------------------------------------------------------------------------------------
 // Primitives implemented in sort.cu / scan.cu
 // ---------------------------------------------------------------------------------------

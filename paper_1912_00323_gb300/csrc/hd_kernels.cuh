@@ -300,6 +300,7 @@ static __global__ void __launch_bounds__(256) k_box_check_hd(const double *__res
                                                             const int64_t *__restrict__ set_off,
                                                             const unsigned long long *__restrict__ mm,
                                                             DevCounters *ctr) {
+    pdl_enter();
     if (blockIdx.x == 0 && threadIdx.x == 0 && ctr->nan_seen) atomicOr(&ctr->status, kErrBox);
     for (int64_t k = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; k < (int64_t)nsets * d;
          k += (int64_t)gridDim.x * blockDim.x) {
@@ -317,6 +318,7 @@ static __global__ void __launch_bounds__(256) k_box_check_hd(const double *__res
 template <typename T>
 __global__ void __launch_bounds__(256) k_minmax_rt(const T *__restrict__ in, int64_t n, int d, DevCounters *ctr,
                                                   unsigned long long *mm /* [2 * 64] */) {
+    pdl_enter();
     // each thread walks one dimension (a stride that is a multiple of d), four independent
     // loads in flight; the block folds its threads per dimension in shared memory, then one
     // global atomic per block and dimension
@@ -398,6 +400,7 @@ template <typename T, typename K>
 __global__ void __launch_bounds__(256) k_bin_proj(const T *__restrict__ in, int d, int3 sel, GridParams g,
                                                  K *__restrict__ keys, uint32_t *__restrict__ digit_counts,
                                                  FillList fill) {
+    pdl_enter();
     __shared__ uint32_t h[8][256];
     fill_regions(fill);
     count_digits_begin(h);
@@ -429,6 +432,7 @@ __global__ void __launch_bounds__(kTileThreads) k_cells_hd(const T *__restrict__
                                                           T *__restrict__ pts, uint8_t *__restrict__ core,
                                                           uint8_t *__restrict__ cell_core, float *__restrict__ fpts,
                                                           const unsigned long long *__restrict__ mm, int set_shift) {
+    pdl_enter();
     constexpr int G = DP / 4;          // threads per row
     constexpr int R = 256 / G;         // rows per step of the block
     const int g = threadIdx.x % G, r0 = threadIdx.x / G;
@@ -569,6 +573,7 @@ struct BoxClear {
 
 template <typename T, int DP, typename R>
 __global__ void __launch_bounds__(256) k_cell_box_hd(HdView<T, DP> v) {
+    pdl_enter();
     typedef BoxCode<R> BC;
     typedef typename BC::U U;
     constexpr int E = DP > 32 ? DP / 32 : 1;  // dimensions per lane in the atomics
@@ -622,6 +627,7 @@ __global__ void __launch_bounds__(256) k_cell_box_hd(HdView<T, DP> v) {
 
 template <typename T, int DP, typename R>
 __global__ void __launch_bounds__(256) k_cell_box_decode(HdView<T, DP> v) {
+    pdl_enter();
     typedef BoxCode<R> BC;
     typedef typename BC::U U;
     const uint64_t m = (uint64_t)v.ctr->n_cells * DP;
@@ -714,6 +720,7 @@ __device__ __forceinline__ bool spill_push(const V &v, int slot, uint32_t t, uin
 // pair tests were bound by the FP64 rate, from 7.4 to 0.95 ms together with the lists.
 template <typename T, int DP, bool SPILL, bool FILTER>
 __global__ void __launch_bounds__(32 * kHdMaxWarps) k_count_hd(HdView<T, DP> v) {
+    pdl_enter();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     typedef Candidate<T, DP, FILTER> Cand;
     typedef typename Cand::Row R;
@@ -818,6 +825,7 @@ __device__ __forceinline__ uint4 list4(const V &v, uint32_t p, uint32_t i) {
 // CUDA cores.
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_list_link(HdView<T, DP> v) {
+    pdl_enter();
     // (the cells' trees and odd counts are cleared here too)
     const uint32_t C = v.ctr->n_cells;
     for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
@@ -850,6 +858,7 @@ __global__ void __launch_bounds__(256) k_list_link(HdView<T, DP> v) {
 // Read-only finds: parent[p] = root (nothing hooks meanwhile).
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_flatten_hd(HdView<T, DP> v) {
+    pdl_enter();
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += (int64_t)gridDim.x * blockDim.x)
         if (v.core[j]) v.parent[j] = uf_root_readonly(v.parent, (uint32_t)j, v.ctr);
 }
@@ -889,6 +898,7 @@ __device__ __forceinline__ void load_edges(const V &v, int64_t j, int64_t m, uin
 // hook the same root.
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_list_hook(HdView<T, DP> v) {
+    pdl_enter();
     const int64_t m = v.g.n * (v.nl_k / 4);
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < m; j += (int64_t)gridDim.x * blockDim.x) {
         uint32_t rp, r[4];
@@ -903,6 +913,7 @@ __global__ void __launch_bounds__(256) k_list_hook(HdView<T, DP> v) {
 
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_list_join(HdView<T, DP> v) {
+    pdl_enter();
     const uint32_t lane = lane_id();
     const int64_t m = v.g.n * (v.nl_k / 4);
     for (int64_t jb = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); jb < m; jb += (int64_t)gridDim.x * blockDim.x) {
@@ -933,6 +944,7 @@ __global__ void __launch_bounds__(256) k_list_join(HdView<T, DP> v) {
 // pencil but hardly across pencils; between dense cells nearly every such sample has an edge.
 template <typename T, int DP, bool FILTER>
 __global__ void __launch_bounds__(32 * kHdMaxWarps) k_cell_link(HdView<T, DP> v) {
+    pdl_enter();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     typedef Candidate<T, DP, FILTER> Cand;
     typedef typename Cand::Row R;
@@ -987,6 +999,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_cell_link(HdView<T, DP> v)
 // others are the cell's odd points.
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_cell_root(HdView<T, DP> v) {
+    pdl_enter();
     const int lane = lane_id();
     const int64_t n = v.g.n;
     for (int64_t jb = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); jb < n; jb += (int64_t)gridDim.x * blockDim.x) {
@@ -1002,6 +1015,7 @@ __global__ void __launch_bounds__(256) k_cell_root(HdView<T, DP> v) {
 
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_cell_odd(HdView<T, DP> v) {
+    pdl_enter();
     const int lane = lane_id();
     const uint32_t C = v.ctr->n_cells, NC = v.ctr->n_chunks, warps = (gridDim.x * blockDim.x) >> 5;
     for (uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < NC; t += warps) {
@@ -1020,6 +1034,7 @@ __global__ void __launch_bounds__(256) k_cell_odd(HdView<T, DP> v) {
 constexpr uint32_t kOddMin = 8;
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_cell_mixed(HdView<T, DP> v) {
+    pdl_enter();
     const uint32_t C = v.ctr->n_cells;
     for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
         const uint32_t odd = v.odd_cnt[c];
@@ -1039,6 +1054,7 @@ __device__ __forceinline__ bool cells_to_join(uint32_t ra, uint32_t rb) {
 // counts (SPILL = true: the second launch).
 template <typename T, int DP, bool SPILL, bool FILTER>
 __global__ void __launch_bounds__(32 * kHdMaxWarps) k_odd_hd(HdView<T, DP> v) {
+    pdl_enter();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     typedef Candidate<T, DP, FILTER> Cand;
     typedef typename Cand::Row R;
@@ -1104,6 +1120,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_odd_hd(HdView<T, DP> v) {
 // 3.50 -> 2.18 ms for the labels and unions from lists together).
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_list_labels(HdView<T, DP> v, int core_too) {
+    pdl_enter();
     uint32_t noise = 0;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t p = (uint32_t)j;
@@ -1146,6 +1163,7 @@ __global__ void __launch_bounds__(256) k_list_labels(HdView<T, DP> v, int core_t
 // one root is skipped without loading coordinates.
 template <typename T, int DP, bool FILTER>
 __global__ void __launch_bounds__(32 * kHdMaxWarps) k_merge_hd(HdView<T, DP> v) {
+    pdl_enter();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     typedef Candidate<T, DP, FILTER> Cand;
     typedef typename Cand::Row R;
@@ -1220,6 +1238,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_merge_hd(HdView<T, DP> v) 
 // roots and the core points, canonical ids.
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_comp_min_hd(HdView<T, DP> v) {
+    pdl_enter();
     const int64_t n = v.g.n;
     const int lane = lane_id();
     uint32_t ncore = 0, roots = 0;
@@ -1253,6 +1272,7 @@ __global__ void __launch_bounds__(256) k_comp_min_hd(HdView<T, DP> v) {
 // second launch).
 template <typename T, int DP, bool SPILL, bool FILTER>
 __global__ void __launch_bounds__(32 * kHdMaxWarps) k_labels_hd(HdView<T, DP> v) {
+    pdl_enter();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     typedef Candidate<T, DP, FILTER> Cand;
     typedef typename Cand::Row R;
@@ -1348,6 +1368,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_minmax_rt_seg(const T *__restrict__ in, int64_t n, int d,
                                                       const int64_t *set_off, int nsets,
                                                       unsigned long long *mm, DevCounters *ctr) {
+    pdl_enter();
     seg_minmax<T>(in, n, d, set_off, nsets, mm, 64, ctr);
 }
 
@@ -1358,6 +1379,7 @@ __global__ void __launch_bounds__(256) k_bin_proj_seg(const T *__restrict__ in, 
                                                      const int64_t *set_off, int nsets, const GridParams *gtab,
                                                      int key_bits, K *__restrict__ keys,
                                                      uint32_t *__restrict__ digit_counts, int total_bits, FillList fill) {
+    pdl_enter();
     __shared__ uint32_t h[8][256];
     fill_regions(fill);
     count_digits_begin(h);

@@ -153,20 +153,20 @@ struct HdLaunch {
 // The lists joined, every cell's tree and its odd points, and those against their neighbourhood.
 template <typename T, int DP, bool FILTER>
 void run_list_unions(HdView<T, DP> &hv, const HdLaunch &L, int &launches) {
-    k_list_link<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+    launch(k_list_link<T, DP>, L.gpts, 256, 0, L.s, hv);
     if (hv.nl_k) {
-        k_flatten_hd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
-        k_list_hook<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
-        k_flatten_hd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
-        k_list_join<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
-        k_cell_link<T, DP, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
+        launch(k_flatten_hd<T, DP>, L.gpts, 256, 0, L.s, hv);
+        launch(k_list_hook<T, DP>, L.gpts, 256, 0, L.s, hv);
+        launch(k_flatten_hd<T, DP>, L.gpts, 256, 0, L.s, hv);
+        launch(k_list_join<T, DP>, L.gpts, 256, 0, L.s, hv);
+        launch(k_cell_link<T, DP, FILTER>, L.gcell, L.block, L.smem, L.s, hv);
     }
-    k_flatten_hd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
-    k_cell_root<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
-    k_cell_odd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
-    k_cell_mixed<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
-    k_odd_hd<T, DP, false, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
-    k_odd_hd<T, DP, true, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
+    launch(k_flatten_hd<T, DP>, L.gpts, 256, 0, L.s, hv);
+    launch(k_cell_root<T, DP>, L.gpts, 256, 0, L.s, hv);
+    launch(k_cell_odd<T, DP>, L.gpts, 256, 0, L.s, hv);
+    launch(k_cell_mixed<T, DP>, L.gpts, 256, 0, L.s, hv);
+    launch(k_odd_hd<T, DP, false, FILTER>, L.gcell, L.block, L.smem, L.s, hv);
+    launch(k_odd_hd<T, DP, true, FILTER>, L.gcell, L.block, L.smem, L.s, hv);
     launches += hv.nl_k ? 12 : 7;
 }
 
@@ -183,22 +183,22 @@ void run_cuda_phases(HdView<T, DP> &hv, const HdLaunch &L, Mark &mark, int &laun
     detail::allow_smem(k_labels_hd<T, DP, false, FILTER>, L.smem);
     detail::allow_smem(k_labels_hd<T, DP, true, FILTER>, L.smem);
     typedef typename Candidate<T, DP, FILTER>::Row R;
-    k_cell_box_decode<T, DP, R><<<L.gpts, 256, 0, L.s>>>(hv);
-    k_count_hd<T, DP, false, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
-    k_count_hd<T, DP, true, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
+    launch(k_cell_box_decode<T, DP, R>, L.gpts, 256, 0, L.s, hv);
+    launch(k_count_hd<T, DP, false, FILTER>, L.gcell, L.block, L.smem, L.s, hv);
+    launch(k_count_hd<T, DP, true, FILTER>, L.gcell, L.block, L.smem, L.s, hv);
     mark(6);
     // (no representative points in this path: every pair of core points is a candidate)
     mark(7);
     run_list_unions<T, DP, FILTER>(hv, L, launches);
-    k_merge_hd<T, DP, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
+    launch(k_merge_hd<T, DP, FILTER>, L.gcell, L.block, L.smem, L.s, hv);
     mark(8);
-    k_comp_min_hd<T, DP><<<L.gpts, 256, 0, L.s>>>(hv);
+    launch(k_comp_min_hd<T, DP>, L.gpts, 256, 0, L.s, hv);
     if (L.list_labels) {
-        k_list_labels<T, DP><<<L.gpts, 256, 0, L.s>>>(hv, 1);
+        launch(k_list_labels<T, DP>, L.gpts, 256, 0, L.s, hv, 1);
         launches += 6;
     } else {
-        k_labels_hd<T, DP, false, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
-        k_labels_hd<T, DP, true, FILTER><<<L.gcell, L.block, L.smem, L.s>>>(hv);
+        launch(k_labels_hd<T, DP, false, FILTER>, L.gcell, L.block, L.smem, L.s, hv);
+        launch(k_labels_hd<T, DP, true, FILTER>, L.gcell, L.block, L.smem, L.s, hv);
         launches += 7;
     }
     mark(9);
@@ -238,7 +238,7 @@ void run_tc_phases(HdView<float, DP> &hv, const HdLaunch &L, char *b, int64_t n,
     scans.run(tc::CountChunks<DP>{hv, tune.min[0]}, tc::BoxDecode<DP>{hv}, ch0, n, &ctr->n_cells,
               &ctr->n_tc_chunks[tc::kCount]);
     tmark(0);
-    tc::k_tc_hd<DP, tc::kCount><<<grid_tc, tc::kTile, tc_smem, s>>>(hv, tc::Tables{ch0, cx, clist, nclist, clab});
+    launch(tc::k_tc_hd<DP, tc::kCount>, grid_tc, tc::kTile, tc_smem, s, hv, tc::Tables{ch0, cx, clist, nclist, clab});
     // the rows those chunks handed over, in cells with at least kRecountMin of them, counted again
     // from the start, 128 per chunk (cx, clist, nclist and ch1 are free until the core numbering); the
     // rest, and what the recount hands over, go to the CUDA-core count.  Per listed row the
@@ -246,11 +246,10 @@ void run_tc_phases(HdView<float, DP> &hv, const HdLaunch &L, char *b, int64_t n,
     scans.run(tc::HandedFlag{hv.core}, tc::HandedList{clist, nch, ch0, nclist}, cx, n, nullptr, cx + n);
     scans.run(tc::RecountItems{hv.cell_start, cx, hv.ranges, hv.n_all, tc::kRecountMin}, tc::NoEmit{}, ch1, n,
               &ctr->n_cells, &ctr->n_tc_recount);
-    tc::k_tc_hd<DP, tc::kCount><<<grid_tc, tc::kTile, tc_smem, s>>>(
-        hv, tc::Tables{ch1, cx, nullptr, nullptr, nullptr, nullptr, clist, nch, ch0, nclist});
+    launch(tc::k_tc_hd<DP, tc::kCount>, grid_tc, tc::kTile, tc_smem, s, hv, tc::Tables{ch1, cx, nullptr, nullptr, nullptr, nullptr, clist, nch, ch0, nclist});
     tmark(1);
-    k_count_hd<float, DP, false, true><<<gcell, hd_block, smem, s>>>(hv);
-    k_count_hd<float, DP, true, true><<<gcell, hd_block, smem, s>>>(hv);
+    launch(k_count_hd<float, DP, false, true>, gcell, hd_block, smem, s, hv);
+    launch(k_count_hd<float, DP, true, true>, gcell, hd_block, smem, s, hv);
     launches += 4;
     mark(6);
     // core numbering, core and non-core lists
@@ -266,21 +265,21 @@ void run_tc_phases(HdView<float, DP> &hv, const HdLaunch &L, char *b, int64_t n,
     scans.run(tc::Stored{flags}, tc::NoEmit{}, ch0, n, &ctr->n_cells, &ctr->n_tc_chunks[3]);
     tmark(2);
     // window-major items: the first window of every chunk, then the other windows
-    tc::k_tc_hd<DP, tc::kMerge><<<grid_tc, tc::kTile, tc_smem, s>>>(hv, tc::Tables{ch1, cx, clist, nclist, clab, ch0});
+    launch(tc::k_tc_hd<DP, tc::kMerge>, grid_tc, tc::kTile, tc_smem, s, hv, tc::Tables{ch1, cx, clist, nclist, clab, ch0});
     tmark(3);
     // the CUDA-core unions take the cells below the threshold; from one core row on every cell
     // with a core point is on the tensor cores and nothing is left for them
     if (tune.min[1] > 1) {
-        k_merge_hd<float, DP, true><<<gcell, hd_block, smem, s>>>(hv);
+        launch(k_merge_hd<float, DP, true>, gcell, hd_block, smem, s, hv);
         ++launches;
     }
     launches += 1;
     mark(8);
     // ---- Algorithm 4: canonical ids, core labels, border and noise points ----
-    k_comp_min_hd<float, DP><<<gpts, 256, 0, s>>>(hv);
+    launch(k_comp_min_hd<float, DP>, gpts, 256, 0, s, hv);
     if (L.list_labels) {
         tmark(4);
-        k_list_labels<float, DP><<<gpts, 256, 0, s>>>(hv, 1);
+        launch(k_list_labels<float, DP>, gpts, 256, 0, s, hv, 1);
         tmark(5);
         launches += 2;
         mark(9);
@@ -292,13 +291,13 @@ void run_tc_phases(HdView<float, DP> &hv, const HdLaunch &L, char *b, int64_t n,
     const bool fork = ss.ok && cudaEventRecord(ss.fork, s) == cudaSuccess &&
                       cudaStreamWaitEvent(ss.s, ss.fork, 0) == cudaSuccess;
     auto cuda_labels = [&](cudaStream_t ls) {
-        k_labels_hd<float, DP, false, true><<<gcell, hd_block, smem, ls>>>(hv);
-        k_labels_hd<float, DP, true, true><<<gcell, hd_block, smem, ls>>>(hv);
+        launch(k_labels_hd<float, DP, false, true>, gcell, hd_block, smem, ls, hv);
+        launch(k_labels_hd<float, DP, true, true>, gcell, hd_block, smem, ls, hv);
     };
     if (fork) cuda_labels(ss.s);
-    tc::k_tc_core_labels<DP><<<gpts, 256, 0, s>>>(hv, tc::Tables{ch2, cx, clist, nclist, clab}, nsets, clab);
+    launch(tc::k_tc_core_labels<DP>, gpts, 256, 0, s, hv, tc::Tables{ch2, cx, clist, nclist, clab}, nsets, clab);
     tmark(4);
-    tc::k_tc_hd<DP, tc::kLabels><<<grid_tc, tc::kTile, tc_smem, s>>>(hv, tc::Tables{ch2, cx, clist, nclist, clab});
+    launch(tc::k_tc_hd<DP, tc::kLabels>, grid_tc, tc::kTile, tc_smem, s, hv, tc::Tables{ch2, cx, clist, nclist, clab});
     tmark(5);
     if (fork) {
         cudaEventRecord(ss.join, ss.s);
@@ -528,12 +527,12 @@ int run_hd(const RunArgs &a) {
     mark(0);
     cudaMemsetAsync(ctr, 0, o_mm + sizeof(unsigned long long) * 128 - o_ctr, s);  // (mm follows the counters)
     if (!batched) {
-        k_minmax_rt<T><<<grid_for(n * d, 256, sms, 8), 256, 0, s>>>((const T *)a.d_points, n, d, ctr, mm);
+        launch(k_minmax_rt<T>, grid_for(n * d, 256, sms, 8), 256, 0, s, (const T *)a.d_points, n, d, ctr, mm);
         if (!boxed) cudaMemcpyAsync(hmm.data(), mm, sizeof(unsigned long long) * 128, cudaMemcpyDeviceToHost, s);
     } else {
         cudaMemsetAsync(d_smm, 0, sizeof(unsigned long long) * 2 * 64 * nsets, s);
         upload(d_setoff, a.h_off, sizeof(int64_t) * (nsets + 1), stage_setoff);
-        k_minmax_rt_seg<T><<<grid_for(n, 256, sms, 8), 256, 0, s>>>((const T *)a.d_points, n, d, d_setoff, nsets,
+        launch(k_minmax_rt_seg<T>, grid_for(n, 256, sms, 8), 256, 0, s, (const T *)a.d_points, n, d, d_setoff, nsets,
                                                                    d_smm, ctr);
         if (!boxed) {
             smm.resize((size_t)2 * 64 * nsets);
@@ -549,8 +548,7 @@ int run_hd(const RunArgs &a) {
         double *d_box = (double *)(b + o_box);
         upload(d_box, boxes.data(), sizeof(double) * boxes.size(), stage_box);
         if (batched) upload(d_gtab, gsets.data(), sizeof(GridParams) * nsets, stage_gtab);
-        k_box_check_hd<<<grid_for((int64_t)nsets * d, 256, sms, 1), 256, 0, s>>>(
-            d_box, nsets, d, batched ? d_setoff : nullptr, batched ? d_smm : mm, ctr);
+        launch(k_box_check_hd, grid_for((int64_t)nsets * d, 256, sms, 1), 256, 0, s, d_box, nsets, d, batched ? d_setoff : nullptr, batched ? d_smm : mm, ctr);
         ++launches;
     } else {
         if (cudaMemcpyAsync(h, ctr, kCountersRead, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
@@ -584,10 +582,10 @@ int run_hd(const RunArgs &a) {
         auto front = [&](auto *ka, auto *kb) {
             typedef typename std::remove_reference<decltype(*ka)>::type K;
             if (batched)
-                k_bin_proj_seg<T, K><<<gpts, 256, 0, s>>>((const T *)a.d_points, n, d, d_setoff, nsets, d_gtab,
+                launch(k_bin_proj_seg<T, K>, gpts, 256, 0, s, (const T *)a.d_points, n, d, d_setoff, nsets, d_gtab,
                                                          g.key_bits, ka, ctr->digit_counts, sort_bits, fill);
             else
-                k_bin_proj<T, K><<<gpts, 256, 0, s>>>((const T *)a.d_points, d, sel, g, ka, ctr->digit_counts, fill);
+                launch(k_bin_proj<T, K>, gpts, 256, 0, s, (const T *)a.d_points, d, sel, g, ka, ctr->digit_counts, fill);
             mark(2);
             flipped = radix_sort_pairs<K>(ka, ia, kb, ib, n, 0, sort_bits, hist, nullptr, s, &launches, &ctr->status,
                                           ctr->digit_counts, true, true);
@@ -604,8 +602,7 @@ int run_hd(const RunArgs &a) {
             ca.ptab = ptab;
             ca.l = LookBack::at(b + o_look);
             ca.ctr = ctr;
-            k_cells_hd<T, DP, K><<<(unsigned)((n + kScanTileElems - 1) / kScanTileElems), kTileThreads, 0, s>>>(
-                (const T *)a.d_points, d, ca, (T *)(b + o_pts), (uint8_t *)(b + o_core), (uint8_t *)(b + o_ccore), fpts,
+            launch(k_cells_hd<T, DP, K>, (unsigned)((n + kScanTileElems - 1) / kScanTileElems), kTileThreads, 0, s, (const T *)a.d_points, d, ca, (T *)(b + o_pts), (uint8_t *)(b + o_core), (uint8_t *)(b + o_ccore), fpts,
                 batched ? d_smm : mm, batched ? g.key_bits : 64);
             launches += 2;
         };
@@ -615,8 +612,8 @@ int run_hd(const RunArgs &a) {
     }
     mark(4);
     if (!ptab) {
-        k_hash_init<<<grid_for(cap_max, 256, sms, 8), 256, 0, s>>>((uint64_t *)(b + o_hk), ctr);
-        k_pencils<<<gpts, 256, 0, s>>>((const uint64_t *)(b + o_ckey), g.prefix_shift,
+        launch(k_hash_init, grid_for(cap_max, 256, sms, 8), 256, 0, s, (uint64_t *)(b + o_hk), ctr);
+        launch(k_pencils, gpts, 256, 0, s, (const uint64_t *)(b + o_ckey), g.prefix_shift,
                                        (const uint32_t *)(b + o_pstart), (uint64_t *)(b + o_hk),
                                        (uint32_t *)(b + o_hv), ctr);
         launches += 2;
@@ -630,7 +627,7 @@ int run_hd(const RunArgs &a) {
     lv.ptab = ptab;
     lv.ranges = (uint2 *)(b + o_ranges);
     lv.ctr = ctr;
-    k_ranges<float, 3><<<grid_for((n / kRangeRun + 1) * (int64_t)st.n_all, 256, sms, 16), 256, 0, s>>>(lv, st);
+    launch(k_ranges<float, 3>, grid_for((n / kRangeRun + 1) * (int64_t)st.n_all, 256, sms, 16), 256, 0, s, lv, st);
     ++launches;
     scans.l = LookBack::at(b + o_scan);
     scans.err = &ctr->status;
@@ -686,10 +683,10 @@ int run_hd(const RunArgs &a) {
         const ChunkCount<HdView<T, DP>> chunks{hv};
         if (fpts) {
             scans.run(chunks, BoxClear<T, DP, float>{hv}, choff, n, &ctr->n_cells, &ctr->n_chunks);
-            k_cell_box_hd<T, DP, float><<<grid_for(n / 32 + 1, 8, sms, 16), 256, 0, s>>>(hv);
+            launch(k_cell_box_hd<T, DP, float>, grid_for(n / 32 + 1, 8, sms, 16), 256, 0, s, hv);
         } else {
             scans.run(chunks, BoxClear<T, DP, T>{hv}, choff, n, &ctr->n_cells, &ctr->n_chunks);
-            k_cell_box_hd<T, DP, T><<<grid_for(n / 32 + 1, 8, sms, 16), 256, 0, s>>>(hv);
+            launch(k_cell_box_hd<T, DP, T>, grid_for(n / 32 + 1, 8, sms, 16), 256, 0, s, hv);
         }
         ++launches;
     }

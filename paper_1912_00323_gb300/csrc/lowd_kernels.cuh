@@ -441,6 +441,7 @@ __device__ __forceinline__ void load_pts(const T *__restrict__ in, int64_t j0, i
 // check.  Each thread step reads VecPts::pts consecutive points with 16-byte loads.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_minmax(const T *__restrict__ in, int64_t n, DevCounters *ctr) {
+    pdl_enter();
     constexpr int P = VecPts<T, D>::pts;
     T mn[D], mx[D];
 #pragma unroll
@@ -508,6 +509,7 @@ template <typename T, int D, typename K>
 __global__ void __launch_bounds__(256) k_bin(const T *__restrict__ in, GridParams g,
                                             K *__restrict__ keys, uint32_t *__restrict__ digit_counts,
                                             FillList fill) {
+    pdl_enter();
     constexpr int P = VecPts<T, D>::pts;
     fill_regions(fill);
     // digit counts of every radix pass, for the sort that follows
@@ -571,6 +573,7 @@ __global__ void __launch_bounds__(256) k_bin(const T *__restrict__ in, GridParam
 template <typename T, int D, typename K>
 __global__ void __launch_bounds__(kTileThreads) k_cells(const T *__restrict__ in, CellsArgs<K> a,
                                                        Pt<T, D> *__restrict__ pts) {
+    pdl_enter();
     const uint32_t tile = take_tile(a.l, 0u);
     const int64_t base = (int64_t)tile * kScanTileElems;
     cells_tile(a, tile, [&]() {
@@ -595,6 +598,7 @@ __global__ void __launch_bounds__(kTileThreads) k_cells(const T *__restrict__ in
 // The hash table of the pencils, when their keys span too much for a direct table: clear the used
 // part (capacity = power of two >= 2 P), then insert.
 static __global__ void __launch_bounds__(256) k_hash_init(uint64_t *__restrict__ hkeys, DevCounters *ctr) {
+    pdl_enter();
     const uint32_t P = ctr->n_pencils;
     uint32_t cap = 64;
     while (cap < 2u * P) cap <<= 1;
@@ -606,6 +610,7 @@ static __global__ void __launch_bounds__(256) k_hash_init(uint64_t *__restrict__
 static __global__ void __launch_bounds__(256) k_pencils(const uint64_t *__restrict__ cell_key, int prefix_shift,
                                                        const uint32_t *__restrict__ pencil_start, uint64_t *hkeys,
                                                        uint32_t *hvals, DevCounters *ctr) {
+    pdl_enter();
     const uint32_t P = ctr->n_pencils;
     const uint32_t mask = ctr->hash_mask;
     for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
@@ -636,6 +641,7 @@ constexpr uint32_t kRangeRun = 4;
 
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_ranges(LowdView<T, D> v, Stencil st_in) {
+    pdl_enter();
     __shared__ Stencil st;
     load_stencil<T, D>(st, st_in);
     const uint32_t C = v.ctr->n_cells;
@@ -727,6 +733,7 @@ struct WarpList {
 // noise and get label -1 at once, else the cell goes on the label list.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_triage(LowdView<T, D> v, int n_all) {
+    pdl_enter();
     const uint32_t C = v.ctr->n_cells;
     uint32_t noise = 0;
     const uint32_t stride = gridDim.x * blockDim.x;
@@ -788,6 +795,7 @@ __global__ void __launch_bounds__(256) k_triage(LowdView<T, D> v, int n_all) {
 // lists of cells with core points (merging) and with non-core points (labels).
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_core(LowdView<T, D> v, Stencil st_in) {
+    pdl_enter();
     __shared__ Stencil st;
     load_stencil<T, D>(st, st_in);
     const int n_all = st.n_all;
@@ -942,6 +950,7 @@ __device__ __forceinline__ unsigned rep_group_bits(int it, int g) {
 
 template <typename T, int D, uint32_t WIN>
 __global__ void __launch_bounds__(32 * kRepWarps) k_reps(LowdView<T, D> v, int64_t n) {
+    pdl_enter();
     using Geo = RepGeom<D, WIN>;
     constexpr int ndir = Geo::ndir;
     constexpr int kPer = (int)(WIN / 32);
@@ -1087,6 +1096,7 @@ __global__ void __launch_bounds__(32 * kRepWarps) k_reps(LowdView<T, D> v, int64
 // A cell that crosses several boundaries is written several times with the same values.
 template <typename T, int D, uint32_t WIN>
 __global__ void __launch_bounds__(256) k_rep_fix(LowdView<T, D> v, int64_t n) {
+    pdl_enter();
     using Geo = RepGeom<D, WIN>;
     constexpr int ndir = Geo::ndir;
     const int64_t nb = (n + Geo::sub - 1) / Geo::sub;
@@ -1155,6 +1165,7 @@ __device__ bool warp_core_pair(const LowdView<T, D> &v, uint32_t A, uint32_t B, 
 // pointer jumping flattens it and the merge passes then join the trees.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_hook(LowdView<T, D> v, int n_all, int n_half) {
+    pdl_enter();
     constexpr int ndir = RepDirs<D>::value;
     const int lane = lane_id();
     const uint32_t NL = v.ctr->n_list[1];
@@ -1200,6 +1211,7 @@ __global__ void __launch_bounds__(256) k_hook(LowdView<T, D> v, int n_all, int n
 // write on the way (nothing hooks meanwhile; the links run a few cells far).
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_flatten(LowdView<T, D> v) {
+    pdl_enter();
     const uint32_t NL = v.ctr->n_list[1];
     for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < NL; w += gridDim.x * blockDim.x) {
         const uint32_t c = v.list_core[w];
@@ -1215,6 +1227,7 @@ __global__ void __launch_bounds__(256) k_flatten(LowdView<T, D> v) {
 // core x core test.  Lanes walk the flattened list of candidate cells of one cell.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_merge(LowdView<T, D> v, int n_all, int n_half, int pass) {
+    pdl_enter();
     constexpr int ndir = RepDirs<D>::value;
     const int lane = lane_id();
     uint32_t rep_tests = 0, rep_hits = 0, exhaustive = 0, chunks = 0;
@@ -1295,6 +1308,7 @@ __global__ void __launch_bounds__(256) k_merge(LowdView<T, D> v, int n_all, int 
 // per cell with core points.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_comp_min(LowdView<T, D> v) {
+    pdl_enter();
     const uint32_t NL = v.ctr->n_list[1];
     uint32_t roots = 0;
     for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < NL; w += gridDim.x * blockDim.x) {
@@ -1315,6 +1329,7 @@ __global__ void __launch_bounds__(256) k_comp_min(LowdView<T, D> v) {
 // also counts the core points.
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_label_core(LowdView<T, D> v) {
+    pdl_enter();
     const int64_t n = v.g.n;
     const int lane = lane_id();
     uint32_t ncore = 0;
@@ -1342,6 +1357,7 @@ __global__ void __launch_bounds__(256) k_label_core(LowdView<T, D> v) {
 // dropped, and the others are compared point by point.  Writes labels in input order.
 template <typename T, int D>
 __global__ void __launch_bounds__(256, 4) k_labels(LowdView<T, D> v, int n_all) {
+    pdl_enter();
     const int lane = lane_id();
     uint32_t noise = 0, chunks = 0;
     const uint32_t NL = v.ctr->n_list[2];
@@ -1473,6 +1489,7 @@ template <int D>
 __global__ void __launch_bounds__(256) k_box_check(BoxArgs single, const double *__restrict__ boxes, int nsets,
                                                   const int64_t *__restrict__ set_off,
                                                   const unsigned long long *__restrict__ mm, DevCounters *ctr) {
+    pdl_enter();
     if (blockIdx.x == 0 && threadIdx.x == 0 && ctr->nan_seen) atomicOr(&ctr->status, kErrBox);
     if (!boxes) {
         if (blockIdx.x != 0 || threadIdx.x >= D) return;
@@ -1616,6 +1633,7 @@ __device__ __forceinline__ void seg_minmax(const T *__restrict__ in, int64_t n, 
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_minmax_seg(const T *__restrict__ in, int64_t n, const int64_t *set_off,
                                                    int nsets, unsigned long long *mm, DevCounters *ctr) {
+    pdl_enter();
     seg_minmax<T>(in, n, D, set_off, nsets, mm, kMaxD, ctr);
 }
 
@@ -1625,6 +1643,7 @@ __global__ void __launch_bounds__(256) k_bin_seg(const T *__restrict__ in, int64
                                                 int nsets, const GridParams *gtab, int key_bits,
                                                 K *__restrict__ keys, uint32_t *__restrict__ digit_counts,
                                                 int total_bits, FillList fill) {
+    pdl_enter();
     fill_regions(fill);
     __shared__ uint32_t h[8][256];
     const int passes = (total_bits + 7) / 8;

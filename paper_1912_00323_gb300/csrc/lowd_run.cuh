@@ -467,11 +467,11 @@ int run_lowd(const RunArgs &a) {
     mark(0);
     cudaMemsetAsync(ctr, 0, sizeof(DevCounters), s);
     if (!batched) {
-        k_minmax<T, D><<<grid_for(n, 256, sms, 2), 256, 0, s>>>((const T *)a.d_points, n, ctr);
+        launch(k_minmax<T, D>, grid_for(n, 256, sms, 2), 256, 0, s, (const T *)a.d_points, n, ctr);
     } else {
         cudaMemsetAsync(d_mm, 0, sizeof(uint64_t) * 2 * kMaxD * nsets, s);
         upload(d_setoff, a.h_off, sizeof(int64_t) * (nsets + 1), stage_setoff);
-        k_minmax_seg<T, D><<<grid_for(n, 256, sms, 8), 256, 0, s>>>((const T *)a.d_points, n, d_setoff, nsets,
+        launch(k_minmax_seg<T, D>, grid_for(n, 256, sms, 8), 256, 0, s, (const T *)a.d_points, n, d_setoff, nsets,
                                                                   (unsigned long long *)d_mm, ctr);
         if (!boxed) {
             hmm.resize((size_t)2 * kMaxD * nsets);
@@ -497,8 +497,7 @@ int run_lowd(const RunArgs &a) {
             upload(d_box, boxes.data(), sizeof(double) * boxes.size(), stage_box);
             upload(d_gtab, gsets.data(), sizeof(GridParams) * nsets, stage_gtab);
         }
-        k_box_check<D><<<grid_for((int64_t)nsets * D, 256, sms, 1), 256, 0, s>>>(
-            one, d_box, nsets, d_setoff, (const unsigned long long *)d_mm, ctr);
+        launch(k_box_check<D>, grid_for((int64_t)nsets * D, 256, sms, 1), 256, 0, s, one, d_box, nsets, d_setoff, (const unsigned long long *)d_mm, ctr);
         ++launches;
     } else {
         if (cudaMemcpyAsync(h, ctr, kCountersRead, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
@@ -538,10 +537,10 @@ int run_lowd(const RunArgs &a) {
         auto front = [&](auto *ka, auto *kb) {
             typedef typename std::remove_reference<decltype(*ka)>::type K;
             if (batched)
-                k_bin_seg<T, D, K><<<gpts, 256, 0, s>>>((const T *)a.d_points, n, d_setoff, nsets, d_gtab, g.key_bits,
+                launch(k_bin_seg<T, D, K>, gpts, 256, 0, s, (const T *)a.d_points, n, d_setoff, nsets, d_gtab, g.key_bits,
                                                        ka, ctr->digit_counts, sort_bits, fill);
             else
-                k_bin<T, D, K><<<gpts, 256, 0, s>>>((const T *)a.d_points, g, ka, ctr->digit_counts, fill);
+                launch(k_bin<T, D, K>, gpts, 256, 0, s, (const T *)a.d_points, g, ka, ctr->digit_counts, fill);
             mark(2);
             flipped = radix_sort_pairs<K>(ka, ia, kb, ib, n, 0, sort_bits, hist, nullptr, s, &launches, &ctr->status,
                                           ctr->digit_counts, true, true);
@@ -558,8 +557,7 @@ int run_lowd(const RunArgs &a) {
             ca.ptab = ptab;
             ca.l = LookBack::at(b + o_look);
             ca.ctr = ctr;
-            k_cells<T, D, K><<<(unsigned)((n + kScanTileElems - 1) / kScanTileElems), kTileThreads, 0, s>>>(
-                (const T *)a.d_points, ca, (Pt<T, D> *)(b + o_pts));
+            launch(k_cells<T, D, K>, (unsigned)((n + kScanTileElems - 1) / kScanTileElems), kTileThreads, 0, s, (const T *)a.d_points, ca, (Pt<T, D> *)(b + o_pts));
             launches += 2;
         };
         if (sort_bits <= 32) front((uint32_t *)(b + o_ka), (uint32_t *)(b + o_kb));
@@ -568,8 +566,8 @@ int run_lowd(const RunArgs &a) {
     }
     mark(4);
     if (!ptab) {
-        k_hash_init<<<grid_for(cap_max, 256, sms, 8), 256, 0, s>>>((uint64_t *)(b + o_hk), ctr);
-        k_pencils<<<gpts, 256, 0, s>>>((const uint64_t *)(b + o_ckey), g.prefix_shift,
+        launch(k_hash_init, grid_for(cap_max, 256, sms, 8), 256, 0, s, (uint64_t *)(b + o_hk), ctr);
+        launch(k_pencils, gpts, 256, 0, s, (const uint64_t *)(b + o_ckey), g.prefix_shift,
                                        (const uint32_t *)(b + o_pstart), (uint64_t *)(b + o_hk),
                                        (uint32_t *)(b + o_hv), ctr);
         launches += 2;
@@ -600,12 +598,12 @@ int run_lowd(const RunArgs &a) {
     v.core_out = a.d_core;
     v.ctr = ctr;
     // ---- neighbour cells of every cell (stencil pencils -> cell ranges) ----
-    k_ranges<T, D><<<grid_for((n / kRangeRun + 1) * (int64_t)st.n_all, 256, sms, 16), 256, 0, s>>>(v, st);
+    launch(k_ranges<T, D>, grid_for((n / kRangeRun + 1) * (int64_t)st.n_all, 256, sms, 16), 256, 0, s, v, st);
     ++launches;
     mark(5);
     // ---- Definition 2: triage of the cells, then dense cells and exact counts ----
-    k_triage<T, D><<<gpts, 256, 0, s>>>(v, st.n_all);
-    k_core<T, D><<<gwarp, 256, 0, s>>>(v, st);
+    launch(k_triage<T, D>, gpts, 256, 0, s, v, st.n_all);
+    launch(k_core<T, D>, gwarp, 256, 0, s, v, st);
     launches += 2;
     // ---- Algorithm 2: representative points and their coordinates (the stage times k_reps
     // alone; the coordinates of boundary-crossing cells are counted with the merge stage) ----
@@ -613,35 +611,34 @@ int run_lowd(const RunArgs &a) {
     {
         auto reps = [&](auto win) {
             constexpr uint32_t W = decltype(win)::value;
-            k_reps<T, D, W><<<(unsigned)((n + (int64_t)W * kRepWarps - 1) / ((int64_t)W * kRepWarps)), 32 * kRepWarps,
-                              0, s>>>(v, n);
+            launch(k_reps<T, D, W>, (unsigned)((n + (int64_t)W * kRepWarps - 1) / ((int64_t)W * kRepWarps)), 32 * kRepWarps, 0, s, v, n);
             mark(7);
-            k_rep_fix<T, D, W><<<grid_for((n / RepGeom<D, W>::sub + 1) * ndir, 256, sms, 8), 256, 0, s>>>(v, n);
+            launch(k_rep_fix<T, D, W>, grid_for((n / RepGeom<D, W>::sub + 1) * ndir, 256, sms, 8), 256, 0, s, v, n);
         };
         if (n < kRepSmall) reps(std::integral_constant<uint32_t, kRepWinSmall>());
         else reps(std::integral_constant<uint32_t, kRepWin>());
     }
     launches += 2;
     // ---- Algorithm 3: first links, flattened, then one merge pass over every pair ----
-    k_hook<T, D><<<gwarp, 256, 0, s>>>(v, st.n_all, st.n_half);
-    k_flatten<T, D><<<gpts, 256, 0, s>>>(v);
-    k_merge<T, D><<<gwarp, 256, 0, s>>>(v, st.n_all, st.n_half, 2);
+    launch(k_hook<T, D>, gwarp, 256, 0, s, v, st.n_all, st.n_half);
+    launch(k_flatten<T, D>, gpts, 256, 0, s, v);
+    launch(k_merge<T, D>, gwarp, 256, 0, s, v, st.n_all, st.n_half, 2);
     launches += 3;
     mark(8);
     // ---- Algorithm 4: cluster ids, border and noise ----
-    k_comp_min<T, D><<<gpts, 256, 0, s>>>(v);
+    launch(k_comp_min<T, D>, gpts, 256, 0, s, v);
     {
         // the core points' labels (point-parallel, bandwidth) on a second stream beside the
         // border search (latency-bound, few cells): they write disjoint points
         const SideStream ss = side_stream();
         if (ss.ok && cudaEventRecord(ss.fork, s) == cudaSuccess && cudaStreamWaitEvent(ss.s, ss.fork, 0) == cudaSuccess) {
-            k_label_core<T, D><<<gpts, 256, 0, ss.s>>>(v);
-            k_labels<T, D><<<gwarp, 256, 0, s>>>(v, st.n_all);
+            launch(k_label_core<T, D>, gpts, 256, 0, ss.s, v);
+            launch(k_labels<T, D>, gwarp, 256, 0, s, v, st.n_all);
             cudaEventRecord(ss.join, ss.s);
             cudaStreamWaitEvent(s, ss.join, 0);
         } else {
-            k_label_core<T, D><<<gpts, 256, 0, s>>>(v);
-            k_labels<T, D><<<gwarp, 256, 0, s>>>(v, st.n_all);
+            launch(k_label_core<T, D>, gpts, 256, 0, s, v);
+            launch(k_labels<T, D>, gwarp, 256, 0, s, v, st.n_all);
         }
     }
     launches += 3;

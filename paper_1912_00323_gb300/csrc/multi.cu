@@ -25,6 +25,7 @@ __global__ void __launch_bounds__(256) k_copy_segments(const E *__restrict__ src
                                                        const int64_t *__restrict__ compact_start,
                                                        const int64_t *__restrict__ far_start, int nseg,
                                                        int64_t total, int to_compact) {
+    pdl_enter();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < total; j += stride) {
         int lo = 0, hi = nseg - 1;
@@ -47,7 +48,7 @@ void copy_segments(const void *src, void *dst, const int64_t *d_compact, const i
     int64_t blocks = (total + 255) / 256;
     const int64_t cap = (int64_t)(sms > 0 ? sms : 148) * 8;
     if (blocks > cap) blocks = cap;
-    k_copy_segments<E><<<(unsigned)blocks, 256, 0, s>>>((const E *)src, (E *)dst, d_compact, d_far, nseg, total,
+    launch(k_copy_segments<E>, (unsigned)blocks, 256, 0, s, (const E *)src, (E *)dst, d_compact, d_far, nseg, total,
                                                         to_compact ? 1 : 0);
 }
 

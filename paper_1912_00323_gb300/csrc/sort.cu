@@ -65,6 +65,7 @@ __device__ __forceinline__ uint64_t os_pack(uint32_t epoch, uint64_t state, uint
 template <typename K>
 __global__ void __launch_bounds__(kHistThreads) k_os_hist(const K *__restrict__ keys, int64_t n, int begin_bit,
                                                          int end_bit, uint32_t *__restrict__ ghist) {
+    pdl_enter();
     __shared__ uint32_t h[kMaxPasses][kRadix];
     for (int i = threadIdx.x; i < kMaxPasses * kRadix; i += kHistThreads) (&h[0][0])[i] = 0;
     __syncthreads();
@@ -117,6 +118,7 @@ __global__ void __launch_bounds__(kSortThreads, 1) k_os_pass(
     uint32_t *__restrict__ vals_out, int64_t n, int shift, int mask_bits,
     const uint32_t *__restrict__ ghist_pass, unsigned long long *status, uint32_t *ticket, uint32_t epoch,
     uint32_t *err, bool full_sum) {
+    pdl_enter();
     constexpr int kSortItems = ITEMS, kSortTile = ITEMS * kSortThreads;
     extern __shared__ __align__(16) unsigned char sm_raw[];
     PassSmem<K, ITEMS> &S = *reinterpret_cast<PassSmem<K, ITEMS> *>(sm_raw);
@@ -339,7 +341,7 @@ bool run_passes(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, int64_
         const int shift = begin_bit + 8 * p;
         const int bits = (end_bit - shift) < 8 ? (end_bit - shift) : 8;
         auto kern = p == 0 && identity ? k_os_pass<K, ITEMS, true> : k_os_pass<K, ITEMS, false>;
-        kern<<<nb, kSortThreads, smem, s>>>(kin, vin, kout, vout, n, shift, bits, ghist + p * kRadix, status, tickets + p,
+        launch(kern, nb, kSortThreads, smem, s, kin, vin, kout, vout, n, shift, bits, ghist + p * kRadix, status, tickets + p,
                                             (uint32_t)(p + 1), err, nb <= kFullSumTiles);
         K *tk = kin; kin = kout; kout = tk;
         uint32_t *tv = vin; vin = vout; vout = tv;
@@ -374,7 +376,7 @@ bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, 
         ghist = const_cast<uint32_t *>(digit_counts);
     } else {
         const int64_t hb = (n + kHistThreads - 1) / kHistThreads;
-        k_os_hist<K><<<hb < 1216 ? (int)hb : 1216, kHistThreads, 0, s>>>(keys, n, begin_bit, end_bit, ghist);
+        launch(k_os_hist<K>, hb < 1216 ? (int)hb : 1216, kHistThreads, 0, s, keys, n, begin_bit, end_bit, ghist);
         if (launches) *launches += 1;
     }
     if (launches) *launches += (end_bit - begin_bit + 7) / 8;

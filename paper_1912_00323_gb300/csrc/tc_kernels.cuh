@@ -466,6 +466,7 @@ __device__ __forceinline__ uint32_t stream_index(const uint32_t *rpre, const uin
 //            the smallest cluster id among the candidates within eps, else -1.
 template <int DP, int MODE>
 __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float, DP> v, Tables tt) {
+    pdl_enter();
     constexpr int KP = Smem<DP>::KP;
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     Smem<DP> &S = *reinterpret_cast<Smem<DP> *>(smem_raw);
@@ -1108,6 +1109,7 @@ struct Stored {
 template <int DP>
 __global__ void __launch_bounds__(256) k_tc_core_labels(HdView<float, DP> v, Tables tt, int nsets,
                                                        uint32_t *__restrict__ core_lab) {
+    pdl_enter();
     const uint32_t n_core = tt.cx[v.g.n];
     for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n_core; k += gridDim.x * blockDim.x) {
         const uint32_t j = tt.core_list[k];
