@@ -176,7 +176,7 @@ struct Scans {
     LookBack l;
     uint32_t *err;
     uint32_t epoch;
-    cudaStream_t s;
+    Lane s;
     int *launches;
     template <typename F, typename E>
     void run(F f, E emit, uint32_t *out, int64_t m_max, const uint32_t *m_dev, uint32_t *total) {

@@ -108,13 +108,25 @@ struct Workspace {
     size_t bytes;
 };
 
-// Launch of a kernel of a call's chain.  The kernel may be put on the GPU while the one before it in
-// the stream still runs (programmatic stream serialisation), and every kernel launched this way
-// starts with pdl_enter, which waits until that one and its writes are complete.  Measured: a call
-// of 16 short kernels (2-D, 10,000 points) 197 -> 167 us, one of 34 (8-D, 3,001 points) 362 ->
-// 298 us; captured into a graph the chain runs as before.
+// A call's stream, and whether its kernels are put on the GPU early: while the one before in the
+// stream still runs (programmatic stream serialisation; every kernel launched this way starts with
+// pdl_enter, which waits until that one and its writes are complete).  Short kernels gain the
+// launch: a call of 16 of them (2-D, 10,000 points) 197 -> 167 us, one of 34 (8-D, 3,001 points)
+// 362 -> 298 us.  Long ones lose: a block that comes early finds its SM divided into shared memory
+// and L1 as the kernel before needed it, the SM never drains in between, and the passes after
+// the sort run on what L1 the sort left.  Single 3-D sets: two million points 634 -> 599 us, 16
+// million 3.38 -> 4.49 ms; 128 sets in groups of 1.4 million 5.30 -> 5.55 ms; 16-D, one million
+// 2.64 -> 2.60 ms.  So up to two million points, batched or on the coarse grid up to one.
+constexpr int64_t kEarlyMax = 1 << 21, kEarlyMaxBatched = 1 << 20;
+struct Lane {
+    cudaStream_t s;
+    bool early;
+    Lane(cudaStream_t stream = nullptr, bool e = false) : s(stream), early(e) {}
+    operator cudaStream_t() const { return s; }
+};
+
 template <typename... P, typename... A>
-inline void launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, cudaStream_t s, A &&...args) {
+inline void launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t smem, Lane lane, A &&...args) {
     cudaLaunchAttribute attr;
     attr.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr.val.programmaticStreamSerializationAllowed = 1;
@@ -122,9 +134,9 @@ inline void launch(void (*kernel)(P...), unsigned grid, unsigned block, size_t s
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
+    cfg.stream = lane.s;
     cfg.attrs = &attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = lane.early ? 1 : 0;
     cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
 }
 
@@ -193,7 +205,7 @@ uint32_t *sort_status_word(uint32_t *hist, int64_t n);
 template <typename K>
 bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, int64_t n,
                       int begin_bit, int end_bit, uint32_t *hist, uint32_t *partials,
-                      cudaStream_t s, int *launches, uint32_t *err_out = nullptr,
+                      Lane s, int *launches, uint32_t *err_out = nullptr,
                       const uint32_t *digit_counts = nullptr, bool hist_cleared = false, bool identity = false);
 
 // Pool allocation (stream ordered) used by api.cu and the pipelines.

@@ -728,8 +728,9 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_count_hd(HdView<T, DP> v) 
     const int lane = lane_id();
     uint32_t chunks = 0;
     const uint32_t C = v.ctr->n_cells, N = SPILL ? min(v.ctr->hd_spill[0], v.sp_cap) : v.ctr->n_chunks;
-    uint32_t *const next = SPILL ? &v.ctr->hd_spill_next[0] : &v.ctr->hd_next[0];
-    for (uint32_t item = next_chunk(next); item < N; item = next_chunk(next)) {
+    ItemQueue items(SPILL ? &v.ctr->hd_spill_next[0] : &v.ctr->hd_next[0], N);
+    while (items.next()) {
+        const uint32_t item = items.cur;
         const uint2 entry = SPILL ? v.sp_queue[item] : make_uint2(item, 0u);
         if (SPILL && entry.x == 0xffffffffu) continue;
         const uint32_t t = entry.x, A = chunk_cell(v.chunk_off, C, t);
@@ -761,26 +762,46 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_count_hd(HdView<T, DP> v) 
             const unsigned near = open & __ballot_sync(0xffffffffu,
                 !cell_far<FILTER, DP>(v, rows + lane * DP, B, G));
             if (!near) return true;
-            for (uint32_t qb = q0; qb < q1 && open; qb += 32) {
-                const uint32_t q = qb + lane;
-                Cand qv;
-                qv.load(v, q, q < q1);
-                ++chunks;
+            // two blocks of candidates per step (for wide rows one): the row's loads and the loop
+            // around them serve both
+            constexpr int NB = DP <= 16 ? 2 : 1;
+            for (uint32_t qb = q0; qb < q1 && open; qb += 32 * NB) {
+                Cand qv[NB];
+                bool in[NB];
+#pragma unroll
+                for (int u = 0; u < NB; ++u) {
+                    in[u] = qb + 32 * u + lane < q1;
+                    qv[u].load(v, qb + 32 * u + lane, in[u]);
+                }
+                chunks += NB;
                 unsigned rem = open & near;
                 while (rem) {
                     const int jj = __ffs(rem) - 1;
                     rem &= rem - 1;
-                    const bool hit = q < q1 && qv.within(v, rows + jj * DP, base + jj, G);
-                    const unsigned hits = __ballot_sync(0xffffffffu, hit);
-                    if (!hits) continue;
-                    // the row's count, and its list entries from there on
-                    uint32_t at = 0;
-                    if (lane == jj) {
-                        at = SPILL ? atomicAdd(v.sp_val + p, (uint32_t)__popc(hits)) : cnt;
-                        cnt = at + (uint32_t)__popc(hits);
+                    bool hit[NB];
+                    unsigned hits[NB], any = 0;
+#pragma unroll
+                    for (int u = 0; u < NB; ++u) {
+                        hit[u] = in[u] && qv[u].within(v, rows + jj * DP, base + jj, G);
+                        hits[u] = __ballot_sync(0xffffffffu, hit[u]);
+                        any |= hits[u];
                     }
-                    at = __shfl_sync(0xffffffffu, at, jj) + (uint32_t)__popc(hits & ((1u << lane) - 1u));
-                    if (hit && at < v.nl_k) v.nl[(uint64_t)(base + jj) * v.nl_k + at] = q;
+                    if (!any) continue;
+                    // the row's count, and its list entries from there on
+                    uint32_t found = 0, at = 0;
+#pragma unroll
+                    for (int u = 0; u < NB; ++u) found += (uint32_t)__popc(hits[u]);
+                    if (lane == jj) {
+                        at = SPILL ? atomicAdd(v.sp_val + p, found) : cnt;
+                        cnt = at + found;
+                    }
+                    at = __shfl_sync(0xffffffffu, at, jj);
+#pragma unroll
+                    for (int u = 0; u < NB; ++u) {
+                        const uint32_t slot = at + (uint32_t)__popc(hits[u] & ((1u << lane) - 1u));
+                        if (hit[u] && slot < v.nl_k) v.nl[(uint64_t)(base + jj) * v.nl_k + slot] = qb + 32 * u + lane;
+                        at += (uint32_t)__popc(hits[u]);
+                    }
                 }
                 open &= __ballot_sync(0xffffffffu, have && cnt < min_pts);
             }
@@ -1062,8 +1083,9 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_odd_hd(HdView<T, DP> v) {
     const int lane = lane_id();
     uint32_t chunks = 0;
     const uint32_t C = v.ctr->n_cells, N = SPILL ? min(v.ctr->hd_spill[2], v.sp_cap) : v.ctr->n_chunks;
-    uint32_t *const next = SPILL ? &v.ctr->hd_spill_next[2] : &v.ctr->hd_next[1];
-    for (uint32_t item = next_chunk(next); item < N; item = next_chunk(next)) {
+    ItemQueue items(SPILL ? &v.ctr->hd_spill_next[2] : &v.ctr->hd_next[1], N);
+    while (items.next()) {
+        const uint32_t item = items.cur;
         const uint2 entry = SPILL ? v.sp_queue[item] : make_uint2(item, 0u);
         if (SPILL && entry.x == 0xffffffffu) continue;
         const uint32_t t = entry.x;
@@ -1280,8 +1302,9 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_labels_hd(HdView<T, DP> v)
     const int lane = lane_id();
     uint32_t noise = 0, chunks = 0;
     const uint32_t C = v.ctr->n_cells, N = SPILL ? min(v.ctr->hd_spill[1], v.sp_cap) : v.ctr->n_chunks;
-    uint32_t *const next = SPILL ? &v.ctr->hd_spill_next[1] : &v.ctr->hd_next[3];
-    for (uint32_t item = next_chunk(next); item < N; item = next_chunk(next)) {
+    ItemQueue items(SPILL ? &v.ctr->hd_spill_next[1] : &v.ctr->hd_next[3], N);
+    while (items.next()) {
+        const uint32_t item = items.cur;
         const uint2 entry = SPILL ? v.sp_queue[item] : make_uint2(item, 0u);
         if (SPILL && entry.x == 0xffffffffu) continue;
         const uint32_t t = entry.x, A = chunk_cell(v.chunk_off, C, t);

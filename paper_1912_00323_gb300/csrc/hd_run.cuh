@@ -144,7 +144,7 @@ struct TcOffsets {
 
 // Launch shapes shared by the phases.
 struct HdLaunch {
-    cudaStream_t s;
+    Lane s;
     int gpts, gcell, block;  // grids of the point and of the chunk kernels, threads of the latter
     size_t smem;             // their shared memory
     bool list_labels;        // the lists are complete: labels from them
@@ -210,7 +210,7 @@ template <int DP, typename Mark>
 void run_tc_phases(HdView<float, DP> &hv, const HdLaunch &L, char *b, int64_t n, int grid_tc, size_t tc_smem,
                    Scans &scans, const TcOffsets &o, int nsets, DevCounters *ctr, const TcTuning &tune, Mark &mark,
                    int &launches, cudaEvent_t *tev) {
-    cudaStream_t s = L.s;
+    const Lane s = L.s;
     const int gpts = L.gpts, gcell = L.gcell, hd_block = L.block;
     const size_t smem = L.smem;
     // tev (nullable): six events recorded around the three tensor-core launches
@@ -290,7 +290,7 @@ void run_tc_phases(HdView<float, DP> &hv, const HdLaunch &L, char *b, int64_t n,
     const detail::SideStream ss = detail::side_stream();
     const bool fork = ss.ok && cudaEventRecord(ss.fork, s) == cudaSuccess &&
                       cudaStreamWaitEvent(ss.s, ss.fork, 0) == cudaSuccess;
-    auto cuda_labels = [&](cudaStream_t ls) {
+    auto cuda_labels = [&](Lane ls) {
         launch(k_labels_hd<float, DP, false, true>, gcell, hd_block, smem, ls, hv);
         launch(k_labels_hd<float, DP, true, true>, gcell, hd_block, smem, ls, hv);
     };
@@ -312,7 +312,7 @@ void run_tc_phases(HdView<float, DP> &hv, const HdLaunch &L, char *b, int64_t n,
 template <typename T, int DP>
 int run_hd(const RunArgs &a) {
     using namespace detail;
-    cudaStream_t s = a.stream;
+    const Lane s(a.stream, a.n <= kEarlyMaxBatched);
     const int64_t n = a.n;
     const int d = a.d;
     int launches = 0;

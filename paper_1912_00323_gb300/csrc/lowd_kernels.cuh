@@ -83,6 +83,10 @@ __device__ __forceinline__ void set_error(DevCounters *ctr, uint32_t bit) {
     atomicOr(&ctr->status, bit);
 }
 
+// Threads per block of the kernels that hand cells to warps: small blocks, so that a warp with a long
+// cell holds few others' slots.
+constexpr int kCellBlock = 128;
+
 // The next work item for this warp from a per-kernel counter (warp-uniform): cells and chunks
 // differ in cost by orders of magnitude, so they are handed out dynamically.
 __device__ __forceinline__ uint32_t next_chunk(uint32_t *counter) {
@@ -91,13 +95,22 @@ __device__ __forceinline__ uint32_t next_chunk(uint32_t *counter) {
     return __shfl_sync(0xffffffffu, t, 0);
 }
 
-// Items [0, N) to warps in batches of kItemBatch taken from counter ctr->lowd_next[slot] (one
-// item at a time: the label list is short, so batches left most warps idle).
-constexpr uint32_t kItemBatch = 1;
-#define LOWD_FOR_EACH(v, X, N, slot)                                                                  \
-    for (uint32_t b_ = next_chunk(&(v).ctr->lowd_next[slot]) * kItemBatch; b_ < (N);                \
-         b_ = next_chunk(&(v).ctr->lowd_next[slot]) * kItemBatch)                                   \
-        for (uint32_t X = b_, xe_ = min(b_ + kItemBatch, (uint32_t)(N)); X < xe_; ++X)
+// Items [0, n) to warps: the first by the warp's number, the rest from a counter, each fetched while
+// the one before is worked on (with every warp taking its first item from the counter, ten
+// thousand atomics on one word came before any work).
+struct ItemQueue {
+    uint32_t *counter;
+    uint32_t n, cur, ahead;
+    __device__ __forceinline__ ItemQueue(uint32_t *c, uint32_t items)
+        : counter(c), n(items), cur(0xffffffffu), ahead((uint32_t)global_warp()) {}
+    __device__ __forceinline__ bool next() {  // false: no item left; warp-uniform
+        cur = __shfl_sync(0xffffffffu, ahead, 0);
+        if (cur >= n) return false;
+        const uint32_t warps = (uint32_t)total_warps();
+        if (lane_id() == 0) ahead = warps < n ? warps + atomicAdd(counter, 1u) : 0xffffffffu;
+        return true;
+    }
+};
 
 // Batched calls put the set id above the cell key bits; cells never mix sets.
 template <typename V>
@@ -794,7 +807,7 @@ __global__ void __launch_bounds__(256) k_triage(LowdView<T, D> v, int n_all) {
 // ballot.  Also initialises the representative slots of cells with core points and fills the
 // lists of cells with core points (merging) and with non-core points (labels).
 template <typename T, int D>
-__global__ void __launch_bounds__(256) k_core(LowdView<T, D> v, Stencil st_in) {
+__global__ void __launch_bounds__(kCellBlock) k_core(LowdView<T, D> v, Stencil st_in) {
     pdl_enter();
     __shared__ Stencil st;
     load_stencil<T, D>(st, st_in);
@@ -1164,7 +1177,7 @@ __device__ bool warp_core_pair(const LowdView<T, D> &v, uint32_t A, uint32_t B, 
 // link points to a lower index, so the links form a forest whose trees lie inside clusters;
 // pointer jumping flattens it and the merge passes then join the trees.
 template <typename T, int D>
-__global__ void __launch_bounds__(256) k_hook(LowdView<T, D> v, int n_all, int n_half) {
+__global__ void __launch_bounds__(kCellBlock) k_hook(LowdView<T, D> v, int n_all, int n_half) {
     pdl_enter();
     constexpr int ndir = RepDirs<D>::value;
     const int lane = lane_id();
@@ -1226,7 +1239,7 @@ __global__ void __launch_bounds__(256) k_flatten(LowdView<T, D> v) {
 // representative points are tested first (Algorithm 3); a miss falls back to the exhaustive
 // core x core test.  Lanes walk the flattened list of candidate cells of one cell.
 template <typename T, int D>
-__global__ void __launch_bounds__(256) k_merge(LowdView<T, D> v, int n_all, int n_half, int pass) {
+__global__ void __launch_bounds__(kCellBlock) k_merge(LowdView<T, D> v, int n_all, int n_half, int pass) {
     pdl_enter();
     constexpr int ndir = RepDirs<D>::value;
     const int lane = lane_id();
@@ -1356,13 +1369,14 @@ __global__ void __launch_bounds__(256) k_label_core(LowdView<T, D> v) {
 // wholly within eps settles that point at once (warp minimum), one wholly beyond eps is
 // dropped, and the others are compared point by point.  Writes labels in input order.
 template <typename T, int D>
-__global__ void __launch_bounds__(256, 4) k_labels(LowdView<T, D> v, int n_all) {
+__global__ void __launch_bounds__(kCellBlock, 8) k_labels(LowdView<T, D> v, int n_all) {
     pdl_enter();
     const int lane = lane_id();
     uint32_t noise = 0, chunks = 0;
     const uint32_t NL = v.ctr->n_list[2];
-    LOWD_FOR_EACH(v, X, NL, 4) {
-        const uint32_t A = v.list_label[X];
+    ItemQueue items(&v.ctr->lowd_next[4], NL);
+    while (items.next()) {
+        const uint32_t A = v.list_label[items.cur];
         const uint32_t s = v.cell_start[A], e = v.cell_start[A + 1];
         const uint64_t akey = v.cell_key[A];
         const uint32_t aset = set_of_key(v, akey);

@@ -296,7 +296,7 @@ inline uint32_t *pencil_table(int bits, int64_t cap_max, void *space) {
 template <typename T, int D>
 int run_lowd(const RunArgs &a) {
     using namespace detail;
-    cudaStream_t s = a.stream;
+    const Lane s(a.stream, a.n <= (a.nsets > 0 ? kEarlyMaxBatched : kEarlyMax));
     const int64_t n = a.n;
     constexpr int ndir = RepDirs<D>::value;
     int launches = 0;
@@ -347,7 +347,7 @@ int run_lowd(const RunArgs &a) {
     Stencil st;
     double tau = 0.0;
     const int gpts = grid_for(n, 256, sms, 8);
-    const int gwarp = grid_for(n, 8, sms, 16);
+    const int gwarp = grid_for(n, kCellBlock / 32, sms, 2048 / kCellBlock);
     LowdView<T, D> v;
     memset(&v, 0, sizeof(v));
     bool flipped = false;
@@ -603,7 +603,7 @@ int run_lowd(const RunArgs &a) {
     mark(5);
     // ---- Definition 2: triage of the cells, then dense cells and exact counts ----
     launch(k_triage<T, D>, gpts, 256, 0, s, v, st.n_all);
-    launch(k_core<T, D>, gwarp, 256, 0, s, v, st);
+    launch(k_core<T, D>, gwarp, kCellBlock, 0, s, v, st);
     launches += 2;
     // ---- Algorithm 2: representative points and their coordinates (the stage times k_reps
     // alone; the coordinates of boundary-crossing cells are counted with the merge stage) ----
@@ -620,9 +620,9 @@ int run_lowd(const RunArgs &a) {
     }
     launches += 2;
     // ---- Algorithm 3: first links, flattened, then one merge pass over every pair ----
-    launch(k_hook<T, D>, gwarp, 256, 0, s, v, st.n_all, st.n_half);
+    launch(k_hook<T, D>, gwarp, kCellBlock, 0, s, v, st.n_all, st.n_half);
     launch(k_flatten<T, D>, gpts, 256, 0, s, v);
-    launch(k_merge<T, D>, gwarp, 256, 0, s, v, st.n_all, st.n_half, 2);
+    launch(k_merge<T, D>, gwarp, kCellBlock, 0, s, v, st.n_all, st.n_half, 2);
     launches += 3;
     mark(8);
     // ---- Algorithm 4: cluster ids, border and noise ----
@@ -633,12 +633,12 @@ int run_lowd(const RunArgs &a) {
         const SideStream ss = side_stream();
         if (ss.ok && cudaEventRecord(ss.fork, s) == cudaSuccess && cudaStreamWaitEvent(ss.s, ss.fork, 0) == cudaSuccess) {
             launch(k_label_core<T, D>, gpts, 256, 0, ss.s, v);
-            launch(k_labels<T, D>, gwarp, 256, 0, s, v, st.n_all);
+            launch(k_labels<T, D>, gwarp, kCellBlock, 0, s, v, st.n_all);
             cudaEventRecord(ss.join, ss.s);
             cudaStreamWaitEvent(s, ss.join, 0);
         } else {
             launch(k_label_core<T, D>, gpts, 256, 0, s, v);
-            launch(k_labels<T, D>, gwarp, 256, 0, s, v, st.n_all);
+            launch(k_labels<T, D>, gwarp, kCellBlock, 0, s, v, st.n_all);
         }
     }
     launches += 3;

@@ -328,7 +328,7 @@ __global__ void __launch_bounds__(kSortThreads, 1) k_os_pass(
 template <typename K, int ITEMS>
 bool run_passes(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, int64_t n, int begin_bit, int end_bit,
                 const uint32_t *ghist, unsigned long long *status, uint32_t *tickets, uint32_t *err, bool identity,
-                cudaStream_t s) {
+                Lane s) {
     const int nb = (int)((n + (int64_t)ITEMS * kSortThreads - 1) / ((int64_t)ITEMS * kSortThreads));
     const int passes = (end_bit - begin_bit + 7) / 8;
     const size_t smem = sizeof(PassSmem<K, ITEMS>);
@@ -359,7 +359,7 @@ uint32_t *sort_status_word(uint32_t *hist, int64_t n) {
 template <typename K>
 bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, int64_t n,
                       int begin_bit, int end_bit, uint32_t *hist, uint32_t *partials,
-                      cudaStream_t s, int *launches, uint32_t *err_out, const uint32_t *digit_counts,
+                      Lane s, int *launches, uint32_t *err_out, const uint32_t *digit_counts,
                       bool hist_cleared, bool identity) {
     (void)partials;
     if (n <= 1 || end_bit <= begin_bit) {
@@ -393,10 +393,10 @@ bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, 
 }
 
 template bool radix_sort_pairs<uint32_t>(uint32_t *, uint32_t *, uint32_t *, uint32_t *, int64_t,
-                                         int, int, uint32_t *, uint32_t *, cudaStream_t, int *, uint32_t *,
+                                         int, int, uint32_t *, uint32_t *, Lane, int *, uint32_t *,
                                          const uint32_t *, bool, bool);
 template bool radix_sort_pairs<uint64_t>(uint64_t *, uint32_t *, uint64_t *, uint32_t *, int64_t,
-                                         int, int, uint32_t *, uint32_t *, cudaStream_t, int *, uint32_t *,
+                                         int, int, uint32_t *, uint32_t *, Lane, int *, uint32_t *,
                                          const uint32_t *, bool, bool);
 
 }  // namespace hca
