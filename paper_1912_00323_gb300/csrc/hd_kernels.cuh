@@ -57,6 +57,7 @@ struct HdView {
     uint8_t *core_out;
     DevCounters *ctr;
     int n_all, n_half;
+    uint8_t near[16];             // the pencils nearest first (n_all of them; the coarse grid has 9)
     // cells left to the tensor-core kernels (float input): those with at least tc_min[phase] rows
     // of a phase (counts, unions, labels; 0: none); cx = exclusive scan of the core flags, for
     // the per-cell core counts; tc_hook: first links also in cells whose unions run there
@@ -647,8 +648,19 @@ __global__ void __launch_bounds__(256) k_cell_box_decode(HdView<T, DP> v) {
                           base = (v).cell_start[A] + 32u * (t_ - (v).chunk_off[A]), o2_ = 1; \
                  o2_; o2_ = 0)
 
-// Length of a cell's candidate stream: its neighbour ranges (at most 32; the coarse grid has 9),
-// one per lane, laid end to end.
+// Candidate stream of a cell: spans of cells laid end to end, the cell itself first, then the rest of
+// its pencil, then the other pencils nearest first.  Points within eps differ by a fraction of
+// eps in each projected coordinate, so nearly half of a point's neighbours are in its own cell
+// (9-D clusters: 44%, in a twentieth of the candidates) and a core point reaches MINPTS early.
+constexpr int kSpansExtra = 2;  // spans beyond one per pencil
+template <typename V>
+__device__ __forceinline__ uint2 stream_span(const V &v, uint32_t A, int k) {
+    if (k >= v.n_all + kSpansExtra) return make_uint2(0u, 0u);
+    const uint2 rg = v.ranges[(uint64_t)A * v.n_all + (k < 3 ? 0 : v.near[k - 2])];
+    return k == 0 ? make_uint2(A, A + 1) : k == 1 ? make_uint2(rg.x, A) : k == 2 ? make_uint2(A + 1, rg.y) : rg;
+}
+
+// Its length, from one span per lane.
 template <typename V>
 __device__ __forceinline__ uint32_t stream_length(const V &v, uint2 rg) {
     return __reduce_add_sync(0xffffffffu, rg.x < rg.y ? v.cell_start[rg.y] - v.cell_start[rg.x] : 0u);
@@ -659,7 +671,7 @@ __device__ __forceinline__ uint32_t stream_length(const V &v, uint2 rg) {
 template <typename V, typename F>
 __device__ __forceinline__ void for_stream_cells(const V &v, uint2 rg, uint32_t p0, uint32_t p1, F f) {
     uint32_t pos = 0;
-    for (int kk = 0; kk < v.n_all; ++kk) {
+    for (int kk = 0; kk < v.n_all + kSpansExtra; ++kk) {
         const uint32_t lo = __shfl_sync(0xffffffffu, rg.x, kk);
         const uint32_t hi = __shfl_sync(0xffffffffu, rg.y, kk);
         if (lo >= hi) continue;
@@ -743,7 +755,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_count_hd(HdView<T, DP> v) 
         if (!rows_m) continue;
         const GridParams &G = params_of(v, set_of_key(v, v.cell_key[A]));
         const uint32_t min_pts = G.min_pts;
-        const uint2 rg = lane < v.n_all ? v.ranges[(uint64_t)A * v.n_all + lane] : make_uint2(0u, 0u);
+        const uint2 rg = stream_span(v, A, lane);
         const uint32_t total = stream_length(v, rg);
         // a row the tensor-core count handed over resumes where it stopped (same candidate order)
         const uint32_t start = tc_cell ? __shfl_sync(0xffffffffu, have ? v.tc_pos[p] : 0u, __ffs(rows_m) - 1) : 0u;
@@ -1095,7 +1107,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_odd_hd(HdView<T, DP> v) {
         if (v.cell_root[A] == kMixedRoot) continue;  // mixed: left to the union kernels
         const uint32_t e = v.cell_start[A + 1], base = v.cell_start[A] + 32u * (t - v.chunk_off[A]), p = base + lane;
         const GridParams &G = params_of(v, set_of_key(v, v.cell_key[A]));
-        const uint2 rg = lane < v.n_all ? v.ranges[(uint64_t)A * v.n_all + lane] : make_uint2(0u, 0u);
+        const uint2 rg = stream_span(v, A, lane);
         const uint32_t total = stream_length(v, rg);
         uint32_t p0 = 0, p1 = min(kSpillWin, total);
         if (SPILL) spill_window(entry.y, p1, total, p0, p1);
@@ -1321,7 +1333,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_labels_hd(HdView<T, DP> v)
         const unsigned smask = __ballot_sync(0xffffffffu, have && !isc);
         bool decide = true;
         if (smask) {
-            const uint2 rg = lane < v.n_all ? v.ranges[(uint64_t)A * v.n_all + lane] : make_uint2(0u, 0u);
+            const uint2 rg = stream_span(v, A, lane);
             const uint32_t total = stream_length(v, rg);
             uint32_t p0 = 0, p1 = min(kSpillWin, total);
             if (SPILL) spill_window(entry.y, p1, total, p0, p1);

@@ -568,6 +568,10 @@ int run_hd(const RunArgs &a) {
         if (rc) goto out;
         if (batched) cudaMemcpyAsync(d_gtab, gsets.data(), sizeof(GridParams) * nsets, cudaMemcpyHostToDevice, s);
     }
+    if (st.n_all > 16) {  // (cells of side eps (1 + 2^-10) have the 3 x 3 pencils around them)
+        rc = HCA_ENOTIMPL;
+        goto out;
+    }
     mark(1);
     // the filter's float copy of double input takes the half of the box space that float boxes
     // leave free
@@ -653,6 +657,7 @@ int run_hd(const RunArgs &a) {
     hv.ctr = ctr;
     hv.n_all = st.n_all;
     hv.n_half = st.n_half;
+    for (int k = 0; k < st.n_all && k < 16; ++k) hv.near[k] = (uint8_t)st.near[k];
     hv.fpts = sizeof(T) == 4 ? (const float *)(b + o_pts) : fpts;
     hv.cell_of = (const uint32_t *)(b + o_flags);
     hv.box_lo = (T *)(b + o_blo);
@@ -691,7 +696,7 @@ int run_hd(const RunArgs &a) {
         ++launches;
     }
     if constexpr (std::is_same<T, float>::value) {
-        if (use_tc && st.n_all <= tc::kMaxRng) {
+        if (use_tc) {
             run_tc_phases<DP>(hv, L, b, n, sms * tc_occ, tc_smem, scans,
                               TcOffsets{o_tnch, o_tnch2, o_tch0, o_tch1, o_tch2, o_tflags, o_cx, o_clist, o_nclist,
                                         o_clab},

@@ -105,7 +105,8 @@ struct Tables {
 // its windows, and the last window to finish decides the row.
 constexpr uint32_t kRecountMin = 32;
 
-// Counts: points of neighbour range k of cell A (the stream is ranges 0 .. n_all - 1 end to end).
+// Counts: points of neighbour range k of cell A (the stream is all of them, in the order of
+// stream_span).
 __device__ __forceinline__ uint32_t count_range_len(const uint2 *ranges, int n_all, const uint32_t *cell_start,
                                                     uint32_t A, int k) {
     const uint2 rg = ranges[(uint64_t)A * n_all + k];
@@ -496,7 +497,7 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
     uint32_t *const next = recount ? &v.ctr->tc_next_recount : &v.ctr->tc_next[MODE];
     const bool split = MODE == kMerge && N0 < kSplitBelow * gridDim.x;
     const uint32_t NC = split ? N0 + v.ctr->n_tc_chunks[3] : N0;  // unions: first windows, then the rest
-    const int n_rng = MODE == kMerge ? v.n_half : v.n_all;
+    const int n_rng = MODE == kMerge ? v.n_half : MODE == kCount ? v.n_all + kSpansExtra : v.n_all;
     uint32_t phase = 0;
     bool failed = false;  // CTA-uniform
     uint32_t n_tiles = 0, n_skip = 0, n_re = 0, n_noise = 0;
@@ -517,7 +518,7 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
                     nwin = merge_windows(__reduce_add_sync(0xffffffffu, len));
                 }
                 if (recount) {
-                    uint32_t len = tid < n_rng ? count_range_len(v.ranges, v.n_all, v.cell_start, A, tid) : 0u;
+                    uint32_t len = tid < v.n_all ? count_range_len(v.ranges, v.n_all, v.cell_start, A, tid) : 0u;
                     nwin = merge_windows(__reduce_add_sync(0xffffffffu, len));
                 }
             }
@@ -646,7 +647,7 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
         if (warp == 0 && !by_cell) {
             uint32_t q0 = 0, len = 0;
             if (tid < n_rng) {
-                uint2 rg = v.ranges[(uint64_t)A * v.n_all + tid];
+                uint2 rg = MODE == kCount ? stream_span(v, A, tid) : v.ranges[(uint64_t)A * v.n_all + tid];
                 if (MODE == kMerge && tid == 0) rg.x = A;  // own pencil: this cell and the ones after it
                 if (rg.x < rg.y) {
                     q0 = v.cell_start[rg.x];
