@@ -239,11 +239,11 @@ void run_tc_phases(HdView<float, DP> &hv, const HdLaunch &L, char *b, int64_t n,
               &ctr->n_tc_chunks[tc::kCount]);
     tmark(0);
     launch(tc::k_tc_hd<DP, tc::kCount>, grid_tc, tc::kTile, tc_smem, s, hv, tc::Tables{ch0, cx, clist, nclist, clab});
-    // the rows those chunks handed over, in cells with at least kRecountMin of them, counted again
-    // from the start, 128 per chunk (cx, clist, nclist and ch1 are free until the core numbering); the
+    // the rows those chunks handed over, in cells with at least kRecountMin of them, counted on, 128
+    // per chunk (cx, clist, nclist and ch1 are free until the core numbering); the
     // rest, and what the recount hands over, go to the CUDA-core count.  Per listed row the
     // tallies summed over its windows and the windows done are in nch, ch0 and nclist.
-    scans.run(tc::HandedFlag{hv.core}, tc::HandedList{clist, nch, ch0, nclist}, cx, n, nullptr, cx + n);
+    scans.run(tc::HandedFlag{hv.core}, tc::HandedList{clist, nch, ch0, nclist, hv.tc_cnt}, cx, n, nullptr, cx + n);
     scans.run(tc::RecountItems{hv.cell_start, cx, hv.ranges, hv.n_all, tc::kRecountMin}, tc::NoEmit{}, ch1, n,
               &ctr->n_cells, &ctr->n_tc_recount);
     launch(tc::k_tc_hd<DP, tc::kCount>, grid_tc, tc::kTile, tc_smem, s, hv, tc::Tables{ch1, cx, nullptr, nullptr, nullptr, nullptr, clist, nch, ch0, nclist});

@@ -55,6 +55,7 @@ constexpr uint32_t kWaitLimit = 1u << 22;  // mbarrier polls before a wait gives
 constexpr size_t kMinSmem = 48 * 1024;     // per CTA: at most 4 CTAs (4 x 128 TMEM columns) per SM
 constexpr int kMaxRng = 32;                // neighbour ranges per cell (the coarse grid has 9)
 constexpr uint32_t kSegCand = 16 * kTile;  // unions: candidates per work item (a window of the stream)
+constexpr uint32_t kRecountSeg = 16 * kTile;  // recount: the same (twice as many made the 16-D recount longer)
 constexpr uint32_t kSplitBelow = 32;       // unions: windows only with fewer chunks per CTA than this
 enum { kCount = 0, kMerge = 1, kLabels = 2 };
 
@@ -82,6 +83,9 @@ __device__ __forceinline__ uint32_t merge_range_len(const HdView<float, DP> &v, 
 __device__ __forceinline__ uint32_t merge_windows(uint32_t len) {
     return len > kSegCand ? (len + kSegCand - 1u) / kSegCand : 1u;
 }
+__device__ __forceinline__ uint32_t recount_windows(uint32_t len) {
+    return len > kRecountSeg ? (len + kRecountSeg - 1u) / kRecountSeg : 1u;
+}
 
 // Row and candidate lists of the three phases.
 struct Tables {
@@ -100,9 +104,10 @@ struct Tables {
 
 // A coarse cell whose first tensor-core count handed over at least this many rows counts them
 // again on the tensor cores (128 per chunk) instead of leaving them to the CUDA-core count.
-// The recount's rows scan their whole neighbourhood (few reach MINPTS early), so each chunk
-// runs as windows of kSegCand candidates, one work item each; a row's tallies are summed over
-// its windows, and the last window to finish decides the row.
+// The recount's rows scan the rest of their neighbourhood (few reach MINPTS early), so each chunk
+// runs as windows of kRecountSeg candidates, one work item each; a row's tallies are summed over
+// its windows, and the last window to finish decides the row.  A row takes part from the position
+// on where the first count left it.
 constexpr uint32_t kRecountMin = 32;
 
 // Counts: points of neighbour range k of cell A (the stream is all of them, in the order of
@@ -298,6 +303,7 @@ struct Smem {
     uint32_t la[3], pad3;      // unions: blocks of a look-ahead round not skippable (rotating)
     uint64_t mbar;
     uint32_t taddr, ref, next, fail;
+    uint32_t from, pad5[3];    // recount: the first stream position that a row of the chunk still needs
 };
 
 template <int DP>
@@ -519,10 +525,11 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
                 }
                 if (recount) {
                     uint32_t len = tid < v.n_all ? count_range_len(v.ranges, v.n_all, v.cell_start, A, tid) : 0u;
-                    nwin = merge_windows(__reduce_add_sync(0xffffffffu, len));
+                    nwin = recount_windows(__reduce_add_sync(0xffffffffu, len));
                 }
             }
             if (tid == 0) {
+                S.from = 0xffffffffu;
                 S.next = t;
                 S.cell = A;
                 S.nwin = nwin;
@@ -556,6 +563,14 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
         const uint32_t rk = k0 + (uint32_t)tid;
         const bool have = rk < rend;
         const uint32_t p = have ? row_point<MODE>(tt, rk) : 0u;
+        // recount: where the first count left this row (a multiple of the block), and the chunk's first
+        uint32_t from = 0, goal = G.min_pts;  // goal: pairs within eps that make the row core
+        if (MODE == kCount && recount) {
+            from = have ? v.tc_pos[p] : 0xffffffffu;
+            if (have) goal -= v.tc_cnt[p];
+            const uint32_t least = __reduce_min_sync(0xffffffffu, from);
+            if ((tid & 31) == 0) atomicMin(&S.from, least);
+        }
         float4 q[DP / 4];
         {
             const float4 *src = reinterpret_cast<const float4 *>(v.pts + (uint64_t)p * DP);
@@ -673,10 +688,12 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
             if (tid == 31) S.rpre[kMaxRng] = incl;  // stream length
         }
         __syncthreads();
-        // the item's part of the stream: all of it, or for the unions window win of kSegCand
+        // the item's part of the stream: all of it, for the unions window win of kSegCand, for the
+        // recount window win of kRecountSeg from the first position on that a row still needs
         const uint32_t L_all = S.rpre[kMaxRng];
-        const uint32_t u0 = MODE == kMerge || recount ? min(L_all, win * kSegCand) : 0u;
-        const uint32_t L = split || recount ? min(L_all, u0 + kSegCand) : L_all;
+        uint32_t u0 = MODE == kMerge ? min(L_all, win * kSegCand) : recount ? min(L_all, win * kRecountSeg) : 0u;
+        const uint32_t L = split ? min(L_all, u0 + kSegCand) : recount ? min(L_all, u0 + kRecountSeg) : L_all;
+        if (recount) u0 = min(L, max(u0, S.from));
         if (MODE == kMerge && u0 >= L && win > 0u) continue;  // the pruning left nothing in this window
         const float na = stage_split<DP, KP>(S.a_hi, S.a_lo, tid, q, S.cen, have);
         const float lo = (float)(G.eps2 * (1.0 - 0x1p-20));
@@ -801,7 +818,7 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
             asm volatile("tcgen05.fence::after_thread_sync;");
             ++n_tiles;
             if (tid == 0) n_pairs += (unsigned long long)min((uint32_t)kTile, rend - k0) * nq;
-            bool need = have && (MODE != kCount || !done);
+            bool need = have && (MODE != kCount || (!done && ub >= from));
             if (MODE == kCount && __any_sync(0xffffffffu, need)) {
                 // 64 columns per wait, the second 32 read even past nq (allocated columns; an empty
                 // candidate's value is below every threshold)
@@ -910,7 +927,7 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
                 }
                 __syncwarp();
             }
-            if (MODE == kCount) done = done || cnt >= G.min_pts;
+            if (MODE == kCount) done = done || cnt >= goal;
             asm volatile("tcgen05.fence::before_thread_sync;");
             int open = 0;
             if (MODE == kCount) open = __syncthreads_count(!done);
@@ -1031,7 +1048,7 @@ struct BoxDecode {
 };
 
 // The recount of handed-over rows: their list (ascending; core = 2, set only by the tensor-core
-// count, the other cells' flags are still 0) with its tallies cleared, and the work items of every
+// count, the other cells' flags are still 0) with its tallies so far, and the work items of every
 // cell with at least min_rows of them.
 struct HandedFlag {
     const uint8_t *core;
@@ -1039,11 +1056,12 @@ struct HandedFlag {
 };
 struct HandedList {
     uint32_t *list, *in, *hi, *done;
+    const uint32_t *cnt;  // the rows' counts so far (both tallies agree on a row that was handed over)
     __device__ void operator()(int64_t j, uint32_t f, uint32_t x) const {
         if (!f) return;
         list[x] = (uint32_t)j;
-        in[x] = 0u;
-        hi[x] = 0u;
+        in[x] = cnt[j];
+        hi[x] = cnt[j];
         done[x] = 0u;
     }
 };
@@ -1057,7 +1075,7 @@ struct RecountItems {
         if (items) {
             uint32_t len = 0;
             for (int k = 0; k < n_all; ++k) len += count_range_len(ranges, n_all, cell_start, (uint32_t)c, k);
-            items *= merge_windows(len);
+            items *= recount_windows(len);
         }
         return items;
     }
