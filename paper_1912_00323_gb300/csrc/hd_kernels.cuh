@@ -1115,7 +1115,16 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_odd_hd(HdView<T, DP> v) {
         const bool mine = (omask >> lane) & 1u;
         uint32_t rp = mine ? uf_find(v.parent, p, v.ctr) : 0xffffffffu;
         auto scan = [&](uint32_t B, uint32_t q0, uint32_t q1) -> bool {
-            const unsigned near = omask & __ballot_sync(0xffffffffu, !cell_far<FILTER, DP>(v, rows + lane * DP, B, G));
+            // nothing to join with a cell without core points, nor for a row in the tree of the cell:
+            // the cell's other core points are in that tree too, but for its odd ones, and those
+            // come to the row's cell themselves (or, where the row's cell has another tree, the
+            // two cells are left to the union kernels)
+            uint32_t rb = v.cell_root[B];
+            if (rb == kNoRoot) return true;
+            if (rb != kMixedRoot) rb = uf_root_readonly(v.parent, rb, v.ctr);
+            unsigned near = __ballot_sync(0xffffffffu, mine && rp != rb);
+            if (!near) return true;
+            near &= __ballot_sync(0xffffffffu, !cell_far<FILTER, DP>(v, rows + lane * DP, B, G));
             if (!near) return true;
             for (uint32_t qb = q0; qb < q1; qb += 32) {
                 const uint32_t q = qb + lane;

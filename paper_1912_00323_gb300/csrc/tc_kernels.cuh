@@ -589,15 +589,15 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
         bool by_cell = false;
         if (MODE != kCount) {
             if (warp == 0) {
-                uint32_t lo = 0, cnt = 0;
+                // (unions: only the cells that still have something to join with A)
+                uint2 rg = make_uint2(0u, 0u);
                 if (tid < n_rng) {
-                    uint2 rg = v.ranges[(uint64_t)A * v.n_all + tid];
+                    rg = v.ranges[(uint64_t)A * v.n_all + tid];
                     if (MODE == kMerge && tid == 0) rg.x = A;  // own pencil: this cell and the ones after it
-                    if (rg.x < rg.y) {
-                        lo = rg.x;
-                        cnt = rg.y - rg.x;
-                    }
                 }
+                const uint32_t ra = MODE == kMerge ? v.cell_root[A] : 0u;
+                uint32_t cnt = 0;
+                for (uint32_t c = rg.x; c < rg.y; ++c) cnt += MODE != kMerge || cells_to_join(ra, v.cell_root[c]) ? 1u : 0u;
                 uint32_t incl = cnt;
 #pragma unroll
                 for (int o = 1; o < 32; o <<= 1) {
@@ -605,8 +605,12 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
                     if (tid >= o) incl += y;
                 }
                 const uint32_t total = __shfl_sync(0xffffffffu, incl, 31);
-                for (uint32_t j = 0; j < cnt; ++j)
-                    if (incl - cnt + j < (uint32_t)kMaxRng) S.bcell[incl - cnt + j] = lo + j;
+                uint32_t at = incl - cnt;
+                for (uint32_t c = rg.x; c < rg.y; ++c) {
+                    if (MODE == kMerge && !cells_to_join(ra, v.cell_root[c])) continue;
+                    if (at < (uint32_t)kMaxRng) S.bcell[at] = c;
+                    ++at;
+                }
                 S.bnear[tid] = 0u;
                 if (tid < 3) S.la[tid] = 0u;
                 if (tid == 0) {
@@ -635,7 +639,6 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
                 if (warp == 0) {
                     uint32_t q0 = 0, len = 0;
                     bool keep = tid < (int)nbc && S.bnear[tid];
-                    if (MODE == kMerge && keep) keep = cells_to_join(v.cell_root[A], v.cell_root[S.bcell[tid]]);
                     if (keep) {
                         const uint32_t c = S.bcell[tid];
                         q0 = tt.cx[v.cell_start[c]];
@@ -819,7 +822,7 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
             ++n_tiles;
             if (tid == 0) n_pairs += (unsigned long long)min((uint32_t)kTile, rend - k0) * nq;
             bool need = have && (MODE != kCount || (!done && ub >= from));
-            if (MODE == kCount && __any_sync(0xffffffffu, need)) {
+            if (__any_sync(0xffffffffu, need)) {
                 // 64 columns per wait, the second 32 read even past nq (allocated columns; an empty
                 // candidate's value is below every threshold)
                 uint32_t in_m[4] = {0u, 0u, 0u, 0u}, near_m[4] = {0u, 0u, 0u, 0u};
@@ -835,69 +838,56 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
                     classify32(dv[0], rt, in_m[c], near_m[c]);
                     classify32(dv[1], rt, in_m[c + 1], near_m[c + 1]);
                 }
-                uint32_t m_in = 0, found = 0;
+                if (MODE == kCount) {
+                    uint32_t m_in = 0, found = 0;
 #pragma unroll
-                for (int c = 0; c < 4; ++c) {
-                    m_in += (uint32_t)__popc(in_m[c]);
-                    found += (uint32_t)__popc(in_m[c] | near_m[c]);
-                }
-                if (need && found) {
-                    // cnt: pairs surely within eps; cnt_hi: pairs not proved outside, which take the
-                    // next entries of the list
-                    uint32_t at = recount ? atomicAdd(tt.rc_hi + rk, found) : cnt_hi;
-                    cnt += m_in;
-                    cnt_hi += found;
-                    // (one loop over the 128 columns: its trip count is the most hits of a lane)
-                    unsigned long long m0 = (unsigned long long)(in_m[1] | near_m[1]) << 32 | in_m[0] | near_m[0];
-                    unsigned long long m1 = (unsigned long long)(in_m[3] | near_m[3]) << 32 | in_m[2] | near_m[2];
-                    const unsigned long long n0 = (unsigned long long)near_m[1] << 32 | near_m[0];
-                    const unsigned long long n1 = (unsigned long long)near_m[3] << 32 | near_m[2];
-                    for (; at < v.nl_k && (m0 | m1); ++at) {
-                        const bool low = m0 != 0ull;
-                        const unsigned long long m = low ? m0 : m1, n = low ? n0 : n1;
-                        const int j = __ffsll((long long)m) - 1;
-                        if (low) m0 &= m0 - 1ull;
-                        else m1 &= m1 - 1ull;
-                        v.nl[(uint64_t)p * v.nl_k + at] = S.cidx[j + (low ? 0 : 64)] | ((n >> j) & 1ull ? kListNear : 0u);
+                    for (int c = 0; c < 4; ++c) {
+                        m_in += (uint32_t)__popc(in_m[c]);
+                        found += (uint32_t)__popc(in_m[c] | near_m[c]);
                     }
-                }
-            }
-            if (MODE != kCount && __any_sync(0xffffffffu, need)) {
-                // labels: 64 columns per wait; unions: 32 (the registers of a second set slowed the
-                // union-find loop)
-                constexpr int NH = MODE == kMerge ? 1 : 2;
-                for (uint32_t c0 = 0; c0 < nq; c0 += 32u * NH) {
-                    __syncwarp();
-                    uint32_t dv[NH][32];
-                    tmem_ld32_issue(t_lane + c0, dv[0]);
-                    if (NH == 2) tmem_ld32_issue(t_lane + c0 + 32, dv[NH - 1]);
-                    tmem_ld_wait(dv[0]);
-                    if (NH == 2) reg_tie(dv[NH - 1]);
+                    if (need && found) {
+                        // cnt: pairs surely within eps; cnt_hi: pairs not proved outside, which take
+                        // the next entries of the list
+                        uint32_t at = recount ? atomicAdd(tt.rc_hi + rk, found) : cnt_hi;
+                        cnt += m_in;
+                        cnt_hi += found;
+                        // (one loop over the 128 columns: its trip count is the most hits of a lane)
+                        unsigned long long m0 = (unsigned long long)(in_m[1] | near_m[1]) << 32 | in_m[0] | near_m[0];
+                        unsigned long long m1 = (unsigned long long)(in_m[3] | near_m[3]) << 32 | in_m[2] | near_m[2];
+                        const unsigned long long n0 = (unsigned long long)near_m[1] << 32 | near_m[0];
+                        const unsigned long long n1 = (unsigned long long)near_m[3] << 32 | near_m[2];
+                        for (; at < v.nl_k && (m0 | m1); ++at) {
+                            const bool low = m0 != 0ull;
+                            const unsigned long long m = low ? m0 : m1, n = low ? n0 : n1;
+                            const int j = __ffsll((long long)m) - 1;
+                            if (low) m0 &= m0 - 1ull;
+                            else m1 &= m1 - 1ull;
+                            v.nl[(uint64_t)p * v.nl_k + at] = S.cidx[j + (low ? 0 : 64)] | ((n >> j) & 1ull ? kListNear : 0u);
+                        }
+                    }
+                } else if (need) {
 #pragma unroll
-                    for (int h = 0; h < NH; ++h) {
-                        const uint32_t cg = c0 + 32u * (uint32_t)h;
-                        if (cg >= nq) break;
-                        uint32_t in_m, near_m;
-                        classify32(dv[h], rt, in_m, near_m);
-                        uint32_t m = need ? in_m | near_m : 0u;  // near: decided by the exact predicate
-                        // candidates sharing the row's tree node need no test; nor do ids
-                        // that cannot lower the row's label
+                    for (int c = 0; c < 4; ++c) {
+                        uint32_t m = in_m[c] | near_m[c];  // near: decided by the exact predicate
+                        if (!m) continue;
+                        // candidates sharing the row's tree node need no test; nor do ids that cannot
+                        // lower the row's label
                         if (MODE == kMerge) {
-                            // (a tile of two clusters' points has hundreds of pairs inside
-                            // either tree: one comparison per node drops them, where the loop
-                            // below took 10 us a tile)
+                            // (a tile of two clusters' points has hundreds of pairs inside either
+                            // tree: one comparison per node drops them, where the loop below took
+                            // 10 us a tile)
 #pragma unroll
                             for (int k2 = 0; k2 < 4; ++k2) {
-                                const uint2 gr = S.groot[cg >> 5][k2];
+                                const uint2 gr = S.groot[c][k2];
                                 if (gr.x == rp) m &= ~gr.y;
                             }
                         }
-                        if (MODE == kLabels && S.gsum[cg >> 5] >= best) m = 0;
+                        if (MODE == kLabels && S.gsum[c] >= best) m = 0;
                         while (m) {
                             const int j = __ffs(m) - 1;
                             m &= m - 1;
-                            const uint32_t col = cg + (uint32_t)j;
-                            const bool inside = (in_m >> j) & 1u;
+                            const uint32_t col = 32u * c + (uint32_t)j;
+                            const bool inside = (in_m[c] >> j) & 1u;
                             const uint32_t ck2 = S.cidx[col];
                             if (MODE == kMerge) {
                                 if (ck2 <= rk || S.cpay[col] == rp) continue;
