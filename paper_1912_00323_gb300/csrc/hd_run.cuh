@@ -528,16 +528,12 @@ int run_hd(const RunArgs &a) {
     cudaMemsetAsync(ctr, 0, o_mm + sizeof(unsigned long long) * 128 - o_ctr, s);  // (mm follows the counters)
     if (!batched) {
         launch(k_minmax_rt<T>, grid_for(n * d, 256, sms, 8), 256, 0, s, (const T *)a.d_points, n, d, ctr, mm);
-        if (!boxed) cudaMemcpyAsync(hmm.data(), mm, sizeof(unsigned long long) * 128, cudaMemcpyDeviceToHost, s);
     } else {
         cudaMemsetAsync(d_smm, 0, sizeof(unsigned long long) * 2 * 64 * nsets, s);
         upload(d_setoff, a.h_off, sizeof(int64_t) * (nsets + 1), stage_setoff);
         launch(k_minmax_rt_seg<T>, grid_for(n, 256, sms, 8), 256, 0, s, (const T *)a.d_points, n, d, d_setoff, nsets,
                                                                    d_smm, ctr);
-        if (!boxed) {
-            smm.resize((size_t)2 * 64 * nsets);
-            cudaMemcpyAsync(smm.data(), d_smm, sizeof(unsigned long long) * smm.size(), cudaMemcpyDeviceToHost, s);
-        }
+        if (!boxed) smm.resize((size_t)2 * 64 * nsets);
     }
     ++launches;
     if (boxed) {
@@ -551,8 +547,15 @@ int run_hd(const RunArgs &a) {
         launch(k_box_check_hd, grid_for((int64_t)nsets * d, 256, sms, 1), 256, 0, s, d_box, nsets, d, batched ? d_setoff : nullptr, batched ? d_smm : mm, ctr);
         ++launches;
     } else {
-        if (cudaMemcpyAsync(h, ctr, kCountersRead, cudaMemcpyDeviceToHost, s) != cudaSuccess ||
-            cudaStreamSynchronize(s) != cudaSuccess) { rc = HCA_ECUDA; goto out; }
+        // the extents come with the counters when they fit the mailbox
+        std::vector<unsigned long long> &ext = batched ? smm : hmm;
+        const void *d_ext = batched ? (const void *)d_smm : (const void *)mm;
+        const bool fits = ext.size() <= kMailExt;
+        if (!mail_read(s, host_mail(), ctr, d_ext, fits ? sizeof(uint64_t) * ext.size() : 0) ||
+            (!fits && cudaMemcpyAsync(ext.data(), d_ext, sizeof(uint64_t) * ext.size(), cudaMemcpyDeviceToHost, s) != cudaSuccess) ||
+            (!fits && cudaStreamSynchronize(s) != cudaSuccess)) { rc = HCA_ECUDA; goto out; }
+        ++launches;
+        if (fits) memcpy(ext.data(), host_mail()->ext, sizeof(uint64_t) * ext.size());
         if (h->nan_seen) { rc = HCA_EINVAL; goto out; }
         if (a.ext_out && !batched)
             for (int i = 0; i < d; ++i) {
@@ -713,14 +716,18 @@ int run_hd(const RunArgs &a) {
         else run_cuda_phases<T, DP, false>(hv, L, mark, launches);
     }
     if (cudaGetLastError() != cudaSuccess) { rc = HCA_ECUDA; goto out; }
-    if (cudaMemcpyAsync(h, ctr, kCountersRead, cudaMemcpyDeviceToHost, s) != cudaSuccess) {
-        rc = HCA_ECUDA;
+    if (a.deferred) {  // the caller synchronises and reads the status from h
+        if (cudaMemcpyAsync(h, ctr, kCountersRead, cudaMemcpyDeviceToHost, s) != cudaSuccess) rc = HCA_ECUDA;
+        else {
+            if (a.launches_out) *a.launches_out = launches;
+            if (a.key_bits_out) *a.key_bits_out = sort_bits;
+        }
         goto out;
     }
+    ++launches;
     if (a.launches_out) *a.launches_out = launches;
     if (a.key_bits_out) *a.key_bits_out = sort_bits;
-    if (a.deferred) goto out;  // the caller synchronises and reads the status from h
-    if (cudaStreamSynchronize(s) != cudaSuccess) { rc = HCA_ECUDA; goto out; }
+    if (!mail_read(s, host_mail(), ctr, nullptr, 0) || (timing && cudaStreamSynchronize(s) != cudaSuccess)) { rc = HCA_ECUDA; goto out; }
     if (boxed && h->nan_seen) { rc = HCA_EINVAL; goto out; }
     if (h->status) { rc = (h->status & kErrBox) ? HCA_ERANGE : HCA_EDEVICE; goto out; }
     if (a.stats) {
