@@ -180,8 +180,10 @@ constexpr int kSortMaxPasses = 8;
 constexpr int sort_items_for(int64_t n) {
     return n <= 150 * kSortThreads * 2 ? 2 : n <= 150 * kSortThreads * 4 ? 4 : n <= 150 * kSortThreads * 8 ? 8 : 13;
 }
+// Threads of a tile: half as many, two tiles on an SM at a time, for more than four million keys.
+constexpr int sort_threads_for(int64_t n) { return n > 4000000 ? kSortThreads / 2 : kSortThreads; }
 constexpr int64_t sort_tiles_for(int64_t n) {
-    const int64_t tile = (int64_t)sort_items_for(n) * kSortThreads;
+    const int64_t tile = (int64_t)sort_items_for(n) * sort_threads_for(n);
     return n <= tile ? 1 : (n + tile - 1) / tile;
 }
 constexpr size_t sort_hist_elems(int64_t n) {

@@ -3,9 +3,9 @@
 // A first kernel counts the digits of every pass over all keys (the counts do not depend on
 // the order, so one read of the keys serves all passes); a caller that produced the keys may
 // pass these counts in instead.  Each pass kernel then takes a tile of 1024 threads x 2, 4, 8
-// or 13 keys (sort_items_for), ranks every key stably among the keys of its tile with the same digit (the
-// lanes of a warp with one digit found by a match instruction or by shared-memory OR masks,
-// per-warp digit counters, an exclusive scan across warps), publishes the tile's digit
+// or 13 keys or 512 threads x 13 keys (sort_items_for, sort_threads_for), ranks every key stably
+// among the keys of its tile with the same digit (the lanes of a warp with one digit found by a
+// match instruction or by shared-memory OR masks, per-warp digit counters, an exclusive scan across warps), publishes the tile's digit
 // counts, scatters the tile through shared memory in digit order, learns how many keys of each
 // digit the earlier tiles hold by decoupled look-back, and writes the digit runs out with
 // coalesced stores.
@@ -14,11 +14,21 @@
 // million keys the ~150 tiles of 13,312 all run at once.  A smaller sort takes smaller tiles, so
 // that it spreads over as many SMs and each ranks fewer keys in turn: four passes over 300,001
 // keys 70 -> 46 us, two over 10,000 28 -> 19 us (one tile of 13,312 before).  Two CTAs of 512
-// threads per SM instead were slower (two million keys 76 -> 109 us).  With every tile running together a published
+// threads per SM instead were slower (two million keys 76 -> 109 us); above four million keys, with
+// many tiles per SM, one of the two loads or stores while the other ranks (five passes over 64-bit
+// keys: 3.4 million 186 -> 191 us, five million 273 -> 261, 16 million 759 -> 734).  With every tile running together a published
 // prefix reaches the later tiles only through their own reads, so the look-back reads 64
 // predecessors per round trip (four thread quarters of 16 words per digit): the last tile of
 // two million keys needs three round trips instead of the dozens that a 4096-key tile with a
 // few words per trip needed.
+//
+// A pass is bound by the wavefronts of shared memory: 13,312 keys take an SM some 37,000 cycles, 7,000
+// to rank, 5,500 to scatter, 7,000 to write out, 3,000 for the digit starts, the rest for the
+// loads and the look-back.  So whole tiles (all but the last) test no bounds, the digit's place in
+// the tile is folded into the per-warp offsets and into the global offset, and both digit scans
+// are one (16 million keys as above 786 -> 759 us; four passes over 32-bit keys, two million 70 -> 66 us,
+// 600,000 45 -> 41, 50,000 28 -> 25).  One vote per digit bit instead of the shared
+// OR was slower (759 -> 857 us).
 //
 // Up to kFullSumTiles tiles (about 3.4 million keys) a tile instead sums the published counts
 // of all earlier tiles (eight loads in flight per thread, no prefix published): with every
@@ -47,9 +57,6 @@ constexpr int kRadix = kSortRadix;
 constexpr int kMaxPasses = kSortMaxPasses;
 constexpr int kLbWords = 16;                      // predecessors per thread per round trip
 constexpr int kHistThreads = 256;
-constexpr int kSortWarps = kSortThreads / 32;
-constexpr int kQuarters = kSortThreads / kRadix;  // threads per digit in the look-back
-static_assert(kQuarters * kRadix == kSortThreads, "whole quarters of digits");
 constexpr uint32_t kSpinLimit = 1u << 24;
 // Up to this many tiles a tile sums the counts of all earlier tiles instead of the decoupled
 // look-back (at two million keys all ~150 tiles run at once, so the look-back finds no
@@ -90,9 +97,11 @@ __global__ void __launch_bounds__(kHistThreads) k_os_hist(const K *__restrict__ 
 }
 
 // Shared memory of a pass (dynamic, 16-byte aligned).
-template <typename K, int ITEMS>
+template <typename K, int ITEMS, int NT>
 struct PassSmem {
-    static constexpr int tile = ITEMS * kSortThreads;
+    // (quarters: the groups of one thread per digit, four of 1024 threads, two of 512)
+    static constexpr int tile = ITEMS * NT, kSortWarps = NT / 32, kQuarters = NT / kRadix;
+    static_assert(kQuarters * kRadix == NT, "whole groups of digits");
     uint32_t whist[kSortWarps][kRadix];       // per-warp digit counts, then per-warp digit offsets
     uint32_t part[kQuarters][kRadix];     // counts of a quarter's warps, per digit
     uint32_t lstart[kRadix];                // first position of each digit in the tile
@@ -101,6 +110,7 @@ struct PassSmem {
     uint32_t lb_used[kQuarters][kRadix];  // predecessors the quarter consumed
     uint32_t lb_kind[kQuarters][kRadix];  // 0 window read through, 1 met a PREFIX, 2 met an unpublished word
     int32_t lb_next[kRadix];                // nearest predecessor not yet added, per digit (-1: done)
+    uint2 wsum[kRadix / 32];                // digit starts: the warps' sums of the tile's and all counts
     uint32_t tile_id, pad[3];
     union {
         uint32_t wmask[kSortWarps][kRadix];   // ranking: per-warp lane masks of each digit
@@ -112,20 +122,21 @@ struct PassSmem {
 // One pass: rank within the tile, publish the tile's digit counts, scatter the tile into
 // shared memory in digit order, look back for the counts of the earlier tiles, write out.
 // IDENT: the values are the positions (first pass of a sort of indices; vals_in is not read).
-template <typename K, int ITEMS, bool IDENT>
-__global__ void __launch_bounds__(kSortThreads, 1) k_os_pass(
+template <typename K, int ITEMS, int NT, bool IDENT>
+__global__ void __launch_bounds__(NT, kSortThreads / NT) k_os_pass(
     const K *__restrict__ keys_in, const uint32_t *__restrict__ vals_in, K *__restrict__ keys_out,
     uint32_t *__restrict__ vals_out, int64_t n, int shift, int mask_bits,
     const uint32_t *__restrict__ ghist_pass, unsigned long long *status, uint32_t *ticket, uint32_t epoch,
     uint32_t *err, bool full_sum) {
     pdl_enter();
-    constexpr int kSortItems = ITEMS, kSortTile = ITEMS * kSortThreads;
+    constexpr int kSortItems = ITEMS, kSortTile = ITEMS * NT;
+    constexpr int kSortWarps = NT / 32, kQuarters = NT / kRadix;
     extern __shared__ __align__(16) unsigned char sm_raw[];
-    PassSmem<K, ITEMS> &S = *reinterpret_cast<PassSmem<K, ITEMS> *>(sm_raw);
+    PassSmem<K, ITEMS, NT> &S = *reinterpret_cast<PassSmem<K, ITEMS, NT> *>(sm_raw);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int dg = threadIdx.x & (kRadix - 1), q = threadIdx.x / kRadix;
     const uint32_t mask = (1u << mask_bits) - 1u;
-    for (int i = threadIdx.x; i < kSortWarps * kRadix; i += kSortThreads) {
+    for (int i = threadIdx.x; i < kSortWarps * kRadix; i += NT) {
         (&S.whist[0][0])[i] = 0;
         (&S.wmask[0][0])[i] = 0;
     }
@@ -135,45 +146,69 @@ __global__ void __launch_bounds__(kSortThreads, 1) k_os_pass(
 
     const int64_t tbase = (int64_t)tile * kSortTile;
     const int64_t wbase = tbase + (int64_t)warp * (32 * kSortItems);
+    const bool full = tbase + kSortTile <= n;  // every tile but the last
+    const uint32_t tile_count = full ? (uint32_t)kSortTile : (uint32_t)(n - tbase);
+    const uint32_t gcount = q == 0 ? ghist_pass[dg] : 0u;
     K k[kSortItems];
     uint32_t v[kSortItems];
     uint32_t rank2[(kSortItems + 1) / 2];  // rank within the warp's digit run, two 16-bit ranks per word
     static_assert(32 * kSortItems < 65536, "16-bit ranks");
+    const K *kin = keys_in + wbase + lane;
+    const uint32_t *vin = vals_in + wbase + lane;
+    const int left = full ? kSortTile : (int)(n - tbase) - warp * (32 * kSortItems);  // from the warp's first key
+    auto load = [&](auto whole) {
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
-        const int64_t i = wbase + r * 32 + lane;
-        k[r] = i < n ? keys_in[i] : K(0);
-    }
-    // ranks within the warp; the values are loaded meanwhile (needed only for the scatter)
+        for (int r = 0; r < kSortItems; ++r) k[r] = decltype(whole)::value || r * 32 + lane < left ? kin[r * 32] : K(0);
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
-        const int64_t i = wbase + r * 32 + lane;
-        const bool valid = i < n;
-        v[r] = IDENT ? (uint32_t)i : valid ? vals_in[i] : 0u;
-        const uint32_t d = valid ? ((uint32_t)(k[r] >> shift) & mask) : (uint32_t)kRadix;
-        // the lanes holding the same digit: a match instruction when lane 0's digit recurs
-        // often (few distinct digits), else one shared-memory OR per lane into the warp's
-        // digit masks (many distinct digits, where the match instruction is slow)
-        const uint32_t d0 = __shfl_sync(0xffffffffu, d, 0);
-        const bool use_match = __popc(__ballot_sync(0xffffffffu, d == d0)) >= 4;
-        unsigned peers = 0u;
-        if (use_match) {
-            peers = __match_any_sync(0xffffffffu, d);
-        } else {
-            if (valid) atomicOr(&S.wmask[warp][d], 1u << lane);
+        for (int r = 0; r < kSortItems; ++r)
+            v[r] = IDENT ? (uint32_t)(wbase + r * 32 + lane)
+                         : decltype(whole)::value || r * 32 + lane < left ? vin[r * 32] : 0u;
+    };
+    if (full) load(std::true_type());
+    else load(std::false_type());
+    // ranks within the warp: the lanes holding the same digit by a match instruction when a digit
+    // recurs often (few distinct digits; judged by the first and the last keys), else by one
+    // shared-memory OR per lane into the warp's digit masks (many distinct digits, where the
+    // match instruction is slow)
+    uint32_t *const wh = S.whist[warp], *const wm = S.wmask[warp];
+    const uint32_t below = (1u << lane) - 1u;
+    auto rank = [&](auto whole, auto by_match) {
+        constexpr bool WHOLE = decltype(whole)::value, MATCH = decltype(by_match)::value;
+#pragma unroll
+        for (int r = 0; r < kSortItems; ++r) {
+            const bool valid = WHOLE || r * 32 + lane < left;
+            const uint32_t d = (uint32_t)(k[r] >> shift) & mask;
+            unsigned peers = 0u;
+            if (MATCH) {
+                peers = __match_any_sync(0xffffffffu, valid ? d : (uint32_t)kRadix);
+            } else {
+                if (valid) atomicOr(wm + d, 1u << lane);
+                __syncwarp();
+                if (valid) peers = wm[d];
+            }
+            const uint32_t before = valid ? wh[d] : 0u;
+            const uint32_t lower = peers & below;
             __syncwarp();
-            if (valid) peers = S.wmask[warp][d];
+            if (valid && lower == 0u) {
+                wh[d] = before + __popc(peers);
+                if (!MATCH) wm[d] = 0u;  // clean for the next key
+            }
+            __syncwarp();
+            const uint32_t rk = before + __popc(lower);
+            if (r & 1) rank2[r >> 1] |= rk << 16;
+            else rank2[r >> 1] = rk;
         }
-        const uint32_t before = valid ? S.whist[warp][d] : 0u;
-        __syncwarp();
-        if (valid && lane == __ffs(peers) - 1) {
-            S.whist[warp][d] = before + __popc(peers);
-            if (!use_match) S.wmask[warp][d] = 0u;  // clean for the next key
+    };
+    {
+        const uint32_t d0 = (uint32_t)(k[0] >> shift) & mask, d1 = (uint32_t)(k[kSortItems - 1] >> shift) & mask;
+        const int same = __popc(__ballot_sync(0xffffffffu, d0 == __shfl_sync(0xffffffffu, d0, 0))) +
+                         __popc(__ballot_sync(0xffffffffu, d1 == __shfl_sync(0xffffffffu, d1, 0)));
+        if (full) {
+            if (same >= 8) rank(std::true_type(), std::true_type());
+            else rank(std::true_type(), std::false_type());
+        } else {
+            rank(std::false_type(), std::true_type());
         }
-        __syncwarp();
-        const uint32_t rk = before + __popc(peers & ((1u << lane) - 1u));
-        if (r & 1) rank2[r >> 1] |= rk << 16;
-        else rank2[r >> 1] = rk;
     }
     __syncthreads();
     // per digit: the count of each quarter's eight warps, then per-warp exclusive offsets
@@ -184,46 +219,58 @@ __global__ void __launch_bounds__(kSortThreads, 1) k_os_pass(
         S.part[q][dg] = c;
     }
     __syncthreads();
-    uint32_t count = 0;  // the tile's count of digit dg
-    {
-        uint32_t base = 0;
+    uint32_t count = 0, base = 0;  // the tile's count of digit dg; that of the quarters before q
 #pragma unroll
-        for (int qq = 0; qq < kQuarters; ++qq) {
-            const uint32_t c = S.part[qq][dg];
-            base += qq < q ? c : 0u;
-            count += c;
-        }
-#pragma unroll
-        for (int w = 0; w < kSortWarps / kQuarters; ++w) {
-            uint32_t &h = S.whist[q * (kSortWarps / kQuarters) + w][dg];
-            const uint32_t t = h;
-            h = base;
-            base += t;
-        }
+    for (int qq = 0; qq < kQuarters; ++qq) {
+        const uint32_t c = S.part[qq][dg];
+        base += qq < q ? c : 0u;
+        count += c;
     }
     // publish this tile's count of the digit at once, so later tiles can read past it
     volatile unsigned long long *st = status;
     if (q == 0) st[(uint64_t)tile * kRadix + dg] = os_pack(epoch, tile == 0 ? kStatePrefix : kStateAgg, count);
     // local and global digit starts (the global one from the pass's digit counts)
-    uint32_t tile_count, total_unused;
-    const uint32_t lst = block_exclusive_scan<kSortThreads>(q == 0 ? count : 0u, &tile_count);
-    const uint32_t gdig = block_exclusive_scan<kSortThreads>(q == 0 ? ghist_pass[dg] : 0u, &total_unused);
+    uint32_t lst = 0, gdig = 0;
+    if (q == 0) {  // the first eight warps
+        lst = warp_inclusive_scan(count);
+        gdig = warp_inclusive_scan(gcount);
+        if (lane == 31) S.wsum[warp] = make_uint2(lst, gdig);
+        lst -= count;
+        gdig -= gcount;
+    }
+    __syncthreads();
     if (q == 0) {
+        for (int w = 0; w < warp; ++w) {
+            lst += S.wsum[w].x;
+            gdig += S.wsum[w].y;
+        }
         S.lstart[dg] = lst;
         S.lb_next[dg] = (int32_t)tile - 1;
     }
     __syncthreads();
-    // the tile in digit order in shared memory (frees the key registers before the look-back)
+    // per warp and digit: the place in the tile of the warp's first key of that digit
+    base += S.lstart[dg];
 #pragma unroll
-    for (int r = 0; r < kSortItems; ++r) {
-        const int64_t i = wbase + r * 32 + lane;
-        if (i < n) {
+    for (int w = 0; w < kSortWarps / kQuarters; ++w) {
+        uint32_t &h = S.whist[q * (kSortWarps / kQuarters) + w][dg];
+        const uint32_t t = h;
+        h = base;
+        base += t;
+    }
+    __syncthreads();
+    // the tile in digit order in shared memory (frees the key registers before the look-back)
+    auto scatter = [&](auto whole) {
+#pragma unroll
+        for (int r = 0; r < kSortItems; ++r) {
+            if (!decltype(whole)::value && r * 32 + lane >= left) continue;
             const uint32_t d = (uint32_t)(k[r] >> shift) & mask;
-            const uint32_t lpos = S.lstart[d] + S.whist[warp][d] + ((rank2[r >> 1] >> (16 * (r & 1))) & 0xffffu);
+            const uint32_t lpos = wh[d] + ((rank2[r >> 1] >> (16 * (r & 1))) & 0xffffu);
             S.keys[lpos] = k[r];
             S.vals[lpos] = v[r];
         }
-    }
+    };
+    if (full) scatter(std::true_type());
+    else scatter(std::false_type());
     // decoupled look-back over the earlier tiles: per round trip, quarter q of digit dg reads
     // the 16 predecessors [j - 16 q - 15, j - 16 q] (j = nearest not yet added), adds the AGG
     // counts from its nearest down to the first PREFIX (included) or unpublished word
@@ -312,36 +359,41 @@ __global__ void __launch_bounds__(kSortThreads, 1) k_os_pass(
     }
     if (q == 0) {
         if (tile > 0 && !full_sum) st[(uint64_t)tile * kRadix + dg] = os_pack(epoch, kStatePrefix, excl + count);
-        S.goff[dg] = gdig + excl;
+        S.goff[dg] = gdig + excl - lst;  // (plus the place in the tile; modulo 2^32)
     }
     __syncthreads();
-    for (uint32_t i = threadIdx.x; i < tile_count; i += kSortThreads) {
+    auto put = [&](uint32_t i) {
         const K key = S.keys[i];
-        const uint32_t d = (uint32_t)(key >> shift) & mask;
-        const uint32_t gpos = S.goff[d] + (i - S.lstart[d]);
+        const uint32_t gpos = S.goff[(uint32_t)(key >> shift) & mask] + i;
         keys_out[gpos] = key;
         vals_out[gpos] = S.vals[i];
+    };
+    if (full) {
+#pragma unroll
+        for (int r = 0; r < kSortItems; ++r) put(r * NT + threadIdx.x);
+    } else {
+        for (uint32_t i = threadIdx.x; i < tile_count; i += NT) put(i);
     }
 }
 
 // The passes of one sort.
-template <typename K, int ITEMS>
+template <typename K, int ITEMS, int NT>
 bool run_passes(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, int64_t n, int begin_bit, int end_bit,
                 const uint32_t *ghist, unsigned long long *status, uint32_t *tickets, uint32_t *err, bool identity,
                 Lane s) {
-    const int nb = (int)((n + (int64_t)ITEMS * kSortThreads - 1) / ((int64_t)ITEMS * kSortThreads));
+    const int nb = (int)((n + (int64_t)ITEMS * NT - 1) / ((int64_t)ITEMS * NT));
     const int passes = (end_bit - begin_bit + 7) / 8;
-    const size_t smem = sizeof(PassSmem<K, ITEMS>);
-    cudaFuncSetAttribute(k_os_pass<K, ITEMS, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    cudaFuncSetAttribute(k_os_pass<K, ITEMS, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    const size_t smem = sizeof(PassSmem<K, ITEMS, NT>);
+    cudaFuncSetAttribute(k_os_pass<K, ITEMS, NT, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaFuncSetAttribute(k_os_pass<K, ITEMS, NT, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     bool flipped = false;
     K *kin = keys, *kout = keys_alt;
     uint32_t *vin = vals, *vout = vals_alt;
     for (int p = 0; p < passes; ++p) {
         const int shift = begin_bit + 8 * p;
         const int bits = (end_bit - shift) < 8 ? (end_bit - shift) : 8;
-        auto kern = p == 0 && identity ? k_os_pass<K, ITEMS, true> : k_os_pass<K, ITEMS, false>;
-        launch(kern, nb, kSortThreads, smem, s, kin, vin, kout, vout, n, shift, bits, ghist + p * kRadix, status, tickets + p,
+        auto kern = p == 0 && identity ? k_os_pass<K, ITEMS, NT, true> : k_os_pass<K, ITEMS, NT, false>;
+        launch(kern, nb, NT, smem, s, kin, vin, kout, vout, n, shift, bits, ghist + p * kRadix, status, tickets + p,
                                             (uint32_t)(p + 1), err, nb <= kFullSumTiles);
         K *tk = kin; kin = kout; kout = tk;
         uint32_t *tv = vin; vin = vout; vout = tv;
@@ -380,16 +432,18 @@ bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, 
         if (launches) *launches += 1;
     }
     if (launches) *launches += (end_bit - begin_bit + 7) / 8;
-    auto run = [&](auto items) {
-        return run_passes<K, decltype(items)::value>(keys, vals, keys_alt, vals_alt, n, begin_bit, end_bit, ghist, status,
+    auto run = [&](auto items, auto threads) {
+        return run_passes<K, decltype(items)::value, decltype(threads)::value>(keys, vals, keys_alt, vals_alt, n, begin_bit, end_bit, ghist, status,
                                                      tickets, err, identity, s);
     };
+    const std::integral_constant<int, kSortThreads> whole;
     switch (sort_items_for(n)) {
-        case 2: return run(std::integral_constant<int, 2>());
-        case 4: return run(std::integral_constant<int, 4>());
-        case 8: return run(std::integral_constant<int, 8>());
+        case 2: return run(std::integral_constant<int, 2>(), whole);
+        case 4: return run(std::integral_constant<int, 4>(), whole);
+        case 8: return run(std::integral_constant<int, 8>(), whole);
     }
-    return run(std::integral_constant<int, 13>());
+    if (sort_threads_for(n) == kSortThreads) return run(std::integral_constant<int, 13>(), whole);
+    return run(std::integral_constant<int, 13>(), std::integral_constant<int, kSortThreads / 2>());
 }
 
 template bool radix_sort_pairs<uint32_t>(uint32_t *, uint32_t *, uint32_t *, uint32_t *, int64_t,
