@@ -46,6 +46,12 @@ struct FillList {
     uint64_t words[4];
     uint32_t value[4];
     int n;
+    // bytes set to 1 (any alignment): the core flags.  Most points are core, and their flags in the
+    // input's order are one scattered byte each; written in a stream here, only the other points'
+    // zeros are scattered later (labels stage of two million points in 3-D 50 -> 38 us, of 16 million
+    // 329 -> 248)
+    uint8_t *ones;
+    uint64_t n_ones;
     void add(void *ptr, size_t bytes, uint32_t v) {
         p[n] = (uint32_t *)ptr;
         words[n] = bytes / 4;
@@ -60,6 +66,15 @@ __device__ __forceinline__ void fill_regions(const FillList &f) {
         const uint32_t x = f.value[r];
         for (uint64_t i = t0; i < quads; i += step) reinterpret_cast<uint4 *>(f.p[r])[i] = make_uint4(x, x, x, x);
         for (uint64_t i = 4 * quads + t0; i < f.words[r]; i += step) f.p[r][i] = x;
+    }
+    if (f.ones) {
+        const uint64_t to_quad = (16u - ((uintptr_t)f.ones & 15u)) & 15u;
+        const uint64_t head = to_quad < f.n_ones ? to_quad : f.n_ones, quads = (f.n_ones - head) / 16;
+        const uint32_t x = 0x01010101u;
+        for (uint64_t i = t0; i < quads; i += step) reinterpret_cast<uint4 *>(f.ones + head)[i] = make_uint4(x, x, x, x);
+        if (t0 < head) f.ones[t0] = 1;
+        const uint64_t tail = head + 16 * quads + t0;
+        if (tail < f.n_ones) f.ones[tail] = 1;
     }
 }
 

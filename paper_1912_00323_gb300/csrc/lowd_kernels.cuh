@@ -1368,8 +1368,7 @@ __global__ void __launch_bounds__(256) k_label_core(LowdView<T, D> v) {
         const uint32_t o = v.perm[j];
         const uint32_t c = v.cell_of[j];
         const uint32_t base = v.gtab ? (uint32_t)v.set_off[set_of_key(v, v.cell_key[c])] : 0u;
-        v.labels[o] = (int32_t)(v.comp_min[v.parent[c]] - base);
-        if (v.core_out) v.core_out[o] = 1;
+        v.labels[o] = (int32_t)(v.comp_min[v.parent[c]] - base);  // (core_out: 1 already, FillList)
     }
     if (lane == 0 && ncore) atomicAdd(&v.ctr->n_core, ncore);
 }

@@ -575,6 +575,8 @@ int run_lowd(const RunArgs &a) {
         fill.add(hist, sizeof(uint32_t) * hist_elems, 0u);
         fill.add(b + o_look, look_bytes(n), 0u);
         if (ptab) fill.add(ptab, sizeof(uint32_t) << (sort_bits - g.prefix_shift), 0xffffffffu);
+        fill.ones = a.d_core;
+        fill.n_ones = a.d_core ? (uint64_t)n : 0;
         auto front = [&](auto *ka, auto *kb) {
             typedef typename std::remove_reference<decltype(*ka)>::type K;
             if (batched)

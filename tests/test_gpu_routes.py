@@ -60,3 +60,18 @@ def test_sort_tile_sizes(env, n, extent):
     got = run(env, X.astype(np.float32), 1.25, 5)
     check(got, want)
     assert (got[2]["key_bits"] > 32) == (extent > 1e5)
+
+
+@pytest.mark.parametrize("n", [1, 14, 15, 16, 17, 31, 33, 1000])
+@pytest.mark.parametrize("offset", [0, 1, 15])
+def test_core_flags_at_any_alignment(env, n, offset):
+    """Core flags are set in 16-byte stores first: unaligned starts, ragged ends, bytes around them."""
+    torch, pkg, oracle = env
+    X = clumps(n, (40.0, 40.0), seed=n)
+    want = oracle.grid(X, 1.25, 5)
+    out = torch.full((n + 48,), 7, dtype=torch.uint8, device="cuda")
+    lab = pkg.hca_dbscan_device(torch.from_numpy(X).cuda(), 1.25, 5, core=out[offset:offset + n])
+    torch.cuda.synchronize()
+    check((lab.cpu().numpy(), out[offset:offset + n].cpu().numpy()), want)
+    rest = torch.cat([out[:offset], out[offset + n:]])
+    assert bool((rest == 7).all())
