@@ -86,7 +86,7 @@ extern "C" {
 #define HCA_STAGE_BIN 1       /* hypercube coordinates and cell keys (Algorithm 1) */
 #define HCA_STAGE_SORT 2      /* radix sort of (key, index) (the pre-sort of Sec. 2) */
 #define HCA_STAGE_CELLS 3     /* gather into cell order, run-length cell offsets */
-#define HCA_STAGE_HASH 4      /* neighbour lookup table */
+#define HCA_STAGE_HASH 4      /* neighbour lookup table, neighbour cells of every cell */
 #define HCA_STAGE_CORE 5      /* dense cells and exact counts (Definition 2); d <= 4: with the
                                  chunk table of the representative pass */
 #define HCA_STAGE_REPS 6      /* representative points (Algorithm 2): the selection kernel alone */
@@ -126,7 +126,7 @@ typedef struct hca_stats {
     int64_t n_core_cells;
     /* d >= 5, float input: point pairs (valid row x valid candidate) of the tensor-core tiles
        computed, and with HCA_FLAG_TIMING the CUDA-event time of the tensor-core kernel of the
-       counts, unions and labels (one launch each) */
+       counts (with the recount), unions and labels */
     int64_t n_tc_pairs;
     float tc_ms[3];
     int32_t reserved2;
@@ -356,11 +356,11 @@ HCA_API int hca_graph_cache_release(void);
  *                  use tensor-core tiles; >= 1.
  *   tc_handoff     open rows at which a tensor-core count chunk hands them to the CUDA cores;
  *                  0..127.
- *   first_links    1: first-link pass in every coarse cell; 0: only in cells whose unions run
- *                  on the CUDA cores.
- *   cta_warps      coarse grid: warps per CTA of the CUDA-core chunk kernels (counts, first
- *                  links, unions, labels; one 32-point chunk per warp, its rows staged in the
- *                  CTA's shared memory): 2, 4 or 8.
+ *   first_links    1: the edges that the counts listed are joined before the unions in every
+ *                  coarse cell; 0: only in cells whose unions run on the CUDA cores.
+ *   cta_warps      coarse grid: warps per CTA of the CUDA-core chunk kernels (counts, odd points,
+ *                  unions, labels; one 32-point chunk per warp, its rows staged in the CTA's
+ *                  shared memory): 2, 4 or 8.
  * Defaults: path 0, tc_handoff 32, first_links 1, cta_warps 4; thresholds 16 / 1 / 4 for
  * d <= 8 and 8 / 1 / 1 for d > 8.
  */
@@ -385,7 +385,7 @@ HCA_API int hca_tuning_set(int32_t d, const hca_tuning *t);
  * (same arguments as hca_dbscan_device; the points are only read) and keep the fastest as the
  * tuning of d.  Each candidate runs once untimed and then `repeats` times (1..16) timed with CUDA
  * events on `stream`, keeping its minimum.  Candidates: both neighbour searches for d = 3, 4;
- * for the coarse grid with float input, first links on / off and several row thresholds; then,
+ * for the coarse grid with float input, first_links on / off and several row thresholds; then,
  * on the coarse grid, 2 and 8 warps per CTA (cta_warps) with the rest of the fastest of those,
  * and with float input the tensor-core handoff at 8, 16, 32 and 64 open rows (tc_handoff).
  *   out       host, nullable: the tuning kept.   best_ms  host, nullable: its time.
@@ -412,7 +412,9 @@ HCA_API int hca_autotune_batched(const void *d_points, int32_t dtype, int32_t n_
  * A batched call takes, per d group, at most this bound for the group's points plus a few
  * hundred bytes per set (more only through the power-of-two rounding of its hash table, below
  * 16 bytes per point), and a group whose sets are not consecutive also a compact copy of its
- * points, labels and core flags.  The paper has no counterpart: the request server admits jobs
+ * points, labels and core flags.  On the coarse grid up to 84 bytes per point of the bound are
+ * neighbour lists; a call that cannot get them runs without (same labels, slower).  The paper has
+ * no counterpart: the request server admits jobs
  * by this bound.  Needs no device.
  *   bytes  host, written on success.
  */

@@ -60,7 +60,7 @@ struct HdView {
     uint8_t near[16];             // the pencils nearest first (n_all of them; the coarse grid has 9)
     // cells left to the tensor-core kernels (float input): those with at least tc_min[phase] rows
     // of a phase (counts, unions, labels; 0: none); cx = exclusive scan of the core flags, for
-    // the per-cell core counts; tc_hook: first links also in cells whose unions run there
+    // the per-cell core counts; tc_hook: listed edges joined in cells whose unions run there too
     uint32_t tc_min[3];
     uint32_t tc_hook;
     uint32_t tc_handoff;  // open count rows at which a tensor-core chunk hands over

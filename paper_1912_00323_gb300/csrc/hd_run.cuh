@@ -129,8 +129,8 @@ inline int tc_launch_shape(size_t &smem) {
 }  // namespace detail
 
 // Rows of a phase (counts, unions, labels) from which a coarse cell goes to the tensor-core
-// kernels, whether the first links also run in cells whose unions are on tensor cores, and the
-// open count rows at which a tensor-core chunk hands over (from the call's hca_tuning).
+// kernels, whether the listed edges are also joined in cells whose unions are on tensor cores, and
+// the open count rows at which a tensor-core chunk hands over (from the call's hca_tuning).
 struct TcTuning {
     uint32_t min[3];
     uint32_t hook;

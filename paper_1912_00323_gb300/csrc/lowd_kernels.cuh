@@ -883,7 +883,9 @@ __global__ void __launch_bounds__(kCellBlock) k_core(LowdView<T, D> v, Stencil s
                                 partial &= partial - 1;
                                 const uint32_t ps = __shfl_sync(0xffffffffu, bs, t);
                                 const uint32_t pe = __shfl_sync(0xffffffffu, be, t);
-                                if (pe - ps <= 32) {  // most cells: one chunk
+                                // most cells: one chunk (four such cells' loads in flight together were
+                                // slower: 101 -> 119 us at two million points, for the tests past MINPTS)
+                                if (pe - ps <= 32) {
                                     const uint32_t q = ps + lane;
                                     const bool hit = q < pe && within_eps<D>(aj, v.pts[q], G);
                                     cj += __popc(__ballot_sync(0xffffffffu, hit));
@@ -1248,9 +1250,9 @@ __global__ void __launch_bounds__(256) k_flatten(LowdView<T, D> v) {
 // Algorithm 3: merge every pair of neighbouring cells that hold core points and have a core
 // pair within eps.  Each unordered pair is visited once (upper half of the stencil).  Pass 0
 // takes the cells at Chebyshev offset 1, pass 1 the rest, pass 2 all of them; a pair already in
-// one set (after the first links and pointer jumping, most pairs of a cluster) is skipped.  The complementary
-// representative points are tested first (Algorithm 3); a miss falls back to the exhaustive
-// core x core test.  Lanes walk the flattened list of candidate cells of one cell.
+// one set (after the flattened first links, most pairs of a cluster) is skipped.  The
+// complementary representative points are tested first (Algorithm 3); a miss falls back to the
+// exhaustive core x core test.  Lanes walk the flattened list of candidate cells of one cell.
 template <typename T, int D>
 __global__ void __launch_bounds__(kCellBlock) k_merge(LowdView<T, D> v, int n_all, int n_half, int pass) {
     pdl_enter();

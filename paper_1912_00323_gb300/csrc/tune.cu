@@ -18,9 +18,8 @@ std::mutex g_tune_mu;
 hca_tuning g_tune[kMaxDim + 1];
 bool g_tune_init = false;
 
-// Defaults per d: the coarse-grid split measured fastest across the workloads, with first
-// links in every cell (leaving them out of tensor-core cells wins a few percent on many small
-// sets but loses up to 8x on a set of a million points) — d <= 8: thresholds 16 / 1 / 4;
+// Defaults per d: the coarse-grid split measured fastest across the workloads, with the list
+// edges joined first in every cell — d <= 8: thresholds 16 / 1 / 4;
 // d > 8 (the 16-D anisotropic clusters): 8 / 1 / 1.  Tensor-core count chunks hand over at 32
 // open rows (the tensor-core recount takes them, in windows: against 8, 5% faster on the d = 8
 // sets of the batched workload, 7-14% on the largest d = 9 and 16 serving jobs, equal on the
