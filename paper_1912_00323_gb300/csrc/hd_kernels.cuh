@@ -888,12 +888,11 @@ __global__ void __launch_bounds__(256) k_list_link(HdView<T, DP> v) {
     }
 }
 
-// Read-only finds: parent[p] = root (nothing hooks meanwhile).
+// parent[p] = root of every core point (nothing hooks meanwhile).
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_flatten_hd(HdView<T, DP> v) {
     pdl_enter();
-    for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += (int64_t)gridDim.x * blockDim.x)
-        if (v.core[j]) v.parent[j] = uf_root_readonly(v.parent, (uint32_t)j, v.ctr);
+    uf_flatten(v.parent, v.g.n, [&](int64_t j) { return v.core[j] ? (uint32_t)j : 0xffffffffu; }, v.ctr);
 }
 
 // Four list entries of one point and its tree against theirs (k_list_hook, k_list_join): the tree

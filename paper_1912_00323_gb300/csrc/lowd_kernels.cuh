@@ -304,6 +304,40 @@ __device__ __forceinline__ uint32_t uf_root_readonly(const uint32_t *parent, uin
     return x;
 }
 
+// Moves x's parent to the grandparent, up to `steps` times or until it is a root (true).  Only x's
+// thread writes parent[x] meanwhile, always an ancestor of x, and nothing hooks.
+__device__ __forceinline__ bool uf_jump(uint32_t *parent, uint32_t x, uint32_t steps) {
+    uint32_t p = __ldcg(parent + x);
+    for (uint32_t it = 0; it < steps; ++it) {
+        const uint32_t gp = __ldcg(parent + p);
+        if (gp == p) return true;
+        __stcg(parent + x, gp);
+        p = gp;
+    }
+    return false;
+}
+
+// parent[x] = root for x = node(i), i < n (node returns ~0 for an item without one); one thread of the
+// grid calls it for each of its items.  Every thread goes round its items until all have
+// arrived, a few jumps each time, so that all nodes jump together and the distances double.  In a
+// filament the first links chain up over the whole cluster, and with each node followed to its root
+// before the next was begun a thread walked link by link over nodes that no thread had come to yet
+// (k_flatten of 2.5 million cells along a line 6.1 ms, now 1.5; calls of two million points along a
+// line 8.4 -> 4.6 ms in 3-D, of ten million in 1-D 11.4 -> 5.8; 2, 4 and 8 jumps a time are alike).
+constexpr uint32_t kJumpSteps = 4;
+template <typename F>
+__device__ __forceinline__ void uf_flatten(uint32_t *parent, int64_t n, F node, DevCounters *ctr) {
+    bool open = true;
+    for (uint32_t round = 0; open; ++round) {
+        open = false;
+        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
+            const uint32_t x = node(i);
+            if (x != 0xffffffffu && !uf_jump(parent, x, kJumpSteps)) open = true;
+        }
+        if (round > kLoopLimit) { set_error(ctr, kErrLoop); return; }
+    }
+}
+
 __device__ __forceinline__ void uf_union(uint32_t *parent, uint32_t a, uint32_t b, DevCounters *ctr) {
     for (uint32_t it = 0; it < kLoopLimit; ++it) {
         a = uf_find(parent, a, ctr);
@@ -1235,16 +1269,11 @@ __global__ void __launch_bounds__(kCellBlock) k_hook(LowdView<T, D> v, int n_all
     }
 }
 
-// The first links flattened: parent[c] = root of every cell with core points, by finds that do not
-// write on the way (nothing hooks meanwhile; the links run a few cells far).
+// The first links flattened: parent[c] = root of every cell with core points (nothing hooks meanwhile).
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_flatten(LowdView<T, D> v) {
     pdl_enter();
-    const uint32_t NL = v.ctr->n_list[1];
-    for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < NL; w += gridDim.x * blockDim.x) {
-        const uint32_t c = v.list_core[w];
-        v.parent[c] = uf_root_readonly(v.parent, c, v.ctr);
-    }
+    uf_flatten(v.parent, v.ctr->n_list[1], [&](int64_t w) { return v.list_core[w]; }, v.ctr);
 }
 
 // Algorithm 3: merge every pair of neighbouring cells that hold core points and have a core
