@@ -892,7 +892,13 @@ __global__ void __launch_bounds__(256) k_list_link(HdView<T, DP> v) {
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_flatten_hd(HdView<T, DP> v) {
     pdl_enter();
-    uf_flatten(v.parent, v.g.n, [&](int64_t j) { return v.core[j] ? (uint32_t)j : 0xffffffffu; }, v.ctr);
+    bool open = true;
+    for (uint32_t round = 0; open; ++round) {
+        open = false;
+        for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += (int64_t)gridDim.x * blockDim.x)
+            if (v.core[j] && !uf_shorten(v.parent, (uint32_t)j)) open = true;
+        if (round > kLoopLimit) { set_error(v.ctr, kErrLoop); return; }
+    }
 }
 
 // Four list entries of one point and its tree against theirs (k_list_hook, k_list_join): the tree

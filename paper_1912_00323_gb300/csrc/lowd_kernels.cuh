@@ -304,38 +304,26 @@ __device__ __forceinline__ uint32_t uf_root_readonly(const uint32_t *parent, uin
     return x;
 }
 
-// Moves x's parent to the grandparent, up to `steps` times or until it is a root (true).  Only x's
-// thread writes parent[x] meanwhile, always an ancestor of x, and nothing hooks.
-__device__ __forceinline__ bool uf_jump(uint32_t *parent, uint32_t x, uint32_t steps) {
-    uint32_t p = __ldcg(parent + x);
-    for (uint32_t it = 0; it < steps; ++it) {
-        const uint32_t gp = __ldcg(parent + p);
-        if (gp == p) return true;
-        __stcg(parent + x, gp);
-        p = gp;
+// Flattening of a forest that nothing hooks meanwhile: the thread of node x walks up to kWalkSteps links
+// up and leaves parent[x] there (only it writes parent[x], always an ancestor of x); true at a root.
+// A kernel whose threads go round their nodes until all have arrived lets the links of all nodes grow
+// by that factor a turn.  In a filament the first links chain up over the whole cluster, and with
+// each node followed to its root before the next was begun a thread walked link by link over
+// nodes that no thread had come to yet (two million points along a line in 3-D 8.4 ms a call, now
+// 4.5; ten million in 1-D 11.4, now 5.3).  Most nodes arrive in the first turn with one write; a
+// write per link (jumps to the grandparent) made that turn wait for the writes (k_flatten of
+// the 3-D benchmark cloud 16 -> 50 us).
+constexpr uint32_t kWalkSteps = 64;
+__device__ __forceinline__ bool uf_shorten(uint32_t *parent, uint32_t x) {
+    uint32_t y = x, p = __ldcg(parent + x), it = 0;
+    bool root = true;
+    while (p != y) {
+        y = p;
+        p = __ldcg(parent + y);
+        if (++it > kWalkSteps) { root = false; break; }
     }
-    return false;
-}
-
-// parent[x] = root for x = node(i), i < n (node returns ~0 for an item without one); one thread of the
-// grid calls it for each of its items.  Every thread goes round its items until all have
-// arrived, a few jumps each time, so that all nodes jump together and the distances double.  In a
-// filament the first links chain up over the whole cluster, and with each node followed to its root
-// before the next was begun a thread walked link by link over nodes that no thread had come to yet
-// (k_flatten of 2.5 million cells along a line 6.1 ms, now 1.5; calls of two million points along a
-// line 8.4 -> 4.6 ms in 3-D, of ten million in 1-D 11.4 -> 5.8; 2, 4 and 8 jumps a time are alike).
-constexpr uint32_t kJumpSteps = 4;
-template <typename F>
-__device__ __forceinline__ void uf_flatten(uint32_t *parent, int64_t n, F node, DevCounters *ctr) {
-    bool open = true;
-    for (uint32_t round = 0; open; ++round) {
-        open = false;
-        for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-            const uint32_t x = node(i);
-            if (x != 0xffffffffu && !uf_jump(parent, x, kJumpSteps)) open = true;
-        }
-        if (round > kLoopLimit) { set_error(ctr, kErrLoop); return; }
-    }
+    parent[x] = p;
+    return root;
 }
 
 __device__ __forceinline__ void uf_union(uint32_t *parent, uint32_t a, uint32_t b, DevCounters *ctr) {
@@ -1273,7 +1261,14 @@ __global__ void __launch_bounds__(kCellBlock) k_hook(LowdView<T, D> v, int n_all
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_flatten(LowdView<T, D> v) {
     pdl_enter();
-    uf_flatten(v.parent, v.ctr->n_list[1], [&](int64_t w) { return v.list_core[w]; }, v.ctr);
+    const uint32_t NL = v.ctr->n_list[1];
+    bool open = true;
+    for (uint32_t round = 0; open; ++round) {
+        open = false;
+        for (uint32_t w = blockIdx.x * blockDim.x + threadIdx.x; w < NL; w += gridDim.x * blockDim.x)
+            if (!uf_shorten(v.parent, v.list_core[w])) open = true;
+        if (round > kLoopLimit) { set_error(v.ctr, kErrLoop); return; }
+    }
 }
 
 // Algorithm 3: merge every pair of neighbouring cells that hold core points and have a core
