@@ -171,8 +171,8 @@ __device__ __forceinline__ bool box_far(const float *a, const float *lo, const f
 #pragma unroll
     for (int i = 0; i < DP; i += 4) {
         const float4 av = *reinterpret_cast<const float4 *>(a + i);
-        const float4 l = __ldg(reinterpret_cast<const float4 *>(lo + i));
-        const float4 h = __ldg(reinterpret_cast<const float4 *>(hi + i));
+        const float4 l = ld(reinterpret_cast<const float4 *>(lo + i));
+        const float4 h = ld(reinterpret_cast<const float4 *>(hi + i));
         float t = fmaxf(fmaxf(__fsub_rn(l.x, av.x), __fsub_rn(av.x, h.x)), 0.f); s = __fmaf_rn(t, t, s);
         t = fmaxf(fmaxf(__fsub_rn(l.y, av.y), __fsub_rn(av.y, h.y)), 0.f);       s = __fmaf_rn(t, t, s);
         t = fmaxf(fmaxf(__fsub_rn(l.z, av.z), __fsub_rn(av.z, h.z)), 0.f);       s = __fmaf_rn(t, t, s);
@@ -185,7 +185,7 @@ __device__ __forceinline__ bool box_far(const double *a, const double *lo, const
     double s = 0.0;
 #pragma unroll
     for (int i = 0; i < DP; ++i) {
-        const double t = fmax(fmax(__dsub_rn(__ldg(lo + i), a[i]), __dsub_rn(a[i], __ldg(hi + i))), 0.0);
+        const double t = fmax(fmax(__dsub_rn(ld(lo + i), a[i]), __dsub_rn(a[i], ld(hi + i))), 0.0);
         s = __fma_rn(t, t, s);
     }
     return s > g.eps2 * (1.0 + 0x1p-40);
@@ -217,7 +217,7 @@ __device__ __noinline__ bool hd_exact(const T *pts, uint32_t i, uint32_t j, doub
     double e = 0.0;
 #pragma unroll 4
     for (int k = 0; k < DP; ++k) {
-        const double t = __dsub_rn((double)__ldg(a + k), (double)__ldg(b + k));
+        const double t = __dsub_rn((double)ld_old(a + k), (double)ld_old(b + k));
         e = __dadd_rn(e, __dmul_rn(t, t));
     }
     return e <= eps2;
@@ -243,7 +243,7 @@ struct Candidate<T, DP, true> {
 #pragma unroll
         for (int i = 0; i < DP / 4; ++i) {
             if (4 * i >= v.d) break;
-            const ulonglong2 x = __ldg(p + i);
+            const ulonglong2 x = ld_old(p + i);
             q[2 * i] = x.x;
             q[2 * i + 1] = x.y;
         }
@@ -297,9 +297,9 @@ __device__ __forceinline__ bool cell_far(const HdView<double, DP> &v, const type
 // Declared extents of a plan against the measured ones (complement of the encoded min of dimension
 // i of set s at mm[s * 64 + i], encoded max at mm[(nsets + s) * 64 + i]; boxes: mins [s * d + i], maxes
 // [(nsets + s) * d + i]): a point outside its box, or a NaN, sets status bit kErrBox.
-static __global__ void __launch_bounds__(256) k_box_check_hd(const double *__restrict__ boxes, int nsets, int d,
-                                                            const int64_t *__restrict__ set_off,
-                                                            const unsigned long long *__restrict__ mm,
+static __global__ void __launch_bounds__(256) k_box_check_hd(const double *boxes, int nsets, int d,
+                                                            const int64_t *set_off,
+                                                            const unsigned long long *mm,
                                                             DevCounters *ctr) {
     pdl_enter();
     if (blockIdx.x == 0 && threadIdx.x == 0 && ctr->nan_seen) atomicOr(&ctr->status, kErrBox);
@@ -317,7 +317,7 @@ static __global__ void __launch_bounds__(256) k_box_check_hd(const double *__res
 // Per-dimension min / max of row-major n x d input (origin shift, Sec. 2).  Each thread keeps
 // one dimension (the stride is a multiple of d).
 template <typename T>
-__global__ void __launch_bounds__(256) k_minmax_rt(const T *__restrict__ in, int64_t n, int d, DevCounters *ctr,
+__global__ void __launch_bounds__(256) k_minmax_rt(const T *in, int64_t n, int d, DevCounters *ctr,
                                                   unsigned long long *mm /* [2 * 64] */) {
     pdl_enter();
     // each thread walks one dimension (a stride that is a multiple of d), four independent
@@ -347,7 +347,7 @@ __global__ void __launch_bounds__(256) k_minmax_rt(const T *__restrict__ in, int
         for (; e + 3 * stride < total; e += 4 * stride) {
             T x[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = __ldg(in + e + u * stride);
+            for (int u = 0; u < 4; ++u) x[u] = ld_old(in + e + u * stride);
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
                 nan |= (x[u] != x[u]);
@@ -356,7 +356,7 @@ __global__ void __launch_bounds__(256) k_minmax_rt(const T *__restrict__ in, int
             }
         }
         for (; e < total; e += stride) {
-            const T x = __ldg(in + e);
+            const T x = ld_old(in + e);
             nan |= (x != x);
             mn[0] = x < mn[0] ? x : mn[0];
             mx[0] = x > mx[0] ? x : mx[0];
@@ -398,7 +398,7 @@ __device__ __forceinline__ void count_digits_end(uint32_t (&h)[8][256], int pass
 // Coarse cell keys from the three projected dimensions (Algorithm 1 on a grid of side >= eps),
 // with the radix digit counts of the sort that follows.
 template <typename T, typename K>
-__global__ void __launch_bounds__(256) k_bin_proj(const T *__restrict__ in, int d, int3 sel, GridParams g,
+__global__ void __launch_bounds__(256) k_bin_proj(const T *in, int d, int3 sel, GridParams g,
                                                  K *__restrict__ keys, uint32_t *__restrict__ digit_counts,
                                                  FillList fill) {
     pdl_enter();
@@ -412,7 +412,7 @@ __global__ void __launch_bounds__(256) k_bin_proj(const T *__restrict__ in, int 
         uint64_t key = 0;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            const double t = __dmul_rn(__dsub_rn((double)in[j * d + dims[i]], g.origin[i]), g.inv_side);
+            const double t = __dmul_rn(__dsub_rn((double)ld_old(in + j * d + dims[i]), g.origin[i]), g.inv_side);
             uint32_t c = (uint32_t)floor(t);
             if (c > g.ncell[i] - 1) c = g.ncell[i] - 1;
             key |= (uint64_t)c << g.shift[i];
@@ -429,10 +429,10 @@ __global__ void __launch_bounds__(256) k_bin_proj(const T *__restrict__ in, int 
 // filter on) writes the float copy of the rows, relative to the set's smallest coordinates (set
 // id above set_shift of the key; complements of their encodings at mm[set * 64 + i]).
 template <typename T, int DP, typename K>
-__global__ void __launch_bounds__(kTileThreads) k_cells_hd(const T *__restrict__ in, int d, CellsArgs<K> a,
+__global__ void __launch_bounds__(kTileThreads) k_cells_hd(const T *in, int d, CellsArgs<K> a,
                                                           T *__restrict__ pts, uint8_t *__restrict__ core,
                                                           uint8_t *__restrict__ cell_core, float *__restrict__ fpts,
-                                                          const unsigned long long *__restrict__ mm, int set_shift) {
+                                                          const unsigned long long *mm, int set_shift) {
     pdl_enter();
     constexpr int G = DP / 4;          // threads per row
     constexpr int R = 256 / G;         // rows per step of the block
@@ -448,7 +448,7 @@ __global__ void __launch_bounds__(kTileThreads) k_cells_hd(const T *__restrict__
             const T *src = in + (int64_t)o * d;
             T x[4];
 #pragma unroll
-            for (int u = 0; u < 4; ++u) x[u] = 4 * g + u < d ? src[4 * g + u] : T(0);
+            for (int u = 0; u < 4; ++u) x[u] = 4 * g + u < d ? ld_old(src + 4 * g + u) : T(0);
             T *dst = pts + j * DP + 4 * g;
             if (sizeof(T) == 4) {
                 *reinterpret_cast<float4 *>(dst) = make_float4((float)x[0], (float)x[1], (float)x[2], (float)x[3]);
@@ -460,7 +460,7 @@ __global__ void __launch_bounds__(kTileThreads) k_cells_hd(const T *__restrict__
                     float f[4];
 #pragma unroll
                     for (int u = 0; u < 4; ++u)
-                        f[u] = 4 * g + u < d ? (float)__dsub_rn((double)x[u], dec_double_dev(~__ldg(mm + set * 64 + 4 * g + u))) : 0.f;
+                        f[u] = 4 * g + u < d ? (float)__dsub_rn((double)x[u], dec_double_dev(~ld_old(mm + set * 64 + 4 * g + u))) : 0.f;
                     *reinterpret_cast<float4 *>(fpts + j * DP + 4 * g) = make_float4(f[0], f[1], f[2], f[3]);
                 }
             }
@@ -507,7 +507,7 @@ __device__ __forceinline__ uint32_t chunk_cell(const uint32_t *off, uint32_t C, 
     while (hi - lo > 1u) {
         const uint32_t step = (hi - lo + 31u) >> 5;
         const uint32_t piv = lo + lane * step;
-        const unsigned ok = __ballot_sync(0xffffffffu, piv < hi && __ldg(off + piv) <= t);
+        const unsigned ok = __ballot_sync(0xffffffffu, piv < hi && ld(off + piv) <= t);
         lo += (uint32_t)(31 - __clz(ok)) * step;  // the ok lanes are a prefix (off is nondecreasing)
         hi = min(hi, lo + step);
     }
@@ -598,12 +598,12 @@ __global__ void __launch_bounds__(256) k_cell_box_hd(HdView<T, DP> v) {
         for (int g0 = 0; g0 < DP; g0 += 4) {
             R x[4];
             if (sizeof(R) == 4) {
-                const float4 f = valid ? __ldg(reinterpret_cast<const float4 *>(pts + (uint64_t)p * DP + g0))
+                const float4 f = valid ? ld_old(reinterpret_cast<const float4 *>(pts + (uint64_t)p * DP + g0))
                                        : make_float4(0.f, 0.f, 0.f, 0.f);
                 x[0] = (R)f.x; x[1] = (R)f.y; x[2] = (R)f.z; x[3] = (R)f.w;
             } else {
 #pragma unroll
-                for (int i = 0; i < 4; ++i) x[i] = valid ? __ldg(pts + (uint64_t)p * DP + g0 + i) : (R)0;
+                for (int i = 0; i < 4; ++i) x[i] = valid ? ld_old(pts + (uint64_t)p * DP + g0 + i) : (R)0;
             }
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
@@ -849,7 +849,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_count_hd(HdView<T, DP> v) 
 // Four list entries of point p from entry i on.
 template <typename V>
 __device__ __forceinline__ uint4 list4(const V &v, uint32_t p, uint32_t i) {
-    return __ldg(reinterpret_cast<const uint4 *>(v.nl + (uint64_t)p * v.nl_k + i));
+    return ld(reinterpret_cast<const uint4 *>(v.nl + (uint64_t)p * v.nl_k + i));
 }
 
 // Union-find over points: every core point starts below the smallest core point on its list (an
@@ -1414,7 +1414,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_labels_hd(HdView<T, DP> v)
 // Batched calls: per-set min / max of every dimension (mm[set * 64 + i] complements of the min
 // encodings, mm[(nsets + set) * 64 + i] max encodings), by seg_minmax.
 template <typename T>
-__global__ void __launch_bounds__(256) k_minmax_rt_seg(const T *__restrict__ in, int64_t n, int d,
+__global__ void __launch_bounds__(256) k_minmax_rt_seg(const T *in, int64_t n, int d,
                                                       const int64_t *set_off, int nsets,
                                                       unsigned long long *mm, DevCounters *ctr) {
     pdl_enter();
@@ -1424,7 +1424,7 @@ __global__ void __launch_bounds__(256) k_minmax_rt_seg(const T *__restrict__ in,
 // Batched calls: coarse cell keys with the set id above them; each set projects on its own
 // three dimensions (GridParams::sel).
 template <typename T, typename K>
-__global__ void __launch_bounds__(256) k_bin_proj_seg(const T *__restrict__ in, int64_t n, int d,
+__global__ void __launch_bounds__(256) k_bin_proj_seg(const T *in, int64_t n, int d,
                                                      const int64_t *set_off, int nsets, const GridParams *gtab,
                                                      int key_bits, K *__restrict__ keys,
                                                      uint32_t *__restrict__ digit_counts, int total_bits, FillList fill) {
@@ -1440,7 +1440,7 @@ __global__ void __launch_bounds__(256) k_bin_proj_seg(const T *__restrict__ in, 
         uint64_t key = (uint64_t)set << key_bits;
 #pragma unroll
         for (int i = 0; i < 3; ++i) {
-            const double t = __dmul_rn(__dsub_rn((double)in[j * d + g.sel[i]], g.origin[i]), g.inv_side);
+            const double t = __dmul_rn(__dsub_rn((double)ld_old(in + j * d + g.sel[i]), g.origin[i]), g.inv_side);
             uint32_t c = (uint32_t)floor(t);
             if (c > g.ncell[i] - 1) c = g.ncell[i] - 1;
             key |= (uint64_t)c << g.shift[i];

@@ -237,8 +237,8 @@ __device__ __forceinline__ uint32_t hash_lookup(const uint64_t *hkeys, const uin
                                                 uint32_t mask, uint64_t key) {
     uint32_t h = (uint32_t)mix64(key) & mask;
     for (uint32_t it = 0; it <= mask; ++it) {
-        uint64_t k = __ldg(hkeys + h);
-        if (k == key) return __ldg(hvals + h);
+        uint64_t k = ld(hkeys + h);
+        if (k == key) return ld(hvals + h);
         if (k == kEmptyKey) return 0xffffffffu;
         h = (h + 1) & mask;
     }
@@ -248,26 +248,26 @@ __device__ __forceinline__ uint32_t hash_lookup(const uint64_t *hkeys, const uin
 // The pencil of a key, ~0 when there is none.
 template <typename V>
 __device__ __forceinline__ uint32_t pencil_of(const V &v, uint64_t key) {
-    return v.ptab ? __ldg(v.ptab + key) : hash_lookup(v.hkeys, v.hvals, v.ctr->hash_mask, key);
+    return v.ptab ? ld(v.ptab + key) : hash_lookup(v.hkeys, v.hvals, v.ctr->hash_mask, key);
 }
 
 // First position in [a, e) of a pencil's cells (keys ascending) whose key is not below kt
 // (Upper: above kt).  A few linear steps first, since the bounds of consecutive cells of a
 // pencil move little, then a binary search over the rest.
 template <bool Upper>
-__device__ __forceinline__ uint32_t key_bound_from(const uint64_t *__restrict__ ck, uint32_t a, uint32_t e,
+__device__ __forceinline__ uint32_t key_bound_from(const uint64_t *ck, uint32_t a, uint32_t e,
                                                    uint64_t kt) {
 #pragma unroll
     for (int step = 0; step < 4; ++step) {
         if (a >= e) return a;
-        const uint64_t x = __ldg(ck + a);
+        const uint64_t x = ld(ck + a);
         if (Upper ? (x > kt) : (x >= kt)) return a;
         ++a;
     }
     uint32_t b = e;
     while (a < b) {
         const uint32_t m = (a + b) >> 1;
-        const uint64_t x = __ldg(ck + m);
+        const uint64_t x = ld(ck + m);
         if (Upper ? (x <= kt) : (x < kt)) a = m + 1;
         else b = m;
     }
@@ -442,8 +442,8 @@ __device__ __forceinline__ void add_counter(unsigned long long *ctr, uint32_t v)
 
 // Results to the host: up to two regions of words into the calling thread's pinned mailbox, then the
 // call's number, which the host waits for (mail_read).
-static __global__ void __launch_bounds__(256) k_mail(const uint32_t *__restrict__ a, uint32_t an, volatile uint32_t *to_a,
-                                                    const uint32_t *__restrict__ b, uint32_t bn, volatile uint32_t *to_b,
+static __global__ void __launch_bounds__(256) k_mail(const uint32_t *a, uint32_t an, volatile uint32_t *to_a,
+                                                    const uint32_t *b, uint32_t bn, volatile uint32_t *to_b,
                                                     volatile uint32_t *number, uint32_t value) {
     pdl_enter();
     for (uint32_t i = threadIdx.x; i < an; i += blockDim.x) to_a[i] = a[i];
@@ -466,7 +466,7 @@ struct VecPts {
 // whole group is in range and `vec_ok` (the input is 16-byte aligned), else element loads;
 // points past n read as zero.
 template <typename T, int D>
-__device__ __forceinline__ void load_pts(const T *__restrict__ in, int64_t j0, int64_t n, bool vec_ok,
+__device__ __forceinline__ void load_pts(const T *in, int64_t j0, int64_t n, bool vec_ok,
                                          T (&x)[VecPts<T, D>::pts * D]) {
     constexpr int P = VecPts<T, D>::pts, V = VecPts<T, D>::vec;
     if (vec_ok && j0 + P <= n) {
@@ -476,19 +476,19 @@ __device__ __forceinline__ void load_pts(const T *__restrict__ in, int64_t j0, i
             T e[P * D];
         } u;
 #pragma unroll
-        for (int k = 0; k < V; ++k) u.v[k] = __ldg(src + k);
+        for (int k = 0; k < V; ++k) u.v[k] = ld_old(src + k);
 #pragma unroll
         for (int k = 0; k < P * D; ++k) x[k] = u.e[k];
     } else {
 #pragma unroll
-        for (int k = 0; k < P * D; ++k) x[k] = j0 + k / D < n ? in[j0 * D + k] : T(0);
+        for (int k = 0; k < P * D; ++k) x[k] = j0 + k / D < n ? ld_old(in + j0 * D + k) : T(0);
     }
 }
 
 // Origin shift (Sec. 2): per-dimension min and max in the input's own precision, plus a NaN
 // check.  Each thread step reads VecPts::pts consecutive points with 16-byte loads.
 template <typename T, int D>
-__global__ void __launch_bounds__(256) k_minmax(const T *__restrict__ in, int64_t n, DevCounters *ctr) {
+__global__ void __launch_bounds__(256) k_minmax(const T *in, int64_t n, DevCounters *ctr) {
     pdl_enter();
     constexpr int P = VecPts<T, D>::pts;
     T mn[D], mx[D];
@@ -554,7 +554,7 @@ __global__ void __launch_bounds__(256) k_minmax(const T *__restrict__ in, int64_
 // key whose order is lexicographic in (c_0, ..., c_{d-1}).  Each thread step bins
 // VecPts::pts consecutive points read with 16-byte loads and stores their keys together.
 template <typename T, int D, typename K>
-__global__ void __launch_bounds__(256) k_bin(const T *__restrict__ in, GridParams g,
+__global__ void __launch_bounds__(256) k_bin(const T *in, GridParams g,
                                             K *__restrict__ keys, uint32_t *__restrict__ digit_counts,
                                             FillList fill) {
     pdl_enter();
@@ -619,7 +619,7 @@ __global__ void __launch_bounds__(256) k_bin(const T *__restrict__ in, GridParam
 // Gather the points into cell order, and the cells and pencils, one block per tile of
 // kScanTileElems points.
 template <typename T, int D, typename K>
-__global__ void __launch_bounds__(kTileThreads) k_cells(const T *__restrict__ in, CellsArgs<K> a,
+__global__ void __launch_bounds__(kTileThreads) k_cells(const T *in, CellsArgs<K> a,
                                                        Pt<T, D> *__restrict__ pts) {
     pdl_enter();
     const uint32_t tile = take_tile(a.l, 0u);
@@ -637,7 +637,7 @@ __global__ void __launch_bounds__(kTileThreads) k_cells(const T *__restrict__ in
             if (j >= a.n) continue;
             Pt<T, D> p = zero_pt<T, D>();
 #pragma unroll
-            for (int i = 0; i < D; ++i) p.x[i] = in[(int64_t)o[k] * D + i];
+            for (int i = 0; i < D; ++i) p.x[i] = ld_old(in + (int64_t)o[k] * D + i);
             pts[j] = p;
         }
     }, [](uint32_t) {});
@@ -655,8 +655,8 @@ static __global__ void __launch_bounds__(256) k_hash_init(uint64_t *__restrict__
     if (blockIdx.x == 0 && threadIdx.x == 0) ctr->hash_mask = cap - 1;
 }
 
-static __global__ void __launch_bounds__(256) k_pencils(const uint64_t *__restrict__ cell_key, int prefix_shift,
-                                                       const uint32_t *__restrict__ pencil_start, uint64_t *hkeys,
+static __global__ void __launch_bounds__(256) k_pencils(const uint64_t *cell_key, int prefix_shift,
+                                                       const uint32_t *pencil_start, uint64_t *hkeys,
                                                        uint32_t *hvals, DevCounters *ctr) {
     pdl_enter();
     const uint32_t P = ctr->n_pencils;
@@ -1526,7 +1526,7 @@ __device__ __forceinline__ uint32_t set_of_point(const int64_t *set_off, int nse
     int lo = 0, hi = nsets;  // last s with set_off[s] <= j
     while (hi - lo > 1) {
         const int mid = (lo + hi) >> 1;
-        if (__ldg(set_off + mid) <= j) lo = mid; else hi = mid;
+        if (ld_old(set_off + mid) <= j) lo = mid; else hi = mid;
     }
     return (uint32_t)lo;
 }
@@ -1538,9 +1538,9 @@ struct BoxArgs {
     double mn[kMaxD], mx[kMaxD];
 };
 template <int D>
-__global__ void __launch_bounds__(256) k_box_check(BoxArgs single, const double *__restrict__ boxes, int nsets,
-                                                  const int64_t *__restrict__ set_off,
-                                                  const unsigned long long *__restrict__ mm, DevCounters *ctr) {
+__global__ void __launch_bounds__(256) k_box_check(BoxArgs single, const double *boxes, int nsets,
+                                                  const int64_t *set_off,
+                                                  const unsigned long long *mm, DevCounters *ctr) {
     pdl_enter();
     if (blockIdx.x == 0 && threadIdx.x == 0 && ctr->nan_seen) atomicOr(&ctr->status, kErrBox);
     if (!boxes) {
@@ -1570,7 +1570,7 @@ __global__ void __launch_bounds__(256) k_box_check(BoxArgs single, const double 
 // lane and lane + 32 for larger d), and the warp folds them into the set's words with one
 // atomic per dimension at each set boundary and at the end of its run.
 template <typename T>
-__device__ __forceinline__ void seg_minmax(const T *__restrict__ in, int64_t n, int d, const int64_t *set_off,
+__device__ __forceinline__ void seg_minmax(const T *in, int64_t n, int d, const int64_t *set_off,
                                            int nsets, unsigned long long *mm, int stride, DevCounters *ctr) {
     const int lane = lane_id();
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1585,7 +1585,7 @@ __device__ __forceinline__ void seg_minmax(const T *__restrict__ in, int64_t n, 
     bool nan = false;
     if (j0 < j1) {
         uint32_t set = set_of_point(set_off, nsets, j0);
-        int64_t next = __ldg(set_off + set + 1);
+        int64_t next = ld_old(set_off + set + 1);
         T mn0 = big, mx0 = -big, mn1 = big, mx1 = -big;
         bool any = false;
         auto flush = [&]() {
@@ -1622,7 +1622,7 @@ __device__ __forceinline__ void seg_minmax(const T *__restrict__ in, int64_t n, 
             while (j >= next) {  // warp-uniform: the run enters the next non-empty set
                 flush();
                 ++set;
-                next = __ldg(set_off + set + 1);
+                next = ld_old(set_off + set + 1);
             }
             const int64_t stop = min(j1, next);
             if (stop - j >= 4 * g) {
@@ -1631,8 +1631,8 @@ __device__ __forceinline__ void seg_minmax(const T *__restrict__ in, int64_t n, 
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
                     const int64_t p = j + u * g + slot;
-                    x0[u] = lane_on && (d <= 32 || lane < d) ? __ldg(in + p * d + dim) : (T)0;
-                    x1[u] = d > 32 && lane + 32 < d ? __ldg(in + p * d + lane + 32) : (T)0;
+                    x0[u] = lane_on && (d <= 32 || lane < d) ? ld_old(in + p * d + dim) : (T)0;
+                    x1[u] = d > 32 && lane + 32 < d ? ld_old(in + p * d + lane + 32) : (T)0;
                 }
 #pragma unroll
                 for (int u = 0; u < 4; ++u) {
@@ -1655,19 +1655,19 @@ __device__ __forceinline__ void seg_minmax(const T *__restrict__ in, int64_t n, 
             const int64_t p = j + slot;
             if (lane_on && slot < take) {
                 if (d <= 32) {
-                    const T x = __ldg(in + p * d + dim);
+                    const T x = ld_old(in + p * d + dim);
                     nan |= (x != x);
                     mn0 = x < mn0 ? x : mn0;
                     mx0 = x > mx0 ? x : mx0;
                 } else {
                     if (lane < d) {
-                        const T x = __ldg(in + p * d + lane);
+                        const T x = ld_old(in + p * d + lane);
                         nan |= (x != x);
                         mn0 = x < mn0 ? x : mn0;
                         mx0 = x > mx0 ? x : mx0;
                     }
                     if (lane + 32 < d) {
-                        const T x = __ldg(in + p * d + lane + 32);
+                        const T x = ld_old(in + p * d + lane + 32);
                         nan |= (x != x);
                         mn1 = x < mn1 ? x : mn1;
                         mx1 = x > mx1 ? x : mx1;
@@ -1683,7 +1683,7 @@ __device__ __forceinline__ void seg_minmax(const T *__restrict__ in, int64_t n, 
 }
 
 template <typename T, int D>
-__global__ void __launch_bounds__(256) k_minmax_seg(const T *__restrict__ in, int64_t n, const int64_t *set_off,
+__global__ void __launch_bounds__(256) k_minmax_seg(const T *in, int64_t n, const int64_t *set_off,
                                                    int nsets, unsigned long long *mm, DevCounters *ctr) {
     pdl_enter();
     seg_minmax<T>(in, n, D, set_off, nsets, mm, kMaxD, ctr);
@@ -1691,7 +1691,7 @@ __global__ void __launch_bounds__(256) k_minmax_seg(const T *__restrict__ in, in
 
 // Algorithm 1 per set, with the set id above the cell key bits.
 template <typename T, int D, typename K>
-__global__ void __launch_bounds__(256) k_bin_seg(const T *__restrict__ in, int64_t n, const int64_t *set_off,
+__global__ void __launch_bounds__(256) k_bin_seg(const T *in, int64_t n, const int64_t *set_off,
                                                 int nsets, const GridParams *gtab, int key_bits,
                                                 K *__restrict__ keys, uint32_t *__restrict__ digit_counts,
                                                 int total_bits, FillList fill) {
@@ -1708,7 +1708,7 @@ __global__ void __launch_bounds__(256) k_bin_seg(const T *__restrict__ in, int64
         uint64_t key = (uint64_t)set << key_bits;
 #pragma unroll
         for (int i = 0; i < D; ++i) {
-            const T x = in[j * D + i];
+            const T x = ld_old(in + j * D + i);
             uint32_t c;
             if (sizeof(T) == 4 && !g.bin_fp64) {
                 float t = __fmul_rn(__fsub_rn((float)x, g.origin_f[i]), g.inv_side_f);

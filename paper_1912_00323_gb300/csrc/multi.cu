@@ -21,9 +21,9 @@ bool finite_pos(double x) { return x > 0.0 && x <= 1.7976931348623157e308; }
 // share their start with the next one; the search takes the last segment starting at or
 // before j, which is the non-empty one holding j.
 template <typename E>
-__global__ void __launch_bounds__(256) k_copy_segments(const E *__restrict__ src, E *__restrict__ dst,
-                                                       const int64_t *__restrict__ compact_start,
-                                                       const int64_t *__restrict__ far_start, int nseg,
+__global__ void __launch_bounds__(256) k_copy_segments(const E *src, E *__restrict__ dst,
+                                                       const int64_t *compact_start,
+                                                       const int64_t *far_start, int nseg,
                                                        int64_t total, int to_compact) {
     pdl_enter();
     const int64_t stride = (int64_t)gridDim.x * blockDim.x;

@@ -70,7 +70,7 @@ __device__ __forceinline__ uint64_t os_pack(uint32_t epoch, uint64_t state, uint
 
 // Digit counts of every pass: ghist[p * 256 + digit].
 template <typename K>
-__global__ void __launch_bounds__(kHistThreads) k_os_hist(const K *__restrict__ keys, int64_t n, int begin_bit,
+__global__ void __launch_bounds__(kHistThreads) k_os_hist(const K *keys, int64_t n, int begin_bit,
                                                          int end_bit, uint32_t *__restrict__ ghist) {
     pdl_enter();
     __shared__ uint32_t h[kMaxPasses][kRadix];
@@ -124,9 +124,9 @@ struct PassSmem {
 // IDENT: the values are the positions (first pass of a sort of indices; vals_in is not read).
 template <typename K, int ITEMS, int NT, bool IDENT>
 __global__ void __launch_bounds__(NT, kSortThreads / NT) k_os_pass(
-    const K *__restrict__ keys_in, const uint32_t *__restrict__ vals_in, K *__restrict__ keys_out,
+    const K *keys_in, const uint32_t *vals_in, K *__restrict__ keys_out,
     uint32_t *__restrict__ vals_out, int64_t n, int shift, int mask_bits,
-    const uint32_t *__restrict__ ghist_pass, unsigned long long *status, uint32_t *ticket, uint32_t epoch,
+    const uint32_t *ghist_pass, unsigned long long *status, uint32_t *ticket, uint32_t epoch,
     uint32_t *err, bool full_sum) {
     pdl_enter();
     constexpr int kSortItems = ITEMS, kSortTile = ITEMS * NT;

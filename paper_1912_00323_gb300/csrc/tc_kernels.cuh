@@ -431,8 +431,8 @@ __device__ __forceinline__ bool within_pts(const float *pts, uint32_t i, uint32_
 
 template <int MODE>
 __device__ __forceinline__ uint32_t row_point(const Tables &tt, uint32_t k) {
-    if (MODE == kCount) return tt.row_list ? __ldg(tt.row_list + k) : k;
-    return MODE == kMerge ? __ldg(tt.core_list + k) : __ldg(tt.nc_list + k);
+    if (MODE == kCount) return tt.row_list ? ld_old(tt.row_list + k) : k;
+    return MODE == kMerge ? ld_old(tt.core_list + k) : ld_old(tt.nc_list + k);
 }
 
 // Candidate u of the chunk's stream: the neighbour ranges laid end to end (list indices
@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
                     const uint32_t i = f / (DP / 2), r = f % (DP / 2);
                     const uint64_t c = S.bcell[i];
                     const float *src = r < DP / 4 ? v.box_lo + c * DP + 4 * r : v.box_hi + c * DP + 4 * (r - DP / 4);
-                    *reinterpret_cast<float4 *>(bx + (size_t)i * 2 * DP + 4 * r) = __ldg(reinterpret_cast<const float4 *>(src));
+                    *reinterpret_cast<float4 *>(bx + (size_t)i * 2 * DP + 4 * r) = ld(reinterpret_cast<const float4 *>(src));
                 }
                 __syncthreads();
                 if (have)
@@ -726,12 +726,12 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
             pre_k = pre_in ? span_off + u : 0u;
             // past the stream: list index 0 (a valid point), zeroed when staged; the loads are
             // not waited for here (no select on their values) but at the staging of the block
-            const uint32_t qp = MODE == kCount ? pre_k : __ldg(tt.core_list + pre_k);
+            const uint32_t qp = MODE == kCount ? pre_k : ld_old(tt.core_list + pre_k);
             const float4 *src = reinterpret_cast<const float4 *>(v.pts + (uint64_t)qp * DP);
 #pragma unroll
             for (int k = 0; k < DP / 4; ++k) q[k] = src[k];
             if (MODE == kMerge) pre_pay = __ldcg(v.parent + qp);  // an ancestor of qp
-            if (MODE == kLabels) pre_pay = __ldg(tt.core_lab + pre_k);
+            if (MODE == kLabels) pre_pay = ld(tt.core_lab + pre_k);
         };
         if (u0 < L) prefetch(u0);
         uint32_t la_r = 0;  // unions: look-ahead rounds of this item
@@ -762,7 +762,7 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
                             const uint32_t u = nb + (uint32_t)j * kTile + (uint32_t)tid;
                             if (u < L) {
                                 const uint32_t k2 = stream_index(S.rpre, S.rq0, nspan, u);
-                                const uint32_t x = __ldcg(v.parent + __ldcg(v.parent + __ldg(tt.core_list + k2)));
+                                const uint32_t x = __ldcg(v.parent + __ldcg(v.parent + ld_old(tt.core_list + k2)));
                                 if (x != ref) bad |= 1u << j;
                             }
                         }
@@ -891,7 +891,7 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
                             const uint32_t ck2 = S.cidx[col];
                             if (MODE == kMerge) {
                                 if (ck2 <= rk || S.cpay[col] == rp) continue;
-                                const uint32_t qp = __ldg(tt.core_list + ck2);
+                                const uint32_t qp = ld_old(tt.core_list + ck2);
                                 bool hit = inside;
                                 if (!hit) {
                                     ++n_re;
@@ -908,7 +908,7 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
                                 bool hit = inside;
                                 if (!hit) {
                                     ++n_re;
-                                    hit = within_pts<DP>(v.pts, p, __ldg(tt.core_list + ck2), G);
+                                    hit = within_pts<DP>(v.pts, p, ld_old(tt.core_list + ck2), G);
                                 }
                                 if (hit) best = lq;
                             }

@@ -1,5 +1,6 @@
 """Kernels that may be put in place early (pdl_enter) overlap the kernel before, whose output they read: no
-load of theirs may take the read-only path, which is for memory that nobody writes while the kernel lives."""
+load of that may take the read-only path, which is for memory that nobody writes while the kernel lives.  The
+read-only load (ld_old) is kept for what is written two or more kernels before any reader."""
 import os
 import re
 
@@ -25,6 +26,9 @@ def test_no_read_only_loads(name):
     src = _code(name)
     assert "__ldg(" not in src and "ld.global.nc" not in src
     assert not re.search(r"const\s+[\w:<>, ]+\*\s*__restrict__", src)
+    # the input and its gathered rows (or a pointer into them), the sets' tables, the lists of points
+    read = set(re.findall(r"ld_old\((?:reinterpret_cast<[^>]*>\()?\(?([\w.]+)", src))
+    assert read <= {"in", "src", "p", "a", "b", "pts", "mm", "set_off", "tt.row_list", "tt.core_list", "tt.nc_list"}
 
 
 @pytest.mark.parametrize("name", EARLY)
