@@ -19,7 +19,7 @@
 
 namespace hca {
 
-constexpr uint32_t kLookSpins = 1u << 24;
+constexpr uint32_t kLookSpins = HCA_LOOK_SPINS;
 constexpr int kTileThreads = 256;
 constexpr int kTileItems = kScanTileElems / kTileThreads;
 constexpr int kMaxScans = 16;  // scans (epochs 1 .. kMaxScans - 1) of one call; epoch 0: cleared words, the cells
@@ -87,10 +87,11 @@ __device__ __forceinline__ void look_publish(const LookBack &l, uint32_t epoch, 
 }
 
 // Sum of the earlier tiles' values, and the sum with this tile's published.  One full warp calls it
-// after look_publish; every lane returns the result.
+// after look_publish; every lane returns the result.  When the wait runs out kErrLook is set, ok is
+// false, nothing is published, and the tile writes nothing; so the later ones, which wait for it.
 template <bool PAIR>
 __device__ __forceinline__ unsigned long long look_back(const LookBack &l, uint32_t epoch, uint32_t tile,
-                                                        unsigned long long own, uint32_t *err) {
+                                                        unsigned long long own, uint32_t *err, bool &ok_all) {
     const int lane = threadIdx.x & 31;
     volatile unsigned long long *st = l.words;
     constexpr int kShift = PAIR ? 62 : 56;
@@ -100,6 +101,7 @@ __device__ __forceinline__ unsigned long long look_back(const LookBack &l, uint3
     unsigned long long sum = 0;
     int64_t base = (int64_t)tile - 1;
     uint32_t spins = 0;
+    ok_all = true;
     while (base >= 0) {
         const int64_t i = base - lane;
         const unsigned long long w = i >= 0 ? st[i] : (tag | kPrefix);
@@ -109,7 +111,8 @@ __device__ __forceinline__ unsigned long long look_back(const LookBack &l, uint3
         const unsigned take = first == 31 ? 0xffffffffu : (2u << first) - 1u;
         if ((okm & take) != take) {  // wait for the nearest ones
             if (++spins > kLookSpins) {
-                if (lane == 0) atomicOr(err, 2u);
+                if (lane == 0) atomicOr(err, kErrLook);
+                ok_all = false;
                 break;
             }
             continue;
@@ -121,8 +124,18 @@ __device__ __forceinline__ unsigned long long look_back(const LookBack &l, uint3
         if (pm) break;
         base -= 32;
     }
-    if (lane == 0 && tile > 0) st[tile] = tag | kPrefix | ((sum + own) & kValue);
+    if (lane == 0 && tile > 0 && ok_all) st[tile] = tag | kPrefix | ((sum + own) & kValue);
     return sum;
+}
+
+// The next tile, for the whole block; ok is false once a wait has run out (here or before).
+__device__ __forceinline__ uint32_t take_tile(const LookBack &l, uint32_t epoch, const uint32_t *err, bool &ok) {
+    __shared__ uint32_t s_tile, s_failed;
+    if (threadIdx.x == 0) s_tile = atomicAdd(l.tickets + epoch, 1u);
+    if (threadIdx.x == 32) s_failed = *(const volatile uint32_t *)err & kErrLook;  // (beside the ticket)
+    __syncthreads();
+    ok = s_failed == 0u;
+    return s_tile;
 }
 
 // out[i] = sum of f(0 .. i - 1) for i < m = min(*m_dev, m_max) (m_max without m_dev), emit(i, f(i),
@@ -134,11 +147,11 @@ __global__ void __launch_bounds__(kTileThreads) k_scan_fn(F f, E emit, uint32_t 
                                                          uint32_t epoch, uint32_t *err) {
     pdl_enter();
     __shared__ uint32_t s_val[kScanTileElems];
-    __shared__ uint32_t s_tile, s_base;
+    __shared__ uint32_t s_base, s_ok;
     const int64_t m = m_dev ? min((int64_t)*m_dev, m_max) : m_max;
-    if (threadIdx.x == 0) s_tile = atomicAdd(l.tickets + epoch, 1u);
-    __syncthreads();
-    const uint32_t tile = s_tile;
+    bool ok;
+    const uint32_t tile = take_tile(l, epoch, err, ok);
+    if (!ok) return;
     const int64_t base = (int64_t)tile * kScanTileElems;
     if (base >= m) {
         if (m == 0 && tile == 0 && threadIdx.x == 0 && total) *total = 0u;
@@ -162,13 +175,16 @@ __global__ void __launch_bounds__(kTileThreads) k_scan_fn(F f, E emit, uint32_t 
     uint32_t run = block_exclusive_scan<kTileThreads>(sum, &all);
     if (threadIdx.x < 32) {
         if (threadIdx.x == 0) look_publish<false>(l, epoch, tile, all);
-        const uint32_t b = (uint32_t)look_back<false>(l, epoch, tile, all, err);
+        bool found;
+        const uint32_t b = (uint32_t)look_back<false>(l, epoch, tile, all, err, found);
         if (threadIdx.x == 0) {
             s_base = b;
-            if (total && base + kScanTileElems >= m) *total = b + all;
+            s_ok = found;
+            if (found && total && base + kScanTileElems >= m) *total = b + all;
         }
     }
     __syncthreads();
+    if (!s_ok) return;
     run += s_base;
 #pragma unroll
     for (int k = 0; k < kTileItems; ++k) {
@@ -226,7 +242,7 @@ __device__ __forceinline__ void cells_tile(const CellsArgs<K> &a, uint32_t tile,
     constexpr int kWarps = kTileThreads / 32, kGroups = kTileItems * kWarps;  // 32-point groups
     static_assert(kGroups == 64, "two groups per lane of the scanning warp");
     __shared__ uint32_t s_cnt[kGroups];  // pencils << 16 | cells, then their exclusive sums
-    __shared__ uint32_t s_cells, s_pencils;
+    __shared__ uint32_t s_cells, s_pencils;  // (s_cells ~0: the look-back failed)
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int64_t base = (int64_t)tile * kScanTileElems;
     unsigned cb[kTileItems], pb[kTileItems];
@@ -263,14 +279,16 @@ __device__ __forceinline__ void cells_tile(const CellsArgs<K> &a, uint32_t tile,
     }
     between();
     if (warp == 0) {
-        const unsigned long long b = look_back<true>(a.l, 0u, tile, own, &a.ctr->status);
+        bool found;
+        const unsigned long long b = look_back<true>(a.l, 0u, tile, own, &a.ctr->status, found);
         if (lane == 0) {
-            s_cells = (uint32_t)(b & 0x7fffffffull);
+            s_cells = found ? (uint32_t)(b & 0x7fffffffull) : 0xffffffffu;
             s_pencils = (uint32_t)(b >> 31);
         }
     }
     __syncthreads();
     const uint32_t c0 = s_cells, p0 = s_pencils;
+    if (c0 == 0xffffffffu) return;
 #pragma unroll
     for (int k = 0; k < kTileItems; ++k) {
         const int64_t j = base + k * kTileThreads + threadIdx.x;
@@ -297,13 +315,6 @@ __device__ __forceinline__ void cells_tile(const CellsArgs<K> &a, uint32_t tile,
             a.ctr->n_pencils = p + 1;
         }
     }
-}
-
-__device__ __forceinline__ uint32_t take_tile(const LookBack &l, uint32_t epoch) {
-    __shared__ uint32_t s_tile;
-    if (threadIdx.x == 0) s_tile = atomicAdd(l.tickets + epoch, 1u);
-    __syncthreads();
-    return s_tile;
 }
 
 }  // namespace hca

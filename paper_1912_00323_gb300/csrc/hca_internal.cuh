@@ -21,6 +21,7 @@ constexpr uint32_t kLoopLimit = 1u << 22;  // cap of every loop that reads concu
 // device-side status word bits (HCA_EDEVICE when non-zero)
 constexpr uint32_t kErrHashFull = 1u;
 constexpr uint32_t kErrLoop = 2u;
+constexpr uint32_t kErrLook = 4u;  // a tile's wait for the earlier tiles ran out (sort, scans, cells)
 constexpr uint32_t kErrBox = 8u;   // a point lies outside the extents a plan declared
 
 // Base tuning (include/hca_dbscan.h): dimension-chosen neighbour search; tensor-core tiles
@@ -57,6 +58,21 @@ struct DevCounters {
     unsigned long long tc_pairs;  // point pairs of the tensor-core tiles computed
     uint32_t digit_counts[8 * 256];  // radix digit counts per pass, filled while binning
 };
+
+// After kErrLook the tables that a sort or scan left are incomplete: permutations, offsets and counts
+// of memory that nobody wrote.  The kernels that follow find nothing to do: every count that they take
+// from such a table is read through unless_failed (one more word of the counters' first line, read
+// along with the count), and sorts and scans return at their start.
+__device__ __forceinline__ bool look_failed(const DevCounters *ctr) { return (ctr->status & kErrLook) != 0u; }
+__device__ __forceinline__ uint32_t unless_failed(const DevCounters *ctr, uint32_t count) {
+    const uint32_t status = ctr->status;
+    return (status & kErrLook) ? 0u : count;
+}
+
+// Polls of one word after which a tile's wait for an earlier tile gives up.
+#ifndef HCA_LOOK_SPINS
+#define HCA_LOOK_SPINS (1u << 24)
+#endif
 
 // Grid of hypercubes (Algorithm 1) and everything a kernel needs to bin, pack and compare.
 struct GridParams {
@@ -210,7 +226,8 @@ constexpr size_t sort_hist_elems(int64_t n) {
 // Ping-pongs between (keys, vals) and (keys_alt, vals_alt); returns true when the sorted
 // result ends up in the alternate buffers.  hist: sort_hist_size(n) uint32 of scratch
 // (8-byte aligned; cleared by the sort itself).  A bounded look-back wait that ran out sets
-// bit 2 of *err_out (device word; NULL: the status word inside hist, sort_status_word).
+// kErrLook in *err_out (device word; NULL: the status word inside hist, sort_status_word); the
+// passes after it return at once.
 // `partials` is not used by the sort (callers may pass NULL).
 inline size_t sort_hist_size(int64_t n) { return sort_hist_elems(n); }
 uint32_t *sort_status_word(uint32_t *hist, int64_t n);

@@ -437,8 +437,13 @@ __global__ void __launch_bounds__(kTileThreads) k_cells_hd(const T *in, int d, C
     constexpr int G = DP / 4;          // threads per row
     constexpr int R = 256 / G;         // rows per step of the block
     const int g = threadIdx.x % G, r0 = threadIdx.x / G;
-    const uint32_t tile = take_tile(a.l, 0u);
+    bool ok;
+    const uint32_t tile = take_tile(a.l, 0u, &a.ctr->status, ok);
     const int64_t base = (int64_t)tile * kScanTileElems;
+    if (!ok) {  // (what follows looks at the flags of all points)
+        for (int64_t j = base + threadIdx.x; j < min(base + kScanTileElems, a.n); j += kTileThreads) core[j] = 0;
+        return;
+    }
     cells_tile(a, tile, [&]() {
 #pragma unroll 4
         for (int k = 0; k < kScanTileElems / R; ++k) {
@@ -579,7 +584,7 @@ __global__ void __launch_bounds__(256) k_cell_box_hd(HdView<T, DP> v) {
     typedef typename BC::U U;
     constexpr int E = DP > 32 ? DP / 32 : 1;  // dimensions per lane in the atomics
     const int lane = lane_id();
-    const uint32_t C = v.ctr->n_cells, NC = v.ctr->n_chunks;
+    const uint32_t C = v.ctr->n_cells, NC = unless_failed(v.ctr, v.ctr->n_chunks);
     const uint32_t warps = (gridDim.x * blockDim.x) >> 5;
     U *lo = reinterpret_cast<U *>(v.box_lo), *hi = reinterpret_cast<U *>(v.box_hi);
     const R *pts = sizeof(R) == sizeof(T) ? reinterpret_cast<const R *>(v.pts) : reinterpret_cast<const R *>(v.fpts);
@@ -631,7 +636,7 @@ __global__ void __launch_bounds__(256) k_cell_box_decode(HdView<T, DP> v) {
     pdl_enter();
     typedef BoxCode<R> BC;
     typedef typename BC::U U;
-    const uint64_t m = (uint64_t)v.ctr->n_cells * DP;
+    const uint64_t m = (uint64_t)unless_failed(v.ctr, v.ctr->n_cells) * DP;
     U *lo = reinterpret_cast<U *>(v.box_lo), *hi = reinterpret_cast<U *>(v.box_hi);
     for (uint64_t i = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; i < m; i += (uint64_t)gridDim.x * blockDim.x) {
         reinterpret_cast<R *>(lo)[i] = BC::dec(lo[i]);
@@ -640,7 +645,7 @@ __global__ void __launch_bounds__(256) k_cell_box_decode(HdView<T, DP> v) {
 }
 
 #define HD_FOR_EACH_CHUNK(v, A, base, e, slot)                                                \
-    const uint32_t C_ = (v).ctr->n_cells, NC_ = (v).ctr->n_chunks;                           \
+    const uint32_t C_ = (v).ctr->n_cells, NC_ = unless_failed((v).ctr, (v).ctr->n_chunks);   \
     for (uint32_t t_ = next_chunk(&(v).ctr->hd_next[slot]); t_ < NC_;                        \
          t_ = next_chunk(&(v).ctr->hd_next[slot]))                                           \
         for (uint32_t A = chunk_cell((v).chunk_off, C_, t_), once_ = 1; once_; once_ = 0)    \
@@ -739,7 +744,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_count_hd(HdView<T, DP> v) 
     R *rows = reinterpret_cast<R *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
     const int lane = lane_id();
     uint32_t chunks = 0;
-    const uint32_t C = v.ctr->n_cells, N = SPILL ? min(v.ctr->hd_spill[0], v.sp_cap) : v.ctr->n_chunks;
+    const uint32_t C = v.ctr->n_cells, N = unless_failed(v.ctr, SPILL ? min(v.ctr->hd_spill[0], v.sp_cap) : v.ctr->n_chunks);
     ItemQueue items(SPILL ? &v.ctr->hd_spill_next[0] : &v.ctr->hd_next[0], N);
     while (items.next()) {
         const uint32_t item = items.cur;
@@ -860,7 +865,7 @@ template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_list_link(HdView<T, DP> v) {
     pdl_enter();
     // (the cells' trees and odd counts are cleared here too)
-    const uint32_t C = v.ctr->n_cells;
+    const uint32_t C = unless_failed(v.ctr, v.ctr->n_cells);
     for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
         v.cell_root[c] = kNoRoot;
         v.odd_cnt[c] = 0u;
@@ -988,7 +993,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_cell_link(HdView<T, DP> v)
     typedef typename Cand::Row R;
     R *rows = reinterpret_cast<R *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
     const int lane = lane_id();
-    const uint64_t N = (uint64_t)v.ctr->n_cells * v.n_half;  // one warp per cell and neighbour pencil
+    const uint64_t N = (uint64_t)unless_failed(v.ctr, v.ctr->n_cells) * v.n_half;  // one warp per cell and neighbour pencil
     for (uint64_t w = global_warp(); w < N; w += total_warps()) {
         const uint32_t A = (uint32_t)(w / v.n_half);
         const int kk = (int)(w % v.n_half);
@@ -1055,7 +1060,7 @@ template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_cell_odd(HdView<T, DP> v) {
     pdl_enter();
     const int lane = lane_id();
-    const uint32_t C = v.ctr->n_cells, NC = v.ctr->n_chunks, warps = (gridDim.x * blockDim.x) >> 5;
+    const uint32_t C = v.ctr->n_cells, NC = unless_failed(v.ctr, v.ctr->n_chunks), warps = (gridDim.x * blockDim.x) >> 5;
     for (uint32_t t = (blockIdx.x * blockDim.x + threadIdx.x) >> 5; t < NC; t += warps) {
         const uint32_t A = chunk_cell(v.chunk_off, C, t);
         const uint32_t e = v.cell_start[A + 1], p = v.cell_start[A] + 32u * (t - v.chunk_off[A]) + lane;
@@ -1073,7 +1078,7 @@ constexpr uint32_t kOddMin = 8;
 template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_cell_mixed(HdView<T, DP> v) {
     pdl_enter();
-    const uint32_t C = v.ctr->n_cells;
+    const uint32_t C = unless_failed(v.ctr, v.ctr->n_cells);
     for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
         const uint32_t odd = v.odd_cnt[c];
         if (odd > kOddMin && odd > (v.cell_start[c + 1] - v.cell_start[c]) / 4u) v.cell_root[c] = kMixedRoot;
@@ -1099,7 +1104,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_odd_hd(HdView<T, DP> v) {
     R *rows = reinterpret_cast<R *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
     const int lane = lane_id();
     uint32_t chunks = 0;
-    const uint32_t C = v.ctr->n_cells, N = SPILL ? min(v.ctr->hd_spill[2], v.sp_cap) : v.ctr->n_chunks;
+    const uint32_t C = v.ctr->n_cells, N = unless_failed(v.ctr, SPILL ? min(v.ctr->hd_spill[2], v.sp_cap) : v.ctr->n_chunks);
     ItemQueue items(SPILL ? &v.ctr->hd_spill_next[2] : &v.ctr->hd_next[1], N);
     while (items.next()) {
         const uint32_t item = items.cur;
@@ -1170,9 +1175,11 @@ template <typename T, int DP>
 __global__ void __launch_bounds__(256) k_list_labels(HdView<T, DP> v, int core_too) {
     pdl_enter();
     uint32_t noise = 0;
+    const bool failed = look_failed(v.ctr);
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t p = (uint32_t)j;
         const bool isc = v.core[p];
+        if (failed) continue;
         if (isc && !core_too) continue;
         const uint32_t set = v.gtab ? set_of_key(v, v.cell_key[v.cell_of[p]]) : 0u;
         uint32_t best = kNoLabel;
@@ -1327,7 +1334,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_labels_hd(HdView<T, DP> v)
     R *rows = reinterpret_cast<R *>(smem_raw) + (threadIdx.x >> 5) * 32 * DP;
     const int lane = lane_id();
     uint32_t noise = 0, chunks = 0;
-    const uint32_t C = v.ctr->n_cells, N = SPILL ? min(v.ctr->hd_spill[1], v.sp_cap) : v.ctr->n_chunks;
+    const uint32_t C = v.ctr->n_cells, N = unless_failed(v.ctr, SPILL ? min(v.ctr->hd_spill[1], v.sp_cap) : v.ctr->n_chunks);
     ItemQueue items(SPILL ? &v.ctr->hd_spill_next[1] : &v.ctr->hd_next[3], N);
     while (items.next()) {
         const uint32_t item = items.cur;

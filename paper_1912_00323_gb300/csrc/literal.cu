@@ -100,7 +100,7 @@ __global__ void __launch_bounds__(256) k_lit_reps(const T *__restrict__ x, const
                                                  const uint32_t *__restrict__ cell_start,
                                                  const uint64_t *__restrict__ cell_key, const DevCounters *ctr,
                                                  LitParams p, uint32_t *__restrict__ rep) {
-    const uint64_t total = (uint64_t)ctr->n_cells * p.ndir;
+    const uint64_t total = (uint64_t)unless_failed(ctr, ctr->n_cells) * p.ndir;
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < total; t += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t c = (uint32_t)(t / p.ndir);
         const int r = (int)(t % p.ndir);
@@ -159,7 +159,7 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_lit_merge(const T *__restrict__ x, const uint64_t *__restrict__ cell_key,
                                                   DevCounters *ctr, LitParams p, const int8_t *__restrict__ offs,
                                                   const uint32_t *__restrict__ rep, uint32_t *parent) {
-    const uint32_t C = ctr->n_cells;
+    const uint32_t C = unless_failed(ctr, ctr->n_cells);
     const uint64_t total = (uint64_t)C * p.noff;
     for (uint64_t t = blockIdx.x * (uint64_t)blockDim.x + threadIdx.x; t < total; t += (uint64_t)gridDim.x * blockDim.x) {
         const uint32_t a = (uint32_t)(t / p.noff);
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(256) k_lit_merge(const T *__restrict__ x, cons
 }
 
 __global__ void __launch_bounds__(256) k_lit_uf_init(const DevCounters *ctr, uint32_t *parent, uint32_t *comp_min) {
-    const uint32_t C = ctr->n_cells;
+    const uint32_t C = unless_failed(ctr, ctr->n_cells);
     for (uint32_t c = blockIdx.x * blockDim.x + threadIdx.x; c < C; c += gridDim.x * blockDim.x) {
         parent[c] = c;
         comp_min[c] = 0xffffffffu;
@@ -203,6 +203,7 @@ __global__ void __launch_bounds__(256) k_lit_uf_init(const DevCounters *ctr, uin
 __global__ void __launch_bounds__(256) k_lit_comp_min(const uint32_t *__restrict__ cell_of, const uint32_t *__restrict__ idx,
                                                      int64_t n, DevCounters *ctr, const uint32_t *parent,
                                                      uint32_t *comp_min) {
+    if (look_failed(ctr)) return;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
         atomicMin(comp_min + uf_root_readonly(parent, cell_of[j], ctr), idx[j]);
 }
@@ -210,6 +211,7 @@ __global__ void __launch_bounds__(256) k_lit_comp_min(const uint32_t *__restrict
 __global__ void __launch_bounds__(256) k_lit_labels(const uint32_t *__restrict__ cell_of, const uint32_t *__restrict__ idx,
                                                    int64_t n, DevCounters *ctr, const uint32_t *parent,
                                                    const uint32_t *__restrict__ comp_min, int32_t *labels) {
+    if (look_failed(ctr)) return;
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < n; j += (int64_t)gridDim.x * blockDim.x)
         labels[idx[j]] = (int32_t)comp_min[uf_root_readonly(parent, cell_of[j], ctr)];
 }

@@ -622,7 +622,9 @@ template <typename T, int D, typename K>
 __global__ void __launch_bounds__(kTileThreads) k_cells(const T *in, CellsArgs<K> a,
                                                        Pt<T, D> *__restrict__ pts) {
     pdl_enter();
-    const uint32_t tile = take_tile(a.l, 0u);
+    bool ok;
+    const uint32_t tile = take_tile(a.l, 0u, &a.ctr->status, ok);
+    if (!ok) return;
     const int64_t base = (int64_t)tile * kScanTileElems;
     cells_tile(a, tile, [&]() {
         uint32_t o[kTileItems];
@@ -647,7 +649,7 @@ __global__ void __launch_bounds__(kTileThreads) k_cells(const T *in, CellsArgs<K
 // part (capacity = power of two >= 2 P), then insert.
 static __global__ void __launch_bounds__(256) k_hash_init(uint64_t *__restrict__ hkeys, DevCounters *ctr) {
     pdl_enter();
-    const uint32_t P = ctr->n_pencils;
+    const uint32_t P = unless_failed(ctr, ctr->n_pencils);
     uint32_t cap = 64;
     while (cap < 2u * P) cap <<= 1;
     for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < cap; i += gridDim.x * blockDim.x)
@@ -659,7 +661,7 @@ static __global__ void __launch_bounds__(256) k_pencils(const uint64_t *cell_key
                                                        const uint32_t *pencil_start, uint64_t *hkeys,
                                                        uint32_t *hvals, DevCounters *ctr) {
     pdl_enter();
-    const uint32_t P = ctr->n_pencils;
+    const uint32_t P = unless_failed(ctr, ctr->n_pencils);
     const uint32_t mask = ctr->hash_mask;
     for (uint32_t p = blockIdx.x * blockDim.x + threadIdx.x; p < P; p += gridDim.x * blockDim.x) {
         const uint64_t key = cell_key[pencil_start[p]] >> prefix_shift;
@@ -692,7 +694,7 @@ __global__ void __launch_bounds__(256) k_ranges(LowdView<T, D> v, Stencil st_in)
     pdl_enter();
     __shared__ Stencil st;
     load_stencil<T, D>(st, st_in);
-    const uint32_t C = v.ctr->n_cells;
+    const uint32_t C = unless_failed(v.ctr, v.ctr->n_cells);
     const int na = st.n_all;
     const uint64_t total = (uint64_t)((C + kRangeRun - 1) / kRangeRun) * na;
     const uint64_t last_mask = (1ull << v.g.bits[D - 1]) - 1ull;
@@ -782,9 +784,11 @@ struct WarpList {
 template <typename T, int D>
 __global__ void __launch_bounds__(256) k_triage(LowdView<T, D> v, int n_all) {
     pdl_enter();
-    const uint32_t C = v.ctr->n_cells;
+    const uint32_t C = unless_failed(v.ctr, v.ctr->n_cells);
     uint32_t noise = 0;
     const uint32_t stride = gridDim.x * blockDim.x;
+    if (C == 0u)  // (no cells after kErrLook: no point is core for those who ask every point)
+        for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += stride) v.core[j] = 0;
     for (uint32_t base = blockIdx.x * blockDim.x + (threadIdx.x & ~31u); base < C; base += stride) {
         const uint32_t A = base + lane_id();
         bool to_count = false, to_label = false;
@@ -1150,13 +1154,14 @@ __global__ void __launch_bounds__(256) k_rep_fix(LowdView<T, D> v, int64_t n) {
     using Geo = RepGeom<D, WIN>;
     constexpr int ndir = Geo::ndir;
     const int64_t nb = (n + Geo::sub - 1) / Geo::sub;
+    const bool failed = look_failed(v.ctr);
     for (int64_t idx = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; idx < nb * ndir;
          idx += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j = (idx / ndir) * Geo::sub;
         const int r = (int)(idx % ndir);
         if (j == 0 || j >= n) continue;
         const uint32_t c = v.cell_of[j];
-        if (c != v.cell_of[j - 1] || !v.cell_core[c]) continue;
+        if (c != v.cell_of[j - 1] || failed || !v.cell_core[c]) continue;
         const uint64_t slot = (uint64_t)c * ndir + r;
         v.rep_pts[slot] = v.pts[(uint32_t)v.reps[slot]];
     }

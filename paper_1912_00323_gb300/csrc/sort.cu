@@ -57,7 +57,7 @@ constexpr int kRadix = kSortRadix;
 constexpr int kMaxPasses = kSortMaxPasses;
 constexpr int kLbWords = 16;                      // predecessors per thread per round trip
 constexpr int kHistThreads = 256;
-constexpr uint32_t kSpinLimit = 1u << 24;
+constexpr uint32_t kSpinLimit = HCA_LOOK_SPINS;
 // Up to this many tiles a tile sums the counts of all earlier tiles instead of the decoupled
 // look-back (at two million keys all ~150 tiles run at once, so the look-back finds no
 // published prefix and reads the same words over three round trips)
@@ -111,13 +111,22 @@ struct PassSmem {
     uint32_t lb_kind[kQuarters][kRadix];  // 0 window read through, 1 met a PREFIX, 2 met an unpublished word
     int32_t lb_next[kRadix];                // nearest predecessor not yet added, per digit (-1: done)
     uint2 wsum[kRadix / 32];                // digit starts: the warps' sums of the tile's and all counts
-    uint32_t tile_id, pad[3];
+    uint32_t tile_id, failed, pad[2];
     union {
         uint32_t wmask[kSortWarps][kRadix];   // ranking: per-warp lane masks of each digit
         K keys[tile];                       // then: the tile in digit order
     };
     uint32_t vals[tile];
 };
+
+// A pass in which a wait ran out leaves places of its output unwritten, with digits that were never
+// counted, so the passes after it are closed: their tickets start at kClosed, and every tile that takes
+// one returns.
+constexpr uint32_t kClosed = 0x80000000u;
+__device__ __forceinline__ void pass_failed(uint32_t *err, uint32_t *ticket, uint32_t epoch) {
+    atomicOr(err, kErrLook);
+    for (uint32_t q = epoch; q < (uint32_t)kMaxPasses; ++q) atomicOr(ticket + (q - epoch + 1u), kClosed);
+}
 
 // One pass: rank within the tile, publish the tile's digit counts, scatter the tile into
 // shared memory in digit order, look back for the counts of the earlier tiles, write out.
@@ -140,9 +149,13 @@ __global__ void __launch_bounds__(NT, kSortThreads / NT) k_os_pass(
         (&S.whist[0][0])[i] = 0;
         (&S.wmask[0][0])[i] = 0;
     }
-    if (threadIdx.x == 0) S.tile_id = atomicAdd(ticket, 1u);
+    if (threadIdx.x == 0) {
+        S.tile_id = atomicAdd(ticket, 1u);
+        S.failed = 0u;
+    }
     __syncthreads();
     const uint32_t tile = S.tile_id;
+    if (tile >= kClosed) return;
 
     const int64_t tbase = (int64_t)tile * kSortTile;
     const int64_t wbase = tbase + (int64_t)warp * (32 * kSortItems);
@@ -294,7 +307,7 @@ __global__ void __launch_bounds__(NT, kSortThreads / NT) k_os_pass(
                 uint32_t tries = 0;
                 while (((uint32_t)(w[u] >> 34)) != epoch || ((uint32_t)(w[u] >> 32) & 3u) == 0u) {
                     if (++tries > kSpinLimit) {
-                        atomicOr(err, 2u);
+                        S.failed = 1u;
                         break;
                     }
                     w[u] = st[(uint64_t)i * kRadix + dg];
@@ -348,7 +361,7 @@ __global__ void __launch_bounds__(NT, kSortThreads / NT) k_os_pass(
                 else if (kind == 2) stalled = true;
             }
             if (stalled && ++spins > kSpinLimit) {
-                atomicOr(err, 2u);
+                S.failed = 1u;
                 done = true;
             }
             next = done ? -1 : nj;
@@ -362,6 +375,10 @@ __global__ void __launch_bounds__(NT, kSortThreads / NT) k_os_pass(
         S.goff[dg] = gdig + excl - lst;  // (plus the place in the tile; modulo 2^32)
     }
     __syncthreads();
+    if (S.failed) {  // no places for this tile's keys
+        if (threadIdx.x == 0) pass_failed(err, ticket, epoch);
+        return;
+    }
     auto put = [&](uint32_t i) {
         const K key = S.keys[i];
         const uint32_t gpos = S.goff[(uint32_t)(key >> shift) & mask] + i;

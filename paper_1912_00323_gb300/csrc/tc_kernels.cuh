@@ -499,10 +499,10 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
     const TileDesc td = {smem_desc<KP>(smem_u32(S.a_hi)), smem_desc<KP>(smem_u32(S.a_lo)),
                          smem_desc<KP>(smem_u32(S.b_hi)), smem_desc<KP>(smem_u32(S.b_lo))};
     const bool recount = MODE == kCount && tt.row_list != nullptr;
-    const uint32_t C = v.ctr->n_cells, N0 = recount ? v.ctr->n_tc_recount : v.ctr->n_tc_chunks[MODE];
+    const uint32_t C = v.ctr->n_cells, N0 = unless_failed(v.ctr, recount ? v.ctr->n_tc_recount : v.ctr->n_tc_chunks[MODE]);
     uint32_t *const next = recount ? &v.ctr->tc_next_recount : &v.ctr->tc_next[MODE];
     const bool split = MODE == kMerge && N0 < kSplitBelow * gridDim.x;
-    const uint32_t NC = split ? N0 + v.ctr->n_tc_chunks[3] : N0;  // unions: first windows, then the rest
+    const uint32_t NC = split ? N0 + unless_failed(v.ctr, v.ctr->n_tc_chunks[3]) : N0;  // unions: first windows, then the rest
     const int n_rng = MODE == kMerge ? v.n_half : MODE == kCount ? v.n_all + kSpansExtra : v.n_all;
     uint32_t phase = 0;
     bool failed = false;  // CTA-uniform
@@ -1119,7 +1119,7 @@ template <int DP>
 __global__ void __launch_bounds__(256) k_tc_core_labels(HdView<float, DP> v, Tables tt, int nsets,
                                                        uint32_t *__restrict__ core_lab) {
     pdl_enter();
-    const uint32_t n_core = tt.cx[v.g.n];
+    const uint32_t n_core = unless_failed(v.ctr, tt.cx[v.g.n]);
     for (uint32_t k = blockIdx.x * blockDim.x + threadIdx.x; k < n_core; k += gridDim.x * blockDim.x) {
         const uint32_t j = tt.core_list[k];
         const uint32_t lab = v.comp_min[v.parent[j]];
