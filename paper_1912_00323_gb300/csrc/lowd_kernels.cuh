@@ -441,16 +441,19 @@ __device__ __forceinline__ void add_counter(unsigned long long *ctr, uint32_t v)
 // ------------------------------------------------------------------------------------------
 
 // Results to the host: up to two regions of words into the calling thread's pinned mailbox, then the
-// call's number, which the host waits for (mail_read).
+// call's number, which the host waits for (mail_read).  The barrier orders the block's words before
+// thread 0's fence, and the fence releases them with the number to the host.
 static __global__ void __launch_bounds__(256) k_mail(const uint32_t *a, uint32_t an, volatile uint32_t *to_a,
                                                     const uint32_t *b, uint32_t bn, volatile uint32_t *to_b,
                                                     volatile uint32_t *number, uint32_t value) {
     pdl_enter();
     for (uint32_t i = threadIdx.x; i < an; i += blockDim.x) to_a[i] = a[i];
     for (uint32_t i = threadIdx.x; i < bn; i += blockDim.x) to_b[i] = b[i];
-    __threadfence_system();
     __syncthreads();
-    if (threadIdx.x == 0) *number = value;
+    if (threadIdx.x == 0) {
+        __threadfence_system();
+        *number = value;
+    }
 }
 
 // Points per thread step of the streaming kernels (min/max, binning): the fewest consecutive

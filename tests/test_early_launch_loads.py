@@ -41,3 +41,12 @@ def test_early_kernels_wait_first(name):
             depth += {"(": 1, ")": -1}.get(src[j], 0)
             j += 1
         assert src[src.index("{", j) + 1:].lstrip().startswith("pdl_enter();"), m.group(1)
+
+
+def test_mail_number_is_released():
+    """The host takes the mailbox's words when it sees the number: the thread that stores the number fences at
+    system scope after the block's barrier."""
+    src = _code("lowd_kernels.cuh")
+    body = src[src.index("k_mail("):src.index("*number = value")]
+    after = body[body.rindex("__syncthreads();"):]
+    assert "if (threadIdx.x == 0)" in after and "__threadfence_system();" in after
