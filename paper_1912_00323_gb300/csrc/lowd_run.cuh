@@ -270,13 +270,17 @@ constexpr size_t kCountersRead = offsetof(DevCounters, digit_counts);
 // and a synchronisation take about 7 us longer, twice a call (10,000 points in 2-D 166 -> 152 us,
 // 8-D 309 -> 282, two million in 3-D 597 -> 584).  A call that runs
 // on for more than kMailWait is waited for by the synchronisation, in the way that the program chose
-// for its device; that also reports a stream that failed or cannot run (capture).
+// for its device; that also reports a stream that failed or cannot run (capture).  A program that
+// chose blocking or yielding waits has nothing but those.
 constexpr std::chrono::microseconds kMailWait(500);
 inline bool mail_read(Lane s, HostMail *m, const DevCounters *ctr, const void *ext, size_t ext_bytes) {
     const uint32_t value = ++m->sent;
     launch(k_mail, 1u, 256u, 0, s, (const uint32_t *)ctr, (uint32_t)(kCountersRead / 4), (uint32_t *)&m->counters,
            (const uint32_t *)ext, (uint32_t)(ext_bytes / 4), (uint32_t *)m->ext, &m->number, value);
     const volatile uint32_t *number = &m->number;
+    unsigned flags = 0;
+    if (cudaGetDeviceFlags(&flags) == cudaSuccess && (flags & (cudaDeviceScheduleBlockingSync | cudaDeviceScheduleYield)))
+        return cudaStreamSynchronize(s) == cudaSuccess && *number == value;
     const auto limit = std::chrono::steady_clock::now() + kMailWait;
     for (uint32_t it = 1; *number != value; ++it)
         if (!(it & 0xffu) && std::chrono::steady_clock::now() > limit) {
