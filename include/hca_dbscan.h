@@ -412,10 +412,10 @@ HCA_API int hca_autotune_batched(const void *d_points, int32_t dtype, int32_t n_
  * A batched call takes, per d group, at most this bound for the group's points plus a few
  * hundred bytes per set (more only through the power-of-two rounding of its hash table, below
  * 16 bytes per point), and a group whose sets are not consecutive also a compact copy of its
- * points, labels and core flags.  On the coarse grid up to 84 bytes per point of the bound are
- * neighbour lists; a call that cannot get them runs without (same labels, slower).  The paper has
- * no counterpart: the request server admits jobs
- * by this bound.  Needs no device.
+ * points, labels and core flags.  On the coarse grid up to 56 bytes per point of the bound are
+ * for the longest neighbour lists; a call that cannot get them runs with shorter ones (same labels,
+ * slower).  The paper has no counterpart: the request server admits jobs by this bound.  Needs no
+ * device.
  *   bytes  host, written on success.
  */
 HCA_API int hca_workspace_bytes(int64_t n, int32_t d, int32_t dtype, int32_t flags, int64_t *bytes);

@@ -319,7 +319,7 @@ extern "C" int hca_workspace_bytes(int64_t n, int32_t d, int32_t dtype, int32_t 
     a.n = n;
     a.d = d;
     a.eps = 1.0;
-    a.min_pts = 1;
+    a.min_pts = INT32_MAX;  // (the bound of any MINPTS)
     a.d_labels = nullptr;
     a.d_core = nullptr;
     a.stream = nullptr;

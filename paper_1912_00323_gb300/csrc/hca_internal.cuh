@@ -274,7 +274,7 @@ struct RunArgs {
     DevCounters *h_ext = nullptr;        // pinned host copy of the counters (nullptr: the thread's)
     void *h_stage = nullptr;             // pinned staging of the batched tables (deferred calls)
     bool deferred = false;               // no host synchronisation: the caller checks the status
-    bool no_lists = false;               // coarse grid: run without neighbour lists (no memory for them)
+    bool short_lists = false;            // coarse grid: neighbour lists no longer than the table space holds
     // optional outputs: the measured extents of a single-set call without declared extents
     // (host, 2 d values: d minima then d maxima), and the launch count and key bits of the call
     double *ext_out = nullptr;

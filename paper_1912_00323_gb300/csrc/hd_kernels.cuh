@@ -82,7 +82,7 @@ struct HdView {
     uint32_t sp_cap;
     // neighbour lists: entry i < min(nl_cnt[p], nl_k) of point p at nl[p * nl_k + i] is a point
     // within eps of p, or with kListNear set one that only the exact predicate can tell; nl_cnt
-    // counts all that were found (nl_k = 0: no lists)
+    // counts all that were found
     uint32_t *nl;
     uint32_t *nl_cnt;
     uint32_t nl_k;
@@ -107,6 +107,17 @@ inline uint32_t list_len(uint32_t min_pts) {
     uint32_t k = min_pts > 1 ? min_pts - 1 : 1;
     k = k < 8 ? 8 : k > kListMax ? kListMax : k;
     return (k + 3u) & ~3u;
+}
+
+// The lists take the space of the pencil table or hash (table_bytes, at least 24 bytes a point), which is
+// free once the neighbour ranges are known, and more where they need it.  Entries that fit without
+// more: 4 or, from 32 bytes a point on, 8.  Without memory for the whole lists a call runs with
+// those (labels by comparison for MINPTS above 5 or 9): 16-D clusters of a million points, MINPTS 20,
+// 2.44 -> 2.96 ms, 128 sets of mixed dimension 5.20 -> 6.00 (with no list at all 5.34 and 7.85).
+inline uint32_t list_len_within(uint32_t min_pts, size_t table_bytes, int64_t n) {
+    const size_t fit = table_bytes / (sizeof(uint32_t) * (size_t)n) & ~(size_t)3;
+    const uint32_t k = list_len(min_pts);
+    return fit < k ? (uint32_t)fit : k;
 }
 
 // A chunk scans the first kSpillWin candidates of its stream itself; what is left of a longer
@@ -843,7 +854,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_count_hd(HdView<T, DP> v) 
         if (decide) {
             const bool is_core = have && cnt >= min_pts;
             if (have) v.core[p] = is_core ? 1 : 0;
-            if (have && v.nl_k) v.nl_cnt[p] = cnt;
+            if (have) v.nl_cnt[p] = cnt;
             if (__any_sync(0xffffffffu, is_core) && lane == 0) v.cell_core[A] = 1;
         }
         __syncwarp();
@@ -873,7 +884,7 @@ __global__ void __launch_bounds__(256) k_list_link(HdView<T, DP> v) {
     for (int64_t j = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; j < v.g.n; j += (int64_t)gridDim.x * blockDim.x) {
         const uint32_t p = (uint32_t)j;
         uint32_t m = p;
-        bool use = v.nl_k && v.core[p];
+        bool use = v.core[p];
         if (use && v.tc_min[1] && !v.tc_hook) {
             const uint32_t A = v.cell_of[p];
             use = v.cx[v.cell_start[A + 1]] - v.cx[v.cell_start[A]] < v.tc_min[1];

@@ -154,20 +154,18 @@ struct HdLaunch {
 template <typename T, int DP, bool FILTER>
 void run_list_unions(HdView<T, DP> &hv, const HdLaunch &L, int &launches) {
     launch(k_list_link<T, DP>, L.gpts, 256, 0, L.s, hv);
-    if (hv.nl_k) {
-        launch(k_flatten_hd<T, DP>, L.gpts, 256, 0, L.s, hv);
-        launch(k_list_hook<T, DP>, L.gpts, 256, 0, L.s, hv);
-        launch(k_flatten_hd<T, DP>, L.gpts, 256, 0, L.s, hv);
-        launch(k_list_join<T, DP>, L.gpts, 256, 0, L.s, hv);
-        launch(k_cell_link<T, DP, FILTER>, L.gcell, L.block, L.smem, L.s, hv);
-    }
+    launch(k_flatten_hd<T, DP>, L.gpts, 256, 0, L.s, hv);
+    launch(k_list_hook<T, DP>, L.gpts, 256, 0, L.s, hv);
+    launch(k_flatten_hd<T, DP>, L.gpts, 256, 0, L.s, hv);
+    launch(k_list_join<T, DP>, L.gpts, 256, 0, L.s, hv);
+    launch(k_cell_link<T, DP, FILTER>, L.gcell, L.block, L.smem, L.s, hv);
     launch(k_flatten_hd<T, DP>, L.gpts, 256, 0, L.s, hv);
     launch(k_cell_root<T, DP>, L.gpts, 256, 0, L.s, hv);
     launch(k_cell_odd<T, DP>, L.gpts, 256, 0, L.s, hv);
     launch(k_cell_mixed<T, DP>, L.gpts, 256, 0, L.s, hv);
     launch(k_odd_hd<T, DP, false, FILTER>, L.gcell, L.block, L.smem, L.s, hv);
     launch(k_odd_hd<T, DP, true, FILTER>, L.gcell, L.block, L.smem, L.s, hv);
-    launches += hv.nl_k ? 12 : 7;
+    launches += 12;
 }
 
 // The three point phases on the CUDA cores: counts (Definition 2), unions (Definitions 3-5) and
@@ -336,7 +334,6 @@ int run_hd(const RunArgs &a) {
     const size_t o_flags = take(4 * n), o_odd = take(4 * n);
     const size_t o_cstart = take(4 * (n + 1)), o_ckey = take(8 * n);
     const size_t o_pend = take(4 * n), o_croot = take(4 * n), o_pstart = take(4 * (n + 1));
-    const size_t o_hk = take(8 * cap_max), o_hv = take(4 * cap_max);
     const size_t o_core = take(n), o_ccore = take(n);
     const size_t o_parent = take(4 * n), o_cmin = take(4 * n);
     const size_t o_ranges = take(sizeof(uint2) * 9 * (size_t)n);
@@ -361,12 +358,13 @@ int run_hd(const RunArgs &a) {
     const size_t o_tflags = take(4 * tc_n), o_cx = take(4 * (tc_n + 1));
     const size_t o_clist = take(4 * tc_n), o_nclist = take(4 * tc_n), o_clab = take(4 * tc_n);
     const size_t o_box = take(sizeof(double) * 2 * (size_t)d * nsets);
-    // the neighbour lists come last: without memory for them the call runs without
+    // the pencil table or hash and, from the counts on, in its place and beyond it the neighbour lists
     uint32_t max_min_pts = (uint32_t)a.min_pts;
     for (int i = 0; batched && i < nsets; ++i) max_min_pts = std::max(max_min_pts, (uint32_t)a.h_minpts[i]);
-    if (a.ws_query && !a.box_mn) max_min_pts = kListMax + 1;  // any MINPTS
-    const bool lists = !a.no_lists;
-    const size_t o_nl = take(lists ? sizeof(uint32_t) * list_len(max_min_pts) * (size_t)n : 0);
+    const size_t o_hk = take(8 * cap_max), o_hv = take(4 * cap_max), o_nl = o_hk;
+    const uint32_t nl_k = a.short_lists ? list_len_within(max_min_pts, off - o_hk, n) : list_len(max_min_pts);
+    const size_t nl_bytes = sizeof(uint32_t) * nl_k * (size_t)n;
+    if (nl_bytes > off - o_hk) take(nl_bytes - (off - o_hk));
     bool use_tc = tc_occ > 0;
     const bool boxed = a.box_mn != nullptr;
     const bool own_ws = a.ws_ext == nullptr;
@@ -380,9 +378,9 @@ int run_hd(const RunArgs &a) {
         ws = a.ws_ext;
     } else if (pool_alloc(&ws, off, s) != cudaSuccess || !ws) {
         cudaGetLastError();
-        if (!lists) return HCA_ENOMEM;
+        if (a.short_lists) return HCA_ENOMEM;
         RunArgs less = a;
-        less.no_lists = true;
+        less.short_lists = true;
         return run_hd<T, DP>(less);
     }
     char *b = (char *)ws;
@@ -677,14 +675,14 @@ int run_hd(const RunArgs &a) {
     hv.odd_cnt = (uint32_t *)(b + o_odd);
     hv.odd_mask = (uint32_t *)(b + o_pstart);
     hv.nl = (uint32_t *)(b + o_nl);
-    hv.nl_k = lists ? list_len(max_min_pts) : 0u;
+    hv.nl_k = nl_k;
     hv.nl_cnt = (uint32_t *)(b + (flipped ? o_ia : o_ib));
     L.s = s;
     L.gpts = gpts;
     L.gcell = gcell;
     L.block = hd_block;
     L.smem = smem;
-    L.list_labels = hv.nl_k && hv.nl_k + 1 >= max_min_pts;
+    L.list_labels = nl_k + 1 >= max_min_pts;
     // the chunks and the box of every coarse cell in all d dimensions (point-to-box distance bounds)
     {
         uint32_t *choff = (uint32_t *)(b + o_choff);

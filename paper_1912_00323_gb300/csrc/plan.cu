@@ -26,7 +26,7 @@ struct PlanPart {
     hca::GroupBuffers gb = {};
     hca::DevCounters *h = nullptr;   // pinned: the counters of the last launch
     void *stage = nullptr;           // pinned: per-set tables the graph copies to the device
-    bool no_lists = false;           // captured without neighbour lists (no memory for them)
+    bool short_lists = false;        // captured with short neighbour lists (no memory for more)
     int32_t flags = 0;               // HCA_FLAG_* of the captured call (no timing)
     int launches = 0;                // kernels the captured call launches
     int key_bits = 0;                // bits of its cell keys
@@ -75,7 +75,7 @@ hca::RunArgs part_args(const PlanPart &pt, const void *pts, int32_t *lab, uint8_
     a.tune = hca::tuning_for(pt.g.d);  // fixed into the graph
     a.box_mn = pt.g.box_mn.data();
     a.box_mx = pt.g.box_mx.data();
-    a.no_lists = pt.no_lists;
+    a.short_lists = pt.short_lists;
     if (pt.batched) {
         a.nsets = (int)pt.g.sets.size();
         a.h_off = pt.g.off.data();
@@ -160,7 +160,7 @@ int create(hca_plan **out, const void *d_points, int32_t dtype, bool batched, st
         if (pool_alloc(&pt.ws, pt.ws_bytes, p->cap) != cudaSuccess || !pt.ws) {
             cudaGetLastError();
             pt.ws = nullptr;
-            a.no_lists = pt.no_lists = true;
+            a.short_lists = pt.short_lists = true;
             rc = dispatch(a, dtype);
             if (rc) break;
             if (pool_alloc(&pt.ws, pt.ws_bytes, p->cap) != cudaSuccess || !pt.ws) {

@@ -961,7 +961,7 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
                         v.tc_pos[p] = 0u;
                     }
                     v.core[p] = undecided ? 2 : (is_core ? 1 : 0);
-                    if (v.nl_k) v.nl_cnt[p] = up;
+                    v.nl_cnt[p] = up;
                     if (is_core) v.cell_core[A] = 1;
                 }
             }
@@ -974,7 +974,7 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
             }
             const bool is_core = have && !handed && cnt >= G.min_pts;
             if (have) v.core[p] = handed ? 2 : (is_core ? 1 : 0);
-            if (have && v.nl_k) v.nl_cnt[p] = cnt_hi;
+            if (have) v.nl_cnt[p] = cnt_hi;
             // the unions of a cell may run on the CUDA cores (fewer core rows than points)
             if (__syncthreads_or(is_core) && tid == 0) v.cell_core[A] = 1;
         } else if (MODE == kLabels) {

@@ -1,0 +1,42 @@
+"""Coarse-grid calls and plans without memory for whole neighbour lists run with short ones in the space of the
+pencil table: same labels, and a workspace no larger than it was without lists."""
+import glob
+import os
+import subprocess
+
+import pytest
+
+from paper_1912_00323_gb300 import build
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+def _objects():
+    build.build()
+    objs = glob.glob(os.path.join(build.BUILD, "*.o"))
+    if len(objs) < len(build.SOURCES):
+        build.build(force=True)
+        objs = glob.glob(os.path.join(build.BUILD, "*.o"))
+    return sorted(objs)
+
+
+@pytest.mark.gpu
+def test_no_memory_for_lists(tmp_path):
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    exe = str(tmp_path / "scratch_limit")
+    subprocess.run([build._nvcc(), *build.ARCH, "-std=c++17", "-I", build.CSRC,
+                    os.path.join(ROOT, "tests", "device", "scratch_limit.cu"), *_objects(),
+                    "-Xlinker", "--wrap=_ZN3hca10pool_allocEPPvmP11CUstream_st", "-o", exe],
+                   check=True, capture_output=True, text=True)
+    r = subprocess.run([exe], capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and "FAIL" not in r.stdout, r.stdout + r.stderr
+
+
+@pytest.mark.parametrize("d,dtype,bytes_per_point", [(8, "float32", 360), (16, "float32", 456), (7, "float64", 416)])
+def test_bound_per_point(d, dtype, bytes_per_point):
+    """The lists share the table's space: 76 bytes a point became 28 to 52."""
+    import paper_1912_00323_gb300 as pkg
+    for n in (200_003, 1_000_000, 2 ** 20, 2 ** 20 + 1):
+        assert pkg.hca_workspace_bytes(n, d, dtype) < bytes_per_point * n
