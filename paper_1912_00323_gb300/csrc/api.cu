@@ -242,10 +242,11 @@ extern "C" int hca_dbscan_device_ex(const void *d_points, int32_t dtype, int64_t
     if (rc != HCA_OK) return rc;
     if (same && !c.plan) {
         // the call repeated: capture it with the extents it measured (a failure, e.g. no memory
-        // for a second workspace, only leaves the calls uncached)
+        // for a second workspace, only leaves the calls uncached; a graph with shorter neighbour
+        // lists than the direct call has would be slower than it)
         hca_plan *p = nullptr;
         if (plan_create_single(&p, d_points, dtype, n, d, eps, min_pts, ext.data(), ext.data() + d, d_labels,
-                               d_core, flags) == HCA_OK)
+                               d_core, flags, true) == HCA_OK)
             c.plan = p;
         cudaGetLastError();
     } else if (!same) {

@@ -289,10 +289,11 @@ hca_tuning tuning_for(int d);
 // driver cannot say (sort_static.cu).
 unsigned long long current_context_id();
 
-// A plan of one set with the given flags (plan.cu; hca_plan_create is this with flags 0).
+// A plan of one set with the given flags (plan.cu; hca_plan_create is this with flags 0).  Without
+// memory for whole neighbour lists it takes short ones, or with whole_lists fails.
 int plan_create_single(hca_plan **out, const void *d_points, int32_t dtype, int64_t n, int32_t d, double eps,
                        int32_t min_pts, const double *box_min, const double *box_max, int32_t *d_labels,
-                       uint8_t *d_core, int32_t flags);
+                       uint8_t *d_core, int32_t flags, bool whole_lists = false);
 
 // api.cu: argument checks, dispatch to the pipelines, and the clustering calls with an
 // explicit tuning.

@@ -102,7 +102,7 @@ void part_buffers(const PlanPart &pt, const void *d_points, int32_t dtype, int32
 }
 
 int create(hca_plan **out, const void *d_points, int32_t dtype, bool batched, std::vector<hca::SetGroup> &groups,
-           int32_t *d_labels, uint8_t *d_core, int32_t flags) {
+           int32_t *d_labels, uint8_t *d_core, int32_t flags, bool whole_lists) {
     using namespace hca;
     hca_plan *p = new hca_plan();
     int rc = HCA_OK;
@@ -160,6 +160,10 @@ int create(hca_plan **out, const void *d_points, int32_t dtype, bool batched, st
         if (pool_alloc(&pt.ws, pt.ws_bytes, p->cap) != cudaSuccess || !pt.ws) {
             cudaGetLastError();
             pt.ws = nullptr;
+            if (whole_lists) {
+                rc = HCA_ENOMEM;
+                break;
+            }
             a.short_lists = pt.short_lists = true;
             rc = dispatch(a, dtype);
             if (rc) break;
@@ -232,7 +236,7 @@ namespace hca {
 
 int plan_create_single(hca_plan **out, const void *d_points, int32_t dtype, int64_t n, int32_t d, double eps,
                        int32_t min_pts, const double *box_min, const double *box_max, int32_t *d_labels,
-                       uint8_t *d_core, int32_t flags) {
+                       uint8_t *d_core, int32_t flags, bool whole_lists) {
     if (!out) return HCA_EINVAL;
     *out = nullptr;
     if (!box_min || !box_max) return HCA_EINVAL;
@@ -253,7 +257,7 @@ int plan_create_single(hca_plan **out, const void *d_points, int32_t dtype, int6
     g.far_pts = {0};
     g.far_lab = {0};
     g.n = n;
-    return create(out, d_points, dtype, false, groups, d_labels, d_core, flags);
+    return create(out, d_points, dtype, false, groups, d_labels, d_core, flags, whole_lists);
 }
 
 }  // namespace hca
@@ -283,7 +287,7 @@ extern "C" int hca_plan_create_batched(hca_plan **out, const void *d_points, int
     if (n == 0 || !d_points || !d_labels) return HCA_EINVAL;
     const size_t esz = dtype == HCA_F32 ? 4 : 8;
     if (((uintptr_t)d_points) % esz || ((uintptr_t)d_labels) % 4) return HCA_EINVAL;
-    return create(out, d_points, dtype, true, groups, d_labels, d_core, 0);
+    return create(out, d_points, dtype, true, groups, d_labels, d_core, 0, false);
 }
 
 extern "C" int hca_plan_launch(hca_plan *plan, void *stream) {

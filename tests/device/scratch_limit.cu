@@ -97,6 +97,21 @@ static void run(int n, int d, int min_pts) {
               what + "its labels");
         hca_plan_destroy(p);
     }
+    if (longer) {
+        // the repeated call: the first two run directly with whole lists, the graph's workspace is refused,
+        // and the third runs directly again
+        hca_graph_cache_release();
+        g_refuse = 2;
+        g_above = 0;
+        bool all = true;
+        for (int k = 0; k < 3; ++k) {
+            rc = call(0, st);
+            all &= rc == HCA_OK && (size_t)st.workspace_bytes == whole && labels() == want;
+        }
+        check(all, what + "repeated calls without memory for a graph's lists");
+        g_refuse = -1;
+        hca_graph_cache_release();
+    }
     cudaFree(dx);
     cudaFree(dl);
 }
