@@ -231,7 +231,9 @@ typedef struct hca_server hca_server;
 
 /* Start a server on `device` with `workers` worker threads (1..16) and a device-memory budget
  * (bytes charged per job: its points and labels, the hca_workspace_bytes bound of its
- * workspace, and 16 bytes per point plus 1 KB of slack for sharing a call).  A job larger than
+ * workspace less the longest neighbour lists, and 16 bytes per point plus 1 KB of slack for
+ * sharing a call; a call whose lists the budget has room for when it starts is charged them too, any
+ * other runs with shorter ones).  A job larger than
  * the whole budget runs alone.  Each worker keeps its staging buffers for the points and labels
  * on the device from batch to batch, and its clustering workspace comes from the library's
  * pool, which keeps freed blocks for the next call; every intermediate (sorted grid,
@@ -414,7 +416,7 @@ HCA_API int hca_autotune_batched(const void *d_points, int32_t dtype, int32_t n_
  * 16 bytes per point), and a group whose sets are not consecutive also a compact copy of its
  * points, labels and core flags.  On the coarse grid up to 56 bytes per point of the bound are
  * for the longest neighbour lists; a call that cannot get them runs with shorter ones (same labels,
- * slower).  The paper has no counterpart: the request server admits jobs by this bound.  Needs no
+ * slower).  The paper has no counterpart; the request server's charges come from it.  Needs no
  * device.
  *   bytes  host, written on success.
  */

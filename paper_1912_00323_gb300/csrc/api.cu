@@ -133,7 +133,7 @@ int device_ex_tuned(const void *d_points, int32_t dtype, int64_t n, int32_t d, d
 
 int batched_tuned(const void *d_points, int32_t dtype, int32_t n_sets, const int64_t *offsets, int32_t d,
                   const double *eps, const int32_t *min_pts, int32_t *d_labels, uint8_t *d_core, void *stream,
-                  hca_stats *stats, int32_t flags, const hca_tuning &tune) {
+                  hca_stats *stats, int32_t flags, const hca_tuning &tune, bool short_lists) {
     if (n_sets < 1 || !offsets || !eps || !min_pts) return HCA_EINVAL;
     if (offsets[0] != 0) return HCA_EINVAL;
     for (int32_t i = 0; i < n_sets; ++i) {
@@ -166,6 +166,7 @@ int batched_tuned(const void *d_points, int32_t dtype, int32_t n_sets, const int
     a.h_eps = eps;
     a.h_minpts = min_pts;
     a.tune = tune;
+    a.short_lists = short_lists;
     return dispatch(a, dtype);
 }
 
@@ -309,7 +310,10 @@ extern "C" int hca_dbscan(const void *points, int32_t dtype, int64_t n, int32_t 
     return rc;
 }
 
-extern "C" int hca_workspace_bytes(int64_t n, int32_t d, int32_t dtype, int32_t flags, int64_t *bytes) {
+namespace hca {
+
+int workspace_bound(int64_t n, int32_t d, int32_t dtype, int32_t flags, int32_t min_pts, bool short_lists,
+                    int64_t *bytes) {
     if (!bytes) return HCA_EINVAL;
     if (n < 0 || n >= ((int64_t)1 << 31) || d < 1 || d > 64) return HCA_EINVAL;
     if (dtype != HCA_F32 && dtype != HCA_F64) return HCA_EINVAL;
@@ -320,7 +324,8 @@ extern "C" int hca_workspace_bytes(int64_t n, int32_t d, int32_t dtype, int32_t 
     a.n = n;
     a.d = d;
     a.eps = 1.0;
-    a.min_pts = INT32_MAX;  // (the bound of any MINPTS)
+    a.min_pts = min_pts;
+    a.short_lists = short_lists;
     a.d_labels = nullptr;
     a.d_core = nullptr;
     a.stream = nullptr;
@@ -332,6 +337,12 @@ extern "C" int hca_workspace_bytes(int64_t n, int32_t d, int32_t dtype, int32_t 
     const int rc = dispatch(a, dtype);
     if (rc == HCA_OK) *bytes = (int64_t)b;
     return rc;
+}
+
+}  // namespace hca
+
+extern "C" int hca_workspace_bytes(int64_t n, int32_t d, int32_t dtype, int32_t flags, int64_t *bytes) {
+    return workspace_bound(n, d, dtype, flags, INT32_MAX, false, bytes);  // (the bound of any MINPTS)
 }
 
 extern "C" int hca_radix_sort_pairs(void *d_keys, uint32_t *d_vals, int64_t n, int32_t key_bytes,

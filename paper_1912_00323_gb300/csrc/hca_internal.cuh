@@ -295,6 +295,11 @@ int plan_create_single(hca_plan **out, const void *d_points, int32_t dtype, int6
                        int32_t min_pts, const double *box_min, const double *box_max, int32_t *d_labels,
                        uint8_t *d_core, int32_t flags, bool whole_lists = false);
 
+// The workspace bound of hca_workspace_bytes for calls of at most min_pts; with short_lists, what a
+// call takes without memory for its whole neighbour lists (api.cu).
+int workspace_bound(int64_t n, int32_t d, int32_t dtype, int32_t flags, int32_t min_pts, bool short_lists,
+                    int64_t *bytes);
+
 // api.cu: argument checks, dispatch to the pipelines, and the clustering calls with an
 // explicit tuning.
 int dispatch(const RunArgs &a, int32_t dtype);
@@ -305,7 +310,7 @@ int device_ex_tuned(const void *d_points, int32_t dtype, int64_t n, int32_t d, d
                     const hca_tuning &tune, double *ext_out = nullptr);
 int batched_tuned(const void *d_points, int32_t dtype, int32_t n_sets, const int64_t *offsets, int32_t d,
                   const double *eps, const int32_t *min_pts, int32_t *d_labels, uint8_t *d_core, void *stream,
-                  hca_stats *stats, int32_t flags, const hca_tuning &tune);
+                  hca_stats *stats, int32_t flags, const hca_tuning &tune, bool short_lists = false);
 // multi.cu: batched calls with one d per set.  The sets are grouped by d (increasing d); a
 // group whose sets are consecutive in the caller's buffers runs in place, any other group is
 // gathered into a compact copy (points, labels, core flags, segment table) and scattered back.
@@ -338,11 +343,12 @@ void group_gather(const SetGroup &g, int32_t dtype, const void *d_points, const 
 void group_scatter(const SetGroup &g, const GroupBuffers &gb, int32_t *d_labels, uint8_t *d_core, cudaStream_t s);
 void add_stats(hca_stats &acc, const hca_stats &x);
 int run_group(const SetGroup &g, const void *d_points, int32_t dtype, int32_t *d_labels, uint8_t *d_core,
-              cudaStream_t s, hca_stats *stats, int32_t flags, const hca_tuning &tune);
+              cudaStream_t s, hca_stats *stats, int32_t flags, const hca_tuning &tune, bool short_lists = false);
 // tune_by_d: nullable, 64 tunings indexed by d - 1 (NULL: the table of tune.cu)
 int batched_mixed(const void *d_points, int32_t dtype, int32_t n_sets, const int64_t *offsets,
                   const int32_t *d_per_set, const double *eps, const int32_t *min_pts, int32_t *d_labels,
-                  uint8_t *d_core, void *stream, hca_stats *stats, int32_t flags, const hca_tuning *tune_by_d);
+                  uint8_t *d_core, void *stream, hca_stats *stats, int32_t flags, const hca_tuning *tune_by_d,
+                  bool short_lists = false);
 
 template <typename T, int D>
 int run_lowd(const RunArgs &a);

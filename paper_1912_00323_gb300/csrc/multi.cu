@@ -180,12 +180,12 @@ void add_stats(hca_stats &acc, const hca_stats &x) {
 }
 
 int run_group(const SetGroup &g, const void *d_points, int32_t dtype, int32_t *d_labels, uint8_t *d_core,
-              cudaStream_t s, hca_stats *stats, int32_t flags, const hca_tuning &tune) {
+              cudaStream_t s, hca_stats *stats, int32_t flags, const hca_tuning &tune, bool short_lists) {
     const size_t esz = dtype == HCA_F32 ? 4 : 8;
     if (!g.gather) {
         return batched_tuned((const char *)d_points + g.first_elem * esz, dtype, (int32_t)g.sets.size(),
                              g.off.data(), g.d, g.eps.data(), g.min_pts.data(), d_labels + g.first_point,
-                             d_core ? d_core + g.first_point : nullptr, s, stats, flags, tune);
+                             d_core ? d_core + g.first_point : nullptr, s, stats, flags, tune, short_lists);
     }
     void *buf = nullptr;
     const bool with_core = d_core != nullptr;
@@ -201,7 +201,7 @@ int run_group(const SetGroup &g, const void *d_points, int32_t dtype, int32_t *d
     if (rc == HCA_OK) {
         group_gather(g, dtype, d_points, gb, s);
         rc = batched_tuned(gb.points, dtype, (int32_t)g.sets.size(), g.off.data(), g.d, g.eps.data(),
-                           g.min_pts.data(), gb.labels, gb.core, s, stats, flags, tune);
+                           g.min_pts.data(), gb.labels, gb.core, s, stats, flags, tune, short_lists);
     }
     if (rc == HCA_OK) {
         group_scatter(g, gb, d_labels, d_core, s);
@@ -215,7 +215,8 @@ int run_group(const SetGroup &g, const void *d_points, int32_t dtype, int32_t *d
 
 int batched_mixed(const void *d_points, int32_t dtype, int32_t n_sets, const int64_t *offsets,
                   const int32_t *d_per_set, const double *eps, const int32_t *min_pts, int32_t *d_labels,
-                  uint8_t *d_core, void *stream, hca_stats *stats, int32_t flags, const hca_tuning *tune_by_d) {
+                  uint8_t *d_core, void *stream, hca_stats *stats, int32_t flags, const hca_tuning *tune_by_d,
+                  bool short_lists) {
     std::vector<SetGroup> groups;
     int rc = group_sets(n_sets, offsets, d_per_set, eps, min_pts, nullptr, nullptr, groups);
     if (rc) return rc;
@@ -234,7 +235,7 @@ int batched_mixed(const void *d_points, int32_t dtype, int32_t n_sets, const int
         if (g.n == 0) continue;
         hca_stats st = {};
         const hca_tuning t = tune_by_d ? tune_by_d[g.d - 1] : tuning_for(g.d);
-        rc = run_group(g, d_points, dtype, d_labels, d_core, s, stats ? &st : nullptr, flags, t);
+        rc = run_group(g, d_points, dtype, d_labels, d_core, s, stats ? &st : nullptr, flags, t, short_lists);
         if (rc) return rc;
         if (stats) add_stats(*stats, st);
     }

@@ -2,9 +2,10 @@
 //
 // Jobs are queued by hca_submit.  Worker threads (each with its own CUDA stream) repeatedly
 // take every queued job that fits the device-memory budget (each charged its points, labels
-// and the hca_workspace_bytes bound of its workspace), group them by (d, dtype), stage each
+// and a bound of the workspace that it cannot do without), group them by (d, dtype), stage each
 // group's points into the worker's resident device buffer, cluster the group with one
-// hca_dbscan_batched call, copy each job's labels to its destination, and complete the jobs.  Jobs that arrive
+// batched call (with whole neighbour lists where the budget has room for them then, else with short
+// ones), copy each job's labels to its destination, and complete the jobs.  Jobs that arrive
 // while a batch is on the GPU join the next batch of a free worker, and the workers keep as many
 // batches in flight.  All waits on the host are condition-variable waits with deadlines.
 #include <algorithm>
@@ -43,14 +44,23 @@ namespace {
 using Clock = std::chrono::steady_clock;
 
 // Device memory a job is charged for: its points and labels in the worker's staging buffers
-// and the bound of hca_workspace_bytes on the clustering workspace, plus 16 bytes per point
+// and the bound on the clustering workspace with short neighbour lists, plus 16 bytes per point
 // for the power-of-two rounding of the hash table when jobs share a call and 1 KB for the
 // per-set tables.
 int64_t job_bytes(const hca_request &r) {
     const int64_t esz = r.dtype == HCA_F32 ? 4 : 8;
     int64_t ws = 0;
-    if (hca_workspace_bytes(r.n, r.d, r.dtype, 0, &ws) != HCA_OK) ws = r.n * 2048;
+    if (hca::workspace_bound(r.n, r.d, r.dtype, 0, r.min_pts, true, &ws) != HCA_OK) ws = r.n * 2048;
     return r.n * (r.d * esz + 4) + ws + 16 * r.n + 1024;
+}
+
+// What whole neighbour lists of a call add to that (0: they add nothing).
+int64_t list_bytes(int64_t n, int32_t d, int32_t dtype, int32_t min_pts) {
+    int64_t whole = 0, part = 0;
+    if (n <= 0 || hca::workspace_bound(n, d, dtype, 0, min_pts, false, &whole) != HCA_OK ||
+        hca::workspace_bound(n, d, dtype, 0, min_pts, true, &part) != HCA_OK)
+        return 0;
+    return whole > part ? whole - part : 0;
 }
 
 // Device buffers a worker keeps from batch to batch: the staged points and the labels of
@@ -92,6 +102,14 @@ void run_group(hca_server *sv, std::vector<int64_t> &ids, cudaStream_t s, Stagin
         mp[i] = reqs[i].min_pts;
     }
     const int64_t n = off.back();
+    int64_t extra = list_bytes(n, d, dtype, *std::max_element(mp.begin(), mp.end()));
+    bool short_lists = false;
+    if (extra > 0) {
+        std::lock_guard<std::mutex> lk(sv->mu);
+        short_lists = sv->in_flight + extra > sv->budget;
+        if (short_lists) extra = 0;
+        sv->in_flight += extra;
+    }
     int rc = HCA_OK;
     if (n > 0 && (!ensure(&stg.dp, &stg.dp_cap, (size_t)n * d * esz, s) ||
                   !ensure(&stg.dl, &stg.dl_cap, (size_t)n * 4, s)))
@@ -105,8 +123,8 @@ void run_group(hca_server *sv, std::vector<int64_t> &ids, cudaStream_t s, Stagin
             rc = HCA_ECUDA;
     }
     if (rc == HCA_OK && n > 0)
-        rc = hca_dbscan_batched(dp, dtype, (int32_t)reqs.size(), off.data(), dims.data(), eps.data(), mp.data(),
-                                (int32_t *)dl, nullptr, (void *)s, nullptr, 0);
+        rc = hca::batched_mixed(dp, dtype, (int32_t)reqs.size(), off.data(), dims.data(), eps.data(), mp.data(),
+                                (int32_t *)dl, nullptr, (void *)s, nullptr, 0, nullptr, short_lists);
     for (size_t i = 0; i < reqs.size() && rc == HCA_OK; ++i) {
         if (reqs[i].n == 0) continue;
         const cudaMemcpyKind kind = reqs[i].on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost;
@@ -117,6 +135,7 @@ void run_group(hca_server *sv, std::vector<int64_t> &ids, cudaStream_t s, Stagin
     const auto now = Clock::now();
     {
         std::lock_guard<std::mutex> lk(sv->mu);
+        sv->in_flight -= extra;
         for (int64_t id : ids) {
             hca_server::Job &j = sv->jobs[id];
             j.state = 2;

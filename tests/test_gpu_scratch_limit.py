@@ -40,3 +40,27 @@ def test_bound_per_point(d, dtype, bytes_per_point):
     import paper_1912_00323_gb300 as pkg
     for n in (200_003, 1_000_000, 2 ** 20, 2 ** 20 + 1):
         assert pkg.hca_workspace_bytes(n, d, dtype) < bytes_per_point * n
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("budget", [1, 64 << 20, 8 << 30])
+def test_server_budgets(budget):
+    """Jobs with whole lists, with short ones (a budget with no room for more, jobs larger than it alone) and
+    mixed: the labels of a call of their own."""
+    torch = pytest.importorskip("torch")
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    import numpy as np
+    import paper_1912_00323_gb300 as pkg
+    rng = np.random.default_rng(3)
+    jobs = []
+    for k in range(40):
+        d, n = [5, 9, 16, 3][k % 4], int(rng.integers(500, 30_000))
+        c = rng.uniform(0, 30, (n // 60 + 1, d)).repeat(60, axis=0)[:n]
+        X = np.round((c + rng.normal(size=(n, d)) * 0.5) * 64) / 64
+        jobs.append((X.astype(np.float32 if k % 3 else np.float64), 0.9 * d ** 0.5, [2, 6, 12, 21, 40][k % 5]))
+    with pkg.Server(hbm_budget_bytes=budget, workers=3) as sv:
+        tickets = [sv.submit(*j) for j in jobs]
+        got = [sv.wait(t)[0] for t in tickets]
+    for (X, eps, mp), lab in zip(jobs, got):
+        np.testing.assert_array_equal(lab, pkg.hca_dbscan(X, eps, mp))
