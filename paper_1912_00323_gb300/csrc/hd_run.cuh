@@ -569,9 +569,15 @@ int run_hd(const RunArgs &a) {
         if (rc) goto out;
         if (batched) cudaMemcpyAsync(d_gtab, gsets.data(), sizeof(GridParams) * nsets, cudaMemcpyHostToDevice, s);
     }
-    if (st.n_all > 16) {  // (cells of side eps (1 + 2^-10) have the 3 x 3 pencils around them)
-        rc = HCA_ENOTIMPL;
-        goto out;
+    {
+        // cells of side eps (1 + 2^-10) have the 3 x 3 x 3 block around them; the tensor-core tiles list
+        // these cells (kMaxRng), the views their pencils
+        int near_cells = 0;
+        for (int k = 0; k < st.n_all; ++k) near_cells += 2 * st.reach[k] + 1;
+        if (st.n_all > 9 || near_cells > 27) {
+            rc = HCA_ENOTIMPL;
+            goto out;
+        }
     }
     mark(1);
     // the filter's float copy of double input takes the half of the box space that float boxes

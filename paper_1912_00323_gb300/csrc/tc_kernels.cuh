@@ -298,7 +298,7 @@ struct Smem {
     uint32_t rpre[kMaxRng + 1];  // stream offset of each span; [kMaxRng] = stream length
     uint32_t bcell[kMaxRng];   // unions, labels: the neighbour cells, range by range
     uint32_t bnear[kMaxRng];   // 1: some row lies within eps of the cell's box
-    uint32_t nbc, bover;       // number of those cells; 1 if they did not fit (no pruning)
+    uint32_t nbc, pad2;        // number of those cells
     uint32_t cell, nwin;       // the item's coarse cell; unions: windows per chunk of it
     uint32_t la[3], pad3;      // unions: blocks of a look-ahead round not skippable (rotating)
     uint64_t mbar;
@@ -586,7 +586,6 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
         // no candidate of this chunk); the stream is one span per kept cell.  Counts keep the
         // whole ranges: the CUDA-core count resumes a handed-over row at a stream position.
         int nspan = n_rng;
-        bool by_cell = false;
         if (MODE != kCount) {
             if (warp == 0) {
                 // (unions: only the cells that still have something to join with A)
@@ -614,68 +613,57 @@ __global__ void __launch_bounds__(kTile, DP <= 16 ? 4 : 1) k_tc_hd(HdView<float,
                 S.bnear[tid] = 0u;
                 if (tid < 3) S.la[tid] = 0u;
                 if (tid == 0) {
-                    S.nbc = total < (uint32_t)kMaxRng ? total : (uint32_t)kMaxRng;
-                    S.bover = total > (uint32_t)kMaxRng ? 1u : 0u;
+                    S.nbc = min(total, (uint32_t)kMaxRng);  // (at most 27)
                 }
             }
             __syncthreads();
-            by_cell = S.bover == 0u;
-            if (by_cell) {
-                const uint32_t nbc = S.nbc;
-                // the boxes of the listed cells, loaded by all threads at once into b_lo (free
-                // until the first block is staged): cell i's lo at 2 DP i, its hi DP further
-                float *bx = S.b_lo;
-                for (uint32_t f = tid; f < nbc * (DP / 2); f += kTile) {
-                    const uint32_t i = f / (DP / 2), r = f % (DP / 2);
-                    const uint64_t c = S.bcell[i];
-                    const float *src = r < DP / 4 ? v.box_lo + c * DP + 4 * r : v.box_hi + c * DP + 4 * (r - DP / 4);
-                    *reinterpret_cast<float4 *>(bx + (size_t)i * 2 * DP + 4 * r) = ld(reinterpret_cast<const float4 *>(src));
-                }
-                __syncthreads();
-                if (have)
-                    for (uint32_t i = 0; i < nbc; ++i)
-                        if (!box_far_sh<DP>(q, bx + (size_t)i * 2 * DP, bx + (size_t)i * 2 * DP + DP, G)) S.bnear[i] = 1u;
-                __syncthreads();
-                if (warp == 0) {
-                    uint32_t q0 = 0, len = 0;
-                    bool keep = tid < (int)nbc && S.bnear[tid];
-                    if (keep) {
-                        const uint32_t c = S.bcell[tid];
-                        q0 = tt.cx[v.cell_start[c]];
-                        const uint32_t q1 = tt.cx[v.cell_start[c + 1]];
-                        if (MODE == kMerge && c == A) q0 = max(q0, k0);  // earlier rows pair from their side
-                        len = q1 > q0 ? q1 - q0 : 0u;
-                    }
-                    uint32_t incl = len;
-#pragma unroll
-                    for (int o = 1; o < 32; o <<= 1) {
-                        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-                        if (tid >= o) incl += y;
-                    }
-                    if (tid < (int)nbc) {
-                        S.rq0[tid] = q0;
-                        S.rpre[tid] = incl - len;
-                    }
-                    if (tid == 31) S.rpre[kMaxRng] = incl;  // stream length
-                }
-                nspan = (int)nbc;
+            const uint32_t nbc = S.nbc;
+            // the boxes of the listed cells, loaded by all threads at once into b_lo (free
+            // until the first block is staged): cell i's lo at 2 DP i, its hi DP further
+            float *bx = S.b_lo;
+            for (uint32_t f = tid; f < nbc * (DP / 2); f += kTile) {
+                const uint32_t i = f / (DP / 2), r = f % (DP / 2);
+                const uint64_t c = S.bcell[i];
+                const float *src = r < DP / 4 ? v.box_lo + c * DP + 4 * r : v.box_hi + c * DP + 4 * (r - DP / 4);
+                *reinterpret_cast<float4 *>(bx + (size_t)i * 2 * DP + 4 * r) = ld(reinterpret_cast<const float4 *>(src));
             }
+            __syncthreads();
+            if (have)
+                for (uint32_t i = 0; i < nbc; ++i)
+                    if (!box_far_sh<DP>(q, bx + (size_t)i * 2 * DP, bx + (size_t)i * 2 * DP + DP, G)) S.bnear[i] = 1u;
+            __syncthreads();
+            if (warp == 0) {
+                uint32_t q0 = 0, len = 0;
+                bool keep = tid < (int)nbc && S.bnear[tid];
+                if (keep) {
+                    const uint32_t c = S.bcell[tid];
+                    q0 = tt.cx[v.cell_start[c]];
+                    const uint32_t q1 = tt.cx[v.cell_start[c + 1]];
+                    if (MODE == kMerge && c == A) q0 = max(q0, k0);  // earlier rows pair from their side
+                    len = q1 > q0 ? q1 - q0 : 0u;
+                }
+                uint32_t incl = len;
+#pragma unroll
+                for (int o = 1; o < 32; o <<= 1) {
+                    const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
+                    if (tid >= o) incl += y;
+                }
+                if (tid < (int)nbc) {
+                    S.rq0[tid] = q0;
+                    S.rpre[tid] = incl - len;
+                }
+                if (tid == 31) S.rpre[kMaxRng] = incl;  // stream length
+            }
+            nspan = (int)nbc;
         }
-        // the candidate stream: one range per warp-0 lane, then a prefix over the ranges
-        if (warp == 0 && !by_cell) {
+        // counts: one span per warp-0 lane, then a prefix over the spans
+        if (MODE == kCount && warp == 0) {
             uint32_t q0 = 0, len = 0;
             if (tid < n_rng) {
-                uint2 rg = MODE == kCount ? stream_span(v, A, tid) : v.ranges[(uint64_t)A * v.n_all + tid];
-                if (MODE == kMerge && tid == 0) rg.x = A;  // own pencil: this cell and the ones after it
+                const uint2 rg = stream_span(v, A, tid);
                 if (rg.x < rg.y) {
                     q0 = v.cell_start[rg.x];
-                    uint32_t q1 = v.cell_start[rg.y];
-                    if (MODE != kCount) {
-                        q0 = tt.cx[q0];
-                        q1 = tt.cx[q1];
-                    }
-                    if (MODE == kMerge && tid == 0) q0 = max(q0, k0);  // earlier rows pair from their side
-                    len = q1 > q0 ? q1 - q0 : 0u;
+                    len = v.cell_start[rg.y] - q0;
                 }
             }
             uint32_t incl = len;
