@@ -365,10 +365,10 @@ extern "C" int hca_radix_sort_pairs(void *d_keys, uint32_t *d_vals, int64_t n, i
     bool flipped;
     if (key_bytes == 4)
         flipped = radix_sort_pairs<uint32_t>((uint32_t *)d_keys, d_vals, (uint32_t *)kalt, valt, n,
-                                             begin_bit, end_bit, h, nullptr, s, nullptr);
+                                             begin_bit, end_bit, h, s, nullptr);
     else
         flipped = radix_sort_pairs<uint64_t>((uint64_t *)d_keys, d_vals, (uint64_t *)kalt, valt, n,
-                                             begin_bit, end_bit, h, nullptr, s, nullptr);
+                                             begin_bit, end_bit, h, s, nullptr);
     int rc = HCA_OK;
     if (flipped) {
         if (cudaMemcpyAsync(d_keys, kalt, (size_t)n * key_bytes, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||

@@ -53,7 +53,7 @@ struct DevCounters {
     uint32_t hd_next[4];      // next unclaimed 32-point chunk: counts, odd rows, unions, labels
     uint32_t hd_spill[3];     // windows queued by the CUDA-core chunks: counts, labels, odd rows
     uint32_t hd_spill_next[3];  // next unclaimed window of each queue
-    uint32_t lowd_next[5];    // next unclaimed batch (labels: [4])
+    uint32_t lowd_next;       // next unclaimed cell of k_labels
     unsigned long long work[8];  // work counters (see hca_stats)
     unsigned long long tc_pairs;  // point pairs of the tensor-core tiles computed
     uint32_t digit_counts[8 * 256];  // radix digit counts per pass, filled while binning
@@ -228,7 +228,6 @@ constexpr size_t sort_hist_elems(int64_t n) {
 // (8-byte aligned; cleared by the sort itself).  A bounded look-back wait that ran out sets
 // kErrLook in *err_out (device word; NULL: the status word inside hist, sort_status_word); the
 // passes after it return at once.
-// `partials` is not used by the sort (callers may pass NULL).
 inline size_t sort_hist_size(int64_t n) { return sort_hist_elems(n); }
 uint32_t *sort_status_word(uint32_t *hist, int64_t n);
 // digit_counts (optional, device): counts of every 8-bit digit of every pass, [pass][256],
@@ -236,9 +235,9 @@ uint32_t *sort_status_word(uint32_t *hist, int64_t n);
 // are 0 .. n - 1 and vals need not hold them.
 template <typename K>
 bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, int64_t n,
-                      int begin_bit, int end_bit, uint32_t *hist, uint32_t *partials,
-                      Lane s, int *launches, uint32_t *err_out = nullptr,
-                      const uint32_t *digit_counts = nullptr, bool hist_cleared = false, bool identity = false);
+                      int begin_bit, int end_bit, uint32_t *hist, Lane s, int *launches,
+                      uint32_t *err_out = nullptr, const uint32_t *digit_counts = nullptr,
+                      bool hist_cleared = false, bool identity = false);
 
 // Pool allocation (stream ordered) used by api.cu and the pipelines.
 cudaError_t pool_alloc(void **p, size_t bytes, cudaStream_t s);

@@ -1178,12 +1178,11 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_odd_hd(HdView<T, DP> v) {
 }
 
 // Labels from complete lists (nl_k >= MINPTS - 1): a non-core point takes the smallest cluster id
-// among its listed core points, core points their cluster id when `core_too` (else they are
-// labelled elsewhere).  One thread per point: at most nl_k scattered loads of a byte, a tree
+// among its listed core points, a core point its cluster id.  One thread per point: at most nl_k scattered loads of a byte, a tree
 // and an id instead of the comparison with the whole neighbourhood (9-D call of 200,003 points
 // 3.50 -> 2.18 ms for the labels and unions from lists together).
 template <typename T, int DP>
-__global__ void __launch_bounds__(256) k_list_labels(HdView<T, DP> v, int core_too) {
+__global__ void __launch_bounds__(256) k_list_labels(HdView<T, DP> v) {
     pdl_enter();
     uint32_t noise = 0;
     const bool failed = look_failed(v.ctr);
@@ -1191,7 +1190,6 @@ __global__ void __launch_bounds__(256) k_list_labels(HdView<T, DP> v, int core_t
         const uint32_t p = (uint32_t)j;
         const bool isc = v.core[p];
         if (failed) continue;
-        if (isc && !core_too) continue;
         const uint32_t set = v.gtab ? set_of_key(v, v.cell_key[v.cell_of[p]]) : 0u;
         uint32_t best = kNoLabel;
         if (isc) {

@@ -192,7 +192,7 @@ void run_cuda_phases(HdView<T, DP> &hv, const HdLaunch &L, Mark &mark, int &laun
     mark(8);
     launch(k_comp_min_hd<T, DP>, L.gpts, 256, 0, L.s, hv);
     if (L.list_labels) {
-        launch(k_list_labels<T, DP>, L.gpts, 256, 0, L.s, hv, 1);
+        launch(k_list_labels<T, DP>, L.gpts, 256, 0, L.s, hv);
         launches += 6;
     } else {
         launch(k_labels_hd<T, DP, false, FILTER>, L.gcell, L.block, L.smem, L.s, hv);
@@ -277,7 +277,7 @@ void run_tc_phases(HdView<float, DP> &hv, const HdLaunch &L, char *b, int64_t n,
     launch(k_comp_min_hd<float, DP>, gpts, 256, 0, s, hv);
     if (L.list_labels) {
         tmark(4);
-        launch(k_list_labels<float, DP>, gpts, 256, 0, s, hv, 1);
+        launch(k_list_labels<float, DP>, gpts, 256, 0, s, hv);
         tmark(5);
         launches += 2;
         mark(9);
@@ -598,7 +598,7 @@ int run_hd(const RunArgs &a) {
             else
                 launch(k_bin_proj<T, K>, gpts, 256, 0, s, (const T *)a.d_points, d, sel, g, ka, ctr->digit_counts, fill);
             mark(2);
-            flipped = radix_sort_pairs<K>(ka, ia, kb, ib, n, 0, sort_bits, hist, nullptr, s, &launches, &ctr->status,
+            flipped = radix_sort_pairs<K>(ka, ia, kb, ib, n, 0, sort_bits, hist, s, &launches, &ctr->status,
                                           ctr->digit_counts, true, true);
             mark(3);
             CellsArgs<K> ca;

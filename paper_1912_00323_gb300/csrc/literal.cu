@@ -310,14 +310,14 @@ int run_literal(const T *d_points, int64_t n, double eps, int32_t *d_labels, cud
         if (key_bits <= 32) {
             uint32_t *ka = (uint32_t *)(b + o_ka), *kb = (uint32_t *)(b + o_kb);
             k_lit_bin<T, uint32_t><<<gpts, 256, 0, s>>>(d_points, n, p, ka, ia);
-            flipped = radix_sort_pairs<uint32_t>(ka, ia, kb, ib, n, 0, key_bits, hist, part, s, &launches, &ctr->status);
+            flipped = radix_sort_pairs<uint32_t>(ka, ia, kb, ib, n, 0, key_bits, hist, s, &launches, &ctr->status);
             const uint32_t *ks = flipped ? kb : ka;
             k_lit_flags<uint32_t><<<gtile, 256, 0, s>>>(ks, n, flags, part);
             cells_from_flags<uint32_t>(ks, flags, n, part, &ctr->n_cells, cstart, ckey, s, &launches);
         } else {
             uint64_t *ka = (uint64_t *)(b + o_ka), *kb = (uint64_t *)(b + o_kb);
             k_lit_bin<T, uint64_t><<<gpts, 256, 0, s>>>(d_points, n, p, ka, ia);
-            flipped = radix_sort_pairs<uint64_t>(ka, ia, kb, ib, n, 0, key_bits, hist, part, s, &launches, &ctr->status);
+            flipped = radix_sort_pairs<uint64_t>(ka, ia, kb, ib, n, 0, key_bits, hist, s, &launches, &ctr->status);
             const uint64_t *ks = flipped ? kb : ka;
             k_lit_flags<uint64_t><<<gtile, 256, 0, s>>>(ks, n, flags, part);
             cells_from_flags<uint64_t>(ks, flags, n, part, &ctr->n_cells, cstart, ckey, s, &launches);

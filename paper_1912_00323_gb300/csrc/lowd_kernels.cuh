@@ -1280,13 +1280,12 @@ __global__ void __launch_bounds__(256) k_flatten(LowdView<T, D> v) {
 }
 
 // Algorithm 3: merge every pair of neighbouring cells that hold core points and have a core
-// pair within eps.  Each unordered pair is visited once (upper half of the stencil).  Pass 0
-// takes the cells at Chebyshev offset 1, pass 1 the rest, pass 2 all of them; a pair already in
+// pair within eps.  Each unordered pair is visited once (upper half of the stencil); a pair already in
 // one set (after the flattened first links, most pairs of a cluster) is skipped.  The
 // complementary representative points are tested first (Algorithm 3); a miss falls back to the
 // exhaustive core x core test.  Lanes walk the flattened list of candidate cells of one cell.
 template <typename T, int D>
-__global__ void __launch_bounds__(kCellBlock) k_merge(LowdView<T, D> v, int n_all, int n_half, int pass) {
+__global__ void __launch_bounds__(kCellBlock) k_merge(LowdView<T, D> v, int n_all, int n_half) {
     pdl_enter();
     constexpr int ndir = RepDirs<D>::value;
     const int lane = lane_id();
@@ -1316,13 +1315,8 @@ __global__ void __launch_bounds__(kCellBlock) k_merge(LowdView<T, D> v, int n_al
                 int bc[D], delta[D];
                 if (pending) {
                     unpack_key<D>(bkey, v.g, bc);
-                    int cheb = 0;
 #pragma unroll
-                    for (int i = 0; i < D; ++i) {
-                        delta[i] = bc[i] - ac[i];
-                        cheb = max(cheb, abs(delta[i]));
-                    }
-                    pending = pass == 2 || (pass == 0) == (cheb <= 1);
+                    for (int i = 0; i < D; ++i) delta[i] = bc[i] - ac[i];
                 }
                 if (pending && uf_find(v.parent, A, v.ctr) == uf_find(v.parent, B, v.ctr)) pending = false;
                 if (pending) {
@@ -1420,7 +1414,7 @@ __global__ void __launch_bounds__(kCellBlock, 8) k_labels(LowdView<T, D> v, int 
     const int lane = lane_id();
     uint32_t noise = 0, chunks = 0;
     const uint32_t NL = v.ctr->n_list[2];
-    ItemQueue items(&v.ctr->lowd_next[4], NL);
+    ItemQueue items(&v.ctr->lowd_next, NL);
     while (items.next()) {
         const uint32_t A = v.list_label[items.cur];
         const uint32_t s = v.cell_start[A], e = v.cell_start[A + 1];

@@ -589,7 +589,7 @@ int run_lowd(const RunArgs &a) {
             else
                 launch(k_bin<T, D, K>, gpts, 256, 0, s, (const T *)a.d_points, g, ka, ctr->digit_counts, fill);
             mark(2);
-            flipped = radix_sort_pairs<K>(ka, ia, kb, ib, n, 0, sort_bits, hist, nullptr, s, &launches, &ctr->status,
+            flipped = radix_sort_pairs<K>(ka, ia, kb, ib, n, 0, sort_bits, hist, s, &launches, &ctr->status,
                                           ctr->digit_counts, true, true);
             mark(3);
             CellsArgs<K> ca;
@@ -669,7 +669,7 @@ int run_lowd(const RunArgs &a) {
     // ---- Algorithm 3: first links, flattened, then one merge pass over every pair ----
     launch(k_hook<T, D>, gwarp, kCellBlock, 0, s, v, st.n_all, st.n_half);
     launch(k_flatten<T, D>, gpts, 256, 0, s, v);
-    launch(k_merge<T, D>, gwarp, kCellBlock, 0, s, v, st.n_all, st.n_half, 2);
+    launch(k_merge<T, D>, gwarp, kCellBlock, 0, s, v, st.n_all, st.n_half);
     launches += 3;
     mark(8);
     // ---- Algorithm 4: cluster ids, border and noise ----

@@ -427,10 +427,8 @@ uint32_t *sort_status_word(uint32_t *hist, int64_t n) {
 
 template <typename K>
 bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, int64_t n,
-                      int begin_bit, int end_bit, uint32_t *hist, uint32_t *partials,
-                      Lane s, int *launches, uint32_t *err_out, const uint32_t *digit_counts,
-                      bool hist_cleared, bool identity) {
-    (void)partials;
+                      int begin_bit, int end_bit, uint32_t *hist, Lane s, int *launches,
+                      uint32_t *err_out, const uint32_t *digit_counts, bool hist_cleared, bool identity) {
     if (n <= 1 || end_bit <= begin_bit) {
         if (identity && n == 1) cudaMemsetAsync(vals, 0, sizeof(uint32_t), s);
         return false;
@@ -464,10 +462,10 @@ bool radix_sort_pairs(K *keys, uint32_t *vals, K *keys_alt, uint32_t *vals_alt, 
 }
 
 template bool radix_sort_pairs<uint32_t>(uint32_t *, uint32_t *, uint32_t *, uint32_t *, int64_t,
-                                         int, int, uint32_t *, uint32_t *, Lane, int *, uint32_t *,
+                                         int, int, uint32_t *, Lane, int *, uint32_t *,
                                          const uint32_t *, bool, bool);
 template bool radix_sort_pairs<uint64_t>(uint64_t *, uint32_t *, uint64_t *, uint32_t *, int64_t,
-                                         int, int, uint32_t *, uint32_t *, Lane, int *, uint32_t *,
+                                         int, int, uint32_t *, Lane, int *, uint32_t *,
                                          const uint32_t *, bool, bool);
 
 }  // namespace hca

@@ -115,10 +115,10 @@ extern "C" int hca_radix_sort_pairs_noalloc(void *d_keys, uint32_t *d_vals, int6
     bool flipped;
     if (key_bytes == 4)
         flipped = radix_sort_pairs<uint32_t>((uint32_t *)d_keys, d_vals, (uint32_t *)b, valt, n,
-                                             begin_bit, end_bit, hist, nullptr, s, nullptr);
+                                             begin_bit, end_bit, hist, s, nullptr);
     else
         flipped = radix_sort_pairs<uint64_t>((uint64_t *)d_keys, d_vals, (uint64_t *)b, valt, n,
-                                             begin_bit, end_bit, hist, nullptr, s, nullptr);
+                                             begin_bit, end_bit, hist, s, nullptr);
     rc = HCA_OK;
     if (flipped) {
         if (cudaMemcpyAsync(d_keys, b, (size_t)n * key_bytes, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||

@@ -286,7 +286,7 @@ static void after_failure() {
     run("k_cell_mixed", [&] { k_cell_mixed<float, 16><<<4, 256>>>(w.h); });
     run("k_odd_hd", [&] { k_odd_hd<float, 16, false, true><<<4, 128, smem>>>(w.h); });
     run("k_merge_hd", [&] { k_merge_hd<float, 16, true><<<4, 128, smem>>>(w.h); });
-    run("k_list_labels", [&] { k_list_labels<float, 16><<<4, 256>>>(w.h, 1); });
+    run("k_list_labels", [&] { k_list_labels<float, 16><<<4, 256>>>(w.h); });
     run("k_labels_hd", [&] { k_labels_hd<float, 16, false, true><<<4, 128, smem>>>(w.h); });
     run("k_tc_core_labels", [&] { tc::k_tc_core_labels<16><<<4, 256>>>(w.h, w.tt, 0, (uint32_t *)w.tt.core_lab); });
     const size_t tsm = tc::smem_bytes<16>();
