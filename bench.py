@@ -50,7 +50,7 @@ L2_FLUSH_BYTES = 256 << 20
 # DRAM traffic (dram__bytes_read.sum + dram__bytes_write.sum) of one radix sort pass
 # (k_os_pass) on the mixed3d workload at n = 2,000,000, from an ncu capture of that kernel;
 # None until a capture of the current kernel exists
-SORT_PASS_TRAFFIC_MIXED3D_2M = 16_050_000  # dram read + write per k_os_pass launch (ncu, mean of 4)
+SORT_PASS_TRAFFIC_MIXED3D_2M = 14_075_000  # dram read + write per k_os_pass launch (ncu, mean of 4: 8.07, 16.06, 16.11, 16.05 MB)
 
 # Nominal dense tensor-core rates of a GB300 (TFLOP/s): the TF32 peak of the tile kernel is the
 # measured bf16 GEMM rate scaled by their ratio
@@ -61,8 +61,9 @@ FP32_LANES_PER_SM, SMS = 128, 152
 
 # Algorithmic bytes per stage, per point (n) and per cell (C) / pencil (P): the data each
 # stage must move at least once (reads + writes), with 4-byte keys for <= 32 key bits.
-#   bin:   read the point (esz d), write key + index (key_bytes + 4)
-#   sort:  per radix pass read and write key + value (2 (key_bytes + 4))
+#   bin:   read the point (esz d), write its key (key_bytes)
+#   sort:  per radix pass read and write key + value (2 (key_bytes + 4)); the first pass reads no
+#          values (they are the positions)
 #   cells: read index (4) + the point (esz d), write the padded point + cell id (4);
 #          per cell write start (4) + key (8)
 #   reps:  read every point, its core flag and its cell id; per cell holding a core point read
@@ -74,9 +75,9 @@ def stage_bytes(stage, n, d, C, P, passes, key_bytes, core_cells=0, esz=4):
     if stage == "minmax":
         return n * pt
     if stage == "bin":
-        return n * (pt + key_bytes + 4)
+        return n * (pt + key_bytes)
     if stage == "sort":
-        return passes * n * 2 * (key_bytes + 4)
+        return passes * n * 2 * (key_bytes + 4) - 4 * n
     if stage == "cells":
         return n * (4 + pt + pad + 4) + C * 12
     if stage == "hash":
@@ -377,12 +378,13 @@ def single_config(pkg, torch, X, eps, min_pts, steps, warmup, flush, stream, pla
 
 def sort_roofline(stats, stage, n, peak, peak_kind, traffic):
     """The radix sort pass (k_os_pass, the largest kernel of the 3-D call): algorithmic bytes
-    per launch = n (key_bytes + 4) read + written; duration = the sort stage's CUDA-event time
+    per launch = n (key_bytes + 4) read + written, the first pass without reading the values,
+    the mean over the passes; duration = the sort stage's CUDA-event time
     over its passes (the stage holds only the passes and the clearing of their look-back words)."""
     key_bytes = 4 if stats["key_bits"] <= 32 else 8
     passes = max(1, stats["sort_passes"])
     per_launch_ms = stage["sort"] / passes
-    bytes_per_launch = n * 2 * (key_bytes + 4)
+    bytes_per_launch = n * 2 * (key_bytes + 4) - 4 * n / passes
     achieved = bytes_per_launch / (per_launch_ms / 1e3) / 1e9
     return {"bound": "hbm", "kernel": "k_os_pass (one radix pass of the cell-key sort)", "achieved": achieved,
             "peak": peak, "unit": "GB/s", "frac": achieved / peak, "traffic": traffic,
