@@ -130,9 +130,16 @@ struct Workspace {
 // launch: a call of 16 of them (2-D, 10,000 points) 197 -> 167 us, one of 34 (8-D, 3,001 points)
 // 362 -> 298 us.  Long ones lose: a block that comes early finds its SM divided into shared memory
 // and L1 as the kernel before needed it, the SM never drains in between, and the passes after
-// the sort run on what L1 the sort left.  Single 3-D sets: two million points 634 -> 599 us, 16
-// million 3.38 -> 4.49 ms; 128 sets in groups of 1.4 million 5.30 -> 5.55 ms; 16-D, one million
-// 2.64 -> 2.60 ms.  So up to two million points, batched or on the coarse grid up to one.
+// the sort run on what L1 the sort left.  Never -> always early:
+//   single 3-D sets of 100,000 points 336 -> 299 us, 500,000 402 -> 366, two million 634 -> 599, three
+//   million 752 -> 736, four million 978 -> 1175, 16 million 3.38 -> 4.49 ms; 2-D, five million 1437 ->
+//   1422 us; 4-D double, 500,000 942 -> 919: up to two million (the crossing lies between three and
+//   four million in 3-D and above five in 2-D)
+//   coarse grid: 9-D sets of 100,000 points 1061 -> 1004 us, 300,000 3.00 -> 3.01 ms, 600,000 6.41 -> 6.48,
+//   a million 13.56 -> 13.80; 16-D, a million 2.64 -> 2.60: up to a million
+//   64 sets in a call, 250,000 points in all: 2-D 368 -> 349 us, 3-D 603 -> 589, 8-D 791 -> 756; a million
+//   527 -> 488, 1003 -> 992, 1942 -> 1933; one and a half million 635 -> 604, 1153 -> 1176, 2712 -> 2797:
+//   up to a million
 constexpr int64_t kEarlyMax = 1 << 21, kEarlyMaxBatched = 1 << 20;
 struct Lane {
     cudaStream_t s;
@@ -203,9 +210,9 @@ void cells_from_flags(const K *keys, uint32_t *flags_cell_of, int64_t n, uint32_
 constexpr int kSortThreads = 1024;
 constexpr int kSortRadix = 256;
 constexpr int kSortMaxPasses = 8;
-// Keys per thread of a tile: 13 for large sorts, and below about two million keys the fewest of 2,
-// 4 and 8 that still leave one tile per SM (152) or less, so that the passes of a small sort are
-// spread over the chip and each tile ranks fewer keys in turn.
+// Keys per thread of a tile: 13 for large sorts, and up to 1,228,800 keys the fewest of 2, 4 and 8
+// that still leave 150 tiles or less (one per SM, with two SMs to spare), so that the passes of a
+// small sort are spread over the chip and each tile ranks fewer keys in turn.
 constexpr int sort_items_for(int64_t n) {
     return n <= 150 * kSortThreads * 2 ? 2 : n <= 150 * kSortThreads * 4 ? 4 : n <= 150 * kSortThreads * 8 ? 8 : 13;
 }

@@ -747,7 +747,7 @@ int run_hd(const RunArgs &a) {
         so->sort_passes = (sort_bits + 7) / 8;
         so->kernel_launches = launches;
         so->n_count_chunks = (int64_t)h->work[0];
-        so->n_rep_tests = (int64_t)h->work[1];   // hook-pass chunks in this path
+        so->n_rep_tests = (int64_t)h->work[1];   // candidate blocks of the odd points in this path
         so->n_rep_hits = (int64_t)h->work[2];    // tiles skipped because every root agreed
         so->n_exhaustive_pairs = (int64_t)h->work[3];
         so->n_exhaustive_chunks = (int64_t)h->work[4];

@@ -977,7 +977,10 @@ __global__ void __launch_bounds__(kCellBlock) k_core(LowdView<T, D> v, Stencil s
 // first, never a label.
 // Points per warp window: 64 (at 128 the window's shared memory leaves too few warps on an SM: 83
 // against 57 us at two million points); below kRepSmall points 32, since there are not enough
-// windows of 64 to fill the chip (18 -> 8 us at 10,000 points of d = 2).
+// windows of 64 to fill the chip (18 -> 8 us at 10,000 points of d = 2).  Stage with 64 -> 32: 3-D,
+// 100,000 points 18 -> 14 us, 350,000 25 -> 18, 500,000 27 -> 22, a million 37 -> 33, two million 57 -> 53,
+// eight million 182 -> 178; but 32 have twice the boundaries for k_rep_fix, and from three
+// million on the whole call is the same (752 and 751 us, 978 and 983, 1760 and 1756 at eight).
 constexpr uint32_t kRepWin = 64, kRepWinSmall = 32;
 constexpr int64_t kRepSmall = 500000;
 constexpr int kRepWarps = 4;          // warps per block

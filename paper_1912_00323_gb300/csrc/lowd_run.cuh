@@ -233,7 +233,8 @@ inline void collect_stencil(int D, double eps, double side, double tau, std::vec
 }
 
 // The calling thread's mailbox in pinned memory that kernels write to: the counters of a call, the
-// extents of up to kMailExt / 128 sets, and the number of the last message.
+// extents of up to 256 sets of d <= 4 (2 kMaxD words a set) or 16 on the coarse grid (128 words), and
+// the number of the last message.
 constexpr size_t kMailExt = 2048;
 struct HostMail {
     DevCounters counters;

@@ -462,7 +462,7 @@ __device__ __forceinline__ uint32_t stream_index(const uint32_t *rpre, const uin
 //            all of them if one saw an undecided pair); a row that ends with MINPTS between
 //            the tallies gets core[p] = 2, zero and zero.  The CUDA-core count continues them
 //            exactly.  With tt.row_list (the recount): rows = the handed-over rows of the cell,
-//            one item per window of kSegCand candidates; the tallies are summed over the
+//            one item per window of kRecountSeg candidates; the tallies are summed over the
 //            windows and the last window of a row decides it the same way.
 //   kMerge:  rows = core points, candidates = core points of the upper half of the
 //            neighbourhood after the row (each unordered pair once); a pair within eps whose
