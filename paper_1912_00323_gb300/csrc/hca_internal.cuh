@@ -54,9 +54,11 @@ struct DevCounters {
     uint32_t hd_spill[3];     // windows queued by the CUDA-core chunks: counts, labels, odd rows
     uint32_t hd_spill_next[3];  // next unclaimed window of each queue
     uint32_t lowd_next;       // next unclaimed cell of k_labels
-    unsigned long long work[8];  // work counters (see hca_stats)
+    // (lines of their own: beside the queue heads above, the work counters' atomics took k_labels of
+    // 250,000 points in 2-D 27.6 -> 29.1 us; digit counts that straddle sectors took k_bin 14.6 -> 16.5)
+    alignas(128) unsigned long long work[8];  // work counters (see hca_stats)
     unsigned long long tc_pairs;  // point pairs of the tensor-core tiles computed
-    uint32_t digit_counts[8 * 256];  // radix digit counts per pass, filled while binning
+    alignas(128) uint32_t digit_counts[8 * 256];  // radix digit counts per pass, filled while binning
 };
 
 // After kErrLook the tables that a sort or scan left are incomplete: permutations, offsets and counts
@@ -176,8 +178,9 @@ __device__ __forceinline__ void pdl_enter() {
 // a plain load.  What was written two or more kernels before is constant: the kernel before lets
 // this one in only after its own wait, when everything earlier is complete and visible.  The
 // input and the tables copied from the host are older still (a memset comes before the first
-// kernel of a call).  ld_old reads such data; plain loads, which the compiler keeps behind earlier
-// stores, took k_cells of 10,000 points 9.5 -> 11.4 us, the 7-D double call 623 -> 658 us.
+// kernel of a call).  ld_old reads such data, and the input's pointer has its __restrict__; plain
+// loads, which the compiler keeps behind earlier stores, took k_cells of 10,000 points 9.5 -> 11.4 us,
+// the 7-D double call 623 -> 658.
 template <typename T>
 __device__ __forceinline__ T ld(const T *p) { return *p; }
 template <typename T>

@@ -331,7 +331,7 @@ static __global__ void __launch_bounds__(256) k_box_check_hd(const double *boxes
 // Per-dimension min / max of row-major n x d input (origin shift, Sec. 2).  Each thread keeps
 // one dimension (the stride is a multiple of d).
 template <typename T>
-__global__ void __launch_bounds__(256) k_minmax_rt(const T *in, int64_t n, int d, DevCounters *ctr,
+__global__ void __launch_bounds__(256) k_minmax_rt(const T *__restrict__ in, int64_t n, int d, DevCounters *ctr,
                                                   unsigned long long *mm /* [2 * 64] */) {
     pdl_enter();
     // each thread walks one dimension (a stride that is a multiple of d), four independent
@@ -412,7 +412,7 @@ __device__ __forceinline__ void count_digits_end(uint32_t (&h)[8][256], int pass
 // Coarse cell keys from the three projected dimensions (Algorithm 1 on a grid of side >= eps),
 // with the radix digit counts of the sort that follows.
 template <typename T, typename K>
-__global__ void __launch_bounds__(256) k_bin_proj(const T *in, int d, int3 sel, GridParams g,
+__global__ void __launch_bounds__(256) k_bin_proj(const T *__restrict__ in, int d, int3 sel, GridParams g,
                                                  K *__restrict__ keys, uint32_t *__restrict__ digit_counts,
                                                  FillList fill) {
     pdl_enter();
@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(256) k_bin_proj(const T *in, int d, int3 sel, 
 // filter on) writes the float copy of the rows, relative to the set's smallest coordinates (set
 // id above set_shift of the key; complements of their encodings at mm[set * 64 + i]).
 template <typename T, int DP, typename K>
-__global__ void __launch_bounds__(kTileThreads) k_cells_hd(const T *in, int d, CellsArgs<K> a,
+__global__ void __launch_bounds__(kTileThreads) k_cells_hd(const T *__restrict__ in, int d, CellsArgs<K> a,
                                                           T *__restrict__ pts, uint8_t *__restrict__ core,
                                                           uint8_t *__restrict__ cell_core, float *__restrict__ fpts,
                                                           const unsigned long long *mm, int set_shift) {
@@ -1433,7 +1433,7 @@ __global__ void __launch_bounds__(32 * kHdMaxWarps) k_labels_hd(HdView<T, DP> v)
 // Batched calls: per-set min / max of every dimension (mm[set * 64 + i] complements of the min
 // encodings, mm[(nsets + set) * 64 + i] max encodings), by seg_minmax.
 template <typename T>
-__global__ void __launch_bounds__(256) k_minmax_rt_seg(const T *in, int64_t n, int d,
+__global__ void __launch_bounds__(256) k_minmax_rt_seg(const T *__restrict__ in, int64_t n, int d,
                                                       const int64_t *set_off, int nsets,
                                                       unsigned long long *mm, DevCounters *ctr) {
     pdl_enter();
@@ -1443,7 +1443,7 @@ __global__ void __launch_bounds__(256) k_minmax_rt_seg(const T *in, int64_t n, i
 // Batched calls: coarse cell keys with the set id above them; each set projects on its own
 // three dimensions (GridParams::sel).
 template <typename T, typename K>
-__global__ void __launch_bounds__(256) k_bin_proj_seg(const T *in, int64_t n, int d,
+__global__ void __launch_bounds__(256) k_bin_proj_seg(const T *__restrict__ in, int64_t n, int d,
                                                      const int64_t *set_off, int nsets, const GridParams *gtab,
                                                      int key_bits, K *__restrict__ keys,
                                                      uint32_t *__restrict__ digit_counts, int total_bits, FillList fill) {

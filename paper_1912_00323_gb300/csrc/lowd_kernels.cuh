@@ -469,7 +469,7 @@ struct VecPts {
 // whole group is in range and `vec_ok` (the input is 16-byte aligned), else element loads;
 // points past n read as zero.
 template <typename T, int D>
-__device__ __forceinline__ void load_pts(const T *in, int64_t j0, int64_t n, bool vec_ok,
+__device__ __forceinline__ void load_pts(const T *__restrict__ in, int64_t j0, int64_t n, bool vec_ok,
                                          T (&x)[VecPts<T, D>::pts * D]) {
     constexpr int P = VecPts<T, D>::pts, V = VecPts<T, D>::vec;
     if (vec_ok && j0 + P <= n) {
@@ -491,7 +491,7 @@ __device__ __forceinline__ void load_pts(const T *in, int64_t j0, int64_t n, boo
 // Origin shift (Sec. 2): per-dimension min and max in the input's own precision, plus a NaN
 // check.  Each thread step reads VecPts::pts consecutive points with 16-byte loads.
 template <typename T, int D>
-__global__ void __launch_bounds__(256) k_minmax(const T *in, int64_t n, DevCounters *ctr) {
+__global__ void __launch_bounds__(256) k_minmax(const T *__restrict__ in, int64_t n, DevCounters *ctr) {
     pdl_enter();
     constexpr int P = VecPts<T, D>::pts;
     T mn[D], mx[D];
@@ -557,7 +557,7 @@ __global__ void __launch_bounds__(256) k_minmax(const T *in, int64_t n, DevCount
 // key whose order is lexicographic in (c_0, ..., c_{d-1}).  Each thread step bins
 // VecPts::pts consecutive points read with 16-byte loads and stores their keys together.
 template <typename T, int D, typename K>
-__global__ void __launch_bounds__(256) k_bin(const T *in, GridParams g,
+__global__ void __launch_bounds__(256) k_bin(const T *__restrict__ in, GridParams g,
                                             K *__restrict__ keys, uint32_t *__restrict__ digit_counts,
                                             FillList fill) {
     pdl_enter();
@@ -622,7 +622,7 @@ __global__ void __launch_bounds__(256) k_bin(const T *in, GridParams g,
 // Gather the points into cell order, and the cells and pencils, one block per tile of
 // kScanTileElems points.
 template <typename T, int D, typename K>
-__global__ void __launch_bounds__(kTileThreads) k_cells(const T *in, CellsArgs<K> a,
+__global__ void __launch_bounds__(kTileThreads) k_cells(const T *__restrict__ in, CellsArgs<K> a,
                                                        Pt<T, D> *__restrict__ pts) {
     pdl_enter();
     bool ok;
@@ -1575,7 +1575,7 @@ __global__ void __launch_bounds__(256) k_box_check(BoxArgs single, const double 
 // lane and lane + 32 for larger d), and the warp folds them into the set's words with one
 // atomic per dimension at each set boundary and at the end of its run.
 template <typename T>
-__device__ __forceinline__ void seg_minmax(const T *in, int64_t n, int d, const int64_t *set_off,
+__device__ __forceinline__ void seg_minmax(const T *__restrict__ in, int64_t n, int d, const int64_t *set_off,
                                            int nsets, unsigned long long *mm, int stride, DevCounters *ctr) {
     const int lane = lane_id();
     const int64_t warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -1688,7 +1688,7 @@ __device__ __forceinline__ void seg_minmax(const T *in, int64_t n, int d, const 
 }
 
 template <typename T, int D>
-__global__ void __launch_bounds__(256) k_minmax_seg(const T *in, int64_t n, const int64_t *set_off,
+__global__ void __launch_bounds__(256) k_minmax_seg(const T *__restrict__ in, int64_t n, const int64_t *set_off,
                                                    int nsets, unsigned long long *mm, DevCounters *ctr) {
     pdl_enter();
     seg_minmax<T>(in, n, D, set_off, nsets, mm, kMaxD, ctr);
@@ -1696,7 +1696,7 @@ __global__ void __launch_bounds__(256) k_minmax_seg(const T *in, int64_t n, cons
 
 // Algorithm 1 per set, with the set id above the cell key bits.
 template <typename T, int D, typename K>
-__global__ void __launch_bounds__(256) k_bin_seg(const T *in, int64_t n, const int64_t *set_off,
+__global__ void __launch_bounds__(256) k_bin_seg(const T *__restrict__ in, int64_t n, const int64_t *set_off,
                                                 int nsets, const GridParams *gtab, int key_bits,
                                                 K *__restrict__ keys, uint32_t *__restrict__ digit_counts,
                                                 int total_bits, FillList fill) {
