@@ -305,7 +305,8 @@ HCA_API int hca_radix_sort_pairs_noalloc(void *d_keys, uint32_t *d_vals, int64_t
  * captured one after another into the one graph (gathering and scattering included), so
  * hca_plan_launch is one graph launch for all of them.
  * hca_plan_create[_batched] synchronises (it sizes and allocates the workspace and captures
- * the graph; no kernel runs).  hca_plan_launch enqueues one clustering on `stream` and returns.
+ * the graph; no kernel runs; on the coarse grid a plan without memory for whole neighbour lists
+ * gets shorter ones: same labels, slower).  hca_plan_launch enqueues one clustering on `stream` and returns.
  * hca_plan_wait synchronises `stream` and returns the launch's code: HCA_OK, HCA_ERANGE (a
  * point outside its box), HCA_EINVAL (a NaN coordinate) or HCA_EDEVICE; `stats` (nullable)
  * receives its counts (every field but the stage and tensor-core times).
