@@ -39,4 +39,4 @@ def test_blocking_waits():
     if not torch.cuda.is_available():
         pytest.skip("no CUDA device")
     spin, block = busy(1), busy(4)  # CU_CTX_SCHED_SPIN, CU_CTX_SCHED_BLOCKING_SYNC
-    assert spin > 0.9 and block < 0.25, (spin, block)  # (with the polls 0.39, without 0.08)
+    assert block < 0.25 and spin > 2 * block, (spin, block)  # (with the polls 0.39, without 0.08; spinning 1)
